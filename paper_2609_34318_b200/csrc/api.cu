@@ -1463,7 +1463,7 @@ int32_t fwd_core(Problem& pb, const void* q, const void* k, const void* v, int32
         // short pairs: one CTA per SM with two work items in flight, K and V in boxes of 64 keys
         CUtensorMap mv_sub;
         if (make_map(&mv_sub, v, pb.Tk, n_kv_heads, D_V, FWD_SHORT_KEYS)) return HYDRA_ERR_CUDA;
-        const int grid = std::min(sms, (plan->n_items2 + 1) / 2);
+        const int grid = std::min(sms, plan->n_items2);      // one item per SM before any SM gets two
         ScopedKernelTimer timer(K_FWD, stream);
         if (ks->launch_fwd_short(mq, mk, mv_sub, fp, grid, stream) != cudaSuccess) return HYDRA_ERR_CUDA;
         g_launches += 1;
@@ -1603,7 +1603,7 @@ int32_t bwd_run(const Problem& pb, int32_t n_kv_heads, int32_t causal, float sof
         bp.accumulate = accumulate_dkv ? 1 : 0;
         bp.debug_stall_ns = g_debug_stall_ns[HYDRA_STALL_BWD_DKV].load();
         ScopedKernelTimer timer(K_DKV, stream);
-        if (ks->launch_bwd_dkv(mq_sub, mk, mv, mdo_sub, bp, sms, stream) != cudaSuccess)
+        if (ks->launch_bwd_dkv(mq_sub, mk, mv, mdo_sub, bp, std::min(sms, bp.n_items), stream) != cudaSuccess)
             return HYDRA_ERR_CUDA;
         g_launches += 1;
     }
@@ -1614,8 +1614,9 @@ int32_t bwd_run(const Problem& pb, int32_t n_kv_heads, int32_t causal, float sof
         bp.accumulate = accumulate_dq ? 1 : 0;
         bp.debug_stall_ns = g_debug_stall_ns[HYDRA_STALL_BWD_DQ].load();
         ScopedKernelTimer timer(K_DQ, stream);
-        const cudaError_t e = hand_off ? ks->launch_bwd_dq_from_ds(mk, bp, sms, stream)
-                                       : ks->launch_bwd_dq(mq, mk, mv, mdo, bp, sms, stream);
+        const int grid = std::min(sms, bp.n_items);
+        const cudaError_t e = hand_off ? ks->launch_bwd_dq_from_ds(mk, bp, grid, stream)
+                                       : ks->launch_bwd_dq(mq, mk, mv, mdo, bp, grid, stream);
         if (e != cudaSuccess)
             return HYDRA_ERR_CUDA;
         g_launches += 1;

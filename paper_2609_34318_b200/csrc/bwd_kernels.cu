@@ -49,6 +49,9 @@ constexpr uint32_t kBox128 = 128 * 128;   // [128 rows x 64 bf16]
 constexpr uint32_t kBox64 = 64 * 128;     // [ 64 rows x 64 bf16]
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kSched = 4;                  // depth of the in-CTA ring of work-item indices
+// Steps before the end of an item at which the next one is popped. Items of sequences up to 512 tokens are popped at
+// the start of the one before: their few steps do not hide the pop, and batches of them have items to spare.
+constexpr int kPopAhead = 8;
 
 __device__ __forceinline__ float neg_inf() { return __int_as_float(0xff800000); }
 __device__ __forceinline__ float pos_inf() { return __int_as_float(0x7f800000); }
@@ -179,6 +182,9 @@ struct TileIter {
         seek();
     }
     __device__ bool valid() const { return li < list_len; }
+    // no more than n steps are left, this one included (pairs after the current one may see nothing: then it is false
+    // to the end, and the caller pops after the last step)
+    __device__ bool ends_within(int n) const { return li == list_len - 1 && t + n >= nt; }
     __device__ void next() { if (++t >= nt) { t = 0; ++li; seek(); } }
 };
 }  // namespace dq
@@ -222,6 +228,7 @@ struct SubIter {
         seek();
     }
     __device__ bool valid() const { return li < list_len; }
+    __device__ bool ends_within(int n) const { return li == list_len - 1 && u + n >= nu; }
     __device__ void next() { if (++u >= nu) { ++li; seek(); } }
 };
 }  // namespace dkv
@@ -276,24 +283,25 @@ HYDRA_K(hydra_bwd_dq_kernel)(const __grid_constant__ CUtensorMap map_q, const __
     // finishes early simply takes more items: no cost model has to predict the run time of an item)
     // and hands it to the other warps of the CTA through a small ring in shared memory.
     volatile int32_t* sched = s_sched;
-    // The pop is split in two: the request to the counter goes out when an item starts, its answer is
-    // looked at after the first loads of that item have been issued; the producer then fetches the
-    // next item's descriptors (three dependent loads from global memory) and puts them in the ring.
+    // A CTA's first item is its own number; every other pop is split in two: the request to the counter goes out a
+    // few steps before the end of an item (not at its start: a CTA with a long item would sit on a second one),
+    // its answer is looked at after that step's loads have been issued; the producer then fetches the next
+    // item's descriptors (three dependent loads from global memory) and puts them in the ring.
     constexpr int kPopFailed = 0x7fffffff;
     auto pop_begin = [&](uint32_t k) -> int {               // producer, one thread
         const int slot = k % kSched;
         if (!mbar_wait(bar(B_ITEMEMPTY + slot), ((k / kSched) ^ 1u) & 1u, abort_p, limit)) return kPopFailed;
-        return atomicAdd(&p.status->next_item[QUEUE_DQ], 1);
+        return k == 0 ? static_cast<int>(blockIdx.x)
+                      : static_cast<int>(gridDim.x) + atomicAdd(&p.status->next_item[QUEUE_DQ], 1);
     };
-    auto pop_end = [&](uint32_t k, int raw, GroupItem& item_out, PairDev& first_out) -> int {
+    auto pop_end = [&](uint32_t k, int raw) -> int {
         if (raw == kPopFailed) return -1;
         const int slot = k % kSched;
         const int idx = raw >= p.n_items ? -1 : raw;
         if (idx >= 0) {
-            item_out = p.items[idx];
-            first_out = p.pairs[p.lists[item_out.list_off]];
-            s_item[slot] = item_out;
-            s_first[slot] = first_out;
+            const GroupItem next = p.items[idx];
+            s_item[slot] = next;
+            s_first[slot] = p.pairs[p.lists[next.list_off]];
         }
         sched[slot] = idx;
         mbar_arrive(bar(B_ITEMFULL + slot));
@@ -318,59 +326,65 @@ HYDRA_K(hydra_bwd_dq_kernel)(const __grid_constant__ CUtensorMap map_q, const __
             bool ok = true;
             ClockProbe probe;
             probe.start();
-            // one item ahead: the round trip to the counter and the descriptor fetch overlap the loads of
-            // the current item
-            GroupItem item_next;
-            PairDev first_next;
             // test hook: idle, then hand out and load nothing; every other role's wait then runs out
             if (p.debug_stall_ns) { debug_stall(p.debug_stall_ns); ok = false; }
-            int it_ahead = ok ? pop_end(0, pop_begin(0), item_next, first_next) : -1;
+            int it_ahead = -1;
+            // round kq loads item kq - 1 (round 0: none) and pops item kq on the way
             for (uint32_t kq = 0; ok; ++kq) {
-                const int it = it_ahead;
-                if (it < 0) break;
-                const GroupItem item = item_next;
-                const PairDev first = first_next;
-                const int raw_next = pop_begin(kq + 1);
-                bool popped = false;
-                const int32_t* list = p.lists + item.list_off;
                 TileIter ti;
-                ti.init(p.pairs, list, item.list_len, min(item.r0 + TILE, first.q_len) - 1, p.causal, first);
-                if (!ti.valid()) { it_ahead = pop_end(kq + 1, raw_next, item_next, first_next); continue; }
-                ok = wait(B_QEMPTY, items ^ 1u);
-                if (!ok) break;
-                ++items;
-                mbar_arrive_expect_tx(bar(B_QFULL), (kQkBoxes + 2) * kBox128);
-                for (int c = 0; c < kQkBoxes; ++c)
-                    tma_load_3d(smem + kQ + c * kBox128, &map_q, bar(B_QFULL), c * 64, item.head,
-                                first.q_tok0 + item.r0);
-                for (int c = 0; c < 2; ++c)
-                    tma_load_3d(smem + kDO + c * kBox128, &map_do, bar(B_QFULL), c * 64, item.head,
-                                first.q_tok0 + item.r0);
-                for (; ti.valid() && ok; ti.next()) {
-                    const int tok = ti.cur.k_tok0 + ti.t * TILE;
-                    // V first: its slots were freed a whole tile ago and dP is the first product of the
-                    // tile; the K stage frees only when the dQ update two tiles back has completed
-                    for (int c = 0; c < 2 && ok; ++c, ++gv) {
-                        const int slot = gv % kVSlots;
-                        ok = wait(B_VEMPTY + slot, (gv / kVSlots) ^ 1u);
+                ti.li = 0; ti.list_len = 0;
+                GroupItem item;
+                if (kq > 0) {
+                    if (it_ahead < 0) break;
+                    item = s_item[(kq - 1) % kSched];
+                    const PairDev first = s_first[(kq - 1) % kSched];
+                    ti.init(p.pairs, p.lists + item.list_off, item.list_len, min(item.r0 + TILE, first.q_len) - 1, p.causal,
+                            first);
+                    if (ti.valid()) {
+                        ok = wait(B_QEMPTY, items ^ 1u);
                         if (!ok) break;
-                        mbar_arrive_expect_tx(bar(B_VFULL + slot), kBox128);
-                        tma_load_3d(smem + kV + slot * kBox128, &map_v, bar(B_VFULL + slot), c * 64,
-                                    item.head / p.kv_group, tok);
+                        ++items;
+                        mbar_arrive_expect_tx(bar(B_QFULL), (kQkBoxes + 2) * kBox128);
+                        for (int c = 0; c < kQkBoxes; ++c)
+                            tma_load_3d(smem + kQ + c * kBox128, &map_q, bar(B_QFULL), c * 64, item.head,
+                                        first.q_tok0 + item.r0);
+                        for (int c = 0; c < 2; ++c)
+                            tma_load_3d(smem + kDO + c * kBox128, &map_do, bar(B_QFULL), c * 64, item.head,
+                                        first.q_tok0 + item.r0);
                     }
-                    if (!ok) break;
-                    const int st = gk % kKStages;
-                    ok = wait(B_KEMPTY + st, (gk / kKStages) ^ 1u);
-                    if (!ok) break;
-                    ++gk;
-                    for (int c = 0; c < kQkBoxes; ++c) {
-                        mbar_arrive_expect_tx(bar(B_KFULL + st * 3 + c), kBox128);
-                        tma_load_3d(smem + kK + st * kQkBoxes * kBox128 + c * kBox128, &map_k, bar(B_KFULL + st * 3 + c),
-                                    c * 64, item.head / p.kv_group, tok);
-                    }
-                    if (!popped) { it_ahead = pop_end(kq + 1, raw_next, item_next, first_next); popped = true; }
                 }
-                if (!popped) it_ahead = pop_end(kq + 1, raw_next, item_next, first_next);
+                int raw_next = 0;
+                bool asked = false, popped = false;
+                for (;;) {
+                    const bool live = ti.valid();
+                    if (!asked && (!live || ti.ends_within(kPopAhead))) { raw_next = pop_begin(kq); asked = true; }
+                    if (live) {
+                        const int tok = ti.cur.k_tok0 + ti.t * TILE;
+                        // V first: its slots were freed a whole tile ago and dP is the first product of the
+                        // tile; the K stage frees only when the dQ update two tiles back has completed
+                        for (int c = 0; c < 2 && ok; ++c, ++gv) {
+                            const int slot = gv % kVSlots;
+                            ok = wait(B_VEMPTY + slot, (gv / kVSlots) ^ 1u);
+                            if (!ok) break;
+                            mbar_arrive_expect_tx(bar(B_VFULL + slot), kBox128);
+                            tma_load_3d(smem + kV + slot * kBox128, &map_v, bar(B_VFULL + slot), c * 64,
+                                        item.head / p.kv_group, tok);
+                        }
+                        if (!ok) break;
+                        const int st = gk % kKStages;
+                        ok = wait(B_KEMPTY + st, (gk / kKStages) ^ 1u);
+                        if (!ok) break;
+                        ++gk;
+                        for (int c = 0; c < kQkBoxes; ++c) {
+                            mbar_arrive_expect_tx(bar(B_KFULL + st * 3 + c), kBox128);
+                            tma_load_3d(smem + kK + st * kQkBoxes * kBox128 + c * kBox128, &map_k, bar(B_KFULL + st * 3 + c),
+                                        c * 64, item.head / p.kv_group, tok);
+                        }
+                        ti.next();
+                    }
+                    if (asked && !popped) { it_ahead = pop_end(kq, raw_next); popped = true; }
+                    if (popped && !ti.valid()) break;
+                }
             }
             if (blockIdx.x == 0) probe.stop(p.status, QUEUE_DQ);
         }
@@ -671,24 +685,25 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
     // finishes early simply takes more items: no cost model has to predict the run time of an item)
     // and hands it to the other warps of the CTA through a small ring in shared memory.
     volatile int32_t* sched = s_sched;
-    // The pop is split in two: the request to the counter goes out when an item starts, its answer is
-    // looked at after the first loads of that item have been issued; the producer then fetches the
-    // next item's descriptors (three dependent loads from global memory) and puts them in the ring.
+    // A CTA's first item is its own number; every other pop is split in two: the request to the counter goes out a
+    // few steps before the end of an item (not at its start: a CTA with a long item would sit on a second one),
+    // its answer is looked at after that step's loads have been issued; the producer then fetches the next
+    // item's descriptors (three dependent loads from global memory) and puts them in the ring.
     constexpr int kPopFailed = 0x7fffffff;
     auto pop_begin = [&](uint32_t k) -> int {               // producer, one thread
         const int slot = k % kSched;
         if (!mbar_wait(bar(B_ITEMEMPTY + slot), ((k / kSched) ^ 1u) & 1u, abort_p, limit)) return kPopFailed;
-        return atomicAdd(&p.status->next_item[QUEUE_DKV], 1);
+        return k == 0 ? static_cast<int>(blockIdx.x)
+                      : static_cast<int>(gridDim.x) + atomicAdd(&p.status->next_item[QUEUE_DKV], 1);
     };
-    auto pop_end = [&](uint32_t k, int raw, GroupItem& item_out, PairDev& first_out) -> int {
+    auto pop_end = [&](uint32_t k, int raw) -> int {
         if (raw == kPopFailed) return -1;
         const int slot = k % kSched;
         const int idx = raw >= p.n_items ? -1 : raw;
         if (idx >= 0) {
-            item_out = p.items[idx];
-            first_out = p.pairs[p.lists[item_out.list_off]];
-            s_item[slot] = item_out;
-            s_first[slot] = first_out;
+            const GroupItem next = p.items[idx];
+            s_item[slot] = next;
+            s_first[slot] = p.pairs[p.lists[next.list_off]];
         }
         sched[slot] = idx;
         mbar_arrive(bar(B_ITEMFULL + slot));
@@ -714,79 +729,86 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
         int it_ahead = -1;
         ClockProbe probe;
         probe.start();
-        GroupItem item_next;                          // lane 0: descriptors of the item popped ahead
-        PairDev first_next;
         // test hook: idle, then hand out and load nothing; every other role's wait then runs out
         if (p.debug_stall_ns) {
             if (lane == 0) debug_stall(p.debug_stall_ns);
             __syncwarp();
             ok = false;
         }
+        // Round kq loads item kq - 1 (round 0: none) and pops item kq on the way. One place each for the two halves of the
+        // pop: the code of the roles together is larger than the instruction cache, and with the pop written out at
+        // the start, in the middle and at the end of an item batches of short sequences ran 4 % slower.
         for (uint32_t kq = 0; ok; ++kq) {
-            int it = 0, raw_next = 0;
-            if (lane == 0) {                          // one pop per CTA, one item ahead, shared with the other lanes
-                if (kq == 0) it_ahead = pop_end(0, pop_begin(0), item_next, first_next);
-                it = it_ahead;
-                if (it >= 0) raw_next = pop_begin(kq + 1);
-            }
-            bool popped = false;
-            it = __shfl_sync(0xffffffffu, it, 0);
-            if (it < 0) break;
-            __syncwarp();
-            // lane 0 wrote this item's descriptors into the ring when it popped it (before the barrier above)
-            const GroupItem item = s_item[kq % kSched];
-            const PairDev first = s_first[kq % kSched];
-            const int32_t* list = p.lists + item.list_off;
             SubIter si;
-            si.init(p.pairs, list, item.list_len, item.r0, p.causal, p.ds != nullptr, first);
-            if (!si.valid()) {
-                if (lane == 0) it_ahead = pop_end(kq + 1, raw_next, item_next, first_next);
-                continue;
+            si.li = 0; si.list_len = 0;
+            GroupItem item;
+            PairDev first;
+            if (kq > 0) {
+                if (__shfl_sync(0xffffffffu, it_ahead, 0) < 0) break;
+                __syncwarp();
+                // lane 0 wrote this item's descriptors into the ring when it popped it (before the barrier above)
+                item = s_item[(kq - 1) % kSched];
+                first = s_first[(kq - 1) % kSched];
+                si.init(p.pairs, p.lists + item.list_off, item.list_len, item.r0, p.causal, p.ds != nullptr, first);
             }
-            ok = wait(B_KVEMPTY, items ^ 1u);
-            if (!ok) break;
-            ++items;
-            if (lane == 0) {
-                mbar_arrive_expect_tx(bar(B_KVFULL), (kQkBoxes + 2) * kBox128);
-                for (int c = 0; c < kQkBoxes; ++c)
-                    tma_load_3d(smem + kK + c * kBox128, &map_k, bar(B_KVFULL), c * 64, item.head / p.kv_group,
-                                first.k_tok0 + item.r0);
-                for (int c = 0; c < 2; ++c)
-                    tma_load_3d(smem + kV + c * kBox128, &map_v, bar(B_KVFULL), c * 64, item.head / p.kv_group,
-                                first.k_tok0 + item.r0);
-            }
-            for (; si.valid() && ok; si.next(), ++gq) {
-                const int st = gq % kStages;
-                ok = wait(B_QEMPTY + st, (gq / kStages) ^ 1u);
-                if (!ok) break;
-                const int tok = si.cur.q_tok0 + si.u * SUB;
-                if (lane == 0) {
-                    mbar_arrive_expect_tx(bar(B_QFULL + st), (kQkBoxes + 2) * kBox64);
-                    for (int c = 0; c < kQkBoxes; ++c)
-                        tma_load_3d(smem + kQ + st * kQkBoxes * kBox64 + c * kBox64, &map_q, bar(B_QFULL + st), c * 64,
-                                    item.head, tok);
-                    for (int c = 0; c < 2; ++c)
-                        tma_load_3d(smem + kDO + st * 2 * kBox64 + c * kBox64, &map_do, bar(B_QFULL + st), c * 64,
-                                    item.head, tok);
+            int raw_next = 0;
+            bool asked = false, popped = false, start = true;
+            for (;;) {
+                const bool live = si.valid();
+                if (!asked && (!live || si.ends_within(kPopAhead))) {
+                    if (lane == 0) raw_next = pop_begin(kq);
+                    asked = true;
                 }
-                // LSE (as log2) and D of the 64 q rows, two rows per lane
+                if (live && start) {
+                    start = false;
+                    ok = wait(B_KVEMPTY, items ^ 1u);
+                    if (!ok) break;
+                    ++items;
+                    if (lane == 0) {
+                        mbar_arrive_expect_tx(bar(B_KVFULL), (kQkBoxes + 2) * kBox128);
+                        for (int c = 0; c < kQkBoxes; ++c)
+                            tma_load_3d(smem + kK + c * kBox128, &map_k, bar(B_KVFULL), c * 64, item.head / p.kv_group,
+                                        first.k_tok0 + item.r0);
+                        for (int c = 0; c < 2; ++c)
+                            tma_load_3d(smem + kV + c * kBox128, &map_v, bar(B_KVFULL), c * 64, item.head / p.kv_group,
+                                        first.k_tok0 + item.r0);
+                    }
+                }
+                if (live) {
+                    const int st = gq % kStages;
+                    ok = wait(B_QEMPTY + st, (gq / kStages) ^ 1u);
+                    if (!ok) break;
+                    const int tok = si.cur.q_tok0 + si.u * SUB;
+                    if (lane == 0) {
+                        mbar_arrive_expect_tx(bar(B_QFULL + st), (kQkBoxes + 2) * kBox64);
+                        for (int c = 0; c < kQkBoxes; ++c)
+                            tma_load_3d(smem + kQ + st * kQkBoxes * kBox64 + c * kBox64, &map_q, bar(B_QFULL + st), c * 64,
+                                        item.head, tok);
+                        for (int c = 0; c < 2; ++c)
+                            tma_load_3d(smem + kDO + st * 2 * kBox64 + c * kBox64, &map_do, bar(B_QFULL + st), c * 64,
+                                        item.head, tok);
+                    }
+                    // LSE (as log2) and D of the 64 q rows, two rows per lane
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int c = lane + 32 * e;
-                    const int i = si.u * SUB + c;
-                    const bool v = i < si.cur.q_len;
-                    const int64_t idx = static_cast<int64_t>(item.head) * p.T + si.cur.q_tok0 + i;
-                    const float l = v ? __ldg(p.lse + idx) : neg_inf();
-                    s_lse2[st][c] = (l == neg_inf()) ? neg_inf() : -(l * kLog2e);
-                    s_dsum[st][c] = v ? -__ldg(p.dsum + idx) : 0.f;
+                    for (int e = 0; e < 2; ++e) {
+                        const int c = lane + 32 * e;
+                        const int i = si.u * SUB + c;
+                        const bool v = i < si.cur.q_len;
+                        const int64_t idx = static_cast<int64_t>(item.head) * p.T + si.cur.q_tok0 + i;
+                        const float l = v ? __ldg(p.lse + idx) : neg_inf();
+                        s_lse2[st][c] = (l == neg_inf()) ? neg_inf() : -(l * kLog2e);
+                        s_dsum[st][c] = v ? -__ldg(p.dsum + idx) : 0.f;
+                    }
+                    mbar_arrive_warp(bar(B_STAT + st));
+                    ++gq;
+                    si.next();
                 }
-                mbar_arrive_warp(bar(B_STAT + st));
-                if (!popped) {
-                    if (lane == 0) it_ahead = pop_end(kq + 1, raw_next, item_next, first_next);
+                if (asked && !popped) {
+                    if (lane == 0) it_ahead = pop_end(kq, raw_next);
                     popped = true;
                 }
+                if (popped && !si.valid()) break;
             }
-            if (!popped && lane == 0) it_ahead = pop_end(kq + 1, raw_next, item_next, first_next);
         }
         if (blockIdx.x == 0 && lane == 0) probe.stop(p.status, QUEUE_DKV);
     } else if (warp == kWarpMma || warp == kWarpMma2) {
@@ -1136,24 +1158,25 @@ HYDRA_K(hydra_bwd_dq_from_ds_kernel)(const __grid_constant__ CUtensorMap map_k,
     volatile int* abort_p = &abort_flag;
     auto wait = [&](int b, uint32_t parity) -> bool { return mbar_wait(bar(b), parity & 1u, abort_p, limit); };
     volatile int32_t* sched = s_sched;
-    // The pop is split in two: the request to the counter goes out when an item starts, its answer is
-    // looked at after the first loads of that item have been issued; the producer then fetches the
-    // next item's descriptors (three dependent loads from global memory) and puts them in the ring.
+    // A CTA's first item is its own number; every other pop is split in two: the request to the counter goes out a
+    // few steps before the end of an item (not at its start: a CTA with a long item would sit on a second one),
+    // its answer is looked at after that step's loads have been issued; the producer then fetches the next
+    // item's descriptors (three dependent loads from global memory) and puts them in the ring.
     constexpr int kPopFailed = 0x7fffffff;
     auto pop_begin = [&](uint32_t k) -> int {               // producer, one thread
         const int slot = k % kSched;
         if (!mbar_wait(bar(B_ITEMEMPTY + slot), ((k / kSched) ^ 1u) & 1u, abort_p, limit)) return kPopFailed;
-        return atomicAdd(&p.status->next_item[QUEUE_DQ], 1);
+        return k == 0 ? static_cast<int>(blockIdx.x)
+                      : static_cast<int>(gridDim.x) + atomicAdd(&p.status->next_item[QUEUE_DQ], 1);
     };
-    auto pop_end = [&](uint32_t k, int raw, GroupItem& item_out, PairDev& first_out) -> int {
+    auto pop_end = [&](uint32_t k, int raw) -> int {
         if (raw == kPopFailed) return -1;
         const int slot = k % kSched;
         const int idx = raw >= p.n_items ? -1 : raw;
         if (idx >= 0) {
-            item_out = p.items[idx];
-            first_out = p.pairs[p.lists[item_out.list_off]];
-            s_item[slot] = item_out;
-            s_first[slot] = first_out;
+            const GroupItem next = p.items[idx];
+            s_item[slot] = next;
+            s_first[slot] = p.pairs[p.lists[next.list_off]];
         }
         sched[slot] = idx;
         mbar_arrive(bar(B_ITEMFULL + slot));
@@ -1179,35 +1202,44 @@ HYDRA_K(hydra_bwd_dq_from_ds_kernel)(const __grid_constant__ CUtensorMap map_k,
             const uint64_t ds_policy = l2_policy_evict_first();   // dS is read once: leave L2 to the K tiles
             ClockProbe probe;
             probe.start();
-            GroupItem item_next;
-            PairDev first_next;
             // test hook: idle, then hand out and load nothing; every other role's wait then runs out
             if (p.debug_stall_ns) { debug_stall(p.debug_stall_ns); ok = false; }
-            int it_ahead = ok ? pop_end(0, pop_begin(0), item_next, first_next) : -1;
+            int it_ahead = -1;
+            // round kq loads item kq - 1 (round 0: none) and pops item kq on the way
             for (uint32_t kq = 0; ok; ++kq) {
-                const int it = it_ahead;
-                if (it < 0) break;
-                const GroupItem item = item_next;
-                const PairDev first = first_next;
-                const int raw_next = pop_begin(kq + 1);
-                bool popped = false;
-                const int32_t* list = p.lists + item.list_off;
                 TileIter ti;
-                ti.init(p.pairs, list, item.list_len, min(item.r0 + TILE, first.q_len) - 1, p.causal, first);
-                const int u0 = item.r0 / SUB;                  // first sub-tile of this q tile
-                for (; ti.valid() && ok; ti.next(), ++g) {
-                    const int st = g % kDsStages;
-                    ok = wait(B_DSEMPTY + st, (g / kDsStages) ^ 1u);
-                    if (!ok) break;
-                    const DsGeom geo = ds_geom(ti.cur.q_len, ti.cur.off, p.causal);
-                    const int64_t blk = static_cast<int64_t>(item.head) * p.ds_head_blocks + ti.cur.ds_base +
-                                        ds_rowstart(geo, ti.t) + (u0 - ds_first(geo, ti.t));
-                    mbar_arrive_expect_tx(bar(B_DSFULL + st), kDsBytes);
-                    bulk_load_hint(smem + st * kDsBytes, static_cast<const uint8_t*>(p.ds) + blk * DS_BLOCK_BYTES,
-                                   kDsBytes, bar(B_DSFULL + st), ds_policy);
-                    if (!popped) { it_ahead = pop_end(kq + 1, raw_next, item_next, first_next); popped = true; }
+                ti.li = 0; ti.list_len = 0;
+                GroupItem item;
+                int u0 = 0;                                    // first sub-tile of this q tile
+                if (kq > 0) {
+                    if (it_ahead < 0) break;
+                    item = s_item[(kq - 1) % kSched];
+                    const PairDev first = s_first[(kq - 1) % kSched];
+                    ti.init(p.pairs, p.lists + item.list_off, item.list_len, min(item.r0 + TILE, first.q_len) - 1, p.causal,
+                            first);
+                    u0 = item.r0 / SUB;
                 }
-                if (!popped) it_ahead = pop_end(kq + 1, raw_next, item_next, first_next);
+                int raw_next = 0;
+                bool asked = false, popped = false;
+                for (;;) {
+                    const bool live = ti.valid();
+                    if (!asked && (!live || ti.ends_within(kPopAhead))) { raw_next = pop_begin(kq); asked = true; }
+                    if (live) {
+                        const int st = g % kDsStages;
+                        ok = wait(B_DSEMPTY + st, (g / kDsStages) ^ 1u);
+                        if (!ok) break;
+                        const DsGeom geo = ds_geom(ti.cur.q_len, ti.cur.off, p.causal);
+                        const int64_t blk = static_cast<int64_t>(item.head) * p.ds_head_blocks + ti.cur.ds_base +
+                                            ds_rowstart(geo, ti.t) + (u0 - ds_first(geo, ti.t));
+                        mbar_arrive_expect_tx(bar(B_DSFULL + st), kDsBytes);
+                        bulk_load_hint(smem + st * kDsBytes, static_cast<const uint8_t*>(p.ds) + blk * DS_BLOCK_BYTES,
+                                       kDsBytes, bar(B_DSFULL + st), ds_policy);
+                        ++g;
+                        ti.next();
+                    }
+                    if (asked && !popped) { it_ahead = pop_end(kq, raw_next); popped = true; }
+                    if (popped && !ti.valid()) break;
+                }
             }
             if (blockIdx.x == 0) probe.stop(p.status, QUEUE_DQ);
         }

@@ -27,6 +27,8 @@
 // memory and hands it to every other role of both CTAs through a ring in (distributed) shared memory.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "hydra_internal.h"
 #include "sm100_ptx.cuh"
 
@@ -66,6 +68,7 @@ constexpr uint32_t kTmS = 0, kTmO = 256, kTmCols = 512;
 constexpr float kRescaleThreshold = 8.f;              // log2 units
 
 constexpr int kSched = 4;                             // depth of the in-cluster ring of work-item indices
+constexpr int kPopAhead = 3;                          // K tiles before the end of an item at which the next one is popped
 
 enum : int {
     B_QFULL = 0, B_QEMPTY = 2, B_KFULL = 4, B_KEMPTY = 7, B_VFULL = 10, B_VEMPTY = 13,
@@ -127,7 +130,9 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
     auto pop_item = [&](uint32_t k) -> int {                 // leader CTA, one thread
         const int slot = k % kSched;
         if (!mbar_wait(bar(B_ITEMEMPTY + slot), ((k / kSched) ^ 1u) & 1u, abort_p, limit)) return -1;
-        int idx = atomicAdd(&p.status->next_item[QUEUE_FWD], 1);
+        // the first item of every cluster is its own number: no round trip before the first load
+        int idx = k == 0 ? static_cast<int>(cluster_id_x())
+                         : static_cast<int>(gridDim.x >> 1) + atomicAdd(&p.status->next_item[QUEUE_FWD], 1);
         if (idx >= p.n_items) idx = -1;
         for (uint32_t r = 0; r < 2; ++r) {
             st_shared_cluster_s32(cluster_map_shared(smem_u32(&s_sched[slot]), r), idx);
@@ -153,14 +158,16 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
             probe.start();
             // test hook: idle, then hand out and load nothing; every other role's wait then runs out
             if (p.debug_stall_ns) { debug_stall(p.debug_stall_ns); ok = false; }
-            // the leader pops one item ahead: the round trip to the counter and the hand-over to the
-            // other CTA then overlap the loads of the current item
+            // The leader pops the next item while the last K tiles of the current one are being asked for: early
+            // enough that the round trip to the counter and the hand-over to the other CTA are hidden, late enough
+            // that a cluster with a long item does not sit on a second one (popped at the start of an item, the
+            // items of a call with fewer than a few per cluster were as good as dealt out in advance: one document
+            // of 8192 tokens, 16 heads, 344 -> 327 us).
             int it_ahead = (leader && ok) ? pop_item(0) : 0;
             for (uint32_t kq = 0; ok; ++kq) {
                 int it;
                 if (leader) {
                     it = it_ahead;
-                    if (it >= 0) it_ahead = pop_item(kq + 1);
                 } else {
                     it = next_item(kq, false);
                 }
@@ -180,6 +187,7 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
                                          item.head, pr.q_tok0 + item.q0 + t * 2 * TILE + rank * TILE);
                 };
                 auto load_k = [&](int j) {
+                    if (leader && j == max(n - kPopAhead, 0)) it_ahead = pop_item(kq + 1);
                     const int slot = gk % kKStages;
                     ok = wait(B_KEMPTY + slot, (gk / kKStages) ^ 1u);
                     if (!ok) return;
@@ -196,6 +204,7 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
                 for (; j < n && j < kKStages - 1 && ok; ++j) load_k(j);
                 load_q(1);
                 for (; j < n && ok; ++j) load_k(j);
+                if (leader && n == 0 && ok) it_ahead = pop_item(kq + 1);     // rows that see no key: nothing to load
             }
             if (blockIdx.x == 0) probe.stop(p.status, QUEUE_FWD);
         }
@@ -532,7 +541,7 @@ int HYDRA_K(fwd_max_clusters)()
 cudaError_t HYDRA_K(launch_fwd)(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
                        const FwdParams& p, int n_clusters, cudaStream_t stream)
 {
-    HYDRA_K(hydra_fwd_kernel)<<<2 * n_clusters, kThreads, HYDRA_K(fwd_smem_bytes)(), stream>>>(mq, mk, mv, p);
+    HYDRA_K(hydra_fwd_kernel)<<<2 * std::min(n_clusters, p.n_items), kThreads, HYDRA_K(fwd_smem_bytes)(), stream>>>(mq, mk, mv, p);
     return cudaGetLastError();
 }
 

@@ -76,6 +76,8 @@ constexpr uint32_t kSmemTotal = kSlots * kSlotBytes;
 constexpr uint32_t kTmSlot = 256, kTmS = 128, kTmCols = 512;
 constexpr float kRescaleThreshold = 8.f;              // log2 units
 constexpr int kSched = 4;                             // depth of a slot's ring of work items
+constexpr int kPopAhead = 4;                          // steps before the end of an item at which the next one is popped
+constexpr int kShortItem = 8;                         // an item of at most so many steps: the pops run two items ahead
 
 enum : int {
     B_QFULL = 0, B_QEMPTY = 1, B_KFULL = 2, B_KEMPTY = 5, B_VFULL = 8, B_VEMPTY = 10, B_SFULL = 12, B_PFULL = 14,
@@ -183,46 +185,50 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
                     tma_load_3d(smem + kOffV + st * kVStage + c * kHalfBox, &map_v, bar(B_VFULL + st), c * 64,
                                 it.head / p.kv_group, it.k_tok0 + j * KV);
             };
-            // The queue is popped two items ahead and the item's descriptor one item ahead, so that neither
-            // the round trip to the counter nor the load of the descriptor is ever waited for: both answers
-            // are looked at one work item after they were asked for.
-            FwdShortItem cur, nxt;
-            int cur_idx = -1, raw1 = 0;
-            if (ok) {
-                const int raw0 = atomicAdd(counter, 1);
-                raw1 = atomicAdd(counter, 1);
-                cur_idx = fetch(raw0, cur);
-                publish(0, cur_idx, cur);
-            }
+            // A slot's first item is its own number (slot 0 of every CTA before any slot 1: while there are no more
+            // items than CTAs, no two share an SM). After a long item the next one is popped, and then its descriptor
+            // asked for, while the long one's last steps are being loaded, each answer looked at a step or more after
+            // it was asked for: always popped two items ahead, a batch with fewer than a few items per slot was as
+            // good as dealt out in advance (64 items of up to 16 steps took 40 us, two in a row on half of the slots,
+            // now 22). Short items are popped two ahead and their descriptors asked for one ahead: an item of a few
+            // steps does not hide both answers (sequences of 64 to 512 tokens: 1-2 % of the kernel).
+            FwdShortItem cur{}, nxt;
+            int raw1 = slot * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x), raw2 = 0;   // pops of the next item and of
+            bool have1 = true, have2 = false;          // the one after it, if they have been asked for
+            const int first_pop = kSlots * static_cast<int>(gridDim.x);
             bool pre = false;                          // Q and the first K tile of `cur` have been requested
-            for (uint32_t kq = 0; ok && cur_idx >= 0; ++kq) {
-                const int nxt_idx = fetch(raw1, nxt);
-                const int raw2 = nxt_idx >= 0 ? atomicAdd(counter, 1) : 0x7fffffff;
+            // round kq loads item kq - 1 (round 0: none) and hands over item kq on the way
+            for (uint32_t kq = 0; ok; ++kq) {
                 const int n = cur.n_kv;
-                const bool nxt_loads = nxt_idx >= 0 && nxt.n_kv > 0;
-                bool handed = false;                   // the next item is in the ring
-                bool pre_next = false;
-                auto hand_over = [&]() {
-                    if (nxt_loads) { load_q(nxt); load_k(nxt, 0); pre_next = true; }
-                    if (ok) publish(kq + 1, nxt_idx, nxt);
-                    handed = true;
-                };
-                if (n > 0) {
-                    if (!pre) { load_q(cur); load_k(cur, 0); }
-                    if (n > 1) load_k(cur, 1);
-                    for (int j = 0; j < n && ok; ++j) {
-                        // The next item's Q and first K tile are released by score products that are long issued
-                        // when the last V stage comes free: ask for them first, and show the item to the issuer.
-                        if (j == n - 1 && n >= 2) hand_over();
-                        if (j + 2 < n) load_k(cur, j + 2);       // its stage came free before V's: S(j) precedes P V(j - 1)
-                        load_v(cur, j);
+                if (n > 0 && !pre) { load_q(cur); load_k(cur, 0); }
+                if (n > 1) load_k(cur, 1);
+                pre = false;
+                bool fetched = false;
+                int nxt_idx = -1;
+                for (int j = 0; ok; ++j) {
+                    // (the pops are used in the order in which they were made: an early one must not be left over
+                    // when a later one finds the queue empty)
+                    if (!have1 && (n <= kShortItem || j >= n - kPopAhead)) {
+                        raw1 = first_pop + atomicAdd(counter, 1);
+                        have1 = true;
                     }
+                    if (!fetched && have1 && (n <= kShortItem || j >= n - 2)) { nxt_idx = fetch(raw1, nxt); fetched = true; }
+                    if (kq > 0 && j == 0 && n <= kShortItem) { raw2 = first_pop + atomicAdd(counter, 1); have2 = true; }
+                    // The next item's Q and first K tile are released by score products that are long issued
+                    // when the last V stage comes free: ask for them first, and show the item to the issuer.
+                    if (j == (n >= 2 ? n - 1 : n)) {
+                        if (n >= 2 && nxt_idx >= 0 && nxt.n_kv > 0) { load_q(nxt); load_k(nxt, 0); pre = true; }
+                        if (ok) publish(kq, nxt_idx, nxt);
+                    }
+                    if (j >= n) break;
+                    if (j + 2 < n) load_k(cur, j + 2);           // its stage came free before V's: S(j) precedes P V(j - 1)
+                    load_v(cur, j);
                 }
-                if (!handed && ok) hand_over();
+                if (nxt_idx < 0) break;
                 cur = nxt;
-                cur_idx = nxt_idx;
                 raw1 = raw2;
-                pre = pre_next;
+                have1 = have2;
+                have2 = false;
             }
             if (blockIdx.x == 0 && slot == 0) probe.stop(p.status, QUEUE_FWD_SHORT);
         }
