@@ -121,7 +121,7 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
     const uint32_t tm = tmem_base_slot;
     const uint64_t limit = p.wait_limit_ns;
     volatile int* abort_p = &abort_flag;
-    auto wait = [&](int b, uint32_t parity) -> bool { return mbar_wait(bar(b), parity & 1u, abort_p, limit); };
+    auto wait = [&](int b, uint32_t parity) -> bool { return mbar_wait_compact(bar(b), parity & 1u, abort_p, limit); };
     // Work queue: the leader's producer pops the next item index from a counter in global memory (a
     // cluster that finishes early simply takes more items: no cost model has to predict the run time
     // of an item) and hands it to every other role of both CTAs through a small ring that exists in
@@ -129,7 +129,7 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
     volatile int32_t* sched = s_sched;
     auto pop_item = [&](uint32_t k) -> int {                 // leader CTA, one thread
         const int slot = k % kSched;
-        if (!mbar_wait(bar(B_ITEMEMPTY + slot), ((k / kSched) ^ 1u) & 1u, abort_p, limit)) return -1;
+        if (!mbar_wait_compact(bar(B_ITEMEMPTY + slot), ((k / kSched) ^ 1u) & 1u, abort_p, limit)) return -1;
         // the first item of every cluster is its own number: no round trip before the first load
         int idx = k == 0 ? static_cast<int>(cluster_id_x())
                          : static_cast<int>(gridDim.x >> 1) + atomicAdd(&p.status->next_item[QUEUE_FWD], 1);
