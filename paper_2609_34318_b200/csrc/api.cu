@@ -1040,11 +1040,6 @@ const KernelSet* kernel_set(int32_t d_qk, int32_t d_v)
     return nullptr;
 }
 
-int32_t reset_status(void* workspace, cudaStream_t s)
-{
-    return cudaMemsetAsync(workspace, 0, sizeof(StatusBlock), s) == cudaSuccess ? HYDRA_OK : HYDRA_ERR_CUDA;
-}
-
 }  // namespace
 
 cudaError_t launch_merge_counted(const MergeParams& p, cudaStream_t stream)
@@ -1431,7 +1426,7 @@ int32_t fwd_core(Problem& pb, const void* q, const void* k, const void* v, int32
     if (int32_t s = lease.acquire(HYDRA_WS_FWD, pb, causal != 0, stream)) return s;
     const Plan* plan = &lease.plan();
     if (plan->n_items == 0 && plan->n_items2 == 0) return HYDRA_OK;
-    if (int32_t s = reset_status(workspace, stream)) return s;
+    if (launch_reset(static_cast<StatusBlock*>(workspace), false, stream) != cudaSuccess) return HYDRA_ERR_CUDA;
     FwdParams fp{};
     fp.pairs = lease.at<PairDev>(plan->off_pairs);
     fp.items = lease.at<FwdItem>(plan->off_items);
@@ -1571,12 +1566,11 @@ int32_t bwd_run(const Problem& pb, int32_t n_kv_heads, int32_t causal, float sof
         make_map(&mq_sub, t.q, pb.Tq, n_heads, pb.dqk, SUB) || make_map(&mdo_sub, t.dout, pb.Tq, n_heads, D_V, SUB))
         return HYDRA_ERR_CUDA;
     if (first) {
-        if (int32_t s = reset_status(workspace, stream)) return s;
         ScopedKernelTimer timer(K_PREP, stream);
-        if (launch_bwd_prep(t.dout, t.out, dsum, pb.Tq, n_heads, stream) != cudaSuccess) return HYDRA_ERR_CUDA;
+        if (launch_bwd_prep(t.dout, t.out, dsum, pb.Tq, n_heads, static_cast<StatusBlock*>(workspace), stream) != cudaSuccess)
+            return HYDRA_ERR_CUDA;
         g_launches += 1;
-    } else if (cudaMemsetAsync(static_cast<uint8_t*>(workspace) + offsetof(StatusBlock, next_item), 0,
-                               sizeof(StatusBlock::next_item), stream) != cudaSuccess) {
+    } else if (launch_reset(static_cast<StatusBlock*>(workspace), true, stream) != cudaSuccess) {
         return HYDRA_ERR_CUDA;
     }
 

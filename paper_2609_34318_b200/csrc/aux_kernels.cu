@@ -77,6 +77,8 @@ template <bool kAccumulate, int kBatch>
 __global__ void __launch_bounds__(kThreads, kBatch == 2 ? 6 : 4)
 hydra_lse_merge_kernel(const MergeParams p)
 {
+    overlap_next_launch();
+    wait_for_previous_launch();
     const MergeItem item = p.items[blockIdx.x];
     const MergeGroup g = p.groups[item.group];
     const int32_t* part_row = p.lists + g.list_off;
@@ -206,6 +208,8 @@ template <bool kAccumulate, int kBatch>
 __global__ void __launch_bounds__(kThreads, kAccumulate ? 3 : 4)
 hydra_lse_merge_wide_kernel(const MergeParams p)
 {
+    overlap_next_launch();
+    wait_for_previous_launch();
     constexpr int kLanes = 8, kUnits = kThreads / kLanes;
     const MergeItem item = p.items[blockIdx.x];
     const MergeGroup g = p.groups[item.group];
@@ -313,11 +317,23 @@ hydra_lse_merge_wide_kernel(const MergeParams p)
 // 64 KB stages and sixteen consumer warps per SM, 3.1-3.8 TB/s. Short-lived blocks in different phases keep
 // more loads in flight than any of those.)
 
-// D[a, t] = sum_e dO[t, a, e] * O[t, a, e]
+// The first n words of what `block` points at become zero (the status block before a forward, the queue heads between
+// the bands of a backward): a launch, not a memset, so that the kernels before and after overlap with it.
+__global__ void __launch_bounds__(32) hydra_reset_kernel(int32_t* block, int n)
+{
+    overlap_next_launch();
+    wait_for_previous_launch();
+    for (int i = threadIdx.x; i < n; i += 32) block[i] = 0;
+}
+
+// D[a, t] = sum_e dO[t, a, e] * O[t, a, e]; block 0 also clears the status block for the kernels that follow
 __global__ void __launch_bounds__(kThreads)
 hydra_bwd_prep_kernel(const uint4* __restrict__ dout, const uint4* __restrict__ out,
-                      float* __restrict__ dsum, int64_t T, int32_t h)
+                      float* __restrict__ dsum, int64_t T, int32_t h, StatusBlock* status)
 {
+    overlap_next_launch();
+    wait_for_previous_launch();
+    if (blockIdx.x == 0 && threadIdx.x < sizeof(StatusBlock) / 4) reinterpret_cast<int32_t*>(status)[threadIdx.x] = 0;
     const int lane = threadIdx.x & (kLanesPerUnit - 1);
     const int64_t units = T * h;
     constexpr int kVecPerRow = D_V / 8;
@@ -342,8 +358,11 @@ hydra_bwd_prep_kernel(const uint4* __restrict__ dout, const uint4* __restrict__ 
 // The same with 32 bytes per lane (8 lanes per (row, head), 256-bit loads), for 32-byte aligned buffers.
 __global__ void __launch_bounds__(kThreads)
 hydra_bwd_prep_wide_kernel(const V8* __restrict__ dout, const V8* __restrict__ out, float* __restrict__ dsum,
-                           int64_t T, int32_t h)
+                           int64_t T, int32_t h, StatusBlock* status)
 {
+    overlap_next_launch();
+    wait_for_previous_launch();
+    if (blockIdx.x == 0 && threadIdx.x < sizeof(StatusBlock) / 4) reinterpret_cast<int32_t*>(status)[threadIdx.x] = 0;
     constexpr int kLanes = 8, kUnits = kThreads / kLanes, kVecPerRow = D_V / 16;
     const int lane = threadIdx.x & (kLanes - 1);
     const int64_t units = T * h;
@@ -371,6 +390,8 @@ __global__ void __launch_bounds__(kThreads)
 hydra_grad_cast_kernel(const float4* acc, uint4* grad, int64_t n8, int64_t n, const float* acc_tail,
                        __nv_bfloat16* grad_tail)
 {
+    overlap_next_launch();
+    wait_for_previous_launch();
     const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; i < n8; i += stride) {
         float4 a, b;
@@ -393,6 +414,8 @@ __global__ void __launch_bounds__(kThreads)
 hydra_grad_cast_wide_kernel(const V8* acc, V8* grad, int64_t n16, int64_t n, const float* acc_tail,
                             __nv_bfloat16* grad_tail)
 {
+    overlap_next_launch();
+    wait_for_previous_launch();
     const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; i < n16; i += stride) {
         const V8 a = ld_stream32(acc + 2 * i), b = ld_stream32(acc + 2 * i + 1);
@@ -417,18 +440,14 @@ cudaError_t launch_grad_cast(const float* acc, void* grad, int64_t n, cudaStream
         const int64_t n16 = n / 16;
         const int64_t blocks = (n16 + kThreads - 1) / kThreads;
         const int grid = static_cast<int>(blocks < 1 ? 1 : (blocks < 148 * 16 ? blocks : 148 * 16));
-        hydra_grad_cast_wide_kernel<<<grid, kThreads, 0, stream>>>(reinterpret_cast<const V8*>(acc),
-                                                               static_cast<V8*>(grad), n16, n, acc,
-                                                               static_cast<__nv_bfloat16*>(grad));
-        return cudaGetLastError();
+        return launch_overlapped(hydra_grad_cast_wide_kernel, grid, kThreads, 0, stream, reinterpret_cast<const V8*>(acc),
+                                 static_cast<V8*>(grad), n16, n, acc, static_cast<__nv_bfloat16*>(grad));
     }
     const int64_t n8 = n / 8;
     const int64_t blocks = (n8 + kThreads - 1) / kThreads;
     const int grid = static_cast<int>(blocks < 1 ? 1 : (blocks < 148 * 16 ? blocks : 148 * 16));
-    hydra_grad_cast_kernel<<<grid, kThreads, 0, stream>>>(reinterpret_cast<const float4*>(acc),
-                                                          static_cast<uint4*>(grad), n8, n, acc,
-                                                          static_cast<__nv_bfloat16*>(grad));
-    return cudaGetLastError();
+    return launch_overlapped(hydra_grad_cast_kernel, grid, kThreads, 0, stream, reinterpret_cast<const float4*>(acc),
+                             static_cast<uint4*>(grad), n8, n, acc, static_cast<__nv_bfloat16*>(grad));
 }
 
 // Ulysses pack / unpack: a permutation of 16-byte units between the token-major layout [n][P][cu] (a row
@@ -450,6 +469,8 @@ __global__ void __launch_bounds__(kThreads)
 hydra_ulysses_kernel(const Vec* __restrict__ src, Vec* __restrict__ dst, uint32_t n, uint32_t P, uint32_t cu,
                      uint32_t rows)
 {
+    overlap_next_launch();
+    wait_for_previous_launch();
     // A warp takes one chunk (row = j * n + t of the block-major side) at a time, four chunks in flight:
     // the two divisions are paid once per chunk, not once per 16 bytes (a flat loop over units spent its
     // time on them: 5.1 TB/s).
@@ -493,13 +514,11 @@ cudaError_t launch_ulysses(bool pack, const void* src, void* dst, int64_t n_toke
         // chunks of whole 32-byte units in 32-byte aligned buffers: half as many, twice as large accesses
         const V8* s32 = static_cast<const V8*>(src);
         V8* d32 = static_cast<V8*>(dst);
-        if (pack) hydra_ulysses_kernel<true, V8><<<grid, kThreads, 0, stream>>>(s32, d32, n, P, cu / 2, r);
-        else hydra_ulysses_kernel<false, V8><<<grid, kThreads, 0, stream>>>(s32, d32, n, P, cu / 2, r);
-        return cudaGetLastError();
+        if (pack) return launch_overlapped(hydra_ulysses_kernel<true, V8>, grid, kThreads, 0, stream, s32, d32, n, P, cu / 2, r);
+        else return launch_overlapped(hydra_ulysses_kernel<false, V8>, grid, kThreads, 0, stream, s32, d32, n, P, cu / 2, r);
     }
-    if (pack) hydra_ulysses_kernel<true, uint4><<<grid, kThreads, 0, stream>>>(s, d, n, P, cu, r);
-    else hydra_ulysses_kernel<false, uint4><<<grid, kThreads, 0, stream>>>(s, d, n, P, cu, r);
-    return cudaGetLastError();
+    if (pack) return launch_overlapped(hydra_ulysses_kernel<true, uint4>, grid, kThreads, 0, stream, s, d, n, P, cu, r);
+    else return launch_overlapped(hydra_ulysses_kernel<false, uint4>, grid, kThreads, 0, stream, s, d, n, P, cu, r);
 }
 
 cudaError_t launch_merge(const MergeParams& p, cudaStream_t stream)
@@ -509,23 +528,29 @@ cudaError_t launch_merge(const MergeParams& p, cudaStream_t stream)
     const bool wide = ((reinterpret_cast<uintptr_t>(p.o_part) | reinterpret_cast<uintptr_t>(p.out)) & 31u) == 0;
     if (wide) {
         if (p.accumulate) {
-            if (four) hydra_lse_merge_wide_kernel<true, 4><<<p.n_items, kThreads, 0, stream>>>(p);
-            else hydra_lse_merge_wide_kernel<true, 2><<<p.n_items, kThreads, 0, stream>>>(p);
+            if (four) return launch_overlapped(hydra_lse_merge_wide_kernel<true, 4>, p.n_items, kThreads, 0, stream, p);
+            else return launch_overlapped(hydra_lse_merge_wide_kernel<true, 2>, p.n_items, kThreads, 0, stream, p);
         } else {
-            if (four) hydra_lse_merge_wide_kernel<false, 4><<<p.n_items, kThreads, 0, stream>>>(p);
-            else hydra_lse_merge_wide_kernel<false, 2><<<p.n_items, kThreads, 0, stream>>>(p);
+            if (four) return launch_overlapped(hydra_lse_merge_wide_kernel<false, 4>, p.n_items, kThreads, 0, stream, p);
+            else return launch_overlapped(hydra_lse_merge_wide_kernel<false, 2>, p.n_items, kThreads, 0, stream, p);
         }
     } else if (p.accumulate) {
-        if (four) hydra_lse_merge_kernel<true, 4><<<p.n_items, kThreads, 0, stream>>>(p);
-        else hydra_lse_merge_kernel<true, 2><<<p.n_items, kThreads, 0, stream>>>(p);
+        if (four) return launch_overlapped(hydra_lse_merge_kernel<true, 4>, p.n_items, kThreads, 0, stream, p);
+        else return launch_overlapped(hydra_lse_merge_kernel<true, 2>, p.n_items, kThreads, 0, stream, p);
     } else {
-        if (four) hydra_lse_merge_kernel<false, 4><<<p.n_items, kThreads, 0, stream>>>(p);
-        else hydra_lse_merge_kernel<false, 2><<<p.n_items, kThreads, 0, stream>>>(p);
+        if (four) return launch_overlapped(hydra_lse_merge_kernel<false, 4>, p.n_items, kThreads, 0, stream, p);
+        else return launch_overlapped(hydra_lse_merge_kernel<false, 2>, p.n_items, kThreads, 0, stream, p);
     }
-    return cudaGetLastError();
 }
 
-cudaError_t launch_bwd_prep(const void* dout, const void* out, float* dsum, int64_t T, int32_t h,
+cudaError_t launch_reset(StatusBlock* status, bool keep_status, cudaStream_t stream)
+{
+    if (keep_status) return launch_overlapped(hydra_reset_kernel, 1, 32, 0, stream, status->next_item, 4);
+    return launch_overlapped(hydra_reset_kernel, 1, 32, 0, stream, reinterpret_cast<int32_t*>(status),
+                             static_cast<int>(sizeof(StatusBlock) / 4));
+}
+
+cudaError_t launch_bwd_prep(const void* dout, const void* out, float* dsum, int64_t T, int32_t h, StatusBlock* status,
                             cudaStream_t stream)
 {
     if (T * h == 0) return cudaSuccess;
@@ -534,13 +559,11 @@ cudaError_t launch_bwd_prep(const void* dout, const void* out, float* dsum, int6
     if (((reinterpret_cast<uintptr_t>(dout) | reinterpret_cast<uintptr_t>(out)) & 31u) == 0) {
         const int64_t wide_passes = (T * h + 2 * kUnitsPerPass - 1) / (2 * kUnitsPerPass);
         const int wide_grid = static_cast<int>(wide_passes < 148 * 16 ? wide_passes : 148 * 16);
-        hydra_bwd_prep_wide_kernel<<<wide_grid, kThreads, 0, stream>>>(static_cast<const V8*>(dout),
-                                                                   static_cast<const V8*>(out), dsum, T, h);
-        return cudaGetLastError();
+        return launch_overlapped(hydra_bwd_prep_wide_kernel, wide_grid, kThreads, 0, stream, static_cast<const V8*>(dout),
+                                 static_cast<const V8*>(out), dsum, T, h, status);
     }
-    hydra_bwd_prep_kernel<<<grid, kThreads, 0, stream>>>(static_cast<const uint4*>(dout),
-                                                         static_cast<const uint4*>(out), dsum, T, h);
-    return cudaGetLastError();
+    return launch_overlapped(hydra_bwd_prep_kernel, grid, kThreads, 0, stream, static_cast<const uint4*>(dout),
+                             static_cast<const uint4*>(out), dsum, T, h, status);
 }
 
 }  // namespace hydra

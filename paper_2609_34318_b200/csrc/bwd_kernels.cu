@@ -240,6 +240,7 @@ HYDRA_K(hydra_bwd_dq_kernel)(const __grid_constant__ CUtensorMap map_q, const __
                     const BwdParams p)
 {
     using namespace dq;
+    overlap_next_launch();
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem = (smem_u32(smem_raw) + 1023u) & ~1023u;
     __shared__ __align__(8) uint64_t bars[B_COUNT];
@@ -268,6 +269,7 @@ HYDRA_K(hydra_bwd_dq_kernel)(const __grid_constant__ CUtensorMap map_q, const __
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
+    wait_for_previous_launch();
     const uint32_t tm = tmem_base_slot;
     const uint64_t limit = p.wait_limit_ns;
     volatile int* abort_p = &abort_flag;
@@ -635,6 +637,7 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                      const BwdParams p)
 {
     using namespace dkv;
+    overlap_next_launch();
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem = (smem_u32(smem_raw) + 1023u) & ~1023u;
     __shared__ __align__(8) uint64_t bars[B_COUNT];
@@ -670,6 +673,7 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
+    wait_for_previous_launch();
     const uint32_t tm = tmem_base_slot;
     const uint64_t limit = p.wait_limit_ns;
     volatile int* abort_p = &abort_flag;
@@ -1121,6 +1125,7 @@ HYDRA_K(hydra_bwd_dq_from_ds_kernel)(const __grid_constant__ CUtensorMap map_k,
 {
     using namespace dqs;
     using dq::TileIter;
+    overlap_next_launch();
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem = (smem_u32(smem_raw) + 1023u) & ~1023u;
     __shared__ __align__(8) uint64_t bars[B_COUNT];
@@ -1148,6 +1153,7 @@ HYDRA_K(hydra_bwd_dq_from_ds_kernel)(const __grid_constant__ CUtensorMap map_k,
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
+    wait_for_previous_launch();
     const uint32_t tm = tmem_base_slot;
     const uint64_t limit = p.wait_limit_ns;
     volatile int* abort_p = &abort_flag;
@@ -1409,8 +1415,7 @@ cudaError_t HYDRA_K(launch_bwd_dq_from_ds)(const CUtensorMap& mk, const BwdParam
 {
     static bool configured[64] = {};
     if (cudaError_t e = configure_once_per_device(HYDRA_K(hydra_bwd_dq_from_ds_kernel), HYDRA_K(bwd_dq_ds_smem_bytes)(), configured)) return e;
-    HYDRA_K(hydra_bwd_dq_from_ds_kernel)<<<grid, dqs::kThreadsS, HYDRA_K(bwd_dq_ds_smem_bytes)(), stream>>>(mk, p);
-    return cudaGetLastError();
+    return launch_overlapped(HYDRA_K(hydra_bwd_dq_from_ds_kernel), grid, dqs::kThreadsS, HYDRA_K(bwd_dq_ds_smem_bytes)(), stream, mk, p);
 }
 
 cudaError_t HYDRA_K(launch_bwd_dq)(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
@@ -1418,8 +1423,7 @@ cudaError_t HYDRA_K(launch_bwd_dq)(const CUtensorMap& mq, const CUtensorMap& mk,
 {
     static bool configured[64] = {};
     if (cudaError_t e = configure_once_per_device(HYDRA_K(hydra_bwd_dq_kernel), HYDRA_K(bwd_dq_smem_bytes)(), configured)) return e;
-    HYDRA_K(hydra_bwd_dq_kernel)<<<grid, kThreads, HYDRA_K(bwd_dq_smem_bytes)(), stream>>>(mq, mk, mv, mdo, p);
-    return cudaGetLastError();
+    return launch_overlapped(HYDRA_K(hydra_bwd_dq_kernel), grid, kThreads, HYDRA_K(bwd_dq_smem_bytes)(), stream, mq, mk, mv, mdo, p);
 }
 
 cudaError_t HYDRA_K(launch_bwd_dkv)(const CUtensorMap& mq_sub, const CUtensorMap& mk, const CUtensorMap& mv,
@@ -1427,8 +1431,8 @@ cudaError_t HYDRA_K(launch_bwd_dkv)(const CUtensorMap& mq_sub, const CUtensorMap
 {
     static bool configured[64] = {};
     if (cudaError_t e = configure_once_per_device(HYDRA_K(hydra_bwd_dkv_kernel), HYDRA_K(bwd_dkv_smem_bytes)(), configured)) return e;
-    HYDRA_K(hydra_bwd_dkv_kernel)<<<grid, kThreads, HYDRA_K(bwd_dkv_smem_bytes)(), stream>>>(mq_sub, mk, mv, mdo_sub, p);
-    return cudaGetLastError();
+    return launch_overlapped(HYDRA_K(hydra_bwd_dkv_kernel), grid, kThreads, HYDRA_K(bwd_dkv_smem_bytes)(), stream, mq_sub, mk, mv,
+                             mdo_sub, p);
 }
 
 }  // namespace hydra

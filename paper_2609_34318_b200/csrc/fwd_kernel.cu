@@ -86,6 +86,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const FwdParams p)
 {
+    overlap_next_launch();
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem = (smem_u32(smem_raw) + 1023u) & ~1023u;
     __shared__ __align__(8) uint64_t bars[B_COUNT];
@@ -118,6 +119,7 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
     __syncthreads();
     cluster_sync_all();                                // both CTAs' barriers exist before anyone signals them
     tc_fence_after_sync();
+    wait_for_previous_launch();
     const uint32_t tm = tmem_base_slot;
     const uint64_t limit = p.wait_limit_ns;
     volatile int* abort_p = &abort_flag;
@@ -541,8 +543,8 @@ int HYDRA_K(fwd_max_clusters)()
 cudaError_t HYDRA_K(launch_fwd)(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
                        const FwdParams& p, int n_clusters, cudaStream_t stream)
 {
-    HYDRA_K(hydra_fwd_kernel)<<<2 * std::min(n_clusters, p.n_items), kThreads, HYDRA_K(fwd_smem_bytes)(), stream>>>(mq, mk, mv, p);
-    return cudaGetLastError();
+    return launch_overlapped(HYDRA_K(hydra_fwd_kernel), 2 * std::min(n_clusters, p.n_items), kThreads, HYDRA_K(fwd_smem_bytes)(),
+                             stream, mq, mk, mv, p);
 }
 
 }  // namespace hydra

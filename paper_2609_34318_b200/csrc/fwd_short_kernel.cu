@@ -94,6 +94,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                                 const __grid_constant__ CUtensorMap map_v, const FwdParams p)
 {
+    overlap_next_launch();
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
     __shared__ __align__(8) uint64_t bars[kSlots * B_PER_SLOT];
@@ -125,6 +126,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
+    wait_for_previous_launch();
     const uint32_t tm = tmem_base_slot + static_cast<uint32_t>(slot) * kTmSlot;
     const uint64_t limit = p.wait_limit_ns;
     volatile int* abort_p = &abort_flag;
@@ -509,8 +511,7 @@ cudaError_t HYDRA_K(launch_fwd_short)(const CUtensorMap& mq, const CUtensorMap& 
         if (e != cudaSuccess) return e;
         configured[dev] = true;
     }
-    HYDRA_K(hydra_fwd_short_kernel)<<<grid, kThreads, HYDRA_K(fwd_short_smem_bytes)(), stream>>>(mq, mk, mv, p);
-    return cudaGetLastError();
+    return launch_overlapped(HYDRA_K(hydra_fwd_short_kernel), grid, kThreads, HYDRA_K(fwd_short_smem_bytes)(), stream, mq, mk, mv, p);
 }
 
 }  // namespace hydra

@@ -137,6 +137,34 @@ struct ClockProbe {
 };
 #endif
 
+// Launches of one stream overlap at their ends: every kernel of the library lets the next one start its blocks as soon
+// as all of its own have started (they take the SMs that its first finished blocks leave) and waits, before it
+// touches global memory, until the launch before it has completed and its results are visible. What is hidden
+// that way is the launch itself, the barriers' and tensor memory's set-up and the wait for the last block: a step of
+// four sequences of 7 to 300 tokens 42 -> 35 us, of 1024 tokens in short ones 49 -> 42 us, the twelve launches around the
+// attention of a 4096-token MLA block 813 -> 794 us. Kernels of other libraries before or after are ordered
+// as usual.
+#ifdef __CUDACC__
+__device__ __forceinline__ void overlap_next_launch() { cudaTriggerProgrammaticLaunchCompletion(); }
+__device__ __forceinline__ void wait_for_previous_launch() { cudaGridDependencySynchronize(); }
+template <class... Params, class... Args>
+cudaError_t launch_overlapped(void (*kernel)(Params...), int grid, int block, size_t smem_bytes, cudaStream_t stream,
+                              Args&&... args)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(static_cast<unsigned>(grid));
+    cfg.blockDim = dim3(static_cast<unsigned>(block));
+    cfg.dynamicSmemBytes = smem_bytes;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+#endif
+
 struct FwdParams {
     const PairDev* pairs;
     const FwdItem* items;
@@ -226,7 +254,10 @@ cudaError_t launch_mla_kv_assemble_bwd(const void* dk, const void* dv, const int
 cudaError_t launch_gate(const void* out, const void* gate, void* y, int64_t n8, cudaStream_t stream);
 cudaError_t launch_gate_bwd(const void* dy, const void* out, const void* gate, void* d_out, void* d_gate, int64_t n8,
                             cudaStream_t stream);
-cudaError_t launch_bwd_prep(const void* dout, const void* out, float* dsum, int64_t T, int32_t h,
+// clears the status block (of which keep_status leaves all but the work-queue heads)
+cudaError_t launch_reset(StatusBlock* status, bool keep_status, cudaStream_t stream);
+// D = rowsum(dO * O); also clears the status block
+cudaError_t launch_bwd_prep(const void* dout, const void* out, float* dsum, int64_t T, int32_t h, StatusBlock* status,
                             cudaStream_t stream);
 
 }  // namespace hydra

@@ -55,6 +55,8 @@ hydra_rope_kernel(const uint32_t* __restrict__ x, const int32_t* __restrict__ po
                   int64_t n_tokens, int32_t n_heads, int32_t head_dim, int32_t rope_offset, int32_t rope_dim,
                   double log_theta, int inverse, int in_place)
 {
+    overlap_next_launch();
+    wait_for_previous_launch();
     __shared__ float s_cos[kMaxRopePairs], s_sin[kMaxRopePairs];
     const int pairs_per_head = head_dim / 2, p0 = rope_offset / 2, p1 = (rope_offset + rope_dim) / 2;
     for (int64_t t = blockIdx.x; t < n_tokens; t += gridDim.x) {
@@ -93,6 +95,8 @@ hydra_mla_kv_assemble_kernel(const uint32_t* __restrict__ kv_up, const uint32_t*
                              int64_t n_tokens, int32_t n_heads, int32_t nope, int32_t rope_dim, int32_t dv,
                              double log_theta)
 {
+    overlap_next_launch();
+    wait_for_previous_launch();
     __shared__ float s_cos[kMaxRopePairs], s_sin[kMaxRopePairs];
     __shared__ uint32_t s_pe[kMaxRopePairs];
     const int np = nope / 2, rp = rope_dim / 2, vp = dv / 2;
@@ -128,6 +132,8 @@ hydra_mla_kv_assemble_bwd_kernel(const uint32_t* __restrict__ dk, const uint32_t
                                  uint32_t* __restrict__ dk_pe, int64_t n_tokens, int32_t n_heads, int32_t nope,
                                  int32_t rope_dim, int32_t dvd, double log_theta)
 {
+    overlap_next_launch();
+    wait_for_previous_launch();
     __shared__ float s_cos[kMaxRopePairs], s_sin[kMaxRopePairs];
     const int np = nope / 2, rp = rope_dim / 2, vp = dvd / 2;
     const int up_pairs = np + vp, k_pairs = np + rp;
@@ -193,9 +199,11 @@ hydra_rope_vec_kernel(const uint4* __restrict__ x, const int32_t* __restrict__ p
                       int64_t n_tokens, int32_t n_heads, int32_t head_dim, int32_t rope_offset, int32_t rope_dim,
                       double log_theta, int inverse, int in_place)
 {
+    overlap_next_launch();
     __shared__ __align__(16) float s_cos[kMaxRopePairs], s_sin[kMaxRopePairs];
     const int vph = head_dim / 8, v0 = rope_offset / 8, nv = rope_dim / 8;
     const double freq = exp(-log_theta * (2.0 * threadIdx.x) / rope_dim);
+    wait_for_previous_launch();
     for (int64_t t = blockIdx.x; t < n_tokens; t += gridDim.x) {
         __syncthreads();                               // the previous token's table is no longer read
         rope_table_fast(s_cos, s_sin, positions[t], rope_dim / 2, freq, inverse);
@@ -231,11 +239,13 @@ hydra_mla_kv_assemble_vec_kernel(const uint4* __restrict__ kv_up, const uint4* _
                                  int64_t n_tokens, int32_t n_heads, int32_t nope, int32_t rope_dim, int32_t dv,
                                  double log_theta)
 {
+    overlap_next_launch();
     __shared__ __align__(16) float s_cos[kMaxRopePairs], s_sin[kMaxRopePairs];
     __shared__ uint4 s_pe[kMaxRopePairs / 4];
     const int nv = nope / 8, rv = rope_dim / 8, vv = dv / 8;
     const int up_vecs = nv + vv, k_vecs = nv + rv;
     const double freq = exp(-log_theta * (2.0 * threadIdx.x) / rope_dim);
+    wait_for_previous_launch();
     for (int64_t t = blockIdx.x; t < n_tokens; t += gridDim.x) {
         __syncthreads();
         rope_table_fast(s_cos, s_sin, positions[t], rope_dim / 2, freq, 0);
@@ -263,10 +273,12 @@ hydra_mla_kv_assemble_bwd_vec_kernel(const uint4* __restrict__ dk, const uint4* 
                                      uint4* __restrict__ dk_pe, int64_t n_tokens, int32_t n_heads, int32_t nope,
                                      int32_t rope_dim, int32_t dvd, double log_theta)
 {
+    overlap_next_launch();
     __shared__ __align__(16) float s_cos[kMaxRopePairs], s_sin[kMaxRopePairs];
     const int nv = nope / 8, rv = rope_dim / 8, vv = dvd / 8;
     const int up_vecs = nv + vv, k_vecs = nv + rv;
     const double freq = exp(-log_theta * (2.0 * threadIdx.x) / rope_dim);
+    wait_for_previous_launch();
     for (int64_t t = blockIdx.x; t < n_tokens; t += gridDim.x) {
         __syncthreads();
         rope_table_fast(s_cos, s_sin, positions[t], rope_dim / 2, freq, 1);
@@ -349,6 +361,8 @@ template <int kWords>
 __global__ void __launch_bounds__(256)
 hydra_gate_kernel(const void* __restrict__ out, const void* __restrict__ gate, void* __restrict__ y, int64_t n)
 {
+    overlap_next_launch();
+    wait_for_previous_launch();
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; i < n; i += static_cast<int64_t>(gridDim.x) * 256) {
         const Words<kWords> o = ld_words<kWords>(out, i), g = ld_words<kWords>(gate, i);
         Words<kWords> r;
@@ -367,6 +381,8 @@ __global__ void __launch_bounds__(256)
 hydra_gate_bwd_kernel(const void* __restrict__ dy, const void* __restrict__ out, const void* __restrict__ gate,
                       void* __restrict__ d_out, void* __restrict__ d_gate, int64_t n)
 {
+    overlap_next_launch();
+    wait_for_previous_launch();
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; i < n; i += static_cast<int64_t>(gridDim.x) * 256) {
         const Words<kWords> d = ld_words<kWords>(dy, i), o = ld_words<kWords>(out, i), g = ld_words<kWords>(gate, i);
         Words<kWords> ro, rg;
@@ -404,15 +420,13 @@ cudaError_t launch_rope(const void* x, const int32_t* positions, void* y, int64_
     if (n_tokens == 0) return cudaSuccess;
     if (head_dim % 8 == 0 && rope_offset % 8 == 0 && rope_dim % 8 == 0 && rope_dim / 2 <= kRopeThreads &&
         aligned16_all({x, y})) {
-        hydra_rope_vec_kernel<<<grid_for(n_tokens, 1), kRopeThreads, 0, stream>>>(
+        return launch_overlapped(hydra_rope_vec_kernel, grid_for(n_tokens, 1), kRopeThreads, 0, stream,
             static_cast<const uint4*>(x), positions, static_cast<uint4*>(y), n_tokens, n_heads, head_dim, rope_offset,
             rope_dim, std::log(static_cast<double>(theta)), inverse, x == y ? 1 : 0);
-        return cudaGetLastError();
     }
-    hydra_rope_kernel<<<grid_for(n_tokens, 1), kRopeThreads, 0, stream>>>(
+    return launch_overlapped(hydra_rope_kernel, grid_for(n_tokens, 1), kRopeThreads, 0, stream,
         static_cast<const uint32_t*>(x), positions, static_cast<uint32_t*>(y), n_tokens, n_heads, head_dim, rope_offset,
         rope_dim, std::log(static_cast<double>(theta)), inverse, x == y ? 1 : 0);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_mla_kv_assemble(const void* kv_up, const void* k_pe, const int32_t* positions, void* k, void* v,
@@ -422,15 +436,13 @@ cudaError_t launch_mla_kv_assemble(const void* kv_up, const void* k_pe, const in
     if (n_tokens == 0) return cudaSuccess;
     if (nope % 8 == 0 && rope_dim % 8 == 0 && dv % 8 == 0 && rope_dim / 2 <= kRopeThreads &&
         aligned16_all({kv_up, k_pe, k, v})) {
-        hydra_mla_kv_assemble_vec_kernel<<<grid_for(n_tokens, 1), kRopeThreads, 0, stream>>>(
+        return launch_overlapped(hydra_mla_kv_assemble_vec_kernel, grid_for(n_tokens, 1), kRopeThreads, 0, stream,
             static_cast<const uint4*>(kv_up), static_cast<const uint4*>(k_pe), positions, static_cast<uint4*>(k),
             static_cast<uint4*>(v), n_tokens, n_heads, nope, rope_dim, dv, std::log(static_cast<double>(theta)));
-        return cudaGetLastError();
     }
-    hydra_mla_kv_assemble_kernel<<<grid_for(n_tokens, 1), kRopeThreads, 0, stream>>>(
+    return launch_overlapped(hydra_mla_kv_assemble_kernel, grid_for(n_tokens, 1), kRopeThreads, 0, stream,
         static_cast<const uint32_t*>(kv_up), static_cast<const uint32_t*>(k_pe), positions, static_cast<uint32_t*>(k),
         static_cast<uint32_t*>(v), n_tokens, n_heads, nope, rope_dim, dv, std::log(static_cast<double>(theta)));
-    return cudaGetLastError();
 }
 
 cudaError_t launch_mla_kv_assemble_bwd(const void* dk, const void* dv, const int32_t* positions, void* dkv_up,
@@ -440,25 +452,22 @@ cudaError_t launch_mla_kv_assemble_bwd(const void* dk, const void* dv, const int
     if (n_tokens == 0) return cudaSuccess;
     if (nope % 8 == 0 && rope_dim % 8 == 0 && dvd % 8 == 0 && rope_dim / 2 <= kRopeThreads &&
         aligned16_all({dk, dv, dkv_up, dk_pe})) {
-        hydra_mla_kv_assemble_bwd_vec_kernel<<<grid_for(n_tokens, 1), kRopeThreads, 0, stream>>>(
+        return launch_overlapped(hydra_mla_kv_assemble_bwd_vec_kernel, grid_for(n_tokens, 1), kRopeThreads, 0, stream,
             static_cast<const uint4*>(dk), static_cast<const uint4*>(dv), positions, static_cast<uint4*>(dkv_up),
             static_cast<uint4*>(dk_pe), n_tokens, n_heads, nope, rope_dim, dvd, std::log(static_cast<double>(theta)));
-        return cudaGetLastError();
     }
-    hydra_mla_kv_assemble_bwd_kernel<<<grid_for(n_tokens, 1), kRopeThreads, 0, stream>>>(
+    return launch_overlapped(hydra_mla_kv_assemble_bwd_kernel, grid_for(n_tokens, 1), kRopeThreads, 0, stream,
         static_cast<const uint32_t*>(dk), static_cast<const uint32_t*>(dv), positions, static_cast<uint32_t*>(dkv_up),
         static_cast<uint32_t*>(dk_pe), n_tokens, n_heads, nope, rope_dim, dvd, std::log(static_cast<double>(theta)));
-    return cudaGetLastError();
 }
 
 cudaError_t launch_gate(const void* out, const void* gate, void* y, int64_t n8, cudaStream_t stream)
 {
     if (n8 == 0) return cudaSuccess;
     if ((n8 & 1) == 0 && all_aligned32({out, gate, y}))
-        hydra_gate_kernel<8><<<grid_for(n8 / 2, 256), 256, 0, stream>>>(out, gate, y, n8 / 2);
+        return launch_overlapped(hydra_gate_kernel<8>, grid_for(n8 / 2, 256), 256, 0, stream, out, gate, y, n8 / 2);
     else
-        hydra_gate_kernel<4><<<grid_for(n8, 256), 256, 0, stream>>>(out, gate, y, n8);
-    return cudaGetLastError();
+        return launch_overlapped(hydra_gate_kernel<4>, grid_for(n8, 256), 256, 0, stream, out, gate, y, n8);
 }
 
 cudaError_t launch_gate_bwd(const void* dy, const void* out, const void* gate, void* d_out, void* d_gate, int64_t n8,
@@ -466,10 +475,9 @@ cudaError_t launch_gate_bwd(const void* dy, const void* out, const void* gate, v
 {
     if (n8 == 0) return cudaSuccess;
     if ((n8 & 1) == 0 && all_aligned32({dy, out, gate, d_out, d_gate}))
-        hydra_gate_bwd_kernel<8><<<grid_for(n8 / 2, 256), 256, 0, stream>>>(dy, out, gate, d_out, d_gate, n8 / 2);
+        return launch_overlapped(hydra_gate_bwd_kernel<8>, grid_for(n8 / 2, 256), 256, 0, stream, dy, out, gate, d_out, d_gate, n8 / 2);
     else
-        hydra_gate_bwd_kernel<4><<<grid_for(n8, 256), 256, 0, stream>>>(dy, out, gate, d_out, d_gate, n8);
-    return cudaGetLastError();
+        return launch_overlapped(hydra_gate_bwd_kernel<4>, grid_for(n8, 256), 256, 0, stream, dy, out, gate, d_out, d_gate, n8);
 }
 
 }  // namespace hydra
