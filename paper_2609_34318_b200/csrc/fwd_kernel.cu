@@ -8,12 +8,13 @@
 // value columns of V for O += P V), so three stages of K and of V fit next to the two Q tiles: deep
 // enough to cover the latency of a TMA load, which two full-size stages could not.
 //
-// Warp roles per CTA (352 threads):
+// Warp roles per CTA (384 threads):
 //   warps 0-3   softmax of this CTA's rows of tile A: thread r owns row r = TMEM lane r
 //   warps 4-7   softmax of this CTA's rows of tile B
 //   warp  8     TMA producer of Q (per item) and K
 //   warp  9     TMA producer of V
 //   warp 10     leader CTA only: UMMA issuer (one thread); both CTAs: TMEM allocation
+//   warp 11     idle
 // Barriers live at the same shared-memory offsets in both CTAs. "Full" barriers are used in the
 // leader's copy (both CTAs' TMA loads count their bytes there; both CTAs' softmax warps arrive
 // there); "done" events of the tensor core are committed to both copies at once.
@@ -52,7 +53,10 @@ namespace {
 
 constexpr int kDqk = HYDRA_KERNEL_DQK;
 constexpr int kQkBoxes = kDqk / 64;                    // 64-column boxes of a q / k row
-constexpr int kThreads = 352;
+constexpr int kThreads = 384;                         // three warpgroups (one warp idle): registers move between whole warpgroups
+// Registers per thread: 168 at launch (65,536 / 384, rounded down to a multiple of 8), then 208 for the two softmax
+// warpgroups and 88 for the producers and the issuer: 256 * 208 + 128 * 88 = 384 * 168.
+constexpr int kRegsSoftmax = 208, kRegsOthers = 88;
 constexpr int kWarpK = 8, kWarpV = 9, kWarpMma = 10;
 constexpr uint32_t kBox = 128 * 128;                  // [128 rows x 64 bf16] = 16 KB
 constexpr uint32_t kHalfBox = 64 * 128;               // [ 64 rows x 64 bf16] =  8 KB
@@ -151,6 +155,8 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
         return idx;
     };
 
+    if (warp >= 8) {
+    regs_decrease<kRegsOthers>();
     if (warp == kWarpK) {
         // ------------------------------------------------------------------ Q and K producer
         if (lane == 0) {
@@ -327,7 +333,9 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
                 }
             }
         }
+    }
     } else {
+        regs_increase<kRegsSoftmax>();
         // ------------------------------------------------------------------ softmax warpgroups
         const int t = warp >> 2;                       // tile A or B
         const int r = tid & 127;                       // row inside this CTA's half of the tile = TMEM lane
@@ -374,27 +382,25 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
                     if (p.causal) jmax = min(jmax, row + pr.off);
                     cmax = jmax - col0;
                 }
-                // pass 1: row maximum, 64 columns at a time (the 168 registers a thread may use do not
-                // hold a whole row of S next to the probabilities without spilling)
+                // The whole row of S goes to registers once: it is read from tensor memory once, masked once, and its
+                // maximum and then its probabilities are taken from there (the 208 registers these warps hold after
+                // the split below have room for it; at 168 it took two passes of 64 columns each).
+                uint32_t s[TILE];
+#pragma unroll
+                for (int c0 = 0; c0 < TILE; c0 += 32) tmem_ld_x32(tm_s + c0, s + c0);
+                tmem_wait_ld();
+                if (need_mask) {
+#pragma unroll
+                    for (int c = 0; c < TILE; ++c)
+                        if (c > cmax) s[c] = __float_as_uint(neg_inf());
+                }
                 float mx0 = neg_inf(), mx1 = neg_inf(), mx2 = neg_inf(), mx3 = neg_inf();
 #pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    uint32_t s[TILE / 2];
-                    tmem_ld_x32(tm_s + half * 64, s);
-                    tmem_ld_x32(tm_s + half * 64 + 32, s + 32);
-                    tmem_wait_ld();
-                    if (need_mask) {
-#pragma unroll
-                        for (int c = 0; c < TILE / 2; ++c)
-                            if (half * 64 + c > cmax) s[c] = __float_as_uint(neg_inf());
-                    }
-#pragma unroll
-                    for (int c = 0; c < TILE / 2; c += 8) {
-                        mx0 = fmax3(mx0, __uint_as_float(s[c]), __uint_as_float(s[c + 1]));
-                        mx1 = fmax3(mx1, __uint_as_float(s[c + 2]), __uint_as_float(s[c + 3]));
-                        mx2 = fmax3(mx2, __uint_as_float(s[c + 4]), __uint_as_float(s[c + 5]));
-                        mx3 = fmax3(mx3, __uint_as_float(s[c + 6]), __uint_as_float(s[c + 7]));
-                    }
+                for (int c = 0; c < TILE; c += 8) {
+                    mx0 = fmax3(mx0, __uint_as_float(s[c]), __uint_as_float(s[c + 1]));
+                    mx1 = fmax3(mx1, __uint_as_float(s[c + 2]), __uint_as_float(s[c + 3]));
+                    mx2 = fmax3(mx2, __uint_as_float(s[c + 4]), __uint_as_float(s[c + 5]));
+                    mx3 = fmax3(mx3, __uint_as_float(s[c + 6]), __uint_as_float(s[c + 7]));
                 }
                 const float m_new = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3)) * p.scale_log2;
                 float alpha = 1.f;
@@ -418,37 +424,22 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
                         tmem_st_x32(tm_o + c0, o);
                     }
                 }
-                // pass 2: P = exp2(S * c - m) as packed bf16, written over the first half of S and handed
-                // to the tensor core in two instalments (columns [0,64), then [64,128)).
+                // P = exp2(S * c - m) as packed bf16, written over the first half of S and handed to the tensor core in
+                // two instalments (columns [0,64), then [64,128)). Masked scores are -inf, their probability is 0 by
+                // itself.
                 float rs0 = 0.f, rs1 = 0.f;
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
-                    uint32_t s[TILE / 2], pk[TILE / 4];
-                    tmem_ld_x32(tm_s + half * 64, s);
-                    tmem_ld_x32(tm_s + half * 64 + 32, s + 32);
-                    tmem_wait_ld();
-                    if (need_mask) {
+                    uint32_t pk[TILE / 4];
 #pragma unroll
-                        for (int c = 0; c < TILE / 2; c += 2) {
-                            float p0 = ex2_approx(fmaf(__uint_as_float(s[c]), p.scale_log2, -m_use));
-                            float p1 = ex2_approx(fmaf(__uint_as_float(s[c + 1]), p.scale_log2, -m_use));
-                            if (half * 64 + c > cmax) p0 = 0.f;
-                            if (half * 64 + c + 1 > cmax) p1 = 0.f;
-                            rs0 += p0;
-                            rs1 += p1;
-                            pk[c >> 1] = pack_bf16x2(p0, p1);
-                        }
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < TILE / 2; c += 2) {
-                            float x0, x1;
-                            ffma2(x0, x1, __uint_as_float(s[c]), __uint_as_float(s[c + 1]), p.scale_log2, p.scale_log2,
-                                  -m_use, -m_use);
-                            const float p0 = ex2_approx(x0);
-                            const float p1 = ex2_approx(x1);
-                            fadd2(rs0, rs1, rs0, rs1, p0, p1);
-                            pk[c >> 1] = pack_bf16x2(p0, p1);
-                        }
+                    for (int c = 0; c < TILE / 2; c += 2) {
+                        float x0, x1;
+                        ffma2(x0, x1, __uint_as_float(s[half * 64 + c]), __uint_as_float(s[half * 64 + c + 1]), p.scale_log2,
+                              p.scale_log2, -m_use, -m_use);
+                        const float p0 = ex2_approx(x0);
+                        const float p1 = ex2_approx(x1);
+                        fadd2(rs0, rs1, rs0, rs1, p0, p1);
+                        pk[c >> 1] = pack_bf16x2(p0, p1);
                     }
                     tmem_st_x32(tm_s + half * 32, pk);
                     tmem_wait_st();

@@ -141,7 +141,7 @@ struct ClockProbe {
 // as all of its own have started (they take the SMs that its first finished blocks leave) and waits, before it
 // touches global memory, until the launch before it has completed and its results are visible. What is hidden
 // that way is the launch itself, the barriers' and tensor memory's set-up and the wait for the last block: a step of
-// four sequences of 7 to 300 tokens 42 -> 35 us, of 1024 tokens in short ones 49 -> 42 us, the twelve launches around the
+// four sequences of 7 to 300 tokens 42 -> 35 us, of 1024 tokens in short ones 49 -> 42 us, the ten launches around the
 // attention of a 4096-token MLA block 813 -> 794 us. Kernels of other libraries before or after are ordered
 // as usual.
 #ifdef __CUDACC__

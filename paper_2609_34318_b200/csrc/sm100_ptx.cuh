@@ -162,6 +162,13 @@ __device__ __forceinline__ bool counter_wait(const volatile uint32_t* counter, u
     return true;
 }
 
+// Registers per thread of the executing warpgroup (all of its warps execute the same one): an increase draws on what
+// the other warpgroups of the block have given up of the registers the block was launched with.
+template <int kRegs>
+__device__ __forceinline__ void regs_increase() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegs)); }
+template <int kRegs>
+__device__ __forceinline__ void regs_decrease() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegs)); }
+
 // ----------------------------------------------------------------------------------------------
 // TMA: tiled loads of a box into shared memory, completion counted in bytes on an mbarrier
 // ----------------------------------------------------------------------------------------------
