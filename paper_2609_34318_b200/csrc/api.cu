@@ -421,15 +421,16 @@ void arena_note_use(const Plan& plan, int device, cudaStream_t stream)
 // Pairs whose q range and kv range are both at most this long go to the short-sequence forward kernel
 // (0: none do; negative: chosen by the library from the head layout). See build_fwd.
 std::atomic<int32_t> g_fwd_short_len{-1};
-// Where the two forward kernels take equal time on sequences of one length (32K tokens, 16 heads, two GPUs of
-// the pool): with a K / V head per query head at d_qk = 192 between 2048 and 3072 tokens; with shared K / V
-// heads, or at d_qk = 128 (where a slot of the short-sequence kernel has room for a second V stage), between
-// 4096 and 8192, and the 32K packed workload (sequences up to 4441 tokens) runs 11-15 % faster on it.
+// Where the two forward kernels take equal time on sequences of one length (32K tokens, 16 heads; ms, short-sequence /
+// CTA pairs): with a K / V head per query head at d_qk = 192, 0.165 / 0.191 at 512 tokens, 0.242 / 0.250 at 1024,
+// 0.326 / 0.316 at 1489, 0.399 / 0.373 at 2048; with shared K / V heads 0.225 / 0.252 at 1024, 0.379 / 0.373 at 2048,
+// 0.677 / 0.620 at 4096; at d_qk = 128 (where a slot of the short-sequence kernel has room for a second V stage)
+// 0.208 / 0.229 at 1024, 0.340 / 0.341 at 2048, 0.608 / 0.561 at 4096.
 int32_t fwd_short_len_for(const Problem& pb)
 {
     const int32_t set = g_fwd_short_len.load();
     if (set >= 0) return set;
-    return (pb.dqk == D_QK && pb.kv_group == 1) ? 2048 : 4608;
+    return (pb.dqk == D_QK && pb.kv_group == 1) ? 1280 : 2048;
 }
 static_assert(FWD_SHORT_KEYS == SUB, "the short forward kernel reads K through the 64-row map of the CTA-pair kernel");
 

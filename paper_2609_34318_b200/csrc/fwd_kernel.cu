@@ -353,18 +353,23 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
             const int row0 = item.q0 + t * 2 * TILE + static_cast<int>(rank) * TILE;   // first row of this CTA
             const int row = row0 + r;                  // q row inside the pair
             const bool row_valid = row < pr.q_len;
-            const int64_t rows_total = pr.to_part ? p.part_rows : p.T;
-            __nv_bfloat16* obase = static_cast<__nv_bfloat16*>(pr.to_part ? p.o_part : p.out);
-            float* lbase = pr.to_part ? p.lse_part : p.lse;
-            const int64_t orow = static_cast<int64_t>(pr.out_row0) + row;
-            uint4* dst = reinterpret_cast<uint4*>(obase + (orow * p.h + item.head) * D_V);
-            float* lse_dst = lbase + static_cast<int64_t>(item.head) * rows_total + orow;
+            const int orow = pr.out_row0 + row;
+            // (formed where they are used: the loop over kv tiles has no registers to spare for pointers)
+            auto out_ptr = [&]() {
+                __nv_bfloat16* obase = static_cast<__nv_bfloat16*>(pr.to_part ? p.o_part : p.out);
+                return reinterpret_cast<uint4*>(obase + (static_cast<int64_t>(orow) * p.h + item.head) * D_V);
+            };
+            auto lse_ptr = [&]() {
+                float* lbase = pr.to_part ? p.lse_part : p.lse;
+                return lbase + static_cast<int64_t>(item.head) * (pr.to_part ? p.part_rows : p.T) + orow;
+            };
 
             if (n_kv <= 0) {                           // rows that see no key: O = 0, LSE = -inf
                 if (row_valid && n_kv == 0) {           // (n_kv < 0: no such tile in this item)
+                    uint4* dst = out_ptr();
 #pragma unroll
                     for (int e = 0; e < D_V / 8; ++e) dst[e] = make_uint4(0u, 0u, 0u, 0u);
-                    *lse_dst = neg_inf();
+                    *lse_ptr() = neg_inf();
                 }
                 continue;
             }
@@ -415,13 +420,13 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
                     // P V of this tile has landed: it was issued before this tile's S, which has
                     // completed, and the tensor pipe runs in issue order.
 #pragma unroll
-                    for (int c0 = 0; c0 < D_V; c0 += 32) {
-                        uint32_t o[32];
-                        tmem_ld_x32(tm_o + c0, o);
+                    for (int c0 = 0; c0 < D_V; c0 += 16) {  // 16 columns: the row of S is in registers next to them
+                        uint32_t o[16];
+                        tmem_ld_x16(tm_o + c0, o);
                         tmem_wait_ld();
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-                        tmem_st_x32(tm_o + c0, o);
+                        for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+                        tmem_st_x16(tm_o + c0, o);
                     }
                 }
                 // P = exp2(S * c - m) as packed bf16, written over the first half of S and handed to the tensor core in
@@ -455,6 +460,7 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
             if (!ok) break;
             tc_fence_after_sync();
             const float inv_l = (l_run > 0.f) ? 1.f / l_run : 0.f;
+            uint4* dst = out_ptr();
             const bool wide = (reinterpret_cast<uintptr_t>(dst) & 31u) == 0;
 #pragma unroll
             for (int c0 = 0; c0 < D_V; c0 += 32) {
@@ -485,7 +491,7 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
                 }
             }
             if (row_valid)
-                *lse_dst = (l_run > 0.f) ? (m_run + __log2f(l_run)) * 0.6931471805599453f : neg_inf();
+                *lse_ptr() = (l_run > 0.f) ? (m_run + __log2f(l_run)) * 0.6931471805599453f : neg_inf();
         }
     }
 
