@@ -195,6 +195,12 @@ constexpr uint32_t kDsStage = kDO + kStages * 2 * kBox64;    // 8 warps x 2 KB: 
 constexpr uint32_t kTotal = kDsStage + 8 * 2048;             // 221,184 B at d_qk = 192
 constexpr uint32_t kTmDK = 0, kTmDV = 192, kTmS = 320, kTmDP = 384, kTmP = 448, kTmDS = 480,
                    kTmCols = 512;
+// What bounds a sub-tile is shared memory: per 64 q rows the score products read 6 KB per UMMA (4 of K or V, 2 of Q or
+// dO), 120 KB at d_qk = 192, the updates 40 KB, and the loads write 40 KB. At d_qk = 128 the columns that dK leaves
+// free are a 128 x 128 bf16 tile: K is copied there once per item, S = K Q^T takes it from tensor memory, and its
+// UMMAs read 2 KB each instead of 6 (a third of what the score products read).
+constexpr bool kKInTmem = kDqk == 128;
+constexpr uint32_t kTmK = kTmDK + 128;
 enum : int { B_KVFULL = 0, B_KVEMPTY = 1, B_QFULL = 2, B_STAT = 5, B_QEMPTY = 8, B_SFULL = 11,
              B_SFREE = 12, B_PFULL = 13, B_PDSFREE = 14, B_ACCFREE = 15, B_ITEMFULL = 16, B_ITEMEMPTY = 16 + kSched,
              B_COUNT = 16 + 2 * kSched };
@@ -837,6 +843,16 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                 if (!si.valid()) continue;
                 if (issue_scores) {
                     ok = wait(B_KVFULL, items);
+                    // (every score product of the previous item has completed: this item's K was loaded behind them)
+                    if (kKInTmem && ok) {
+                        tc_fence_after_sync();
+                        if (elect_one()) {
+#pragma unroll
+                            for (int kk = 0; kk < kDqk / 16; ++kk)
+                                umma_copy_a_w(tm + kTmK + kk * 8, k_lo + (kk >> 2) * (kBox128 >> 4) + (kk & 3) * 2, hi_kmaj);
+                        }
+                        __syncwarp();
+                    }
                     for (; si.valid() && ok;) {
                         // the poll that is almost always satisfied (Q / dO landed stages ago) and the
                         // address arithmetic come first; the wait on the critical path (S / dP of the
@@ -853,9 +869,12 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                         tc_fence_after_sync();
                         if (elect_one()) {
 #pragma unroll
-                            for (int kk = 0; kk < kDqk / 16; ++kk)
-                                umma_ss_w(tm + kTmS, k_lo + (kk >> 2) * (kBox128 >> 4) + (kk & 3) * 2, hi_kmaj,
-                                          q_lo + (kk >> 2) * (kBox64 >> 4) + (kk & 3) * 2, hi_kmaj, idesc_st, kk > 0);
+                            for (int kk = 0; kk < kDqk / 16; ++kk) {
+                                const uint32_t b_lo = q_lo + (kk >> 2) * (kBox64 >> 4) + (kk & 3) * 2;
+                                if (kKInTmem) umma_ts_w(tm + kTmS, tm + kTmK + kk * 8, b_lo, hi_kmaj, idesc_st, kk > 0);
+                                else umma_ss_w(tm + kTmS, k_lo + (kk >> 2) * (kBox128 >> 4) + (kk & 3) * 2, hi_kmaj, b_lo, hi_kmaj,
+                                               idesc_st, kk > 0);
+                            }
 #pragma unroll
                             for (int kk = 0; kk < D_V / 16; ++kk)
                                 umma_ss_w(tm + kTmDP, v_lo + (kk >> 2) * (kBox128 >> 4) + (kk & 3) * 2, hi_kmaj,

@@ -417,6 +417,16 @@ __device__ __forceinline__ void umma_ts_w(uint32_t d_tmem, uint32_t a_tmem, uint
         "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+// Shared memory -> tensor memory: 128 rows x 32 bytes of a K-major tile, the descriptor of a UMMA's A operand, to 8
+// columns, where a UMMA takes them as its A operand. Issued by the thread that issues the UMMAs; a copy and the UMMAs
+// after it execute in issue order.
+__device__ __forceinline__ void umma_copy_a_w(uint32_t tmem, uint32_t a_lo, uint32_t a_hi) {
+    asm volatile(
+        "{\n\t.reg .b64 da;\n\t"
+        "mov.b64 da, {%1, %2};\n\t"
+        "tcgen05.cp.cta_group::1.128x256b [%0], da;\n\t}" ::"r"(tmem), "r"(a_lo), "r"(a_hi)
+        : "memory");
+}
 // The mbarrier gets one arrival when every UMMA issued so far by this thread has completed.
 // Implies tcgen05.fence::before_thread_sync.
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
