@@ -886,19 +886,22 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                     }
                 } else {
                     bool first_step = true;
-                    for (; si.valid() && ok; si.next()) {
-                        ok = wait(B_PFULL, n_step);
-                        if (ok && first_step && items > 0) ok = wait(B_ACCFREE, items - 1u);
+                    while (si.valid() && ok) {
+                        // Everything that can be formed before P and dS are there is: what follows the wait stands between
+                        // them and their updates (with the step to the next sub-tile behind the wait the tensor pipe
+                        // idled 250 cycles per sub-tile at d_qk = 128).
+                        const int st = n_step % kStages;
+                        si.next();
+                        const bool more = si.valid();
+                        if (first_step && items > 0) ok = wait(B_ACCFREE, items - 1u);
                         // Order hint, not a data dependency: let the score products of the NEXT sub-tile of
                         // this item enter the tensor pipe first. They are what the elementwise warps wait
                         // for next; these updates then fill the gap in which S / dP are copied out,
                         // instead of interleaving with the score products and delaying them.
-                        SubIter peek = si;
-                        peek.next();
-                        if (ok && peek.valid()) ok = counter_wait(bursts_p, n_step + 2u, abort_p, limit);
+                        if (ok && more) ok = counter_wait(bursts_p, n_step + 2u, abort_p, limit);
+                        if (ok) ok = wait(B_PFULL, n_step);
                         if (!ok) break;
                         tc_fence_after_sync();
-                        const int st = n_step % kStages;
                         const uint32_t do_lo = domn_lo0 + st * (2 * kBox64 >> 4), q_lo = qmn_lo0 + st * (kQkBoxes * kBox64 >> 4);
                         const uint32_t acc = first_step ? 0u : 1u;
                         if (elect_one()) {
