@@ -195,26 +195,40 @@ KERNEL_KINDS = ("fwd", "merge", "bwd_prep", "bwd_dkv", "bwd_dq", "grad_cast", "u
 # ------------------------------------------------------------------------------------------------
 def _ptr(x) -> Optional[int]:
     """Device pointer of a torch tensor, or the integer / None passed through."""
-    if x is None:
-        return None
-    if isinstance(x, int):
+    if x is None or isinstance(x, int):
         return x
     if not x.is_cuda or not x.is_contiguous():
         raise ValueError("tensors must be contiguous CUDA tensors")
     return x.data_ptr()
 
 
+_current_raw_stream = None      # current stream of the current device, as an integer
+
+
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        global _current_raw_stream
+        if _current_raw_stream is None:
+            import torch
+            # without the Stream object that torch.cuda.current_stream() makes (1 us of a call that takes 10)
+            raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+            _current_raw_stream = (lambda: torch.cuda.current_stream().cuda_stream) if raw is None else \
+                (lambda: raw(torch.cuda.current_device()))
+        return _current_raw_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
 
 
 def _cu(cu_seqlens) -> np.ndarray:
+    if type(cu_seqlens) is np.ndarray and cu_seqlens.dtype == np.int32 and cu_seqlens.flags.c_contiguous:
+        return cu_seqlens
     return np.ascontiguousarray(np.asarray(cu_seqlens, dtype=np.int32))
+
+
+def _addr(array: np.ndarray) -> int:
+    """Address of an array's data (array.ctypes.data makes a ctypes object on the way: three times as long)."""
+    return array.__array_interface__["data"][0]
 
 
 def as_pairs(pairs) -> Optional[np.ndarray]:
@@ -239,7 +253,7 @@ def _pairs_arg(pairs) -> Tuple[Optional[int], int, Optional[np.ndarray]]:
     arr = as_pairs(pairs)
     if arr is None:
         return None, 0, None
-    return arr.ctypes.data, len(arr), arr
+    return _addr(arr), len(arr), arr
 
 
 def _check(status: int, where: str) -> None:
@@ -283,7 +297,7 @@ def hydra_plan_build_seconds(which: int, cu_seqlens, n_heads: int, pairs=None, c
     """Host-only: seconds to build the (uncached) work tables of one call of kind `which` for this problem."""
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
-    return float(_lib.hydra_plan_build_seconds(which, cu.ctypes.data, len(cu) - 1, n_heads, pp, npairs, int(bool(causal))))
+    return float(_lib.hydra_plan_build_seconds(which, _addr(cu), len(cu) - 1, n_heads, pp, npairs, int(bool(causal))))
 
 
 def hydra_set_plan_prefetch(on: bool) -> None:
@@ -317,7 +331,7 @@ def hydra_zigzag_pairs(cu_seqlens, cp_r):
     per_seq = None if isinstance(cp_r, (int, np.integer)) else np.ascontiguousarray(cp_r, dtype=np.int32)
     all_r = int(cp_r) if per_seq is None else 0
     n_pairs, part_rows = ctypes.c_int32(0), ctypes.c_int64(0)
-    s = _lib.hydra_zigzag_pairs(cu.ctypes.data, n, None if per_seq is None else per_seq.ctypes.data, all_r,
+    s = _lib.hydra_zigzag_pairs(_addr(cu), n, None if per_seq is None else per_seq.ctypes.data, all_r,
                                 None, 0, ctypes.addressof(n_pairs), ctypes.addressof(part_rows), None, None)
     if s not in (HYDRA_OK, HYDRA_ERR_WORKSPACE_TOO_SMALL):
         raise HydraError(s, "hydra_zigzag_pairs")
@@ -325,7 +339,7 @@ def hydra_zigzag_pairs(cu_seqlens, cp_r):
     rank = np.zeros(n_pairs.value, dtype=np.int32)
     step = np.zeros(n_pairs.value, dtype=np.int32)
     if n_pairs.value:
-        _check(_lib.hydra_zigzag_pairs(cu.ctypes.data, n, None if per_seq is None else per_seq.ctypes.data,
+        _check(_lib.hydra_zigzag_pairs(_addr(cu), n, None if per_seq is None else per_seq.ctypes.data,
                                        all_r, pairs.ctypes.data, len(pairs), ctypes.addressof(n_pairs),
                                        ctypes.addressof(part_rows), rank.ctypes.data, step.ctypes.data),
                "hydra_zigzag_pairs")
@@ -337,7 +351,7 @@ def hydra_bwd_bands(cu_seqlens, n_heads: int, pairs, causal: bool, scratch_bytes
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
     n_out, n_bands = ctypes.c_int32(0), ctypes.c_int32(0)
-    args = (cu.ctypes.data, len(cu) - 1, n_heads, pp, npairs, int(bool(causal)), int(scratch_bytes))
+    args = (_addr(cu), len(cu) - 1, n_heads, pp, npairs, int(bool(causal)), int(scratch_bytes))
     s = _lib.hydra_bwd_bands(*args, None, None, 0, ctypes.addressof(n_out), ctypes.addressof(n_bands))
     if s not in (HYDRA_OK, HYDRA_ERR_WORKSPACE_TOO_SMALL):
         raise HydraError(s, "hydra_bwd_bands")
@@ -352,7 +366,7 @@ def hydra_bwd_bands(cu_seqlens, n_heads: int, pairs, causal: bool, scratch_bytes
 def hydra_workspace_bytes(which: int, cu_seqlens, n_heads: int, pairs=None) -> int:
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
-    return int(_lib.hydra_workspace_bytes(which, cu.ctypes.data, len(cu) - 1, n_heads, pp, npairs))
+    return int(_lib.hydra_workspace_bytes(which, _addr(cu), len(cu) - 1, n_heads, pp, npairs))
 
 
 def hydra_attn_fwd(q, k, v, cu_seqlens, n_heads: int, pairs, causal: bool, softmax_scale: float, out, lse,
@@ -361,9 +375,9 @@ def hydra_attn_fwd(q, k, v, cu_seqlens, n_heads: int, pairs, causal: bool, softm
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
     if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
-    s = _lib.hydra_attn_fwd(_ptr(q), _ptr(k), _ptr(v), cu.ctypes.data, len(cu) - 1, n_heads, pp, npairs,
-                            int(bool(causal)), ctypes.c_float(float(softmax_scale)), _ptr(out), _ptr(lse),
+        workspace_bytes = workspace.nbytes
+    s = _lib.hydra_attn_fwd(_ptr(q), _ptr(k), _ptr(v), _addr(cu), len(cu) - 1, n_heads, pp, npairs,
+                            int(bool(causal)), float(softmax_scale), _ptr(out), _ptr(lse),
                             _ptr(o_part), _ptr(lse_part), int(part_rows), _ptr(workspace),
                             int(workspace_bytes), _stream(stream))
     if check:
@@ -376,8 +390,8 @@ def hydra_lse_merge(o_part, lse_part, part_rows: int, cu_seqlens, n_heads: int, 
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
     if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
-    s = _lib.hydra_lse_merge(_ptr(o_part), _ptr(lse_part), int(part_rows), cu.ctypes.data, len(cu) - 1,
+        workspace_bytes = workspace.nbytes
+    s = _lib.hydra_lse_merge(_ptr(o_part), _ptr(lse_part), int(part_rows), _addr(cu), len(cu) - 1,
                              n_heads, pp, npairs, _ptr(out), _ptr(lse), _ptr(workspace),
                              int(workspace_bytes), _stream(stream))
     if check:
@@ -392,8 +406,8 @@ def hydra_lse_merge_accumulate(o_part, lse_part, part_rows: int, cu_seqlens, n_h
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
     if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
-    s = _lib.hydra_lse_merge_accumulate(_ptr(o_part), _ptr(lse_part), int(part_rows), cu.ctypes.data,
+        workspace_bytes = workspace.nbytes
+    s = _lib.hydra_lse_merge_accumulate(_ptr(o_part), _ptr(lse_part), int(part_rows), _addr(cu),
                                         len(cu) - 1, n_heads, pp, npairs, _ptr(out), _ptr(lse), _ptr(workspace),
                                         int(workspace_bytes), _stream(stream))
     if check:
@@ -407,10 +421,10 @@ def hydra_attn_bwd(q, k, v, out, lse, dout, cu_seqlens, n_heads: int, pairs, cau
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
     if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
-    s = _lib.hydra_attn_bwd(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), _ptr(dout), cu.ctypes.data,
+        workspace_bytes = workspace.nbytes
+    s = _lib.hydra_attn_bwd(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), _ptr(dout), _addr(cu),
                             len(cu) - 1, n_heads, pp, npairs, int(bool(causal)),
-                            ctypes.c_float(float(softmax_scale)), _ptr(dq), _ptr(dk), _ptr(dv),
+                            float(softmax_scale), _ptr(dq), _ptr(dk), _ptr(dv),
                             _ptr(workspace), int(workspace_bytes), _stream(stream))
     if check:
         _check(s, "hydra_attn_bwd")
@@ -424,10 +438,10 @@ def hydra_attn_bwd_accumulate(q, k, v, out, lse, dout, cu_seqlens, n_heads: int,
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
     if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
+        workspace_bytes = workspace.nbytes
     s = _lib.hydra_attn_bwd_accumulate(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), _ptr(dout),
-                                       cu.ctypes.data, len(cu) - 1, n_heads, pp, npairs, int(bool(causal)),
-                                       ctypes.c_float(float(softmax_scale)), _ptr(dq_acc), _ptr(dk_acc),
+                                       _addr(cu), len(cu) - 1, n_heads, pp, npairs, int(bool(causal)),
+                                       float(softmax_scale), _ptr(dq_acc), _ptr(dk_acc),
                                        _ptr(dv_acc), _ptr(workspace), int(workspace_bytes), _stream(stream))
     if check:
         _check(s, "hydra_attn_bwd_accumulate")
@@ -441,9 +455,9 @@ def hydra_attn_fwd_gqa(q, k, v, cu_seqlens, n_heads: int, n_kv_heads: int, pairs
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
     if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
-    s = _lib.hydra_attn_fwd_gqa(_ptr(q), _ptr(k), _ptr(v), cu.ctypes.data, len(cu) - 1, n_heads, n_kv_heads, pp,
-                                npairs, int(bool(causal)), ctypes.c_float(float(softmax_scale)), _ptr(out),
+        workspace_bytes = workspace.nbytes
+    s = _lib.hydra_attn_fwd_gqa(_ptr(q), _ptr(k), _ptr(v), _addr(cu), len(cu) - 1, n_heads, n_kv_heads, pp,
+                                npairs, int(bool(causal)), float(softmax_scale), _ptr(out),
                                 _ptr(lse), _ptr(o_part), _ptr(lse_part), int(part_rows), _ptr(workspace),
                                 int(workspace_bytes), _stream(stream))
     if check:
@@ -454,7 +468,7 @@ def hydra_attn_fwd_gqa(q, k, v, cu_seqlens, n_heads: int, n_kv_heads: int, pairs
 def hydra_workspace_bytes_gqa(which: int, cu_seqlens, n_heads: int, n_kv_heads: int, pairs=None) -> int:
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
-    return int(_lib.hydra_workspace_bytes_gqa(which, cu.ctypes.data, len(cu) - 1, n_heads, n_kv_heads, pp, npairs))
+    return int(_lib.hydra_workspace_bytes_gqa(which, _addr(cu), len(cu) - 1, n_heads, n_kv_heads, pp, npairs))
 
 
 def hydra_attn_bwd_gqa(q, k, v, out, lse, dout, cu_seqlens, n_heads: int, n_kv_heads: int, pairs, causal: bool,
@@ -464,10 +478,10 @@ def hydra_attn_bwd_gqa(q, k, v, out, lse, dout, cu_seqlens, n_heads: int, n_kv_h
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
     if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
-    s = _lib.hydra_attn_bwd_gqa(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), _ptr(dout), cu.ctypes.data,
+        workspace_bytes = workspace.nbytes
+    s = _lib.hydra_attn_bwd_gqa(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), _ptr(dout), _addr(cu),
                                 len(cu) - 1, n_heads, n_kv_heads, pp, npairs, int(bool(causal)),
-                                ctypes.c_float(float(softmax_scale)), _ptr(dq), _ptr(dk), _ptr(dv),
+                                float(softmax_scale), _ptr(dq), _ptr(dk), _ptr(dv),
                                 _ptr(workspace), int(workspace_bytes), _stream(stream))
     if check:
         _check(s, "hydra_attn_bwd_gqa")
@@ -481,10 +495,10 @@ def hydra_attn_bwd_accumulate_gqa(q, k, v, out, lse, dout, cu_seqlens, n_heads: 
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
     if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
+        workspace_bytes = workspace.nbytes
     s = _lib.hydra_attn_bwd_accumulate_gqa(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), _ptr(dout),
-                                           cu.ctypes.data, len(cu) - 1, n_heads, n_kv_heads, pp, npairs,
-                                           int(bool(causal)), ctypes.c_float(float(softmax_scale)), _ptr(dq_acc),
+                                           _addr(cu), len(cu) - 1, n_heads, n_kv_heads, pp, npairs,
+                                           int(bool(causal)), float(softmax_scale), _ptr(dq_acc),
                                            _ptr(dk_acc), _ptr(dv_acc), _ptr(workspace), int(workspace_bytes),
                                            _stream(stream))
     if check:
@@ -496,7 +510,7 @@ def hydra_workspace_bytes_dims(which: int, cu_seqlens, n_heads: int, n_kv_heads:
                                pairs=None) -> int:
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
-    return int(_lib.hydra_workspace_bytes_dims(which, cu.ctypes.data, len(cu) - 1, n_heads, n_kv_heads, int(d_qk),
+    return int(_lib.hydra_workspace_bytes_dims(which, _addr(cu), len(cu) - 1, n_heads, n_kv_heads, int(d_qk),
                                                int(d_v), pp, npairs))
 
 
@@ -507,10 +521,10 @@ def hydra_attn_fwd_dims(q, k, v, cu_seqlens, n_heads: int, n_kv_heads: int, d_qk
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
     if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
-    s = _lib.hydra_attn_fwd_dims(_ptr(q), _ptr(k), _ptr(v), cu.ctypes.data, len(cu) - 1, n_heads, n_kv_heads,
+        workspace_bytes = workspace.nbytes
+    s = _lib.hydra_attn_fwd_dims(_ptr(q), _ptr(k), _ptr(v), _addr(cu), len(cu) - 1, n_heads, n_kv_heads,
                                  int(d_qk), int(d_v), pp, npairs, int(bool(causal)),
-                                 ctypes.c_float(float(softmax_scale)), _ptr(out), _ptr(lse), _ptr(o_part),
+                                 float(softmax_scale), _ptr(out), _ptr(lse), _ptr(o_part),
                                  _ptr(lse_part), int(part_rows), _ptr(workspace), int(workspace_bytes),
                                  _stream(stream))
     if check:
@@ -523,10 +537,10 @@ def _bwd_dims(fn_name, q, k, v, out, lse, dout, cu_seqlens, n_heads, n_kv_heads,
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
     if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
-    s = getattr(_lib, fn_name)(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), _ptr(dout), cu.ctypes.data,
+        workspace_bytes = workspace.nbytes
+    s = getattr(_lib, fn_name)(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), _ptr(dout), _addr(cu),
                                len(cu) - 1, n_heads, n_kv_heads, int(d_qk), int(d_v), pp, npairs,
-                               int(bool(causal)), ctypes.c_float(float(softmax_scale)), _ptr(dq), _ptr(dk),
+                               int(bool(causal)), float(softmax_scale), _ptr(dq), _ptr(dk),
                                _ptr(dv), _ptr(workspace), int(workspace_bytes), _stream(stream))
     if check:
         _check(s, fn_name)
@@ -555,7 +569,7 @@ def hydra_mla_rope(x, positions, n_tokens: int, n_heads: int, head_dim: int, rop
                    theta: float, inverse: bool, y, stream=None, check: bool = True) -> int:
     """Rotary embedding of columns [rope_offset, rope_offset + rope_dim) of every head (y may be x)."""
     s = _lib.hydra_mla_rope(_ptr(x), _ptr(positions), int(n_tokens), n_heads, head_dim, rope_offset, rope_dim,
-                            ctypes.c_float(float(theta)), int(bool(inverse)), _ptr(y), _stream(stream))
+                            float(theta), int(bool(inverse)), _ptr(y), _stream(stream))
     if check:
         _check(s, "hydra_mla_rope")
     return s
@@ -565,7 +579,7 @@ def hydra_mla_kv_assemble(kv_up, k_pe, positions, n_tokens: int, n_heads: int, d
                           theta: float, k, v, stream=None, check: bool = True) -> int:
     """k = [key part of kv_up | rope(k_pe) shared by all heads], v = value part of kv_up."""
     s = _lib.hydra_mla_kv_assemble(_ptr(kv_up), _ptr(k_pe), _ptr(positions), int(n_tokens), n_heads, d_nope, d_rope,
-                                   d_v, ctypes.c_float(float(theta)), _ptr(k), _ptr(v), _stream(stream))
+                                   d_v, float(theta), _ptr(k), _ptr(v), _stream(stream))
     if check:
         _check(s, "hydra_mla_kv_assemble")
     return s
@@ -574,7 +588,7 @@ def hydra_mla_kv_assemble(kv_up, k_pe, positions, n_tokens: int, n_heads: int, d
 def hydra_mla_kv_assemble_bwd(dk, dv, positions, n_tokens: int, n_heads: int, d_nope: int, d_rope: int, d_v: int,
                               theta: float, dkv_up, dk_pe, stream=None, check: bool = True) -> int:
     s = _lib.hydra_mla_kv_assemble_bwd(_ptr(dk), _ptr(dv), _ptr(positions), int(n_tokens), n_heads, d_nope, d_rope,
-                                       d_v, ctypes.c_float(float(theta)), _ptr(dkv_up), _ptr(dk_pe), _stream(stream))
+                                       d_v, float(theta), _ptr(dkv_up), _ptr(dk_pe), _stream(stream))
     if check:
         _check(s, "hydra_mla_kv_assemble_bwd")
     return s
@@ -605,7 +619,7 @@ def hydra_workspace_bytes_local(which: int, cu_seqlens, n_heads: int, n_kv_heads
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
     t, _k2 = _tables(q_chunks, q_rows, kv_chunks, kv_rows)
-    return int(_lib.hydra_workspace_bytes_local(which, cu.ctypes.data, len(cu) - 1, n_heads, n_kv_heads, int(d_qk),
+    return int(_lib.hydra_workspace_bytes_local(which, _addr(cu), len(cu) - 1, n_heads, n_kv_heads, int(d_qk),
                                                 int(d_v), *t, pp, npairs))
 
 
@@ -618,10 +632,10 @@ def hydra_attn_fwd_local(q, k, v, cu_seqlens, n_heads: int, n_kv_heads: int, d_q
     pp, npairs, _keep = _pairs_arg(pairs)
     t, _k2 = _tables(q_chunks, q_rows, kv_chunks, kv_rows)
     if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
-    s = _lib.hydra_attn_fwd_local(_ptr(q), _ptr(k), _ptr(v), cu.ctypes.data, len(cu) - 1, n_heads, n_kv_heads,
+        workspace_bytes = workspace.nbytes
+    s = _lib.hydra_attn_fwd_local(_ptr(q), _ptr(k), _ptr(v), _addr(cu), len(cu) - 1, n_heads, n_kv_heads,
                                   int(d_qk), int(d_v), *t, pp, npairs, int(bool(causal)),
-                                  ctypes.c_float(float(softmax_scale)), _ptr(out), _ptr(lse), _ptr(o_part),
+                                  float(softmax_scale), _ptr(out), _ptr(lse), _ptr(o_part),
                                   _ptr(lse_part), int(part_rows), _ptr(workspace), int(workspace_bytes),
                                   _stream(stream))
     if check:
@@ -636,8 +650,8 @@ def hydra_lse_merge_local(o_part, lse_part, part_rows: int, cu_seqlens, n_heads:
     pp, npairs, _keep = _pairs_arg(pairs)
     qc = as_chunks(q_chunks)
     if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
-    s = _lib.hydra_lse_merge_local(_ptr(o_part), _ptr(lse_part), int(part_rows), cu.ctypes.data, len(cu) - 1, n_heads,
+        workspace_bytes = workspace.nbytes
+    s = _lib.hydra_lse_merge_local(_ptr(o_part), _ptr(lse_part), int(part_rows), _addr(cu), len(cu) - 1, n_heads,
                                    qc.ctypes.data, len(qc), int(q_rows), pp, npairs, int(bool(accumulate)), _ptr(out),
                                    _ptr(lse), _ptr(workspace), int(workspace_bytes), _stream(stream))
     if check:
@@ -653,10 +667,10 @@ def hydra_attn_bwd_accumulate_local(q, k, v, out, lse, dout, cu_seqlens, n_heads
     pp, npairs, _keep = _pairs_arg(pairs)
     t, _k2 = _tables(q_chunks, q_rows, kv_chunks, kv_rows)
     if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
+        workspace_bytes = workspace.nbytes
     s = _lib.hydra_attn_bwd_accumulate_local(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), _ptr(dout),
-                                             cu.ctypes.data, len(cu) - 1, n_heads, n_kv_heads, int(d_qk), int(d_v), *t,
-                                             pp, npairs, int(bool(causal)), ctypes.c_float(float(softmax_scale)),
+                                             _addr(cu), len(cu) - 1, n_heads, n_kv_heads, int(d_qk), int(d_v), *t,
+                                             pp, npairs, int(bool(causal)), float(softmax_scale),
                                              _ptr(dq_acc), _ptr(dk_acc), _ptr(dv_acc), _ptr(workspace),
                                              int(workspace_bytes), _stream(stream))
     if check:
@@ -737,7 +751,7 @@ def hydra_profile_collect():
 def hydra_host_step_arena_bytes(cu_seqlens, n_heads: int, pairs=None) -> int:
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
-    return int(_lib.hydra_host_step_arena_bytes(cu.ctypes.data, len(cu) - 1, n_heads, pp, npairs))
+    return int(_lib.hydra_host_step_arena_bytes(_addr(cu), len(cu) - 1, n_heads, pp, npairs))
 
 
 def _host_ptr(x) -> int:
@@ -761,8 +775,8 @@ def hydra_attn_fwd_bwd_host(q_host, k_host, v_host, dout_host, cu_seqlens, n_hea
     if arena_bytes is None:
         arena_bytes = device_arena.numel() * device_arena.element_size()
     s = _lib.hydra_attn_fwd_bwd_host(_host_ptr(q_host), _host_ptr(k_host), _host_ptr(v_host),
-                                     _host_ptr(dout_host), cu.ctypes.data, len(cu) - 1, n_heads, pp, npairs,
-                                     int(bool(causal)), ctypes.c_float(float(softmax_scale)),
+                                     _host_ptr(dout_host), _addr(cu), len(cu) - 1, n_heads, pp, npairs,
+                                     int(bool(causal)), float(softmax_scale),
                                      _host_ptr(out_host), _host_ptr(lse_host), _host_ptr(dq_host),
                                      _host_ptr(dk_host), _host_ptr(dv_host), _ptr(device_arena),
                                      int(arena_bytes), _stream(stream))
@@ -781,7 +795,7 @@ def hydra_lse_merge_noalloc(o_part, lse_part, part_rows: int, cu_seqlens, n_head
     arrays the next call overwrites). Host-side table building is serialised per process."""
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
-    s = _lib.hydra_lse_merge_noalloc(_ptr(o_part), _ptr(lse_part), int(part_rows), cu.ctypes.data, len(cu) - 1,
+    s = _lib.hydra_lse_merge_noalloc(_ptr(o_part), _ptr(lse_part), int(part_rows), _addr(cu), len(cu) - 1,
                                      n_heads, pp, npairs, _ptr(out), _ptr(lse), _stream(stream))
     if check:
         _check(s, "hydra_lse_merge_noalloc")
