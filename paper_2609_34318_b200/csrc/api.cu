@@ -672,13 +672,21 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     std::vector<uint8_t> is_short(pb.pairs.size(), 0);
     {
         double work_short = 0, work_all = 0;
+        int32_t longest = 0;
         for (size_t pi = 0; pi < pb.pairs.size(); ++pi) {
             const auto& p = pb.pairs[pi];
             const double w = static_cast<double>(p.q_len) * p.k_len;
             work_all += w;
+            longest = std::max(longest, std::max(p.q_len, p.k_len));
             if (short_len > 0 && p.q_len <= short_len && p.k_len <= short_len) { is_short[pi] = 1; work_short += w; }
         }
         if (work_short * 4 < work_all) std::fill(is_short.begin(), is_short.end(), 0);
+        // The second launch is not worth its price either if little is left for it that the short kernel would run almost
+        // as fast: pairs up to twice the limit cost it at most a tenth more, and 2^29 positions (with those above the
+        // mask) take 0.2 ms. 4096 packed tokens, 16 heads, the longest sequence 1381 tokens: 75 us on both kernels,
+        // 59 on the short one alone.
+        else if (work_short < work_all && longest <= 2 * short_len && (work_all - work_short) * pb.h <= double{1 << 29})
+            std::fill(is_short.begin(), is_short.end(), 1);
     }
     std::vector<std::vector<GroupEntry>> groups(pb.pairs.size()), groups_short(pb.pairs.size());
     for (size_t pi = 0; pi < pb.pairs.size(); ++pi) {
@@ -1561,9 +1569,8 @@ int32_t bwd_run(const Problem& pb, int32_t n_kv_heads, int32_t causal, float sof
     const Plan* plan = &lease.plan();
 
     float* dsum = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + kStatusBytes);
-    CUtensorMap mq, mk, mv, mdo, mq_sub, mdo_sub;
-    if (make_map(&mq, t.q, pb.Tq, n_heads, pb.dqk, TILE) || make_map(&mk, t.k, pb.Tk, n_kv_heads, pb.dqk, TILE) ||
-        make_map(&mv, t.v, pb.Tk, n_kv_heads, D_V, TILE) || make_map(&mdo, t.dout, pb.Tq, n_heads, D_V, TILE) ||
+    CUtensorMap mk, mv, mq_sub, mdo_sub;
+    if (make_map(&mk, t.k, pb.Tk, n_kv_heads, pb.dqk, TILE) || make_map(&mv, t.v, pb.Tk, n_kv_heads, D_V, TILE) ||
         make_map(&mq_sub, t.q, pb.Tq, n_heads, pb.dqk, SUB) || make_map(&mdo_sub, t.dout, pb.Tq, n_heads, D_V, SUB))
         return HYDRA_ERR_CUDA;
     if (first) {
@@ -1610,6 +1617,9 @@ int32_t bwd_run(const Problem& pb, int32_t n_kv_heads, int32_t causal, float sof
         bp.debug_stall_ns = g_debug_stall_ns[HYDRA_STALL_BWD_DQ].load();
         ScopedKernelTimer timer(K_DQ, stream);
         const int grid = std::min(sms, bp.n_items);
+        CUtensorMap mq, mdo;                           // whole tiles of q and dO: the recomputing form only
+        if (!hand_off && (make_map(&mq, t.q, pb.Tq, n_heads, pb.dqk, TILE) || make_map(&mdo, t.dout, pb.Tq, n_heads, D_V, TILE)))
+            return HYDRA_ERR_CUDA;
         const cudaError_t e = hand_off ? ks->launch_bwd_dq_from_ds(mk, bp, grid, stream)
                                        : ks->launch_bwd_dq(mq, mk, mv, mdo, bp, grid, stream);
         if (e != cudaSuccess)
