@@ -1265,10 +1265,12 @@ std::atomic<uint64_t> g_ds_limit_bytes{uint64_t{4} << 30};
 // smallest scratch the banded backward is worth running with
 constexpr uint64_t kMinBandBytes = uint64_t{1} << 20;
 // Band scratch: a byte count, 0 (bands off) or HYDRA_BAND_AUTO: as much as the dS limit, for problems whose
-// whole dS buffer is at most 16 times that (a band boundary costs about as much as 1 / 30 of a 48 GB band,
-// so hundreds of small bands would cost more than the recomputation they save).
+// whole dS buffer is at most 8 times that. The longer the sequence, the narrower a band of that size: 16 to 21 key
+// tiles at 48K to 64K tokens, two waves of work items of which the second is half empty, and beside the stores of dS
+// that costs more than the recomputation it saves. One sequence, 16 heads, 4 GiB, step in bands / recomputing: 24K
+// tokens 10.96 / 11.21 ms, 32K (5 bands) 18.9 / 19.6, 48K (10 bands) 45.2 / 43.6, 64K (17 bands) 83.1 / 78.2.
 std::atomic<uint64_t> g_band_bytes{HYDRA_BAND_AUTO};
-constexpr uint64_t kAutoBandsMax = 16;
+constexpr uint64_t kAutoBandsMax = 8;
 uint64_t band_scratch_for(int64_t head_blocks, int32_t n_heads)
 {
     const uint64_t set = g_band_bytes.load();
