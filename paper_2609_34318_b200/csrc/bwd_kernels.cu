@@ -275,7 +275,6 @@ HYDRA_K(hydra_bwd_dq_kernel)(const __grid_constant__ CUtensorMap map_q, const __
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    wait_for_previous_launch();
     const uint32_t tm = tmem_base_slot;
     const uint64_t limit = p.wait_limit_ns;
     volatile int* abort_p = &abort_flag;
@@ -386,11 +385,13 @@ HYDRA_K(hydra_bwd_dq_kernel)(const __grid_constant__ CUtensorMap map_q, const __
                     if (asked && !popped) { it_ahead = pop_end(kq, raw_next); popped = true; }
                     if (popped && !ti.valid()) break;
                 }
+                if (kq == 0) wait_for_previous_launch();
             }
             if (blockIdx.x == 0) probe.stop(p.status, QUEUE_DQ);
         }
     } else if (warp == kWarpMma || warp == kWarpMma2) {
         // ------------------------------------------------------------------ UMMA issuers
+        wait_for_previous_launch();
         // Two issuing threads, so that neither kind of UMMA waits behind the other's operands:
         // warp 9 issues S = Q K^T and dP = dO V^T of tile j+1 as soon as S/dP of tile j have been
         // copied out and K, V have landed; warp 10 issues dQ += dS K of tile j as soon as dS is there.
@@ -503,6 +504,7 @@ HYDRA_K(hydra_bwd_dq_kernel)(const __grid_constant__ CUtensorMap map_q, const __
         }
     } else {
         // ------------------------------------------------------------------ elementwise warpgroups
+        wait_for_previous_launch();
         const int g = warp >> 2;                       // column half
         const int r = tid & 127;
         const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
@@ -679,7 +681,6 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    wait_for_previous_launch();
     const uint32_t tm = tmem_base_slot;
     const uint64_t limit = p.wait_limit_ns;
     volatile int* abort_p = &abort_flag;
@@ -812,10 +813,12 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                 }
                 if (popped && !si.valid()) break;
             }
+            if (kq == 0) wait_for_previous_launch();
         }
         if (blockIdx.x == 0 && lane == 0) probe.stop(p.status, QUEUE_DKV);
     } else if (warp == kWarpMma || warp == kWarpMma2) {
         // ------------------------------------------------------------------ UMMA issuers
+        wait_for_previous_launch();
         // warp 9 issues S^T = K Q^T and dP^T = V dO^T of sub-tile u+1 as soon as those of sub-tile u
         // have been copied out; warp 10 issues dV += P^T dO and dK += dS^T Q of sub-tile u as soon
         // as P and dS are in tensor memory. Neither waits behind the other's operands.
@@ -926,6 +929,7 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
         }
     } else {
         // ------------------------------------------------------------------ elementwise warpgroups
+        wait_for_previous_launch();
         const int g = warp >> 2;                       // column half: q rows [32 g, 32 g + 32) of the sub-tile
         const int r = tid & 127;
         const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
@@ -1175,7 +1179,6 @@ HYDRA_K(hydra_bwd_dq_from_ds_kernel)(const __grid_constant__ CUtensorMap map_k,
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    wait_for_previous_launch();
     const uint32_t tm = tmem_base_slot;
     const uint64_t limit = p.wait_limit_ns;
     volatile int* abort_p = &abort_flag;
@@ -1263,11 +1266,13 @@ HYDRA_K(hydra_bwd_dq_from_ds_kernel)(const __grid_constant__ CUtensorMap map_k,
                     if (asked && !popped) { it_ahead = pop_end(kq, raw_next); popped = true; }
                     if (popped && !ti.valid()) break;
                 }
+                if (kq == 0) wait_for_previous_launch();
             }
             if (blockIdx.x == 0) probe.stop(p.status, QUEUE_DQ);
         }
     } else if (warp == 6) {
         // ------------------------------------------------------------------ K producer
+        wait_for_previous_launch();
         uint32_t g = 0;
         bool ok = true;
         for (uint32_t kq = 0; ok; ++kq) {
@@ -1292,6 +1297,7 @@ HYDRA_K(hydra_bwd_dq_from_ds_kernel)(const __grid_constant__ CUtensorMap map_k,
         }
     } else if (warp == 5) {
         // ------------------------------------------------------------------ UMMA issuer
+        wait_for_previous_launch();
         constexpr uint32_t idesc = umma_idesc_bf16(TILE, kDqk, true, true);
         // dS^T without swizzle: 8 kv rows are 128 bytes, chunks of 8 q rows are 2 KB apart (two blocks in a row)
         constexpr uint32_t hi_ds = umma_desc_plain_hi(128, 2048);
@@ -1335,6 +1341,7 @@ HYDRA_K(hydra_bwd_dq_from_ds_kernel)(const __grid_constant__ CUtensorMap map_k,
         }
     } else if (warp < 4) {
         // ------------------------------------------------------------------ epilogue warps
+        wait_for_previous_launch();
         const int r = tid;                             // q row inside the tile = TMEM lane
         const uint32_t lane_base = static_cast<uint32_t>(warp * 32) << 16;
         uint32_t n_acc = 0;

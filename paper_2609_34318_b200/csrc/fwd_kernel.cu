@@ -123,7 +123,6 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
     __syncthreads();
     cluster_sync_all();                                // both CTAs' barriers exist before anyone signals them
     tc_fence_after_sync();
-    wait_for_previous_launch();
     const uint32_t tm = tmem_base_slot;
     const uint64_t limit = p.wait_limit_ns;
     volatile int* abort_p = &abort_flag;
@@ -184,6 +183,7 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
                 const PairDev pr = p.pairs[item.pair];
                 const int n_t[2] = {item.n_a, item.n_b};
                 const int n = max(item.n_a, item.n_b);
+                if (kq == 0) wait_for_previous_launch();
                 auto load_q = [&](int t) {
                     if (n_t[t] <= 0 || !ok) return;
                     ok = wait(B_QEMPTY + t, q_use[t] ^ 1u);
@@ -218,6 +218,7 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
         }
     } else if (warp == kWarpV) {
         // ------------------------------------------------------------------ V producer
+        wait_for_previous_launch();
         if (lane == 0) {
             uint32_t gv = 0;
             bool ok = true;
@@ -239,6 +240,7 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
         }
     } else if (warp == kWarpMma) {
         // ------------------------------------------------------------------ UMMA issuer (leader CTA)
+        wait_for_previous_launch();
         if (leader && elect_one()) {
             constexpr uint32_t idesc_s = umma_idesc_bf16(2 * TILE, TILE, false, false);
             constexpr uint32_t idesc_o = umma_idesc_bf16(2 * TILE, D_V, false, true);
@@ -337,6 +339,7 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
     } else {
         regs_increase<kRegsSoftmax>();
         // ------------------------------------------------------------------ softmax warpgroups
+        wait_for_previous_launch();
         const int t = warp >> 2;                       // tile A or B
         const int r = tid & 127;                       // row inside this CTA's half of the tile = TMEM lane
         const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;

@@ -126,7 +126,6 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    wait_for_previous_launch();
     const uint32_t tm = tmem_base_slot + static_cast<uint32_t>(slot) * kTmSlot;
     const uint64_t limit = p.wait_limit_ns;
     volatile int* abort_p = &abort_flag;
@@ -226,6 +225,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
                     if (j + 2 < n) load_k(cur, j + 2);           // its stage came free before V's: S(j) precedes P V(j - 1)
                     load_v(cur, j);
                 }
+                if (kq == 0) wait_for_previous_launch();
                 if (nxt_idx < 0) break;
                 cur = nxt;
                 raw1 = raw2;
@@ -236,6 +236,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
         }
     } else if (warp == kWarpMma + slot) {
         // ------------------------------------------------------------------ UMMA issuer
+        wait_for_previous_launch();
         if (elect_one()) {
             constexpr uint32_t idesc_s = umma_idesc_bf16(TILE, KV, false, false);
             constexpr uint32_t idesc_o = umma_idesc_bf16(TILE, D_V, false, true);
@@ -336,6 +337,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
         const uint32_t tm_s0 = tm + kTmS + lane_base;
         uint32_t g = 0;                                // steps of this slot so far
         bool ok = true;
+        wait_for_previous_launch();
         for (uint32_t kq = 0; ok; ++kq) {
             const int rs = kq % kSched;
             ok = wait(B_ITEMFULL + rs, kq / kSched);

@@ -139,7 +139,10 @@ struct ClockProbe {
 
 // Launches of one stream overlap at their ends: every kernel of the library lets the next one start its blocks as soon
 // as all of its own have started (they take the SMs that its first finished blocks leave) and waits, before it
-// touches global memory, until the launch before it has completed and its results are visible. What is hidden
+// touches global memory, until the launch before it has completed and its results are visible. (The work tables are the
+// exception: no kernel writes them, and their copy to the device is ordered before the call's first launch, so the
+// producer of a thread block fetches its first work item before it waits. The other roles wait first thing, so that
+// the limit of their bounded waits does not run while the launch before is still at work.) What is hidden
 // that way is the launch itself, the barriers' and tensor memory's set-up and the wait for the last block: a step of
 // four sequences of 7 to 300 tokens 42 -> 35 us, of 1024 tokens in short ones 49 -> 42 us, the ten launches around the
 // attention of a 4096-token MLA block 813 -> 794 us. Kernels of other libraries before or after are ordered
