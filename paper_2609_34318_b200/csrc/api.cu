@@ -249,6 +249,7 @@ struct Plan {
     std::vector<uint8_t> blob;       // the tables, as they go to the device
     size_t off_pairs = 0, off_items = 0, off_lists = 0, off_groups = 0, off_items2 = 0, off_lists2 = 0;
     int32_t n_items = 0, n_items2 = 0;
+    int32_t halves = 0;              // forward: the short kernel's items are halves of tiles, two per thread block
     int64_t ds_head_blocks = 0;      // backward: blocks of the dS hand-off buffer per head; -1: not usable
     // residency on the device (guarded by g_plan_mutex)
     int half = -1;                   // arena half the tables were last copied to
@@ -670,7 +671,21 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     // tail), so the short kernel is used only if the short pairs carry at least a quarter of the call's work.
     const int32_t short_len = fwd_short_len_for(pb);
     std::vector<uint8_t> is_short(pb.pairs.size(), 0);
-    {
+    // A call with no more q tiles than SMs: what it takes is its longest tile's chain of steps. The short kernel then has
+    // an idle slot beside every busy one and gives it the second half of the tile's keys, whatever their number (the
+    // CTA-pair kernel would leave more than half of the SMs idle).
+    // (A limit set by the caller is kept to.)
+    int64_t n_tiles = 0;
+    bool within = true;
+    for (const auto& p : pb.pairs) {
+        n_tiles += (p.q_len + TILE - 1) / TILE;
+        within = within && p.q_len <= short_len && p.k_len <= short_len;
+    }
+    n_tiles *= pb.h;
+    const bool halves = short_len > 0 && n_tiles <= plan_workers(1) && (within || g_fwd_short_len.load() < 0);
+    if (halves) {
+        std::fill(is_short.begin(), is_short.end(), 1);
+    } else {
         double work_short = 0, work_all = 0;
         int32_t longest = 0;
         for (size_t pi = 0; pi < pb.pairs.size(); ++pi) {
@@ -744,6 +759,35 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
         return it;
     };
     const int short_workers = 2 * plan_workers(1);
+    if (halves) {
+        // the first parts, then the second parts in the same order: slots 0 take items [0, n), slots 1 [n, 2 n)
+        std::vector<FwdShortItem> first, second;
+        for (size_t g = 0; g < groups_short.size(); ++g)
+            for (int32_t a = 0; a < pb.h; ++a)
+                for (const GroupEntry& e : groups_short[g]) {
+                    FwdShortItem it = make_short(static_cast<int32_t>(g), a, e), rest = it;
+                    const int32_t n0 = (e.b + 1) / 2;
+                    rest.n_kv = static_cast<uint16_t>(e.b - n0);
+                    if (rest.n_kv > 0) {
+                        const int32_t skip = n0 * FWD_SHORT_KEYS;
+                        it.n_kv = static_cast<uint16_t>(n0);
+                        it.half = 1;
+                        rest.half = 2;
+                        rest.k_tok0 += skip;
+                        rest.k_len -= skip;
+                        rest.off -= skip;
+                    } else {
+                        rest.rows = 0;                      // nothing left for the other slot: it writes nothing
+                    }
+                    first.push_back(it);
+                    second.push_back(rest);
+                }
+        first.insert(first.end(), second.begin(), second.end());
+        plan.off_items2 = append(blob, first);
+        plan.n_items2 = static_cast<int32_t>(first.size());
+        plan.halves = 1;
+        return;
+    }
     const GroupOrder go = order_groups(groups_short, pb.h, short_workers);
     if (go.settled) {
         const size_t off = align_up(blob.size(), 16);
@@ -1030,7 +1074,7 @@ struct KernelSet {
     int (*fwd_max_clusters)();
     cudaError_t (*launch_fwd)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const FwdParams&, int,
                               cudaStream_t);
-    cudaError_t (*launch_fwd_short)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const FwdParams&, int,
+    cudaError_t (*launch_fwd_short)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const FwdParams&, bool, int,
                                     cudaStream_t);
     cudaError_t (*launch_bwd_dq)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const CUtensorMap&,
                                  const BwdParams&, int, cudaStream_t);
@@ -1469,9 +1513,10 @@ int32_t fwd_core(Problem& pb, const void* q, const void* k, const void* v, int32
         // short pairs: one CTA per SM with two work items in flight, K and V in boxes of 64 keys
         CUtensorMap mv_sub;
         if (make_map(&mv_sub, v, pb.Tk, n_kv_heads, D_V, FWD_SHORT_KEYS)) return HYDRA_ERR_CUDA;
-        const int grid = std::min(sms, plan->n_items2);      // one item per SM before any SM gets two
+        // one item per SM before any SM gets two, or both halves of a tile on one SM
+        const int grid = plan->halves ? plan->n_items2 / 2 : std::min(sms, plan->n_items2);
         ScopedKernelTimer timer(K_FWD, stream);
-        if (ks->launch_fwd_short(mq, mk, mv_sub, fp, grid, stream) != cudaSuccess) return HYDRA_ERR_CUDA;
+        if (ks->launch_fwd_short(mq, mk, mv_sub, fp, plan->halves != 0, grid, stream) != cudaSuccess) return HYDRA_ERR_CUDA;
         g_launches += 1;
     }
     lease.release();                                   // the tables have their reader on record

@@ -81,7 +81,8 @@ constexpr int kShortItem = 8;                         // an item of at most so m
 
 enum : int {
     B_QFULL = 0, B_QEMPTY = 1, B_KFULL = 2, B_KEMPTY = 5, B_VFULL = 8, B_VEMPTY = 10, B_SFULL = 12, B_PFULL = 14,
-    B_PVDONE = 16, B_OFREE = 17, B_ITEMFULL = 18, B_ITEMEMPTY = 18 + kSched, B_PER_SLOT = 18 + 2 * kSched
+    B_PVDONE = 16, B_OFREE = 17, B_ITEMFULL = 18, B_ITEMEMPTY = 18 + kSched, B_HALF = 18 + 2 * kSched,
+    B_PER_SLOT = 19 + 2 * kSched
 };
 
 __device__ __forceinline__ float neg_inf() { return __int_as_float(0xff800000); }
@@ -90,6 +91,9 @@ __device__ __forceinline__ float neg_inf() { return __int_as_float(0xff800000); 
 
 size_t HYDRA_K(fwd_short_smem_bytes)() { return kSmemTotal + 1024; }
 
+// kHalves: every thread block has one q tile, whose keys its two slots share. (A build of its own: the join of the two parts
+// in the epilogue of the other would cost it 7 % on sequences of 64 to 512 tokens in instruction-cache misses.)
+template <bool kHalves>
 __global__ void __launch_bounds__(kThreads, 1)
 HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                                 const __grid_constant__ CUtensorMap map_v, const FwdParams p)
@@ -115,7 +119,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
         for (int s = 0; s < kSlots; ++s)
             for (int i = 0; i < B_PER_SLOT; ++i) {
                 uint32_t count = 1u;
-                if ((i >= B_PFULL && i < B_PFULL + 2) || i == B_OFREE) count = 4u;        // the slot's softmax warps
+                if ((i >= B_PFULL && i < B_PFULL + 2) || i == B_OFREE || i == B_HALF) count = 4u;   // softmax warps
                 if (i >= B_ITEMEMPTY && i < B_ITEMEMPTY + kSched) count = 5u;             // + its issuer
                 mbar_init(base + 8u * static_cast<uint32_t>(s * B_PER_SLOT + i), count);
             }
@@ -447,6 +451,40 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
             ok = wait(B_PVDONE, g - 1u);
             if (!ok) break;
             tc_fence_after_sync();
+            // A tile whose keys the two slots share: slot 1 leaves its unscaled O, maximum and sum in its own (now unused)
+            // operand space, a column of 128 rows after the other, and slot 0 joins them to its own. In such a launch
+            // every thread block has this one tile.
+            const uint32_t half_buf = smem0 + kSlotBytes + r * 4u;
+            constexpr uint32_t kColumn = TILE * 4;
+            float mul0 = 1.f, mul1 = 0.f;
+            if (kHalves && item.half == 2) {
+                st_shared_f32(half_buf + D_V * kColumn, m_run);
+                st_shared_f32(half_buf + (D_V + 1) * kColumn, l_run);
+#pragma unroll 1
+                for (int c0 = 0; c0 < D_V; c0 += 32) {
+                    uint32_t o[32];
+                    tmem_ld_x32(tm_o + c0, o);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) st_shared_f32(half_buf + (c0 + e) * kColumn, __uint_as_float(o[e]));
+                }
+                tc_fence_before_sync();
+                mbar_arrive_warp(bar(B_OFREE));
+                mbar_arrive_warp(smem_u32(&bars[B_HALF]));
+                continue;
+            }
+            if (kHalves && item.half == 1) {
+                ok = wait(B_HALF, 0u);
+                if (!ok) break;
+                const float m1 = ld_shared_f32(half_buf + D_V * kColumn), l1 = ld_shared_f32(half_buf + (D_V + 1) * kColumn);
+                const float m = fmaxf(m_run, m1);
+                if (m != neg_inf()) {                  // (a part without visible keys has maximum -inf: weight 0)
+                    mul0 = ex2_approx(m_run - m);
+                    mul1 = ex2_approx(m1 - m);
+                }
+                m_run = m;
+                l_run = l_run * mul0 + l1 * mul1;
+            }
             const float inv_l = (l_run > 0.f) ? 1.f / l_run : 0.f;
             const bool wide = (reinterpret_cast<uintptr_t>(dst) & 31u) == 0;   // the interface asks for 16 bytes only
 #pragma unroll
@@ -457,6 +495,11 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
                 if (c0 + 32 == D_V) {                  // every column has left TMEM: O may be overwritten
                     tc_fence_before_sync();
                     mbar_arrive_warp(bar(B_OFREE));
+                }
+                if (kHalves && item.half == 1) {
+#pragma unroll
+                    for (int e = 0; e < 32; ++e)
+                        o[e] = __float_as_uint(__uint_as_float(o[e]) * mul0 + ld_shared_f32(half_buf + (c0 + e) * kColumn) * mul1);
                 }
                 if (row_valid) {
                     // 32 bytes per store: a thread's row is 4 KB away from its neighbour's, so every store of the
@@ -499,21 +542,21 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
 }
 
 cudaError_t HYDRA_K(launch_fwd_short)(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
-                                      const FwdParams& p, int grid, cudaStream_t stream)
+                                      const FwdParams& p, bool halves, int grid, cudaStream_t stream)
 {
     // the opt-in to more than 48 KB of dynamic shared memory is made once per device ordinal
-    static bool configured[64] = {};
+    static bool configured[64][2] = {};
+    const auto kernel = halves ? HYDRA_K(hydra_fwd_short_kernel)<true> : HYDRA_K(hydra_fwd_short_kernel)<false>;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!configured[dev]) {
-        e = cudaFuncSetAttribute(HYDRA_K(hydra_fwd_short_kernel), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(HYDRA_K(fwd_short_smem_bytes)()));
+    if (!configured[dev][halves]) {
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(HYDRA_K(fwd_short_smem_bytes)()));
         if (e != cudaSuccess) return e;
-        configured[dev] = true;
+        configured[dev][halves] = true;
     }
-    return launch_overlapped(HYDRA_K(hydra_fwd_short_kernel), grid, kThreads, HYDRA_K(fwd_short_smem_bytes)(), stream, mq, mk, mv, p);
+    return launch_overlapped(kernel, grid, kThreads, HYDRA_K(fwd_short_smem_bytes)(), stream, mq, mk, mv, p);
 }
 
 }  // namespace hydra

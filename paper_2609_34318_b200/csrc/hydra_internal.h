@@ -79,8 +79,9 @@ struct alignas(16) FwdShortItem {
     uint16_t n_kv;     // steps of FWD_SHORT_KEYS keys the tile visits; 0: its rows see no key
     uint8_t rows;      // q rows of the tile that exist (1..128)
     uint8_t to_part;   // 1: partial buffers, 0: out / lse
-    uint16_t pad;
-    int32_t pad2;
+    uint16_t half;     // 0: all keys of the tile; 1, 2: its first and second part, run by the two slots of one thread
+                       // block (the second hands its result to the first)
+    int32_t pad;
 };
 static_assert(sizeof(FwdShortItem) == 32, "two 16-byte loads per work item");
 
@@ -228,7 +229,7 @@ struct MergeParams {
                                    const FwdParams& p, int grid, cudaStream_t stream);                                \
     size_t fwd_short_smem_bytes##SUFFIX();                                                                            \
     cudaError_t launch_fwd_short##SUFFIX(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv_sub,     \
-                                         const FwdParams& p, int grid, cudaStream_t stream);                          \
+                                         const FwdParams& p, bool halves, int grid, cudaStream_t stream);             \
     cudaError_t launch_bwd_dq##SUFFIX(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,            \
                                       const CUtensorMap& mdo, const BwdParams& p, int grid, cudaStream_t stream);     \
     cudaError_t launch_bwd_dq_from_ds##SUFFIX(const CUtensorMap& mk, const BwdParams& p, int grid,                    \

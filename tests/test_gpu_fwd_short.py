@@ -57,6 +57,24 @@ def test_short_sequences_against_the_oracle(lengths):
     check(got, ref, label=f"{lengths[:5]} ")
 
 
+@pytest.mark.parametrize("lengths,h", [
+    ([1], 1),                     # one row, one step: nothing for the second slot
+    ([64], 2), ([65], 2),         # one step and two
+    ([128], 3), ([129, 192], 2),  # two steps; three and four, rows that see nothing of the second part
+    ([700, 33, 1], 3),            # an odd number of steps beside single ones
+    ([3000], 2),                  # longer than the limit of the short-sequence kernel: 24 tiles, up to 47 steps
+    ([128] * 37, 4),              # 148 tiles: as many as the GPU has SMs
+    ([128] * 37 + [1], 4),        # one more: no halves
+])
+def test_tiles_shared_by_the_two_slots(lengths, h):
+    """A call with no more q tiles than SMs gives each slot of a thread block half of a tile's keys. The two parts are
+    joined in fp32 before the one rounding to bf16, so the tolerance is that of the whole tile."""
+    cu = hw.cu_seqlens(lengths)
+    x = rand_inputs(sum(lengths) + h, int(cu[-1]), h)
+    got = run_gpu(x, cu, h)
+    check(got, run_oracle(x, cu), label=f"{lengths[:4]} ")
+
+
 def test_random_length_mixes_and_both_kernels_agree():
     import paper_2609_34318_b200 as P
     rng = np.random.default_rng(11)
