@@ -249,7 +249,8 @@ struct Plan {
     std::vector<uint8_t> blob;       // the tables, as they go to the device
     size_t off_pairs = 0, off_items = 0, off_lists = 0, off_groups = 0, off_items2 = 0, off_lists2 = 0;
     int32_t n_items = 0, n_items2 = 0;
-    int32_t halves = 0;              // forward: the short kernel's items are halves of tiles, two per thread block
+    int32_t halves = 0;              // forward: the short kernel's items are halves of tiles, two per thread block;
+                                     // backward: two CTAs share every key-side item
     int64_t ds_head_blocks = 0;      // backward: blocks of the dS hand-off buffer per head; -1: not usable
     // residency on the device (guarded by g_plan_mutex)
     int half = -1;                   // arena half the tables were last copied to
@@ -867,7 +868,9 @@ int64_t ds_layout(const Problem& pb, int causal, std::vector<PairDev>* dev)
 void build_bwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& blob)
 {
     const int32_t n = static_cast<int32_t>(pb.pairs.size());
+    int32_t longest = 0;                                   // q sub-tiles of the longest key-side item (the last side built)
     auto group_by = [&](bool by_q, std::vector<int32_t>& lists, std::vector<GroupItem>& items) {
+        longest = 0;
         std::vector<int32_t> order(n);
         for (int32_t i = 0; i < n; ++i) order[i] = i;
         auto key = [&](int32_t i) {
@@ -914,6 +917,7 @@ void build_bwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
                         }
                     }
                     groups.back().push_back(GroupEntry{r0, 0, 0, c});
+                    longest = std::max(longest, c);
                 }
             }
             i = j;
@@ -926,6 +930,10 @@ void build_bwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     std::vector<GroupItem> items_q, items_k;
     group_by(true, lists_q, items_q);
     group_by(false, lists_k, items_k);
+    // Two CTAs per key-side item where there are enough for that and the longest is worth the exchange at the end: it and the
+    // cluster's start cost 2 us, a sub-tile takes 1.1. Step with sequences of 300 tokens (5 sub-tiles) 30.5 us with one CTA,
+    // 31.8 with two; of 512 (8) 36.6 and 36.4; of 1024 tokens, 8 heads, 54.8 and 51.4; of 2048, 4 heads, 84.7 and 73.4.
+    plan.halves = longest > 8 && 2 * static_cast<int64_t>(items_k.size()) <= plan_workers(1);
     std::vector<PairDev> dev = device_pairs(pb);
     plan.ds_head_blocks = ds_layout(pb, causal, &dev);
     plan.off_pairs = append(blob, dev);
@@ -1080,7 +1088,7 @@ struct KernelSet {
                                  const BwdParams&, int, cudaStream_t);
     cudaError_t (*launch_bwd_dq_from_ds)(const CUtensorMap&, const BwdParams&, int, cudaStream_t);
     cudaError_t (*launch_bwd_dkv)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const CUtensorMap&,
-                                  const BwdParams&, int, cudaStream_t);
+                                  const BwdParams&, bool, int, cudaStream_t);
 };
 const KernelSet* kernel_set(int32_t d_qk, int32_t d_v)
 {
@@ -1652,7 +1660,9 @@ int32_t bwd_run(const Problem& pb, int32_t n_kv_heads, int32_t causal, float sof
         bp.accumulate = accumulate_dkv ? 1 : 0;
         bp.debug_stall_ns = g_debug_stall_ns[HYDRA_STALL_BWD_DKV].load();
         ScopedKernelTimer timer(K_DKV, stream);
-        if (ks->launch_bwd_dkv(mq_sub, mk, mv, mdo_sub, bp, std::min(sms, bp.n_items), stream) != cudaSuccess)
+        const bool halves = plan->halves != 0;
+        if (ks->launch_bwd_dkv(mq_sub, mk, mv, mdo_sub, bp, halves, halves ? 2 * bp.n_items : std::min(sms, bp.n_items),
+                               stream) != cudaSuccess)
             return HYDRA_ERR_CUDA;
         g_launches += 1;
     }

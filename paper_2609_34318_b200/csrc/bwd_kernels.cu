@@ -202,8 +202,9 @@ constexpr uint32_t kTmDK = 0, kTmDV = 192, kTmS = 320, kTmDP = 384, kTmP = 448, 
 constexpr bool kKInTmem = kDqk == 128;
 constexpr uint32_t kTmK = kTmDK + 128;
 enum : int { B_KVFULL = 0, B_KVEMPTY = 1, B_QFULL = 2, B_STAT = 5, B_QEMPTY = 8, B_SFULL = 11,
-             B_SFREE = 12, B_PFULL = 13, B_PDSFREE = 14, B_ACCFREE = 15, B_ITEMFULL = 16, B_ITEMEMPTY = 16 + kSched,
-             B_COUNT = 16 + 2 * kSched };
+             B_SFREE = 12, B_PFULL = 13, B_PDSFREE = 14, B_ACCFREE = 15, B_PEERFREE = 16, B_PEERDATA = 17,
+             B_ITEMFULL = 18, B_ITEMEMPTY = 18 + kSched, B_COUNT = 18 + 2 * kSched };
+static_assert(kDqk * TILE * 4u <= kDsStage, "the other CTA's part of dK fits the operand space");
 
 // Iterator over (pair of the kv chunk, 64-row q sub-tile).
 struct SubIter {
@@ -639,6 +640,10 @@ HYDRA_K(hydra_bwd_dq_kernel)(const __grid_constant__ CUtensorMap map_q, const __
 // =============================================================================================
 // dK / dV
 // =============================================================================================
+// kHalves: the two CTAs of a cluster share one kv tile, each visiting every other of its q sub-tiles; at the end CTA 0 gets
+// the other's dK through distributed shared memory and writes the tile's dK, CTA 1 its dV. For calls with no more than
+// half as many kv tiles as SMs, which take as long as their longest tile.
+template <bool kHalves>
 __global__ void __launch_bounds__(kThreads, 1)
 HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                      const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do,
@@ -669,8 +674,8 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
         for (int i = 0; i < B_COUNT; ++i) {
             uint32_t count = 1u;
             if (i == B_SFREE || i == B_PFULL || i == B_ACCFREE) count = 8u;   // elementwise warps
+            if (i == B_PEERFREE || i == B_PEERDATA) count = 8u;
             if (i >= B_ITEMEMPTY && i < B_ITEMEMPTY + kSched) count = 10u;   // + the two issuer warps
-            
             mbar_init(bar(i), count);
         }
         fence_mbar_init();
@@ -680,8 +685,14 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
     if (warp == kWarpMma) { tmem_alloc(smem_u32(&tmem_base_slot), kTmCols); tmem_relinquish(); }
     tc_fence_before_sync();
     __syncthreads();
+    if (kHalves) cluster_sync_all();                   // both CTAs' barriers exist before anyone signals them
     tc_fence_after_sync();
     const uint32_t tm = tmem_base_slot;
+    const uint32_t rank = kHalves ? cluster_cta_rank() : 0u;
+    const int worker = kHalves ? static_cast<int>(cluster_id_x()) : static_cast<int>(blockIdx.x);
+    const int n_workers = static_cast<int>(kHalves ? gridDim.x >> 1 : gridDim.x);
+    auto sub_begin = [&](SubIter& si) { if (kHalves && rank != 0 && si.valid()) si.next(); };   // this CTA's first sub-tile
+    auto sub_next = [&](SubIter& si) { si.next(); if (kHalves && si.valid()) si.next(); };
     const uint64_t limit = p.wait_limit_ns;
     volatile int* abort_p = &abort_flag;
     auto wait = [&](int b, uint32_t parity) -> bool { return mbar_wait(bar(b), parity & 1u, abort_p, limit); };
@@ -697,8 +708,7 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
     auto pop_begin = [&](uint32_t k) -> int {               // producer, one thread
         const int slot = k % kSched;
         if (!mbar_wait(bar(B_ITEMEMPTY + slot), ((k / kSched) ^ 1u) & 1u, abort_p, limit)) return kPopFailed;
-        return k == 0 ? static_cast<int>(blockIdx.x)
-                      : static_cast<int>(gridDim.x) + atomicAdd(&p.status->next_item[QUEUE_DKV], 1);
+        return k == 0 ? worker : n_workers + atomicAdd(&p.status->next_item[QUEUE_DKV], 1);
     };
     auto pop_end = [&](uint32_t k, int raw) -> int {
         if (raw == kPopFailed) return -1;
@@ -754,6 +764,7 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                 item = s_item[(kq - 1) % kSched];
                 first = s_first[(kq - 1) % kSched];
                 si.init(p.pairs, p.lists + item.list_off, item.list_len, item.r0, p.causal, p.ds != nullptr, first);
+                sub_begin(si);
             }
             int raw_next = 0;
             bool asked = false, popped = false, start = true;
@@ -805,7 +816,7 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                     }
                     mbar_arrive_warp(bar(B_STAT + st));
                     ++gq;
-                    si.next();
+                    sub_next(si);
                 }
                 if (asked && !popped) {
                     if (lane == 0) it_ahead = pop_end(kq, raw_next);
@@ -843,6 +854,7 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                 const int32_t* list = p.lists + item.list_off;
                 SubIter si;
                 si.init(p.pairs, list, item.list_len, item.r0, p.causal, p.ds != nullptr, first);
+                sub_begin(si);
                 if (!si.valid()) continue;
                 if (issue_scores) {
                     ok = wait(B_KVFULL, items);
@@ -866,7 +878,7 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                         const uint32_t q_lo = q_lo0 + st * (kQkBoxes * kBox64 >> 4), do_lo = do_lo0 + st * (2 * kBox64 >> 4);
                         const uint32_t prev = n_step;
                         ++n_step;
-                        si.next();
+                        sub_next(si);
                         if (prev > 0) ok = wait(B_SFREE, prev - 1u);
                         if (!ok) break;
                         tc_fence_after_sync();
@@ -894,7 +906,7 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                         // them and their updates (with the step to the next sub-tile behind the wait the tensor pipe
                         // idled 250 cycles per sub-tile at d_qk = 128).
                         const int st = n_step % kStages;
-                        si.next();
+                        sub_next(si);
                         const bool more = si.valid();
                         if (first_step && items > 0) ok = wait(B_ACCFREE, items - 1u);
                         // Order hint, not a data dependency: let the score products of the NEXT sub-tile of
@@ -962,6 +974,14 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
             float* dvp_acc = static_cast<float*>(p.dv) + dv_off;
             SubIter si;
             si.init(p.pairs, list, item.list_len, item.r0, p.causal, p.ds != nullptr, first);
+            bool joint = false;                        // the other CTA of the cluster has sub-tiles of this tile too
+            if (kHalves) {
+                SubIter second = si;
+                if (second.valid()) second.next();
+                joint = second.valid();
+                if (rank != 0) si = second;
+                if (rank != 0 && !joint) continue;     // CTA 0 does what there is to do
+            }
             if (!si.valid()) {                         // no q row sees this tile: dK = dV = 0 (nothing to add)
                 if (row_valid && !p.accumulate) {
                     uint4* a4 = reinterpret_cast<uint4*>(dkp);
@@ -973,7 +993,7 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                 }
                 continue;
             }
-            for (; si.valid() && ok; si.next(), ++gq) {
+            for (; si.valid() && ok; sub_next(si), ++gq) {
                 const int st = gq % kStages;
                 ok = wait(B_SFULL, c_s);
                 ++c_s;
@@ -1066,15 +1086,51 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                 return c < kDkChunks ? tm + kTmDK + lane_base + g * (kDqk / 2) + c * 32
                                      : tm + kTmDV + lane_base + g * 64 + (c - kDkChunks) * 32;
             };
-            uint32_t v[32];
-            tmem_ld_x32(chunk_addr(0), v);
+            int c_begin = 0, c_end = kChunks;
+            // the other CTA's part of a column of dK or dV: 128 rows after one another, this thread's row
+            const uint32_t part = smem + r * 4u;
+            auto part_col = [&](int c) -> uint32_t {   // chunk c's first column of this warpgroup
+                return (c < kDkChunks ? g * (kDqk / 2) + c * 32 : g * 64 + (c - kDkChunks) * 32) * (TILE * 4u);
+            };
+            if (kHalves && joint) {
+                // Nothing of this CTA reads its operand space any more: let the other one write there. CTA 0 sends its part
+                // of dV and finishes dK, CTA 1 the other way round.
+                const uint32_t peer = rank ^ 1u;
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster_release(cluster_map_shared(bar(B_PEERFREE), peer));
+                ok = mbar_wait_acquire_cluster(bar(B_PEERFREE), 0u, abort_p, limit);
+                if (!ok) break;
+                const uint32_t remote = cluster_map_shared(part, peer);
 #pragma unroll 1
-            for (int c = 0; c < kChunks; ++c) {
+                for (int c = rank == 0 ? kDkChunks : 0; c < (rank == 0 ? kChunks : kDkChunks); ++c) {
+                    uint32_t v[32];
+                    tmem_ld_x32(chunk_addr(c), v);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < 32; ++e)
+                        st_shared_cluster_f32(remote + part_col(c) + e * (TILE * 4u), __uint_as_float(v[e]));
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster_release(cluster_map_shared(bar(B_PEERDATA), peer));
+                ok = mbar_wait_acquire_cluster(bar(B_PEERDATA), 0u, abort_p, limit);
+                if (!ok) break;
+                if (rank == 0) c_end = kDkChunks;
+                else c_begin = kDkChunks;
+            }
+            uint32_t v[32];
+            tmem_ld_x32(chunk_addr(c_begin), v);
+#pragma unroll 1
+            for (int c = c_begin; c < c_end; ++c) {
                 const bool is_dk = c < kDkChunks;
                 const int c0 = is_dk ? c * 32 : (c - kDkChunks) * 32;
                 const int64_t stride = kv_heads * (is_dk ? kDqk : D_V);
                 const float mul = is_dk ? p.scale : 1.f;
                 tmem_wait_ld();
+                if (kHalves && joint) {
+#pragma unroll
+                    for (int e = 0; e < 32; ++e)
+                        v[e] = __float_as_uint(__uint_as_float(v[e]) + ld_shared_f32(part + part_col(c) + e * (TILE * 4u)));
+                }
                 if (p.accumulate) {
                     float* dst = (is_dk ? dkp_acc : dvp_acc) + c0;
 #pragma unroll
@@ -1087,7 +1143,7 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
 #pragma unroll
                 for (int e = 0; e < 16; ++e)
                     w[e] = pack_bf16x2(__uint_as_float(v[2 * e]) * mul, __uint_as_float(v[2 * e + 1]) * mul);
-                if (c + 1 < kChunks) {
+                if (c + 1 < c_end) {
                     tmem_ld_x32(chunk_addr(c + 1), v);
                 } else {                                         // every column has left tensor memory
                     tc_fence_before_sync();
@@ -1103,6 +1159,7 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
     __syncwarp();
     tc_fence_before_sync();
     __syncthreads();
+    if (kHalves) cluster_sync_all();                   // nobody leaves while the other may still write to it
     if (abort_flag) {
         const uint64_t t0 = global_timer_ns();
         while (global_timer_ns() - t0 < 50000ull) { }
@@ -1456,12 +1513,13 @@ cudaError_t HYDRA_K(launch_bwd_dq)(const CUtensorMap& mq, const CUtensorMap& mk,
 }
 
 cudaError_t HYDRA_K(launch_bwd_dkv)(const CUtensorMap& mq_sub, const CUtensorMap& mk, const CUtensorMap& mv,
-                           const CUtensorMap& mdo_sub, const BwdParams& p, int grid, cudaStream_t stream)
+                           const CUtensorMap& mdo_sub, const BwdParams& p, bool halves, int grid, cudaStream_t stream)
 {
-    static bool configured[64] = {};
-    if (cudaError_t e = configure_once_per_device(HYDRA_K(hydra_bwd_dkv_kernel), HYDRA_K(bwd_dkv_smem_bytes)(), configured)) return e;
-    return launch_overlapped(HYDRA_K(hydra_bwd_dkv_kernel), grid, kThreads, HYDRA_K(bwd_dkv_smem_bytes)(), stream, mq_sub, mk, mv,
-                             mdo_sub, p);
+    static bool configured[2][64] = {};
+    const auto kernel = halves ? HYDRA_K(hydra_bwd_dkv_kernel)<true> : HYDRA_K(hydra_bwd_dkv_kernel)<false>;
+    if (cudaError_t e = configure_once_per_device(kernel, HYDRA_K(bwd_dkv_smem_bytes)(), configured[halves])) return e;
+    return launch_overlapped_clusters(kernel, halves ? 2 : 1, grid, kThreads, HYDRA_K(bwd_dkv_smem_bytes)(), stream, mq_sub, mk, mv,
+                                      mdo_sub, p);
 }
 
 }  // namespace hydra

@@ -151,21 +151,31 @@ struct ClockProbe {
 #ifdef __CUDACC__
 __device__ __forceinline__ void overlap_next_launch() { cudaTriggerProgrammaticLaunchCompletion(); }
 __device__ __forceinline__ void wait_for_previous_launch() { cudaGridDependencySynchronize(); }
+// (cluster: CTAs per cluster of a kernel that does not state it itself; 1 for all others)
 template <class... Params, class... Args>
-cudaError_t launch_overlapped(void (*kernel)(Params...), int grid, int block, size_t smem_bytes, cudaStream_t stream,
-                              Args&&... args)
+cudaError_t launch_overlapped_clusters(void (*kernel)(Params...), int cluster, int grid, int block, size_t smem_bytes,
+                                       cudaStream_t stream, Args&&... args)
 {
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2] = {};
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = static_cast<unsigned>(cluster);
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(static_cast<unsigned>(grid));
     cfg.blockDim = dim3(static_cast<unsigned>(block));
     cfg.dynamicSmemBytes = smem_bytes;
     cfg.stream = stream;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+template <class... Params, class... Args>
+cudaError_t launch_overlapped(void (*kernel)(Params...), int grid, int block, size_t smem_bytes, cudaStream_t stream,
+                              Args&&... args)
+{
+    return launch_overlapped_clusters(kernel, 1, grid, block, smem_bytes, stream, static_cast<Args&&>(args)...);
 }
 #endif
 
@@ -235,7 +245,8 @@ struct MergeParams {
     cudaError_t launch_bwd_dq_from_ds##SUFFIX(const CUtensorMap& mk, const BwdParams& p, int grid,                    \
                                               cudaStream_t stream);                                                   \
     cudaError_t launch_bwd_dkv##SUFFIX(const CUtensorMap& mq_sub, const CUtensorMap& mk, const CUtensorMap& mv,       \
-                                       const CUtensorMap& mdo_sub, const BwdParams& p, int grid, cudaStream_t stream);
+                                       const CUtensorMap& mdo_sub, const BwdParams& p, bool halves, int grid,             \
+                                       cudaStream_t stream);
 HYDRA_DECLARE_KERNEL_SET()
 HYDRA_DECLARE_KERNEL_SET(_d128)
 #undef HYDRA_DECLARE_KERNEL_SET

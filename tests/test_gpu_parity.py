@@ -349,3 +349,18 @@ def test_non_causal_backward_with_room_for_the_dense_hand_off(backward_form):
            "dq": step.dq[:T].float().cpu().numpy().astype(np.float64), "dk": step.dk[:T].float().cpu().numpy().astype(np.float64),
            "dv": step.dv[:T].float().cpu().numpy().astype(np.float64)}
     check(got, run_oracle(x, cu, False), label="non-causal, roomy workspace: ")
+
+
+@pytest.mark.parametrize("lengths,h,cp_r,causal", [
+    ([577], 1, 0, True),              # ten q sub-tiles for the first kv tile, one for the last
+    ([700, 64, 1], 2, 0, True),       # kv tiles of a single sub-tile beside long ones: nothing for the second CTA
+    ([1300], 3, 0, True),             # 33 kv tiles; an odd number of sub-tiles
+    ([640], 2, 0, False),             # every kv tile visits every sub-tile
+    ([1500], 2, 1, True),             # a kv chunk seen by two q chunks: the two CTAs alternate across pairs
+    ([577] * 7 + [64], 2, 0, True),   # 72 kv tiles of the 74 that pairs of CTAs take; with one more sequence, below,
+    ([577] * 7 + [64] * 3, 2, 0, True),   # too many: one CTA per tile
+])
+def test_key_tiles_shared_by_two_ctas(lengths, h, cp_r, causal):
+    """In calls with no more than half as many kv tiles as SMs two CTAs share a tile's q sub-tiles. Their parts of dK and dV
+    are added in fp32 before the one rounding, so the tolerance is that of the whole tile."""
+    run_case(lengths, h, cp_r, causal, seed=sum(lengths) + h, label=f"{lengths[:3]} h={h} ")
