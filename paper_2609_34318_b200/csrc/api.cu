@@ -865,12 +865,44 @@ int64_t ds_layout(const Problem& pb, int causal, std::vector<PairDev>* dev)
     return blocks + 1;                                  // one spare block: a q tile is read as two blocks
 }
 
+// q sub-tiles of pair p that a kv tile starting at row k0 of the pair's keys meets
+inline int32_t q_subs(const hydra_pair_t& p, int32_t k0, int causal)
+{
+    const int32_t n_sub = (p.q_len + SUB - 1) / SUB;
+    const int32_t i_min = causal ? k0 - (p.q_start - p.k_start) : 0;
+    return std::max(0, n_sub - (i_min > 0 ? i_min / SUB : 0));
+}
+
+// Two CTAs per key-side item where there are enough for that and the longest is worth the exchange at the end: it and the
+// cluster's start cost 2 us, a sub-tile takes 1.1. Step with sequences of 300 tokens (5 sub-tiles) 30.5 us with one CTA,
+// 31.8 with two; of 512 (8) 36.6 and 36.4; of 1024 tokens, 8 heads, 54.8 and 51.4; of 2048, 4 heads, 84.7 and 73.4.
+// Decided for a call as a whole, so that its bands add up dk and dv in the same order as one launch would.
+bool key_tiles_halved(const Problem& pb, int causal)
+{
+    std::vector<const hydra_pair_t*> by_k;
+    for (const auto& p : pb.pairs)
+        if (p.q_len > 0 && p.k_len > 0) by_k.push_back(&p);
+    auto range = [](const hydra_pair_t* p) { return Range{p->seq, p->k_start, p->k_len}; };
+    std::sort(by_k.begin(), by_k.end(), [&](const hydra_pair_t* a, const hydra_pair_t* b) { return range_less(range(a), range(b)); });
+    int64_t items = 0;
+    int32_t longest = 0;
+    for (size_t i = 0, j = 0; i < by_k.size(); i = j) {
+        for (j = i; j < by_k.size() && !range_less(range(by_k[i]), range(by_k[j])); ++j) {}
+        for (int32_t r0 = 0; r0 < by_k[i]->k_len; r0 += TILE) {
+            items += pb.h;
+            if (2 * items > plan_workers(1)) return false;
+            int32_t c = 0;
+            for (size_t t = i; t < j; ++t) c += q_subs(*by_k[t], r0, causal);
+            longest = std::max(longest, c);
+        }
+    }
+    return longest > 8;
+}
+
 void build_bwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& blob)
 {
     const int32_t n = static_cast<int32_t>(pb.pairs.size());
-    int32_t longest = 0;                                   // q sub-tiles of the longest key-side item (the last side built)
     auto group_by = [&](bool by_q, std::vector<int32_t>& lists, std::vector<GroupItem>& items) {
-        longest = 0;
         std::vector<int32_t> order(n);
         for (int32_t i = 0; i < n; ++i) order[i] = i;
         auto key = [&](int32_t i) {
@@ -904,20 +936,9 @@ void build_bwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
                     int32_t c = 0;
                     for (int32_t t = 0; t < list_len; ++t) {
                         const auto& p = pb.pairs[lists[list_off + t]];
-                        if (by_q) {
-                            c += kv_tiles(p, r0, causal);
-                        } else {
-                            const int32_t n_sub = (p.q_len + SUB - 1) / SUB;
-                            int32_t first = 0;
-                            if (causal) {
-                                const int32_t i_min = r0 - (p.q_start - p.k_start);
-                                first = i_min > 0 ? i_min / SUB : 0;
-                            }
-                            c += std::max(0, n_sub - first);
-                        }
+                        c += by_q ? kv_tiles(p, r0, causal) : q_subs(p, r0, causal);
                     }
                     groups.back().push_back(GroupEntry{r0, 0, 0, c});
-                    longest = std::max(longest, c);
                 }
             }
             i = j;
@@ -930,10 +951,7 @@ void build_bwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     std::vector<GroupItem> items_q, items_k;
     group_by(true, lists_q, items_q);
     group_by(false, lists_k, items_k);
-    // Two CTAs per key-side item where there are enough for that and the longest is worth the exchange at the end: it and the
-    // cluster's start cost 2 us, a sub-tile takes 1.1. Step with sequences of 300 tokens (5 sub-tiles) 30.5 us with one CTA,
-    // 31.8 with two; of 512 (8) 36.6 and 36.4; of 1024 tokens, 8 heads, 54.8 and 51.4; of 2048, 4 heads, 84.7 and 73.4.
-    plan.halves = longest > 8 && 2 * static_cast<int64_t>(items_k.size()) <= plan_workers(1);
+    plan.halves = key_tiles_halved(pb, causal);
     std::vector<PairDev> dev = device_pairs(pb);
     plan.ds_head_blocks = ds_layout(pb, causal, &dev);
     plan.off_pairs = append(blob, dev);
@@ -1611,10 +1629,10 @@ struct BwdTensors {
 // One backward over the pairs of `pb`: D = rowsum(dO*O) (if `first`), the key-side kernel, the query-side
 // kernel. dq and dk/dv are bf16 outputs or fp32 accumulators, each by its own flag. `ds` / `ds_room` is
 // where a dS hand-off buffer may go. With `first` false the status block keeps its flags and only the
-// work-queue counters are cleared.
+// work-queue counters are cleared. `halves_of_call` is key_tiles_halved of the whole call, -1 if `pb` is all of it.
 int32_t bwd_run(const Problem& pb, int32_t n_kv_heads, int32_t causal, float softmax_scale, const BwdTensors& t,
-                bool accumulate_dq, bool accumulate_dkv, void* workspace, uint8_t* ds, size_t ds_room, uint64_t ds_limit, bool first, int sms,
-                cudaStream_t stream)
+                bool accumulate_dq, bool accumulate_dkv, void* workspace, uint8_t* ds, size_t ds_room, uint64_t ds_limit, bool first,
+                int halves_of_call, int sms, cudaStream_t stream)
 {
     const int32_t n_heads = pb.h;
     const KernelSet* ks = kernel_set(pb.dqk, D_V);
@@ -1660,7 +1678,7 @@ int32_t bwd_run(const Problem& pb, int32_t n_kv_heads, int32_t causal, float sof
         bp.accumulate = accumulate_dkv ? 1 : 0;
         bp.debug_stall_ns = g_debug_stall_ns[HYDRA_STALL_BWD_DKV].load();
         ScopedKernelTimer timer(K_DKV, stream);
-        const bool halves = plan->halves != 0;
+        const bool halves = halves_of_call >= 0 ? halves_of_call != 0 : plan->halves != 0;
         if (ks->launch_bwd_dkv(mq_sub, mk, mv, mdo_sub, bp, halves, halves ? 2 * bp.n_items : std::min(sms, bp.n_items),
                                stream) != cudaSuccess)
             return HYDRA_ERR_CUDA;
@@ -1844,7 +1862,7 @@ int32_t bwd_core(Problem& pb, const void* q, const void* k, const void* v, const
         if (cudaMemsetAsync(dk_acc, 0, kv_bytes, stream) != cudaSuccess) return HYDRA_ERR_CUDA;
         const BwdTensors tg{q, k, v, out, dout, lse, dq, dk_acc, dv_acc};
         if (int32_t s = bwd_run(pb, n_kv_heads, causal, softmax_scale, tg, false, true, workspace,
-                                ws + ds_off + kv_bytes, room - kv_bytes, g_ds_limit_bytes.load(), true, sms, stream))
+                                ws + ds_off + kv_bytes, room - kv_bytes, g_ds_limit_bytes.load(), true, -1, sms, stream))
             return s;
         const size_t rk = static_cast<size_t>(n_kv_heads) * pb.dqk, rv = static_cast<size_t>(n_kv_heads) * D_V;
         for (const auto& run : covered_rows(pb, true)) {
@@ -1878,11 +1896,12 @@ int32_t bwd_core(Problem& pb, const void* q, const void* k, const void* v, const
                 const BwdTensors tb{q, k, v, out, dout, lse, dq_acc, dk, dv};
                 Problem band_pb;
                 band_pb.cu = pb.cu; band_pb.n_seqs = pb.n_seqs; band_pb.h = pb.h; band_pb.T = pb.T; band_pb.Tq = pb.Tq; band_pb.Tk = pb.Tk; band_pb.dqk = pb.dqk;
+                const int halves = key_tiles_halved(pb, causal);
                 bool first = true;
                 for (const auto& band : bands) {
                     band_pb.pairs = band;
                     if (int32_t s = bwd_run(band_pb, n_heads, causal, softmax_scale, tb, true, false, workspace,
-                                            ws + ds_off + acc_bytes, scratch, scratch, first, sms, stream))
+                                            ws + ds_off + acc_bytes, scratch, scratch, first, halves, sms, stream))
                         return s;
                     first = false;
                 }
@@ -1902,7 +1921,7 @@ int32_t bwd_core(Problem& pb, const void* q, const void* k, const void* v, const
         }
     }
     return bwd_run(pb, n_kv_heads, causal, softmax_scale, t, accumulate, accumulate, workspace, ws + ds_off, room,
-                   g_ds_limit_bytes.load(), true, sms, stream);
+                   g_ds_limit_bytes.load(), true, -1, sms, stream);
 }
 }  // namespace
 
