@@ -440,13 +440,13 @@ cudaError_t launch_grad_cast(const float* acc, void* grad, int64_t n, cudaStream
         const int64_t n16 = n / 16;
         const int64_t blocks = (n16 + kThreads - 1) / kThreads;
         const int grid = static_cast<int>(blocks < 1 ? 1 : (blocks < 148 * 16 ? blocks : 148 * 16));
-        return launch_overlapped(hydra_grad_cast_wide_kernel, grid, kThreads, 0, stream, reinterpret_cast<const V8*>(acc),
+        return launch_overlapped_spread<hydra_grad_cast_wide_kernel>(grid, kThreads, stream, reinterpret_cast<const V8*>(acc),
                                  static_cast<V8*>(grad), n16, n, acc, static_cast<__nv_bfloat16*>(grad));
     }
     const int64_t n8 = n / 8;
     const int64_t blocks = (n8 + kThreads - 1) / kThreads;
     const int grid = static_cast<int>(blocks < 1 ? 1 : (blocks < 148 * 16 ? blocks : 148 * 16));
-    return launch_overlapped(hydra_grad_cast_kernel, grid, kThreads, 0, stream, reinterpret_cast<const float4*>(acc),
+    return launch_overlapped_spread<hydra_grad_cast_kernel>(grid, kThreads, stream, reinterpret_cast<const float4*>(acc),
                              static_cast<uint4*>(grad), n8, n, acc, static_cast<__nv_bfloat16*>(grad));
 }
 
@@ -528,18 +528,18 @@ cudaError_t launch_merge(const MergeParams& p, cudaStream_t stream)
     const bool wide = ((reinterpret_cast<uintptr_t>(p.o_part) | reinterpret_cast<uintptr_t>(p.out)) & 31u) == 0;
     if (wide) {
         if (p.accumulate) {
-            if (four) return launch_overlapped(hydra_lse_merge_wide_kernel<true, 4>, p.n_items, kThreads, 0, stream, p);
-            else return launch_overlapped(hydra_lse_merge_wide_kernel<true, 2>, p.n_items, kThreads, 0, stream, p);
+            if (four) return launch_overlapped_spread<hydra_lse_merge_wide_kernel<true, 4>>(p.n_items, kThreads, stream, p);
+            else return launch_overlapped_spread<hydra_lse_merge_wide_kernel<true, 2>>(p.n_items, kThreads, stream, p);
         } else {
-            if (four) return launch_overlapped(hydra_lse_merge_wide_kernel<false, 4>, p.n_items, kThreads, 0, stream, p);
-            else return launch_overlapped(hydra_lse_merge_wide_kernel<false, 2>, p.n_items, kThreads, 0, stream, p);
+            if (four) return launch_overlapped_spread<hydra_lse_merge_wide_kernel<false, 4>>(p.n_items, kThreads, stream, p);
+            else return launch_overlapped_spread<hydra_lse_merge_wide_kernel<false, 2>>(p.n_items, kThreads, stream, p);
         }
     } else if (p.accumulate) {
-        if (four) return launch_overlapped(hydra_lse_merge_kernel<true, 4>, p.n_items, kThreads, 0, stream, p);
-        else return launch_overlapped(hydra_lse_merge_kernel<true, 2>, p.n_items, kThreads, 0, stream, p);
+        if (four) return launch_overlapped_spread<hydra_lse_merge_kernel<true, 4>>(p.n_items, kThreads, stream, p);
+        else return launch_overlapped_spread<hydra_lse_merge_kernel<true, 2>>(p.n_items, kThreads, stream, p);
     } else {
-        if (four) return launch_overlapped(hydra_lse_merge_kernel<false, 4>, p.n_items, kThreads, 0, stream, p);
-        else return launch_overlapped(hydra_lse_merge_kernel<false, 2>, p.n_items, kThreads, 0, stream, p);
+        if (four) return launch_overlapped_spread<hydra_lse_merge_kernel<false, 4>>(p.n_items, kThreads, stream, p);
+        else return launch_overlapped_spread<hydra_lse_merge_kernel<false, 2>>(p.n_items, kThreads, stream, p);
     }
 }
 
@@ -559,10 +559,10 @@ cudaError_t launch_bwd_prep(const void* dout, const void* out, float* dsum, int6
     if (((reinterpret_cast<uintptr_t>(dout) | reinterpret_cast<uintptr_t>(out)) & 31u) == 0) {
         const int64_t wide_passes = (T * h + 2 * kUnitsPerPass - 1) / (2 * kUnitsPerPass);
         const int wide_grid = static_cast<int>(wide_passes < 148 * 16 ? wide_passes : 148 * 16);
-        return launch_overlapped(hydra_bwd_prep_wide_kernel, wide_grid, kThreads, 0, stream, static_cast<const V8*>(dout),
+        return launch_overlapped_spread<hydra_bwd_prep_wide_kernel>(wide_grid, kThreads, stream, static_cast<const V8*>(dout),
                                  static_cast<const V8*>(out), dsum, T, h, status);
     }
-    return launch_overlapped(hydra_bwd_prep_kernel, grid, kThreads, 0, stream, static_cast<const uint4*>(dout),
+    return launch_overlapped_spread<hydra_bwd_prep_kernel>(grid, kThreads, stream, static_cast<const uint4*>(dout),
                              static_cast<const uint4*>(out), dsum, T, h, status);
 }
 
