@@ -2,12 +2,13 @@
 // (Section 5.2, "Exposed All-to-All Overlap": the query's rotary embedding; the split of the KV
 // up-projection's output into the value and the key's position-free part; the key's rotary embedding and
 // concatenation; the output gate), forward and backward. All are bound by HBM: every byte moves once, with
-// 16-byte or 4-byte accesses that are contiguous per warp. The paper names the steps, not their formulas;
+// 32-, 16- or 4-byte accesses that are contiguous per warp. The paper names the steps, not their formulas;
 // the readings taken (rotary pairs (2i, 2i+1), angle = position * theta^(-2i/rope_dim); one rotary key
 // vector per token shared by all heads; up-projection rows laid out [key part | value]; gate = sigmoid)
 // are stated with each entry point in the header.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <initializer_list>
 
 #include <cmath>
@@ -159,172 +160,12 @@ hydra_mla_kv_assemble_bwd_kernel(const uint32_t* __restrict__ dk, const uint32_t
     }
 }
 
-// ---------------------------------------------------------------------------------------------
-// 16-byte forms of the three kernels above (8 bf16 = 4 rotary pairs per access), used when the head
-// dimensions are multiples of 8 and the buffers 16-byte aligned: with 4-byte accesses a thread has 4 bytes
-// in flight (key / value assembly 2.0 TB/s on 262 144 tokens x 16 heads, 5.9 with a vector per thread), and the
-// pair's frequency is formed once per thread instead of once per token. Flat loops over a token's vectors with
-// one integer division per vector: a (head, column) assignment made once per thread and a float reciprocal were
-// both measured and are slower (4.5 TB/s).
-// ---------------------------------------------------------------------------------------------
-// cos / sin table of one token with the pair's frequency already in a register (one pair per thread)
-__device__ __forceinline__ void rope_table_fast(float* s_cos, float* s_sin, int32_t pos, int pairs, double freq,
-                                                int inverse)
-{
-    if (static_cast<int>(threadIdx.x) < pairs) {
-        double ang = static_cast<double>(pos) * freq;
-        ang -= 6.283185307179586476925 * floor(ang / 6.283185307179586476925);
-        float sn, cs;
-        sincosf(static_cast<float>(ang), &sn, &cs);
-        s_cos[threadIdx.x] = cs;
-        s_sin[threadIdx.x] = inverse ? -sn : sn;
-    }
-}
-__device__ __forceinline__ uint4 rotate_vec(const uint4& w, const float* cp, const float* sp)
-{
-    const float4 c4 = *reinterpret_cast<const float4*>(cp), s4 = *reinterpret_cast<const float4*>(sp);
-    const float c[4] = {c4.x, c4.y, c4.z, c4.w}, sn[4] = {s4.x, s4.y, s4.z, s4.w};
-    const uint32_t in[4] = {w.x, w.y, w.z, w.w};
-    uint32_t out[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const float2 v = bf2_to_f2(in[j]);
-        out[j] = f2_to_bf2(v.x * c[j] - v.y * sn[j], v.x * sn[j] + v.y * c[j]);
-    }
-    return make_uint4(out[0], out[1], out[2], out[3]);
-}
-
-__global__ void __launch_bounds__(kRopeThreads)
-hydra_rope_vec_kernel(const uint4* __restrict__ x, const int32_t* __restrict__ positions, uint4* __restrict__ y,
-                      int64_t n_tokens, int32_t n_heads, int32_t head_dim, int32_t rope_offset, int32_t rope_dim,
-                      double log_theta, int inverse, int in_place)
-{
-    overlap_next_launch();
-    __shared__ __align__(16) float s_cos[kMaxRopePairs], s_sin[kMaxRopePairs];
-    const int vph = head_dim / 8, v0 = rope_offset / 8, nv = rope_dim / 8;
-    const double freq = exp(-log_theta * (2.0 * threadIdx.x) / rope_dim);
-    wait_for_previous_launch();
-    for (int64_t t = blockIdx.x; t < n_tokens; t += gridDim.x) {
-        __syncthreads();                               // the previous token's table is no longer read
-        rope_table_fast(s_cos, s_sin, positions[t], rope_dim / 2, freq, inverse);
-        __syncthreads();
-        const int64_t row0 = t * n_heads * vph;
-        if (in_place) {                                // only the rotary columns move
-            for (int e = threadIdx.x; e < n_heads * nv; e += kRopeThreads) {
-                const int a = e / nv, i = e - a * nv;
-                const int64_t idx = row0 + static_cast<int64_t>(a) * vph + v0 + i;
-                y[idx] = rotate_vec(x[idx], s_cos + 4 * i, s_sin + 4 * i);
-            }
-        } else {
-            // the rotary vectors and the others in loops of their own: no lane waits for a rotation it does not
-            // do (one loop with a branch per vector: 4.4 instead of 5.65 TB/s)
-            const int n_copy = vph - nv;
-            for (int e = threadIdx.x; e < n_heads * nv; e += kRopeThreads) {
-                const int a = e / nv, i = e - a * nv;
-                const int64_t idx = row0 + static_cast<int64_t>(a) * vph + v0 + i;
-                y[idx] = rotate_vec(x[idx], s_cos + 4 * i, s_sin + 4 * i);
-            }
-            for (int e = threadIdx.x; e < n_heads * n_copy; e += kRopeThreads) {
-                const int a = e / n_copy, j = e - a * n_copy;
-                const int64_t idx = row0 + static_cast<int64_t>(a) * vph + (j < v0 ? j : j + nv);
-                y[idx] = x[idx];
-            }
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kRopeThreads)
-hydra_mla_kv_assemble_vec_kernel(const uint4* __restrict__ kv_up, const uint4* __restrict__ k_pe,
-                                 const int32_t* __restrict__ positions, uint4* __restrict__ k, uint4* __restrict__ v,
-                                 int64_t n_tokens, int32_t n_heads, int32_t nope, int32_t rope_dim, int32_t dv,
-                                 double log_theta)
-{
-    overlap_next_launch();
-    __shared__ __align__(16) float s_cos[kMaxRopePairs], s_sin[kMaxRopePairs];
-    __shared__ uint4 s_pe[kMaxRopePairs / 4];
-    const int nv = nope / 8, rv = rope_dim / 8, vv = dv / 8;
-    const int up_vecs = nv + vv, k_vecs = nv + rv;
-    const double freq = exp(-log_theta * (2.0 * threadIdx.x) / rope_dim);
-    wait_for_previous_launch();
-    for (int64_t t = blockIdx.x; t < n_tokens; t += gridDim.x) {
-        __syncthreads();
-        rope_table_fast(s_cos, s_sin, positions[t], rope_dim / 2, freq, 0);
-        __syncthreads();
-        if (static_cast<int>(threadIdx.x) < rv)
-            s_pe[threadIdx.x] = rotate_vec(k_pe[t * rv + threadIdx.x], s_cos + 4 * threadIdx.x, s_sin + 4 * threadIdx.x);
-        __syncthreads();
-        const int64_t up0 = t * n_heads * up_vecs, k0 = t * n_heads * k_vecs, v0 = t * n_heads * vv;
-        for (int e = threadIdx.x; e < n_heads * up_vecs; e += kRopeThreads) {
-            const int a = e / up_vecs, c = e - a * up_vecs;
-            const uint4 w = kv_up[up0 + e];
-            if (c < nv) k[k0 + static_cast<int64_t>(a) * k_vecs + c] = w;
-            else v[v0 + static_cast<int64_t>(a) * vv + (c - nv)] = w;
-        }
-        for (int e = threadIdx.x; e < n_heads * rv; e += kRopeThreads) {
-            const int a = e / rv, i = e - a * rv;
-            k[k0 + static_cast<int64_t>(a) * k_vecs + nv + i] = s_pe[i];
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kRopeThreads)
-hydra_mla_kv_assemble_bwd_vec_kernel(const uint4* __restrict__ dk, const uint4* __restrict__ dv,
-                                     const int32_t* __restrict__ positions, uint4* __restrict__ dkv_up,
-                                     uint4* __restrict__ dk_pe, int64_t n_tokens, int32_t n_heads, int32_t nope,
-                                     int32_t rope_dim, int32_t dvd, double log_theta)
-{
-    overlap_next_launch();
-    __shared__ __align__(16) float s_cos[kMaxRopePairs], s_sin[kMaxRopePairs];
-    const int nv = nope / 8, rv = rope_dim / 8, vv = dvd / 8;
-    const int up_vecs = nv + vv, k_vecs = nv + rv;
-    const double freq = exp(-log_theta * (2.0 * threadIdx.x) / rope_dim);
-    wait_for_previous_launch();
-    for (int64_t t = blockIdx.x; t < n_tokens; t += gridDim.x) {
-        __syncthreads();
-        rope_table_fast(s_cos, s_sin, positions[t], rope_dim / 2, freq, 1);
-        __syncthreads();
-        const int64_t up0 = t * n_heads * up_vecs, k0 = t * n_heads * k_vecs, v0 = t * n_heads * vv;
-        for (int e = threadIdx.x; e < n_heads * up_vecs; e += kRopeThreads) {
-            const int a = e / up_vecs, c = e - a * up_vecs;
-            dkv_up[up0 + e] = c < nv ? dk[k0 + static_cast<int64_t>(a) * k_vecs + c]
-                                     : dv[v0 + static_cast<int64_t>(a) * vv + (c - nv)];
-        }
-        // the shared rotary key's gradient: the sum over the heads, in fp32, rotated back (one vector per thread)
-        if (static_cast<int>(threadIdx.x) < rv) {
-            const int i = threadIdx.x;
-            float acc[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) acc[j] = 0.f;
-            for (int a = 0; a < n_heads; ++a) {
-                const uint4 w = dk[k0 + static_cast<int64_t>(a) * k_vecs + nv + i];
-                const uint32_t in[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float2 f = bf2_to_f2(in[j]);
-                    acc[2 * j] += f.x;
-                    acc[2 * j + 1] += f.y;
-                }
-            }
-            uint32_t out[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float c = s_cos[4 * i + j], sn = s_sin[4 * i + j];
-                out[j] = f2_to_bf2(acc[2 * j] * c - acc[2 * j + 1] * sn, acc[2 * j] * sn + acc[2 * j + 1] * c);
-            }
-            dk_pe[t * rv + i] = make_uint4(out[0], out[1], out[2], out[3]);
-        }
-    }
-}
-
 inline bool aligned16_all(std::initializer_list<const void*> ptrs)
 {
     uintptr_t bits = 0;
     for (const void* p : ptrs) bits |= reinterpret_cast<uintptr_t>(p);
     return (bits & 15u) == 0;
 }
-
-// (exp and reciprocal of the special-function unit: a relative error of 2^-21, far below the bf16 result's 2^-9)
-__device__ __forceinline__ float sigmoidf_(float x) { return __fdividef(1.f, 1.f + __expf(-x)); }
 
 // kWords 32-bit words (pairs of bf16) per thread and access: 4 (16 bytes), or 8 (32 bytes) where the element
 // count and the buffers allow it. Half as many threads then share the loop and address arithmetic.
@@ -346,6 +187,19 @@ __device__ __forceinline__ Words<kWords> ld_words(const void* base, int64_t i)
     }
     return v;
 }
+// the same from memory that this kernel writes
+template <int kWords>
+__device__ __forceinline__ Words<kWords> ld_words_coherent(const void* base, int64_t i)
+{
+    Words<kWords> v;
+    const uint4* p = reinterpret_cast<const uint4*>(static_cast<const Words<kWords>*>(base) + i);
+#pragma unroll
+    for (int j = 0; j < kWords / 4; ++j) {
+        const uint4 t = p[j];
+        v.w[4 * j] = t.x; v.w[4 * j + 1] = t.y; v.w[4 * j + 2] = t.z; v.w[4 * j + 3] = t.w;
+    }
+    return v;
+}
 template <int kWords>
 __device__ __forceinline__ void st_words(void* base, int64_t i, const Words<kWords>& v)
 {
@@ -355,6 +209,264 @@ __device__ __forceinline__ void st_words(void* base, int64_t i, const Words<kWor
         static_cast<uint4*>(base)[i] = make_uint4(v.w[0], v.w[1], v.w[2], v.w[3]);
     }
 }
+
+// ---------------------------------------------------------------------------------------------
+// Vector forms of the three kernels above (kWords rotary pairs, 16 or 32 bytes, per access), used when the head
+// dimensions are multiples of the vector and the buffers aligned to it. All three are bound by memory, and what keeps
+// them from its rate is the time in which a block has no access in flight. So: a block takes several tokens at once where
+// a token is short, and forms their cos / sin (or rotated keys) in one pass with a thread per (token, pair); what needs no
+// table is moved while that is done; vector numbers are split with a multiplication. Against one token, 128 threads and
+// 16 bytes at a time (and, in the backward, 8 threads adding up the rotary columns of all heads): 4096 tokens, 128 heads
+// of 128 + 64 / 128, rotary embedding 77.2 -> 66.6 us (6.05 TB/s), assembly 119.3 -> 97.3 (6.2), its backward
+// 155 -> 99.3 (6.1); 16384 tokens, 8 heads 20.8 -> 20.5, 31.3 -> 26.8 and 41.2 -> 31.3; 100 tokens, 128 heads 6.7 -> 5.7,
+// 9.7 -> 6.4 and 20.1 -> 6.1. A copy of as many bytes runs at 6.3 TB/s.
+// ---------------------------------------------------------------------------------------------
+constexpr int kVecThreads = 256;
+// Vectors of a thread in flight. The assembly gains from four (two: 100 us instead of 97.3); the other two need their registers
+// for more blocks (rotary embedding with four, two, one: 71.5, 66.6, 68.3 us; assembly backward 113, 99.3, 104).
+constexpr int kAsmUnroll = 4, kRopeUnroll = 2, kAsmBwdUnroll = 2;
+
+// n / d for n * d < 2^32 (`fits` below): the error of n * m / 2^32, m = floor(2^32 / d) + 1, is under 1 / d
+struct Div {
+    uint32_t d, m;
+    explicit Div(uint32_t div) : d(div), m(div > 1 ? static_cast<uint32_t>((uint64_t{1} << 32) / div) + 1 : 0) {}
+    __device__ __forceinline__ uint32_t operator()(uint32_t n) const { return m ? __umulhi(n, m) : n; }
+};
+
+// cos / sin of position * freq, the angle reduced as in rope_table
+__device__ __forceinline__ void rope_angle(int32_t pos, double freq, float& cs, float& sn)
+{
+    double ang = static_cast<double>(pos) * freq;
+    ang -= 6.283185307179586476925 * floor(ang / 6.283185307179586476925);
+    sincosf(static_cast<float>(ang), &sn, &cs);
+}
+
+// A block takes `per_item` tokens at once; thread (token of the item) * pairs + pair forms that pair's angle.
+struct VecItems {
+    int64_t n_tokens;
+    int32_t n_heads, per_item, pairs;
+    double log_theta;
+    Div by_heads;
+    VecItems(int64_t n, int32_t h, int32_t rope_dim, int64_t vecs_per_token, float theta)
+        : n_tokens(n), n_heads(h), per_item(1), pairs(rope_dim / 2), log_theta(std::log(static_cast<double>(theta))),
+          by_heads(static_cast<uint32_t>(h))
+    {
+        // eight vectors per thread where the tokens are short, but no fewer than two blocks per SM for that (4096 tokens of
+        // 8 heads: assembly backward 6.9 us, with four vectors and four blocks per SM 9.8)
+        const int64_t want = 8 * kVecThreads / vecs_per_token;
+        per_item = static_cast<int32_t>(std::max<int64_t>(1, std::min({want, int64_t{kVecThreads / pairs}, n / (148 * 2)})));
+    }
+    // are all vector and row numbers of an item in the range of Div?
+    bool fits(int32_t vecs_per_head) const
+    {
+        const double rows = static_cast<double>(per_item) * n_heads, vecs = rows * vecs_per_head;
+        return std::max(vecs * vecs_per_head, rows * n_heads) < 4294967296.0;
+    }
+    int grid() const
+    {
+        const int64_t items = (n_tokens + per_item - 1) / per_item;
+        return static_cast<int>(std::min<int64_t>(items, 148 * 32));
+    }
+};
+
+template <int kWords>
+__device__ __forceinline__ Words<kWords> rotate_vec(const Words<kWords>& w, const float* cp, const float* sp)
+{
+    Words<kWords> out;
+#pragma unroll
+    for (int j = 0; j < kWords; ++j) {
+        const float2 v = bf2_to_f2(w.w[j]);
+        out.w[j] = f2_to_bf2(v.x * cp[j] - v.y * sp[j], v.x * sp[j] + v.y * cp[j]);
+    }
+    return out;
+}
+
+// n vectors of a block: load(e) gives vector e and where it goes, store(at, v) puts it there
+template <int kWords, int kVecUnroll, class Load, class Store>
+__device__ __forceinline__ void move_vecs(uint32_t n, Load load, Store store)
+{
+    for (uint32_t e0 = threadIdx.x; e0 < n; e0 += kVecUnroll * kVecThreads) {
+        Words<kWords> v[kVecUnroll];
+        uint32_t at[kVecUnroll];
+#pragma unroll
+        for (int u = 0; u < kVecUnroll; ++u)
+            if (e0 + u * kVecThreads < n) v[u] = load(e0 + u * kVecThreads, at[u]);
+#pragma unroll
+        for (int u = 0; u < kVecUnroll; ++u)
+            if (e0 + u * kVecThreads < n) store(at[u], v[u]);
+    }
+}
+
+// the rotary vectors and the others in loops of their own: no lane waits for a rotation it does not do. In place (x == y)
+// only the rotary columns move.
+template <int kWords, bool kInPlace>
+__global__ void __launch_bounds__(kVecThreads)
+hydra_rope_vec_kernel(const uint32_t* x, const int32_t* __restrict__ positions, uint32_t* y, const VecItems it, int32_t v0,
+                      const Div by_rot, const Div by_copy, int inverse)
+{
+    overlap_next_launch();
+    __shared__ __align__(16) float s_cos[kVecThreads], s_sin[kVecThreads];
+    const uint32_t nv = by_rot.d, vph = by_rot.d + by_copy.d;
+    const int my_tok = threadIdx.x / it.pairs, my_pair = threadIdx.x - my_tok * it.pairs;
+    const double freq = exp(-it.log_theta * my_pair / it.pairs);
+    wait_for_previous_launch();
+    for (int64_t t0 = static_cast<int64_t>(blockIdx.x) * it.per_item; t0 < it.n_tokens;
+         t0 += static_cast<int64_t>(gridDim.x) * it.per_item) {
+        const int n_tok = static_cast<int>(min(static_cast<int64_t>(it.per_item), it.n_tokens - t0));
+        const uint32_t rows = n_tok * it.n_heads;
+        const uint32_t* xb = x + t0 * it.n_heads * vph * kWords;
+        uint32_t* yb = y + t0 * it.n_heads * vph * kWords;
+        if (!kInPlace)
+            move_vecs<kWords, kRopeUnroll>(rows * by_copy.d, [&](uint32_t e, uint32_t& at) {
+                const uint32_t r = by_copy(e), j = e - r * by_copy.d;
+                at = r * vph + (j < static_cast<uint32_t>(v0) ? j : j + nv);
+                return ld_words<kWords>(xb, at);
+            }, [&](uint32_t at, const Words<kWords>& v) { st_words<kWords>(yb, at, v); });
+        bool tables = false;
+        for (uint32_t e0 = threadIdx.x; !tables || e0 < rows * nv; e0 += kRopeUnroll * kVecThreads) {
+            Words<kWords> w[kRopeUnroll];
+#pragma unroll
+            for (int u = 0; u < kRopeUnroll; ++u) {
+                const uint32_t e = e0 + u * kVecThreads, r = by_rot(e), at = r * vph + v0 + e - r * nv;
+                if (e < rows * nv) w[u] = kInPlace ? ld_words_coherent<kWords>(xb, at) : ld_words<kWords>(xb, at);
+            }
+            if (!tables) {                             // the angles while the first vectors are on their way
+                tables = true;
+                __syncthreads();                       // the tables of the tokens before are no longer read
+                if (my_tok < n_tok) {
+                    float cs, sn;
+                    rope_angle(positions[t0 + my_tok], freq, cs, sn);
+                    s_cos[threadIdx.x] = cs;
+                    s_sin[threadIdx.x] = inverse ? -sn : sn;
+                }
+                __syncthreads();
+            }
+#pragma unroll
+            for (int u = 0; u < kRopeUnroll; ++u) {
+                const uint32_t e = e0 + u * kVecThreads, r = by_rot(e), i = e - r * nv;
+                const uint32_t c = it.by_heads(r) * it.pairs + i * kWords;
+                if (e < rows * nv) st_words<kWords>(yb, r * vph + v0 + i, rotate_vec<kWords>(w[u], s_cos + c, s_sin + c));
+            }
+        }
+    }
+}
+
+template <int kWords>
+__global__ void __launch_bounds__(kVecThreads)
+hydra_mla_kv_assemble_vec_kernel(const uint32_t* __restrict__ kv_up, const uint32_t* __restrict__ k_pe,
+                                 const int32_t* __restrict__ positions, uint32_t* __restrict__ k, uint32_t* __restrict__ v,
+                                 const VecItems it, uint32_t nv, const Div by_up, const Div by_rot)
+{
+    overlap_next_launch();
+    __shared__ __align__(32) uint32_t s_pe[kVecThreads];
+    const uint32_t vv = by_up.d - nv, rv = by_rot.d, k_vecs = nv + rv;
+    const int my_tok = threadIdx.x / it.pairs, my_pair = threadIdx.x - my_tok * it.pairs;
+    const double freq = exp(-it.log_theta * my_pair / it.pairs);
+    wait_for_previous_launch();
+    for (int64_t t0 = static_cast<int64_t>(blockIdx.x) * it.per_item; t0 < it.n_tokens;
+         t0 += static_cast<int64_t>(gridDim.x) * it.per_item) {
+        const int n_tok = static_cast<int>(min(static_cast<int64_t>(it.per_item), it.n_tokens - t0));
+        const uint32_t rows = n_tok * it.n_heads;
+        const int64_t row0 = t0 * it.n_heads;
+        const uint32_t* ub = kv_up + row0 * by_up.d * kWords;
+        uint32_t* kb = k + row0 * k_vecs * kWords;
+        uint32_t* vb = v + row0 * vv * kWords;
+        __syncthreads();                               // the rotated keys of the tokens before are no longer read
+        if (my_tok < n_tok) {
+            float cs, sn;
+            rope_angle(positions[t0 + my_tok], freq, cs, sn);
+            const float2 w = bf2_to_f2(k_pe[t0 * it.pairs + threadIdx.x]);
+            s_pe[threadIdx.x] = f2_to_bf2(w.x * cs - w.y * sn, w.x * sn + w.y * cs);
+        }
+        move_vecs<kWords, kAsmUnroll>(rows * by_up.d, [&](uint32_t e, uint32_t& at) {
+            at = e;
+            return ld_words<kWords>(ub, e);
+        }, [&](uint32_t e, const Words<kWords>& w) {
+            const uint32_t r = by_up(e), c = e - r * by_up.d;
+            if (c < nv) st_words<kWords>(kb, r * k_vecs + c, w);
+            else st_words<kWords>(vb, r * vv + (c - nv), w);
+        });
+        __syncthreads();
+        for (uint32_t e = threadIdx.x; e < rows * rv; e += kVecThreads) {
+            const uint32_t r = by_rot(e), i = e - r * rv;
+            const uint32_t* pe = s_pe + it.by_heads(r) * it.pairs + i * kWords;
+            Words<kWords> w;
+#pragma unroll
+            for (int j = 0; j < kWords; ++j) w.w[j] = pe[j];
+            st_words<kWords>(kb, r * k_vecs + nv + i, w);
+        }
+    }
+}
+
+// The shared rotary key's gradient is the sum over the heads: each thread adds up one vector over every n-th head of its
+// token, a thread per (token, pair) adds those partial sums in order, and rotates back.
+template <int kWords>
+__global__ void __launch_bounds__(kVecThreads)
+hydra_mla_kv_assemble_bwd_vec_kernel(const uint32_t* __restrict__ dk, const uint32_t* __restrict__ dv,
+                                     const int32_t* __restrict__ positions, uint32_t* __restrict__ dkv_up,
+                                     uint32_t* __restrict__ dk_pe, const VecItems it, uint32_t nv, const Div by_up, uint32_t rv)
+{
+    overlap_next_launch();
+    __shared__ __align__(16) float s_part[kVecThreads * 2 * kWords];
+    const uint32_t vv = by_up.d - nv, k_vecs = nv + rv;
+    const int my_tok = threadIdx.x / it.pairs, my_pair = threadIdx.x - my_tok * it.pairs;
+    const int part = threadIdx.x / rv, vec = threadIdx.x - part * rv;      // this thread's partial sum and vector of it
+    const int parts = kVecThreads / static_cast<int>(rv) / it.per_item;    // partial sums per token
+    const int part_tok = part / parts, first_head = part - part_tok * parts;
+    const double freq = exp(-it.log_theta * my_pair / it.pairs);
+    wait_for_previous_launch();
+    for (int64_t t0 = static_cast<int64_t>(blockIdx.x) * it.per_item; t0 < it.n_tokens;
+         t0 += static_cast<int64_t>(gridDim.x) * it.per_item) {
+        const int n_tok = static_cast<int>(min(static_cast<int64_t>(it.per_item), it.n_tokens - t0));
+        const uint32_t rows = n_tok * it.n_heads;
+        const int64_t row0 = t0 * it.n_heads;
+        const uint32_t* kb = dk + row0 * k_vecs * kWords;
+        const uint32_t* vb = dv + row0 * vv * kWords;
+        uint32_t* ub = dkv_up + row0 * by_up.d * kWords;
+        float acc[2 * kWords];
+#pragma unroll
+        for (int j = 0; j < 2 * kWords; ++j) acc[j] = 0.f;
+        if (part_tok < n_tok) {
+#pragma unroll 2
+            for (int a = first_head; a < it.n_heads; a += parts) {
+                const Words<kWords> w = ld_words<kWords>(kb, (part_tok * it.n_heads + a) * k_vecs + nv + vec);
+#pragma unroll
+                for (int j = 0; j < kWords; ++j) {
+                    const float2 f = bf2_to_f2(w.w[j]);
+                    acc[2 * j] += f.x;
+                    acc[2 * j + 1] += f.y;
+                }
+            }
+        }
+        __syncthreads();                               // the partial sums of the tokens before are no longer read
+        if (part_tok < n_tok) {
+#pragma unroll
+            for (int j = 0; j < 2 * kWords; j += 4)
+                *reinterpret_cast<float4*>(s_part + threadIdx.x * 2 * kWords + j) =
+                    make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
+        }
+        move_vecs<kWords, kAsmBwdUnroll>(rows * by_up.d, [&](uint32_t e, uint32_t& at) {
+            const uint32_t r = by_up(e), c = e - r * by_up.d;
+            at = e;
+            return c < nv ? ld_words<kWords>(kb, r * k_vecs + c) : ld_words<kWords>(vb, r * vv + (c - nv));
+        }, [&](uint32_t at, const Words<kWords>& w) { st_words<kWords>(ub, at, w); });
+        __syncthreads();
+        if (my_tok < n_tok) {
+            float sx = 0.f, sy = 0.f;
+            for (int q = 0; q < parts; ++q) {
+                const float2 f = *reinterpret_cast<const float2*>(s_part + ((my_tok * parts + q) * it.pairs + my_pair) * 2);
+                sx += f.x;
+                sy += f.y;
+            }
+            float cs, sn;
+            rope_angle(positions[t0 + my_tok], freq, cs, sn);
+            dk_pe[t0 * it.pairs + threadIdx.x] = f2_to_bf2(sx * cs + sy * sn, sy * cs - sx * sn);
+        }
+    }
+}
+
+// (exp and reciprocal of the special-function unit: a relative error of 2^-21, far below the bf16 result's 2^-9)
+__device__ __forceinline__ float sigmoidf_(float x) { return __fdividef(1.f, 1.f + __expf(-x)); }
 
 // y = out * sigmoid(gate)
 template <int kWords>
@@ -413,19 +525,40 @@ int grid_for(int64_t work_items, int per_block)
 
 }  // namespace
 
+// kWords of the vector kernels that the dimensions and buffers admit: 8, 4 or 0 (the four-byte kernels)
+static int words_for(std::initializer_list<int32_t> dims, std::initializer_list<const void*> ptrs)
+{
+    int32_t bits = 0;
+    for (int32_t d : dims) bits |= d;
+    if (bits % 16 == 0 && all_aligned32(ptrs)) return 8;
+    return bits % 8 == 0 && aligned16_all(ptrs) ? 4 : 0;
+}
+
+template <int kWords>
+static cudaError_t launch_rope_vec(const VecItems& it, const uint32_t* x, const int32_t* positions, uint32_t* y, int32_t head_dim,
+                                   int32_t rope_offset, int32_t rope_dim, int inverse, cudaStream_t stream)
+{
+    constexpr int32_t kElems = 2 * kWords;
+    const Div by_rot(rope_dim / kElems), by_copy((head_dim - rope_dim) / kElems);
+    return launch_overlapped(x == y ? hydra_rope_vec_kernel<kWords, true> : hydra_rope_vec_kernel<kWords, false>, it.grid(),
+                             kVecThreads, 0, stream, x, positions, y, it, rope_offset / kElems, by_rot, by_copy, inverse);
+}
+
 cudaError_t launch_rope(const void* x, const int32_t* positions, void* y, int64_t n_tokens, int32_t n_heads,
                         int32_t head_dim, int32_t rope_offset, int32_t rope_dim, float theta, int inverse,
                         cudaStream_t stream)
 {
     if (n_tokens == 0) return cudaSuccess;
-    if (head_dim % 8 == 0 && rope_offset % 8 == 0 && rope_dim % 8 == 0 && rope_dim / 2 <= kRopeThreads &&
-        aligned16_all({x, y})) {
-        return launch_overlapped(hydra_rope_vec_kernel, grid_for(n_tokens, 1), kRopeThreads, 0, stream,
-            static_cast<const uint4*>(x), positions, static_cast<uint4*>(y), n_tokens, n_heads, head_dim, rope_offset,
-            rope_dim, std::log(static_cast<double>(theta)), inverse, x == y ? 1 : 0);
+    const uint32_t* x32 = static_cast<const uint32_t*>(x);
+    uint32_t* y32 = static_cast<uint32_t*>(y);
+    if (const int words = words_for({head_dim, rope_offset, rope_dim}, {x, y})) {
+        const VecItems it(n_tokens, n_heads, rope_dim, int64_t{n_heads} * (head_dim / (2 * words)), theta);
+        if (it.fits(head_dim / (2 * words)))
+            return words == 8 ? launch_rope_vec<8>(it, x32, positions, y32, head_dim, rope_offset, rope_dim, inverse, stream)
+                              : launch_rope_vec<4>(it, x32, positions, y32, head_dim, rope_offset, rope_dim, inverse, stream);
     }
     return launch_overlapped(hydra_rope_kernel, grid_for(n_tokens, 1), kRopeThreads, 0, stream,
-        static_cast<const uint32_t*>(x), positions, static_cast<uint32_t*>(y), n_tokens, n_heads, head_dim, rope_offset,
+        x32, positions, y32, n_tokens, n_heads, head_dim, rope_offset,
         rope_dim, std::log(static_cast<double>(theta)), inverse, x == y ? 1 : 0);
 }
 
@@ -434,15 +567,20 @@ cudaError_t launch_mla_kv_assemble(const void* kv_up, const void* k_pe, const in
                                    float theta, cudaStream_t stream)
 {
     if (n_tokens == 0) return cudaSuccess;
-    if (nope % 8 == 0 && rope_dim % 8 == 0 && dv % 8 == 0 && rope_dim / 2 <= kRopeThreads &&
-        aligned16_all({kv_up, k_pe, k, v})) {
-        return launch_overlapped(hydra_mla_kv_assemble_vec_kernel, grid_for(n_tokens, 1), kRopeThreads, 0, stream,
-            static_cast<const uint4*>(kv_up), static_cast<const uint4*>(k_pe), positions, static_cast<uint4*>(k),
-            static_cast<uint4*>(v), n_tokens, n_heads, nope, rope_dim, dv, std::log(static_cast<double>(theta)));
+    const uint32_t *up32 = static_cast<const uint32_t*>(kv_up), *pe32 = static_cast<const uint32_t*>(k_pe);
+    uint32_t *k32 = static_cast<uint32_t*>(k), *v32 = static_cast<uint32_t*>(v);
+    if (const int words = words_for({nope, rope_dim, dv}, {kv_up, k, v})) {
+        const int32_t per_head = (nope + std::max(dv, rope_dim)) / (2 * words);
+        const VecItems it(n_tokens, n_heads, rope_dim, int64_t{n_heads} * ((nope + dv) / (2 * words)), theta);
+        if (it.fits(per_head)) {
+            const uint32_t nv = nope / (2 * words);
+            const Div by_up((nope + dv) / (2 * words)), by_rot(rope_dim / (2 * words));
+            return launch_overlapped(words == 8 ? hydra_mla_kv_assemble_vec_kernel<8> : hydra_mla_kv_assemble_vec_kernel<4>,
+                                     it.grid(), kVecThreads, 0, stream, up32, pe32, positions, k32, v32, it, nv, by_up, by_rot);
+        }
     }
     return launch_overlapped(hydra_mla_kv_assemble_kernel, grid_for(n_tokens, 1), kRopeThreads, 0, stream,
-        static_cast<const uint32_t*>(kv_up), static_cast<const uint32_t*>(k_pe), positions, static_cast<uint32_t*>(k),
-        static_cast<uint32_t*>(v), n_tokens, n_heads, nope, rope_dim, dv, std::log(static_cast<double>(theta)));
+        up32, pe32, positions, k32, v32, n_tokens, n_heads, nope, rope_dim, dv, std::log(static_cast<double>(theta)));
 }
 
 cudaError_t launch_mla_kv_assemble_bwd(const void* dk, const void* dv, const int32_t* positions, void* dkv_up,
@@ -450,15 +588,20 @@ cudaError_t launch_mla_kv_assemble_bwd(const void* dk, const void* dv, const int
                                        int32_t dvd, float theta, cudaStream_t stream)
 {
     if (n_tokens == 0) return cudaSuccess;
-    if (nope % 8 == 0 && rope_dim % 8 == 0 && dvd % 8 == 0 && rope_dim / 2 <= kRopeThreads &&
-        aligned16_all({dk, dv, dkv_up, dk_pe})) {
-        return launch_overlapped(hydra_mla_kv_assemble_bwd_vec_kernel, grid_for(n_tokens, 1), kRopeThreads, 0, stream,
-            static_cast<const uint4*>(dk), static_cast<const uint4*>(dv), positions, static_cast<uint4*>(dkv_up),
-            static_cast<uint4*>(dk_pe), n_tokens, n_heads, nope, rope_dim, dvd, std::log(static_cast<double>(theta)));
+    const uint32_t *dk32 = static_cast<const uint32_t*>(dk), *dv32 = static_cast<const uint32_t*>(dv);
+    uint32_t *up32 = static_cast<uint32_t*>(dkv_up), *pe32 = static_cast<uint32_t*>(dk_pe);
+    if (const int words = words_for({nope, rope_dim, dvd}, {dk, dv, dkv_up})) {
+        const int32_t per_head = (nope + std::max(dvd, rope_dim)) / (2 * words);
+        const VecItems it(n_tokens, n_heads, rope_dim, int64_t{n_heads} * ((nope + dvd) / (2 * words)), theta);
+        if (it.fits(per_head)) {
+            const uint32_t nv = nope / (2 * words), rv = rope_dim / (2 * words);
+            const Div by_up((nope + dvd) / (2 * words));
+            return launch_overlapped(words == 8 ? hydra_mla_kv_assemble_bwd_vec_kernel<8> : hydra_mla_kv_assemble_bwd_vec_kernel<4>,
+                                     it.grid(), kVecThreads, 0, stream, dk32, dv32, positions, up32, pe32, it, nv, by_up, rv);
+        }
     }
     return launch_overlapped(hydra_mla_kv_assemble_bwd_kernel, grid_for(n_tokens, 1), kRopeThreads, 0, stream,
-        static_cast<const uint32_t*>(dk), static_cast<const uint32_t*>(dv), positions, static_cast<uint32_t*>(dkv_up),
-        static_cast<uint32_t*>(dk_pe), n_tokens, n_heads, nope, rope_dim, dvd, std::log(static_cast<double>(theta)));
+        dk32, dv32, positions, up32, pe32, n_tokens, n_heads, nope, rope_dim, dvd, std::log(static_cast<double>(theta)));
 }
 
 cudaError_t launch_gate(const void* out, const void* gate, void* y, int64_t n8, cudaStream_t stream)

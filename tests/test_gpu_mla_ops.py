@@ -163,3 +163,40 @@ def test_dimensions_that_are_not_multiples_of_eight_take_the_four_byte_kernels(i
     torch.cuda.synchronize()
     assert np.array_equal(f64(dup), up_ref)
     close(f64(dpe), pe_ref, np.abs(pe_ref).max(), "rotary key gradient, odd dimensions")
+
+
+@pytest.mark.parametrize("T,h,nope,rope,dv,in_place", [
+    (1500, 2, 128, 64, 128, False),     # 32-byte vectors, several tokens per block, a last block with fewer
+    (650, 3, 24, 24, 8, True),          # 16-byte vectors, three rotary vectors per head (256 threads: one left over)
+    (601, 1, 8, 8, 8, False),           # one vector of each kind per head
+    (3, 5, 16, 256, 32, True),          # the most rotary columns: two tokens' angles fill a block
+    (5, 130, 128, 64, 128, False)])     # more vectors per token than a block takes in one sweep
+def test_vector_kernels_at_the_edges_of_their_blocks(T, h, nope, rope, dv, in_place):
+    import paper_2609_34318_b200 as P
+    rng = np.random.default_rng(55)
+    pos = rng.integers(0, 262144, T).astype(np.int32)
+    pd = torch.from_numpy(pos).cuda()
+    nan = lambda *shape: torch.full(shape, float("nan"), dtype=torch.bfloat16, device="cuda")
+    xb = bits(rng, (T, h, nope + rope))
+    x = hw.bf16_bits_to_f64(xb)
+    ref = M.rope(x, pos, nope, rope, THETA)
+    xd = dev(xb)
+    yd = xd if in_place else nan(T, h, nope + rope)
+    P.hydra_mla_rope(xd, pd, T, h, nope + rope, nope, rope, THETA, False, yd)
+    torch.cuda.synchronize()
+    assert np.array_equal(f64(yd)[..., :nope], x[..., :nope])
+    close(f64(yd)[..., nope:], ref[..., nope:], np.abs(x).max(), "rope")
+    up_b, pe_b = bits(rng, (T, h, nope + dv)), bits(rng, (T, rope))
+    k_ref, v_ref = M.kv_assemble(hw.bf16_bits_to_f64(up_b), hw.bf16_bits_to_f64(pe_b), pos, nope, rope, dv, THETA)
+    k, v = nan(T, h, nope + rope), nan(T, h, dv)
+    P.hydra_mla_kv_assemble(dev(up_b), dev(pe_b), pd, T, h, nope, rope, dv, THETA, k, v)
+    torch.cuda.synchronize()
+    assert np.array_equal(f64(k)[..., :nope], k_ref[..., :nope]) and np.array_equal(f64(v), v_ref)
+    close(f64(k)[..., nope:], k_ref[..., nope:], np.abs(hw.bf16_bits_to_f64(pe_b)).max(), "assembled key, rotary part")
+    dk_b, dv_b = bits(rng, (T, h, nope + rope)), bits(rng, (T, h, dv))
+    up_ref, pe_ref = M.kv_assemble_bwd(hw.bf16_bits_to_f64(dk_b), hw.bf16_bits_to_f64(dv_b), pos, nope, rope, dv, THETA)
+    dup, dpe = nan(T, h, nope + dv), nan(T, rope)
+    P.hydra_mla_kv_assemble_bwd(dev(dk_b), dev(dv_b), pd, T, h, nope, rope, dv, THETA, dup, dpe)
+    torch.cuda.synchronize()
+    assert np.array_equal(f64(dup), up_ref)
+    close(f64(dpe), pe_ref, np.abs(pe_ref).max(), "rotary key gradient (summed over heads)")
