@@ -203,7 +203,7 @@ constexpr bool kKInTmem = kDqk == 128;
 constexpr uint32_t kTmK = kTmDK + 128;
 enum : int { B_KVFULL = 0, B_KVEMPTY = 1, B_QFULL = 2, B_STAT = 5, B_QEMPTY = 8, B_SFULL = 11,
              B_SFREE = 12, B_PFULL = 13, B_PDSFREE = 14, B_ACCFREE = 15, B_PEERFREE = 16, B_PEERDATA = 17,
-             B_ITEMFULL = 18, B_ITEMEMPTY = 18 + kSched, B_COUNT = 18 + 2 * kSched };
+             B_VFULL = 18, B_ITEMFULL = 19, B_ITEMEMPTY = 19 + kSched, B_COUNT = 19 + 2 * kSched };
 static_assert(kDqk * TILE * 4u <= kDsStage, "the other CTA's part of dK fits the operand space");
 
 // Iterator over (pair of the kv chunk, 64-row q sub-tile).
@@ -774,21 +774,6 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                     if (lane == 0) raw_next = pop_begin(kq);
                     asked = true;
                 }
-                if (live && start) {
-                    start = false;
-                    ok = wait(B_KVEMPTY, items ^ 1u);
-                    if (!ok) break;
-                    ++items;
-                    if (lane == 0) {
-                        mbar_arrive_expect_tx(bar(B_KVFULL), (kQkBoxes + 2) * kBox128);
-                        for (int c = 0; c < kQkBoxes; ++c)
-                            tma_load_3d(smem + kK + c * kBox128, &map_k, bar(B_KVFULL), c * 64, item.head / p.kv_group,
-                                        first.k_tok0 + item.r0);
-                        for (int c = 0; c < 2; ++c)
-                            tma_load_3d(smem + kV + c * kBox128, &map_v, bar(B_KVFULL), c * 64, item.head / p.kv_group,
-                                        first.k_tok0 + item.r0);
-                    }
-                }
                 if (live) {
                     const int st = gq % kStages;
                     ok = wait(B_QEMPTY + st, (gq / kStages) ^ 1u);
@@ -802,6 +787,26 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                         for (int c = 0; c < 2; ++c)
                             tma_load_3d(smem + kDO + st * 2 * kBox64 + c * kBox64, &map_do, bar(B_QFULL + st), c * 64,
                                         item.head, tok);
+                    }
+                    // The item's K and V come after its first Q and dO, which find a free stage while the item before still
+                    // reads its K and V (80 KB that take some 3000 cycles to arrive then: between items this is what the
+                    // tensor core waits for), and S does not wait for V. Sequences of 64 to 512 tokens, 32 heads
+                    // 1.104 -> 1.094 ms, whole step on 32K packed tokens 1.870 -> 1.863.
+                    if (start) {
+                        start = false;
+                        ok = wait(B_KVEMPTY, items ^ 1u);
+                        if (!ok) break;
+                        ++items;
+                        if (lane == 0) {
+                            mbar_arrive_expect_tx(bar(B_KVFULL), kQkBoxes * kBox128);
+                            mbar_arrive_expect_tx(bar(B_VFULL), 2 * kBox128);
+                            for (int c = 0; c < kQkBoxes; ++c)
+                                tma_load_3d(smem + kK + c * kBox128, &map_k, bar(B_KVFULL), c * 64, item.head / p.kv_group,
+                                            first.k_tok0 + item.r0);
+                            for (int c = 0; c < 2; ++c)
+                                tma_load_3d(smem + kV + c * kBox128, &map_v, bar(B_VFULL), c * 64, item.head / p.kv_group,
+                                            first.k_tok0 + item.r0);
+                        }
                     }
                     // LSE (as log2) and D of the 64 q rows, two rows per lane
 #pragma unroll
@@ -858,6 +863,7 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                 if (!si.valid()) continue;
                 if (issue_scores) {
                     ok = wait(B_KVFULL, items);
+                    bool v_here = false;
                     // (every score product of the previous item has completed: this item's K was loaded behind them)
                     if (kKInTmem && ok) {
                         tc_fence_after_sync();
@@ -890,6 +896,14 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                                 else umma_ss_w(tm + kTmS, k_lo + (kk >> 2) * (kBox128 >> 4) + (kk & 3) * 2, hi_kmaj, b_lo, hi_kmaj,
                                                idesc_st, kk > 0);
                             }
+                        }
+                        if (!v_here) {
+                            ok = wait(B_VFULL, items);
+                            if (!ok) break;
+                            tc_fence_after_sync();
+                            v_here = true;
+                        }
+                        if (elect_one()) {
 #pragma unroll
                             for (int kk = 0; kk < D_V / 16; ++kk)
                                 umma_ss_w(tm + kTmDP, v_lo + (kk >> 2) * (kBox128 >> 4) + (kk & 3) * 2, hi_kmaj,
