@@ -464,19 +464,35 @@ __device__ __forceinline__ void st_unit(V8* p, const V8& v)
                  "r"(v.w[2]), "r"(v.w[3]), "r"(v.w[4]), "r"(v.w[5]), "r"(v.w[6]), "r"(v.w[7])
                  : "memory");
 }
-template <bool kPack, class Vec>
+template <bool kPack, class Vec, bool kLong>
 __global__ void __launch_bounds__(kThreads)
 hydra_ulysses_kernel(const Vec* __restrict__ src, Vec* __restrict__ dst, uint32_t n, uint32_t P, uint32_t cu,
                      uint32_t rows)
 {
     overlap_next_launch();
     wait_for_previous_launch();
-    // A warp takes one chunk (row = j * n + t of the block-major side) at a time, four chunks in flight:
+    // kLong: a warp takes one chunk (row = j * n + t of the block-major side) at a time, four units per lane in flight.
+    // Otherwise (a chunk is at most one unit per lane) four chunks in flight:
     // the two divisions are paid once per chunk, not once per 16 bytes (a flat loop over units spent its
     // time on them: 5.1 TB/s).
     constexpr int kUnroll = 4;
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t n_warps = gridDim.x * (kThreads / 32);
+    if (kLong) {
+        for (uint32_t r = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); r < rows; r += n_warps) {
+            const uint32_t j = r / n, t = r - j * n, blk = r * cu, tok = (t * P + j) * cu;
+            for (uint32_t w0 = lane; w0 < cu; w0 += 32 * kUnroll) {
+                Vec v[kUnroll];
+#pragma unroll
+                for (int e = 0; e < kUnroll; ++e)
+                    if (w0 + e * 32 < cu) v[e] = ld_unit(src + (kPack ? tok : blk) + w0 + e * 32);
+#pragma unroll
+                for (int e = 0; e < kUnroll; ++e)
+                    if (w0 + e * 32 < cu) st_unit(dst + (kPack ? blk : tok) + w0 + e * 32, v[e]);
+            }
+        }
+        return;
+    }
     for (uint32_t r0 = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); r0 < rows; r0 += n_warps * kUnroll) {
         uint32_t blk[kUnroll], tok[kUnroll];
 #pragma unroll
@@ -503,22 +519,28 @@ cudaError_t launch_ulysses(bool pack, const void* src, void* dst, int64_t n_toke
 {
     const int64_t rows = n_tokens * cp_u;
     if (rows <= 0 || chunk_units <= 0) return cudaSuccess;
-    const int64_t blocks = (rows + (kThreads / 32) * 4 - 1) / ((kThreads / 32) * 4);
-    const int grid = static_cast<int>(blocks < 148 * 8 ? blocks : 148 * 8);
+    const bool wide = (chunk_units & 1) == 0 && ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 31u) == 0;
+    // Chunks of more than one unit per lane: a warp per chunk. 8192 tokens, 64 heads of 128, eight ranks (64 units) pack /
+    // unpack 43.9 / 42.3 -> 42.2 / 41.4 us, 32 heads of 192 (48) 34.0 / 34.0 -> 32.0 / 31.7; of 128 (32 units) 19.5 / 19.1
+    // with four chunks per warp, 21.3 / 21.0 with one. 1024 tokens, 128 heads of 192: 18.4 -> 12.5 (four times the warps).
+    const bool is_long = (wide ? chunk_units / 2 : chunk_units) > 32;
+    const int64_t per = (kThreads / 32) * (is_long ? 1 : 4), cap = is_long ? 148 * 32 : 148 * 8;
+    const int64_t blocks = (rows + per - 1) / per;
+    const int grid = static_cast<int>(blocks < cap ? blocks : cap);
     const uint4* s = static_cast<const uint4*>(src);
     uint4* d = static_cast<uint4*>(dst);
     // 32-bit index arithmetic: the caller has checked that the units (plus one sweep of the grid) fit
     const uint32_t n = static_cast<uint32_t>(n_tokens), P = static_cast<uint32_t>(cp_u),
                    cu = static_cast<uint32_t>(chunk_units), r = static_cast<uint32_t>(rows);
-    if ((cu & 1u) == 0 && ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 31u) == 0) {
+    if (wide) {
         // chunks of whole 32-byte units in 32-byte aligned buffers: half as many, twice as large accesses
         const V8* s32 = static_cast<const V8*>(src);
         V8* d32 = static_cast<V8*>(dst);
-        if (pack) return launch_overlapped(hydra_ulysses_kernel<true, V8>, grid, kThreads, 0, stream, s32, d32, n, P, cu / 2, r);
-        else return launch_overlapped(hydra_ulysses_kernel<false, V8>, grid, kThreads, 0, stream, s32, d32, n, P, cu / 2, r);
+        if (pack) return launch_overlapped(is_long ? hydra_ulysses_kernel<true, V8, true> : hydra_ulysses_kernel<true, V8, false>, grid, kThreads, 0, stream, s32, d32, n, P, cu / 2, r);
+        else return launch_overlapped(is_long ? hydra_ulysses_kernel<false, V8, true> : hydra_ulysses_kernel<false, V8, false>, grid, kThreads, 0, stream, s32, d32, n, P, cu / 2, r);
     }
-    if (pack) return launch_overlapped(hydra_ulysses_kernel<true, uint4>, grid, kThreads, 0, stream, s, d, n, P, cu, r);
-    else return launch_overlapped(hydra_ulysses_kernel<false, uint4>, grid, kThreads, 0, stream, s, d, n, P, cu, r);
+    if (pack) return launch_overlapped(is_long ? hydra_ulysses_kernel<true, uint4, true> : hydra_ulysses_kernel<true, uint4, false>, grid, kThreads, 0, stream, s, d, n, P, cu, r);
+    else return launch_overlapped(is_long ? hydra_ulysses_kernel<false, uint4, true> : hydra_ulysses_kernel<false, uint4, false>, grid, kThreads, 0, stream, s, d, n, P, cu, r);
 }
 
 cudaError_t launch_merge(const MergeParams& p, cudaStream_t stream)
