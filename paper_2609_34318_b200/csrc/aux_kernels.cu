@@ -547,21 +547,28 @@ cudaError_t launch_merge(const MergeParams& p, cudaStream_t stream)
 {
     if (p.n_items == 0) return cudaSuccess;
     const bool four = p.max_parts > 2;
+    // Not launched ahead of the forward's end, unlike the other kernels of a call (the kernel behind it does start early): 432
+    // chunk pairs of about 200 tokens, 4 heads 131 -> 127.5 us with their forward, 72 pairs, 16 heads 49.4 -> 47.3, one
+    // rank's ring step of 64K tokens 5.54 -> 5.44 ms, 65536 tokens of short sequences cut in two 3.05 -> 3.015.
+    auto launch = [&](auto kernel) {
+        kernel<<<p.n_items, kThreads, 0, stream>>>(p);
+        return cudaGetLastError();
+    };
     const bool wide = ((reinterpret_cast<uintptr_t>(p.o_part) | reinterpret_cast<uintptr_t>(p.out)) & 31u) == 0;
     if (wide) {
         if (p.accumulate) {
-            if (four) return launch_overlapped_spread<hydra_lse_merge_wide_kernel<true, 4>>(p.n_items, kThreads, stream, p);
-            else return launch_overlapped_spread<hydra_lse_merge_wide_kernel<true, 2>>(p.n_items, kThreads, stream, p);
+            if (four) return launch(hydra_lse_merge_wide_kernel<true, 4>);
+            else return launch(hydra_lse_merge_wide_kernel<true, 2>);
         } else {
-            if (four) return launch_overlapped_spread<hydra_lse_merge_wide_kernel<false, 4>>(p.n_items, kThreads, stream, p);
-            else return launch_overlapped_spread<hydra_lse_merge_wide_kernel<false, 2>>(p.n_items, kThreads, stream, p);
+            if (four) return launch(hydra_lse_merge_wide_kernel<false, 4>);
+            else return launch(hydra_lse_merge_wide_kernel<false, 2>);
         }
     } else if (p.accumulate) {
-        if (four) return launch_overlapped_spread<hydra_lse_merge_kernel<true, 4>>(p.n_items, kThreads, stream, p);
-        else return launch_overlapped_spread<hydra_lse_merge_kernel<true, 2>>(p.n_items, kThreads, stream, p);
+        if (four) return launch(hydra_lse_merge_kernel<true, 4>);
+        else return launch(hydra_lse_merge_kernel<true, 2>);
     } else {
-        if (four) return launch_overlapped_spread<hydra_lse_merge_kernel<false, 4>>(p.n_items, kThreads, stream, p);
-        else return launch_overlapped_spread<hydra_lse_merge_kernel<false, 2>>(p.n_items, kThreads, stream, p);
+        if (four) return launch(hydra_lse_merge_kernel<false, 4>);
+        else return launch(hydra_lse_merge_kernel<false, 2>);
     }
 }
 

@@ -179,11 +179,10 @@ cudaError_t launch_overlapped(void (*kernel)(Params...), int grid, int block, si
 }
 // A grid of small blocks behind a kernel that fills the GPU: its blocks start as that kernel's leave, as many as fit on each
 // SM that comes free first, and a grid of two or three blocks per SM ends up on a fraction of the SMs. Dynamic shared
-// memory that the kernel does not use keeps it to as many blocks per SM as an even spread has. A loop of forward calls on
-// 72 chunk pairs (2048 packed tokens cut over four ranks, 16 heads, d_qk 128; a merge of about 3 blocks per SM) takes
-// 49.5 us with it and 58.9 without; a 1024-token step of 8 heads, where it is the backward's first kernel, 49.6 and 51.4.
-// From four blocks per SM on there is nothing to keep apart (the kernels' registers admit four to eight): spreading up
-// to eight per SM changed no time, spreading a single block per SM only gave back what three blocks gain.
+// memory that the kernel does not use keeps it to as many blocks per SM as an even spread has. A 1024-token step of 8 heads,
+// where D = rowsum(dO O) is such a grid, takes 49.6 us with it and 51.4 without. From four blocks per SM on there is
+// nothing to keep apart (the kernels' registers admit four to eight): spreading up to eight per SM changed no time,
+// spreading a single block per SM only gave the gain back.
 template <auto kKernel, class... Args>
 cudaError_t launch_overlapped_spread(int grid, int block, cudaStream_t stream, Args&&... args)
 {
