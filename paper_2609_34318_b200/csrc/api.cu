@@ -676,24 +676,28 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     // an idle slot beside every busy one and gives it the second half of the tile's keys, whatever their number (the
     // CTA-pair kernel would leave more than half of the SMs idle).
     // (A limit set by the caller is kept to.)
+    // (A work item counts its steps in 16 bits: more keys than two items hold stay with the CTA-pair kernel.)
+    constexpr int64_t kMostKeys = int64_t{UINT16_MAX} * FWD_SHORT_KEYS;
     int64_t n_tiles = 0;
+    int32_t longest = 0, most_keys = 0;
     bool within = true;
     for (const auto& p : pb.pairs) {
         n_tiles += (p.q_len + TILE - 1) / TILE;
+        longest = std::max(longest, std::max(p.q_len, p.k_len));
+        most_keys = std::max(most_keys, p.k_len);
         within = within && p.q_len <= short_len && p.k_len <= short_len;
     }
     n_tiles *= pb.h;
-    const bool halves = short_len > 0 && n_tiles <= plan_workers(1) && (within || g_fwd_short_len.load() < 0);
+    const bool halves = short_len > 0 && n_tiles <= plan_workers(1) && most_keys <= 2 * kMostKeys &&
+                        (within || g_fwd_short_len.load() < 0);
     if (halves) {
         std::fill(is_short.begin(), is_short.end(), 1);
     } else {
         double work_short = 0, work_all = 0;
-        int32_t longest = 0;
         for (size_t pi = 0; pi < pb.pairs.size(); ++pi) {
             const auto& p = pb.pairs[pi];
             const double w = static_cast<double>(p.q_len) * p.k_len;
             work_all += w;
-            longest = std::max(longest, std::max(p.q_len, p.k_len));
             if (short_len > 0 && p.q_len <= short_len && p.k_len <= short_len) { is_short[pi] = 1; work_short += w; }
         }
         if (work_short * 4 < work_all) std::fill(is_short.begin(), is_short.end(), 0);
@@ -701,7 +705,8 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
         // as fast: pairs up to twice the limit cost it at most a tenth more, and 2^29 positions (with those above the
         // mask) take 0.2 ms. 4096 packed tokens, 16 heads, the longest sequence 1381 tokens: 75 us on both kernels,
         // 59 on the short one alone.
-        else if (work_short < work_all && longest <= 2 * short_len && (work_all - work_short) * pb.h <= double{1 << 29})
+        else if (work_short < work_all && longest <= 2 * short_len && most_keys <= kMostKeys &&
+                 (work_all - work_short) * pb.h <= double{1 << 29})
             std::fill(is_short.begin(), is_short.end(), 1);
     }
     std::vector<std::vector<GroupEntry>> groups(pb.pairs.size()), groups_short(pb.pairs.size());

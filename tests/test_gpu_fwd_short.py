@@ -75,6 +75,40 @@ def test_tiles_shared_by_the_two_slots(lengths, h):
     check(got, run_oracle(x, cu), label=f"{lengths[:4]} ")
 
 
+@pytest.mark.parametrize("keys", [
+    131070 * 64,              # the most that two halves of a tile count in 16 bits each (8.4M keys)
+    131071 * 64 + 5,          # one step and a ragged one more: not a matter of this kernel any more
+])
+def test_as_many_keys_as_a_work_item_counts_and_more(keys):
+    """A few q rows against millions of keys is a call with no more q tiles than SMs, which shares a tile's keys between
+    two slots, as long as their steps of 64 keys fit the 16 bits of a work item."""
+    import paper_2609_34318_b200 as P
+    q_len = 3
+    cu = np.array([0, keys], dtype=np.int32)
+    gen = torch.Generator(device="cuda").manual_seed(keys)
+    normal = lambda *shape: torch.randn(shape, generator=gen, device="cuda", dtype=torch.bfloat16)
+    q, k, v = normal(q_len, 1, DQK), normal(keys, 1, DQK), normal(keys, 1, DV)
+    pairs = [dict(seq=0, q_start=keys - q_len, q_len=q_len, k_start=0, k_len=keys, part_row=-1, group=0)]
+    q_chunks, kv_chunks = [(0, keys - q_len, q_len, 0)], [(0, 0, keys, 0)]
+    out = torch.full((q_len, 1, DV), float("nan"), dtype=torch.bfloat16, device="cuda")
+    lse = torch.full((1, q_len), float("nan"), dtype=torch.float32, device="cuda")
+    ws = torch.zeros(4096, dtype=torch.uint8, device="cuda")
+    scale = 1.0 / np.sqrt(DQK)
+    P.hydra_attn_fwd_local(q, k, v, cu, 1, 1, DQK, DV, q_chunks, q_len, kv_chunks, keys, pairs, True, scale, out, lse,
+                           None, None, 0, ws)
+    assert P.hydra_poll_status(ws)[0] == 0
+    # the same in fp64, a block of keys at a time
+    block = 1 << 20
+    s = torch.cat([q[:, 0].double() @ k[i:i + block, 0].double().T for i in range(0, keys, block)], 1) * scale
+    s.masked_fill_(torch.arange(keys, device="cuda")[None] > torch.arange(keys - q_len, keys, device="cuda")[:, None],
+                   -float("inf"))
+    ref_l = s.logsumexp(1)
+    w = torch.exp(s - ref_l[:, None])
+    ref_o = sum(w[:, i:i + block] @ v[i:i + block, 0].double() for i in range(0, keys, block))
+    assert float((lse[0].double() - ref_l).abs().max()) <= TOL_LSE
+    assert float((out[:, 0].double() - ref_o).abs().max()) <= TOL_REL * float(ref_o.abs().max())
+
+
 def test_random_length_mixes_and_both_kernels_agree():
     import paper_2609_34318_b200 as P
     rng = np.random.default_rng(11)
