@@ -72,6 +72,7 @@ struct Problem {
     int64_t T = 0;
     int32_t dqk = D_QK;     // q / k head dimension of the call: 192 or 128 (the value dimension is 128)
     int32_t kv_group = 1;   // query heads per K / V head (the forward's routing looks at it)
+    int32_t fwd_short_set = -1;     // hydra_set_fwd_short_len as it stood when a forward call began
     // Local layouts (a rank of a ring holds only its own q chunks and the visiting kv chunks): where the
     // chunks of the sequences sit in the q-side tensors (q, out, lse, dout, dq) and in the kv-side tensors
     // (k, v, dk, dv). Empty tables = the packed layout, row = cu[seq] + position, Tq = Tk = T.
@@ -430,8 +431,7 @@ std::atomic<int32_t> g_fwd_short_len{-1};
 // 0.208 / 0.229 at 1024, 0.340 / 0.341 at 2048, 0.608 / 0.561 at 4096.
 int32_t fwd_short_len_for(const Problem& pb)
 {
-    const int32_t set = g_fwd_short_len.load();
-    if (set >= 0) return set;
+    if (pb.fwd_short_set >= 0) return pb.fwd_short_set;
     return (pb.dqk == D_QK && pb.kv_group == 1) ? 1280 : 2048;
 }
 static_assert(FWD_SHORT_KEYS == SUB, "the short forward kernel reads K through the 64-row map of the CTA-pair kernel");
@@ -443,8 +443,10 @@ std::vector<uint8_t> make_key(int kind, int device, const Problem& pb, int causa
         const uint8_t* b = static_cast<const uint8_t*>(p);
         key.insert(key.end(), b, b + n);
     };
-    // the forward's tables depend on which pairs go to the short-sequence kernel
-    const int32_t head[6] = {kind, device, pb.h, causal, pb.n_seqs, kind == HYDRA_WS_FWD ? fwd_short_len_for(pb) : 0};
+    // the forward's tables depend on which pairs go to the short-sequence kernel: on the limit, and on who chose it
+    const bool fwd = kind == HYDRA_WS_FWD;
+    const int32_t head[7] = {kind, device, pb.h, causal, pb.n_seqs, fwd ? fwd_short_len_for(pb) : 0,
+                             fwd && pb.fwd_short_set < 0};
     put(head, sizeof head);
     put(pb.cu.data(), pb.cu.size() * sizeof(int32_t));
     put(pb.pairs.data(), pb.pairs.size() * sizeof(hydra_pair_t));
@@ -689,7 +691,7 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     }
     n_tiles *= pb.h;
     const bool halves = short_len > 0 && n_tiles <= plan_workers(1) && most_keys <= 2 * kMostKeys &&
-                        (within || g_fwd_short_len.load() < 0);
+                        (within || pb.fwd_short_set < 0);
     if (halves) {
         std::fill(is_short.begin(), is_short.end(), 1);
     } else {
@@ -1268,6 +1270,7 @@ double hydra_plan_build_seconds(int32_t which, const int32_t* cu, int32_t n_seqs
 {
     Problem pb;
     if (make_problem(cu, n_seqs, n_heads, pairs, n_pairs, pb) != HYDRA_OK) return -1.0;
+    pb.fwd_short_set = g_fwd_short_len.load();
     Plan plan;
     const auto t0 = std::chrono::steady_clock::now();
     if (which == HYDRA_WS_FWD) build_fwd(pb, causal != 0, plan, plan.blob);
@@ -1495,6 +1498,7 @@ int32_t fwd_core(Problem& pb, const void* q, const void* k, const void* v, int32
     const KernelSet* ks = kernel_set(pb.dqk, D_V);
     if (n_kv_heads < 1 || n_heads % n_kv_heads) return HYDRA_ERR_INVALID_ARG;
     pb.kv_group = n_heads / n_kv_heads;
+    pb.fwd_short_set = g_fwd_short_len.load();          // once: another thread may set it meanwhile
     if (!(softmax_scale > 0.f) || !std::isfinite(softmax_scale)) return HYDRA_ERR_INVALID_ARG;
     if (!workspace || !aligned16(workspace)) return HYDRA_ERR_INVALID_ARG;
     if (workspace_bytes < kStatusBytes) return HYDRA_ERR_WORKSPACE_TOO_SMALL;

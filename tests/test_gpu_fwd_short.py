@@ -109,6 +109,29 @@ def test_as_many_keys_as_a_work_item_counts_and_more(keys):
     assert float((out[:, 0].double() - ref_o).abs().max()) <= TOL_REL * float(ref_o.abs().max())
 
 
+@pytest.mark.parametrize("order", [(0, -1, 1280, -1), (0, 1280, -1, 1280)])
+def test_a_limit_set_to_the_library_s_own_value_is_kept_to(order):
+    """A 3000-token call of two heads has fewer tiles than SMs: the library sends it to the short-sequence kernel, halved.
+    A caller who sets the limit, to 1280 like the library, keeps it on CTA pairs, whichever of the two came first."""
+    import paper_2609_34318_b200 as P
+    from paper_2609_34318_b200.runner import AttnStep, bits_to_tensor
+    h, T = 2, 3000 + (order[1] < 0)                      # (a shape per order: no tables from the other one)
+    cu = hw.cu_seqlens([T])
+    x = rand_inputs(T, T, h)
+    step = AttnStep(cu, h)
+    q, k, v = (bits_to_tensor(x[n]) for n in ("q", "k", "v"))
+    got = {}
+    for limit in order:
+        P.hydra_set_fwd_short_len(limit)
+        step.forward(q, k, v)
+        assert step.poll()[0] == 0
+        bits = step.out.view(torch.uint8).clone()
+        assert limit not in got or torch.equal(bits, got[limit]), limit
+        got[limit] = bits
+    assert torch.equal(got[1280], got[0]), "not the CTA-pair kernel's result"
+    assert not torch.equal(got[-1], got[0]), "the two kernels' sums differ in their last bits"
+
+
 def test_random_length_mixes_and_both_kernels_agree():
     import paper_2609_34318_b200 as P
     rng = np.random.default_rng(11)
