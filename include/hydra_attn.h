@@ -571,8 +571,9 @@ void hydra_set_plan_prefetch(int32_t on);
  * (not bit for bit: their summation orders differ). len = 0 switches the short-sequence kernel off; a negative
  * len (the default) lets the library choose: 1280 for heads of 192 with a K / V head per query head, 2048 with
  * shared K / V heads or heads of 128 (where the kernels were measured to take equal time on sequences of one
- * length), and any length for a call with no more 128-row q tiles (times heads) than the GPU has SMs, whose tiles
- * the short-sequence kernel splits between its two slots. Takes effect with the next call.
+ * length), any length for a call with no more 128-row q tiles (times heads) than the GPU has SMs, whose tiles
+ * the short-sequence kernel splits between its two slots, and up to twice that limit where the pairs above it are
+ * too little work for a second launch. A limit set by the caller is kept to exactly. Takes effect with the next call.
  */
 void hydra_set_fwd_short_len(int32_t len);
 /*

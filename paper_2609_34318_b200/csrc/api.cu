@@ -706,8 +706,8 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
         // The second launch is not worth its price either if little is left for it that the short kernel would run almost
         // as fast: pairs up to twice the limit cost it at most a tenth more, and 2^29 positions (with those above the
         // mask) take 0.2 ms. 4096 packed tokens, 16 heads, the longest sequence 1381 tokens: 75 us on both kernels,
-        // 59 on the short one alone.
-        else if (work_short < work_all && longest <= 2 * short_len && most_keys <= kMostKeys &&
+        // 59 on the short one alone. (Not against a limit set by the caller.)
+        else if (pb.fwd_short_set < 0 && work_short < work_all && longest <= 2 * short_len &&
                  (work_all - work_short) * pb.h <= double{1 << 29})
             std::fill(is_short.begin(), is_short.end(), 1);
     }

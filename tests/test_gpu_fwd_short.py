@@ -167,6 +167,23 @@ def test_one_call_uses_both_kernels_when_short_pairs_carry_enough_work():
         check(got, run_oracle(x, cu, backward=False), names=("out", "lse"), label=f"{lengths[:3]} ")
 
 
+def test_a_limit_set_by_the_caller_is_kept_to_by_a_few_longer_pairs_too():
+    """With the library's own limit a few pairs of up to twice its length stay on the short-sequence kernel, for the sake of
+    one launch; a caller's limit sends every longer pair to CTA pairs."""
+    import paper_2609_34318_b200 as P
+    from paper_2609_34318_b200.runner import AttnStep, bits_to_tensor
+    h, lengths = 2, [200] * 80 + [500] * 20              # 480 q tiles: not a call for halved ones
+    cu = hw.cu_seqlens(lengths)
+    x = rand_inputs(3, int(cu[-1]), h)
+    step = AttnStep(cu, h)
+    q, k, v = (bits_to_tensor(x[n]) for n in ("q", "k", "v"))
+    for limit, launches in ((256, 2), (499, 2), (500, 1), (FWD_SHORT_LEN_DEFAULT, 1), (0, 1)):
+        P.hydra_set_fwd_short_len(limit)
+        assert forward_launches(lambda: step.forward(q, k, v)) == launches, limit
+        if limit == 256:
+            check(run_gpu(x, cu, h, backward=False), run_oracle(x, cu, backward=False), names=("out", "lse"))
+
+
 def test_chunked_short_pairs_write_partials_and_merge():
     """Short sequences cut into zigzag chunks: diagonal and full pairs with offsets, partial outputs, the merge."""
     h = 2
