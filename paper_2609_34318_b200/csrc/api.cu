@@ -252,6 +252,7 @@ struct Plan {
     int32_t n_items = 0, n_items2 = 0;
     int32_t halves = 0;              // forward: the short kernel's items are halves of tiles, two per thread block;
                                      // backward: two CTAs share every key-side item
+    int32_t early_pops = 0;          // forward: FwdParams::early_pops
     int64_t ds_head_blocks = 0;      // backward: blocks of the dS hand-off buffer per head; -1: not usable
     // residency on the device (guarded by g_plan_mutex)
     int half = -1;                   // arena half the tables were last copied to
@@ -711,6 +712,14 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
                  (work_all - work_short) * pb.h <= double{1 << 29})
             std::fill(is_short.begin(), is_short.end(), 1);
     }
+    // How far ahead the short kernel's slots pop: items of up to 8 steps two ahead, longer ones late, so that no slot sits on
+    // an item while others run dry. In a call whose tiles are all of up to 16 steps (1024 keys) two ahead throughout is
+    // better: late / two ahead us, 16384 tokens, 8 heads of 192, sequences of 520 tokens 66.7 / 64.9, of 900 84.6 / 77.5, of
+    // 1000 80.3 / 78.0; heads of 128 53.5 / 48.1, 68.9 / 58.6, 58.7 / 58.4. Longer tiles: 6000 tokens, 16 heads, sequences
+    // of 1100 tokens 54.8 / 64.6; 4096 tokens of 1500 36.2 / 42.2; 8192 log-normal ones 105.9 / 124.5. (A fixed line
+    // inside a call, at 12, 16 or 24 steps, was worse than either way on 1500-token sequences.)
+    constexpr int32_t kShortTile = 16, kShortItem = 8;
+    int32_t longest_tile = 0;
     std::vector<std::vector<GroupEntry>> groups(pb.pairs.size()), groups_short(pb.pairs.size());
     for (size_t pi = 0; pi < pb.pairs.size(); ++pi) {
         const auto& p = pb.pairs[pi];
@@ -719,6 +728,7 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
                 const int32_t rows = std::min(TILE, p.q_len - q0);
                 const int32_t n_kv = kv_steps_short(p, q0, rows, causal);
                 groups_short[pi].push_back(GroupEntry{q0, n_kv, rows, n_kv});
+                longest_tile = std::max(longest_tile, n_kv);
             }
             continue;
         }
@@ -741,6 +751,7 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
             groups[pi].push_back(GroupEntry{qa, n_a, n_b, 2 * std::max(n_a, std::max(n_b, 0))});
         }
     }
+    plan.early_pops = longest_tile > kShortTile ? kShortItem : kShortTile;
     const std::vector<FwdItem> items = order_by_groups<FwdItem>(
         groups, pb.h, plan_workers(2),
         [](int32_t g, int32_t a, const GroupEntry& e) { return FwdItem{g, a, e.a, e.b, e.c, {0, 0, 0}}; });
@@ -1525,6 +1536,7 @@ int32_t fwd_core(Problem& pb, const void* q, const void* k, const void* v, int32
     fp.n_items = plan->n_items;
     fp.short_items = lease.at<FwdShortItem>(plan->off_items2);
     fp.n_short = plan->n_items2;
+    fp.early_pops = plan->early_pops;
     fp.out = out; fp.lse = lse; fp.o_part = o_part; fp.lse_part = lse_part;
     fp.T = pb.Tq; fp.part_rows = part_rows; fp.h = n_heads; fp.causal = causal != 0;
     fp.kv_group = n_heads / n_kv_heads;

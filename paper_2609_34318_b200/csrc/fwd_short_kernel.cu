@@ -78,7 +78,6 @@ constexpr uint32_t kTmSlot = 256, kTmS = 128, kTmCols = 512;
 constexpr float kRescaleThreshold = 8.f;              // log2 units
 constexpr int kSched = 4;                             // depth of a slot's ring of work items
 constexpr int kPopAhead = 4;                          // steps before the end of an item at which the next one is popped
-constexpr int kShortItem = 8;                         // an item of at most so many steps: the pops run two items ahead
 
 enum : int {
     B_QFULL = 0, B_QEMPTY = 1, B_KFULL = 2, B_KEMPTY = 5, B_VFULL = 8, B_VEMPTY = 10, B_SFULL = 12, B_PFULL = 14,
@@ -196,8 +195,10 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
             // asked for, while the long one's last steps are being loaded, each answer looked at a step or more after
             // it was asked for: always popped two items ahead, a batch with fewer than a few items per slot was as
             // good as dealt out in advance (64 items of up to 16 steps took 40 us, two in a row on half of the slots,
-            // now 22). Short items are popped two ahead and their descriptors asked for one ahead: an item of a few
-            // steps does not hide both answers (sequences of 64 to 512 tokens: 1-2 % of the kernel).
+            // now 22). Items of up to p.early_pops steps are popped two ahead and their descriptors asked for one ahead: a
+            // few steps do not hide both answers (sequences of 64 to 512 tokens: 1-2 % of the kernel). The host chooses
+            // where that line lies in a call (build_fwd).
+            const int early = p.early_pops;
             FwdShortItem cur{}, nxt;
             int raw1 = slot * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x), raw2 = 0;   // pops of the next item and of
             bool have1 = true, have2 = false;          // the one after it, if they have been asked for
@@ -214,12 +215,12 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
                 for (int j = 0; ok; ++j) {
                     // (the pops are used in the order in which they were made: an early one must not be left over
                     // when a later one finds the queue empty)
-                    if (!have1 && (n <= kShortItem || j >= n - kPopAhead)) {
+                    if (!have1 && (n <= early || j >= n - kPopAhead)) {
                         raw1 = first_pop + atomicAdd(counter, 1);
                         have1 = true;
                     }
-                    if (!fetched && have1 && (n <= kShortItem || j >= n - 2)) { nxt_idx = fetch(raw1, nxt); fetched = true; }
-                    if (kq > 0 && j == 0 && n <= kShortItem) { raw2 = first_pop + atomicAdd(counter, 1); have2 = true; }
+                    if (!fetched && have1 && (n <= early || j >= n - 2)) { nxt_idx = fetch(raw1, nxt); fetched = true; }
+                    if (kq > 0 && j == 0 && n <= early) { raw2 = first_pop + atomicAdd(counter, 1); have2 = true; }
                     // The next item's Q and first K tile are released by score products that are long issued
                     // when the last V stage comes free: ask for them first, and show the item to the issuer.
                     if (j == (n >= 2 ? n - 1 : n)) {

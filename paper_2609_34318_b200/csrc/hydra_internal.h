@@ -212,6 +212,7 @@ struct FwdParams {
     int32_t n_items;
     const FwdShortItem* short_items;   // the pairs that go to the short-sequence kernel
     int32_t n_short;
+    int32_t early_pops;         // short-sequence kernel: items of up to so many steps are popped two items ahead
     void* out; float* lse; void* o_part; float* lse_part;
     int64_t T; int64_t part_rows;
     int32_t h; int32_t causal;

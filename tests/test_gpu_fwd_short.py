@@ -47,6 +47,8 @@ def default_routing():
     [129, 257, 64, 500, 127],     # one row more than a tile, one more than two
     [2048],                       # the longest sequence the default routing sends here: 16 tiles, up to 32 steps
     [200] * 40,                   # more work items than the two slots of every SM hold at once
+    [1024] * 7,                   # tiles of up to 16 steps, the longest call whose slots pop two items ahead throughout
+    [1025] * 6,                   # one step more: popped near the end of an item (162 tiles: not a halved call either)
 ])
 def test_short_sequences_against_the_oracle(lengths):
     h = 3
