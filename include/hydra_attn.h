@@ -119,9 +119,10 @@ int32_t hydra_zigzag_pairs(const int32_t* cu_seqlens_host, int32_t n_seqs, const
  *
  * Banded form, for problems whose dS buffer is over that limit (long sequences). The band scratch is set
  * with hydra_set_bwd_band_scratch(bytes): a byte count >= 1 MiB, 0 (bands off), or HYDRA_BAND_AUTO (the
- * default): as much as the dS limit, for problems whose whole dS buffer is at most 8 times the limit,
- * and off for larger ones (hundreds of small bands cost more than the recomputation they save: give
- * those an explicit scratch of tens of GB). With a scratch in effect HYDRA_WS_BWD asks, for a problem over
+ * default): as much as the dS limit, for problems whose whole dS buffer is at most 16 times the limit
+ * and whose longest sequence's own at most 7 times, and off for others (a band of a long sequence is few key
+ * tiles, of equal length, and leaves much of the GPU idle at its end, which costs more than the recomputation
+ * it saves: give those an explicit scratch of tens of GB). With a scratch in effect HYDRA_WS_BWD asks, for a problem over
  * the limit, for the base size + an fp32 accumulator of dq (4 * 192 bytes per token and head) +
  * min(scratch, the full dS buffer). hydra_attn_bwd, given that much, cuts the key rows of every chunk into
  * bands of 128-row tiles whose own dS buffer fits the scratch and runs every band with the hand-off

@@ -708,7 +708,7 @@ HYDRA_BAND_AUTO = (1 << 64) - 1
 
 def hydra_set_bwd_band_scratch(n_bytes: int) -> None:
     """Scratch for the banded backward of problems whose dS buffer is over the limit (0: off;
-    HYDRA_BAND_AUTO, the default: the dS limit, for problems of at most 8 such bands)."""
+    HYDRA_BAND_AUTO, the default: the dS limit, for problems of at most 16 such bands, no sequence over 7)."""
     _lib.hydra_set_bwd_band_scratch(int(n_bytes))
 
 

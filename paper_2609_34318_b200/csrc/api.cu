@@ -1355,21 +1355,35 @@ std::atomic<uint64_t> g_ds_limit_bytes{uint64_t{4} << 30};
 
 // smallest scratch the banded backward is worth running with
 constexpr uint64_t kMinBandBytes = uint64_t{1} << 20;
-// Band scratch: a byte count, 0 (bands off) or HYDRA_BAND_AUTO: as much as the dS limit, for problems whose
-// whole dS buffer is at most 8 times that. The longer the sequence, the narrower a band of that size: 16 to 21 key
-// tiles at 48K to 64K tokens, two waves of work items of which the second is half empty, and beside the stores of dS
-// that costs more than the recomputation it saves. One sequence, 16 heads, 4 GiB, step in bands / recomputing: 24K
-// tokens 10.96 / 11.21 ms, 32K (5 bands) 18.9 / 19.6, 48K (10 bands) 45.2 / 43.6, 64K (17 bands) 83.1 / 78.2.
+// Band scratch: a byte count, 0 (bands off) or HYDRA_BAND_AUTO: as much as the dS limit, for problems whose whole dS buffer
+// is at most 16 times that and whose longest sequence's own is at most 7 times. The longer a sequence, the fewer of its key
+// tiles a band holds, all nearly as long: 16 to 21 at 48K to 64K tokens, two waves of work items of which the second is
+// half empty, and beside the stores of dS that costs more than the recomputation it saves. How many sequences there are
+// costs nothing. Backward in bands of 4 GiB / recomputing, ms, 16 heads, one sequence: 28000 tokens (2.9 times the limit) 10.4 /
+// 11.2, 36000 (4.9) 18.5 / 18.7, 40000 (6.0) 22.7 / 22.9, 44000 (7.2) 28.7 / 27.8, 49152 (9.0) 35.3 / 34.4, 64K (16) 65.1 /
+// 61.3; several: ten of 16384 (10.1, each 1.0) 36.9 / 39.2, fourteen 51.5 / 55.5, forty of 8192 39.3 / 41.3, two of 40000
+// (12, each 6.0) 45.9 / 46.1; 32 heads, four of 16384 (8.1, each 2.0) 29.7 / 31.3.
 std::atomic<uint64_t> g_band_bytes{HYDRA_BAND_AUTO};
-constexpr uint64_t kAutoBandsMax = 8;
-uint64_t band_scratch_for(int64_t head_blocks, int32_t n_heads)
+constexpr uint64_t kAutoBandsMax = 16, kAutoBandsLongest = 7;
+// blocks per head of the dS of the sequence that has most of them
+int64_t longest_ds_blocks(const Problem& pb, int causal)
+{
+    std::vector<int64_t> blocks(pb.n_seqs, 0);
+    for (const auto& p : pb.pairs)
+        if (p.q_len > 0 && p.k_len > 0)
+            blocks[p.seq] += ds_rowstart(ds_geom(p.q_len, p.q_start - p.k_start, causal), (p.k_len + TILE - 1) / TILE);
+    return blocks.empty() ? 0 : *std::max_element(blocks.begin(), blocks.end());
+}
+uint64_t band_scratch_for(const Problem& pb, int causal, int64_t head_blocks)
 {
     const uint64_t set = g_band_bytes.load();
     if (set != HYDRA_BAND_AUTO) return set;
     if (head_blocks <= 0) return 0;
     const uint64_t limit = g_ds_limit_bytes.load();
-    const uint64_t full = static_cast<uint64_t>(head_blocks) * n_heads * DS_BLOCK_BYTES;
-    return (limit >= kMinBandBytes && full <= kAutoBandsMax * limit) ? limit : 0;
+    const uint64_t block = static_cast<uint64_t>(pb.h) * DS_BLOCK_BYTES;
+    const bool bands = limit >= kMinBandBytes && head_blocks * block <= kAutoBandsMax * limit &&
+                       longest_ds_blocks(pb, causal) * block <= kAutoBandsLongest * limit;
+    return bands ? limit : 0;
 }
 
 size_t bwd_acc_bytes(const Problem& pb)
@@ -1431,7 +1445,7 @@ size_t hydra_workspace_bytes_dims(int32_t which, const int32_t* cu, int32_t n_se
             const size_t ds = bwd_ds_bytes(head_blocks, n_heads, g_ds_limit_bytes.load());
             if (ds) return base + ds;
             // over the limit: the banded form, if switched on, wants an fp32 dq and its scratch
-            const uint64_t band = band_scratch_for(head_blocks, n_heads);
+            const uint64_t band = band_scratch_for(pb, 1, head_blocks);
             if (head_blocks > 0 && band >= kMinBandBytes) {
                 const uint64_t full = static_cast<uint64_t>(head_blocks) * n_heads * DS_BLOCK_BYTES;
                 return base + bwd_acc_bytes(pb) + static_cast<size_t>(std::min(band, full));
@@ -1908,7 +1922,7 @@ int32_t bwd_core(Problem& pb, const void* q, const void* k, const void* v, const
     const size_t acc_bytes = bwd_acc_bytes(pb);
     if (!accumulate && room >= acc_bytes + kMinBandBytes) {
         const int64_t head_blocks = ds_layout(pb, causal, nullptr);
-        const uint64_t band_limit = band_scratch_for(head_blocks, n_heads);
+        const uint64_t band_limit = band_scratch_for(pb, causal, head_blocks);
         if (head_blocks > 0 && band_limit >= kMinBandBytes &&
             bwd_ds_bytes(head_blocks, n_heads, g_ds_limit_bytes.load()) == 0) {
             const size_t scratch = static_cast<size_t>(std::min<uint64_t>(band_limit, room - acc_bytes));

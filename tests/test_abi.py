@@ -270,6 +270,34 @@ def test_workspace_bytes_with_the_band_scratch():
         P.hydra_set_bwd_band_scratch(P.HYDRA_BAND_AUTO)
 
 
+@pytest.mark.parametrize("lengths,h,ring,bands", [
+    ([16384] * 10, 16, 0, True),      # 10 limits of dS, no sequence over one of them
+    ([16384] * 17, 16, 0, False),     # 17 limits
+    ([43000], 16, 0, True),           # one sequence of 6.9 limits
+    ([44000], 16, 0, False),          # of 7.2
+    ([44000, 300, 300], 16, 0, False),
+    ([44000], 16, 2, False),          # a ring's chunk pairs count for their sequence
+    ([20000, 20000], 16, 2, True),
+    ([1, 0], 16, 0, False),           # under the limit
+])
+def test_automatic_bands_look_at_the_longest_sequence(lengths, h, ring, bands):
+    """Many documents whose dS together is over the limit run in bands; a long one recomputes (a band of it is a few key
+    tiles of equal length)."""
+    cu = [int(c) for c in np.concatenate([[0], np.cumsum(lengths)])]
+    pairs = P.hydra_zigzag_pairs(np.array(cu, dtype=np.int32), ring)[0] if ring else None
+    try:
+        automatic = P.hydra_workspace_bytes(P.HYDRA_WS_BWD, cu, h, pairs)
+        P.hydra_set_bwd_band_scratch(0)
+        off = P.hydra_workspace_bytes(P.HYDRA_WS_BWD, cu, h, pairs)
+    finally:
+        P.hydra_set_bwd_band_scratch(P.HYDRA_BAND_AUTO)
+    acc = sum(lengths) * h * 192 * 4
+    if bands:
+        assert off + acc + (4 << 30) <= automatic <= off + acc + (4 << 30) + 8192
+    else:
+        assert automatic == off
+
+
 @pytest.mark.parametrize("seed", range(12))
 def test_bands_cover_random_problems_exactly_once(seed):
     rng = np.random.default_rng(7000 + seed)
