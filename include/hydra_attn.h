@@ -322,7 +322,9 @@ int32_t hydra_attn_bwd_accumulate_gqa(const void* q, const void* k, const void* 
  * `cuda_stream`, the copies in and out on two internal streams (created once per device, on the
  * first call), so that both directions of the host link are busy at once. Work enqueued on
  * `cuda_stream` before the call precedes all of it, and `cuda_stream` completes only when the last
- * copy out has: host outputs are valid once the stream has been synchronised. Host buffers have
+ * copy out has: host outputs are valid once the stream has been synchronised. out_host and dv_host may be
+ * v_host or dout_host, dq_host and dk_host may be q_host or k_host: a group's results are copied out after
+ * its inputs of that memory have been copied in. Host buffers have
  * the tensor layouts above; pinned memory makes the copies asynchronous. `device_arena` is device
  * memory, 256-byte aligned, of at least hydra_host_step_arena_bytes(...) bytes, owned by the
  * caller; the library carves every device tensor, the partial buffers and the workspace out of it

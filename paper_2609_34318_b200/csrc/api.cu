@@ -2236,6 +2236,13 @@ int32_t hydra_attn_fwd_bwd_host(const void* q_host, const void* k_host, const vo
         return to_device ? cudaMemcpy2DAsync(dev, width, host, H * row_bytes, width, rows, kind, st)
                          : cudaMemcpy2DAsync(host, H * row_bytes, dev, width, width, rows, kind, st);
     };
+    // (an output buffer may be an input's: the results of a group then wait until its inputs have been read)
+    auto share = [](const void* a, size_t na, const void* b, size_t nb) {
+        const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+        return x < y + nb && y < x + na;
+    };
+    const bool out_over_dout = share(out_host, th * D_V * 2, dout_host, th * D_V * 2) ||
+                               share(lse_host, th * 4, dout_host, th * D_V * 2);
     if (cudaEventRecord(pipe->start, stream) || cudaStreamWaitEvent(pipe->in, pipe->start, 0) ||
         cudaStreamWaitEvent(pipe->out, pipe->start, 0))
         return HYDRA_ERR_CUDA;
@@ -2285,6 +2292,7 @@ int32_t hydra_attn_fwd_bwd_host(const void* q_host, const void* k_host, const vo
         // link is busy (before the first copy out and after the last copy in): 12288 tokens, 16 heads 6.47 -> 6.35 ms, 8192
         // packed tokens 4.77 -> 4.53, 8192 tokens of short sequences, 8 heads 2.55 -> 2.42, 1024 tokens, 4 heads 0.252 -> 0.235
         if (cudaEventRecord(pipe->fwd_done[g], stream) || cudaStreamWaitEvent(pipe->out, pipe->fwd_done[g], 0) ||
+            (out_over_dout && cudaStreamWaitEvent(pipe->out, pipe->dout_done[g], 0)) ||
             move(G, out + ov, static_cast<const uint8_t*>(out_host), D_V * 2, false, pipe->out) ||
             cudaMemcpy2DAsync(lse_host + static_cast<size_t>(G.h0) * pb.T + G.t0, static_cast<size_t>(pb.T) * 4, lse_g,
                               static_cast<size_t>(G.tn) * 4, static_cast<size_t>(G.tn) * 4, G.hn, cudaMemcpyDeviceToHost,
