@@ -469,7 +469,6 @@ __global__ void __launch_bounds__(kThreads)
 hydra_ulysses_kernel(const Vec* __restrict__ src, Vec* __restrict__ dst, uint32_t n, uint32_t P, uint32_t cu,
                      uint32_t rows)
 {
-    overlap_next_launch();
     wait_for_previous_launch();
     // kLong: a warp takes one chunk (row = j * n + t of the block-major side) at a time, four units per lane in flight.
     // Otherwise (a chunk is at most one unit per lane) four chunks in flight:
@@ -491,6 +490,7 @@ hydra_ulysses_kernel(const Vec* __restrict__ src, Vec* __restrict__ dst, uint32_
                     if (w0 + e * 32 < cu) st_unit(dst + (kPack ? blk : tok) + w0 + e * 32, v[e]);
             }
         }
+        overlap_next_launch();
         return;
     }
     for (uint32_t r0 = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); r0 < rows; r0 += n_warps * kUnroll) {
@@ -512,6 +512,7 @@ hydra_ulysses_kernel(const Vec* __restrict__ src, Vec* __restrict__ dst, uint32_
                 if (r0 + e * n_warps < rows) st_unit(dst + (kPack ? blk[e] : tok[e]) + w, v[e]);
         }
     }
+    overlap_next_launch();
 }
 
 cudaError_t launch_ulysses(bool pack, const void* src, void* dst, int64_t n_tokens, int32_t cp_u, int64_t chunk_units,

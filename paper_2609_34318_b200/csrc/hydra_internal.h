@@ -148,6 +148,10 @@ struct ClockProbe {
 // four sequences of 7 to 300 tokens 42 -> 35 us, of 1024 tokens in short ones 49 -> 42 us, the ten launches around the
 // attention of a 4096-token MLA block 813 -> 794 us. Kernels of other libraries before or after are ordered
 // as usual.
+// The elementwise steps of the MLA block and the Ulysses permutation let the next launch start at their end only. Their grids
+// are a few blocks per SM, of which many fit: started at once, a grid fills the SMs that come free first and leaves the
+// others empty. Rotary embedding, key / value assembly and its backward of 800 tokens, 63 heads of 126 + 62 / 126 (the
+// four-byte kernels) 101 us started at once, 78 plainly, 72 at the end; 1200 tokens, 128 heads 214, 182, 177.
 #ifdef __CUDACC__
 __device__ __forceinline__ void overlap_next_launch() { cudaTriggerProgrammaticLaunchCompletion(); }
 __device__ __forceinline__ void wait_for_previous_launch() { cudaGridDependencySynchronize(); }

@@ -56,7 +56,6 @@ hydra_rope_kernel(const uint32_t* __restrict__ x, const int32_t* __restrict__ po
                   int64_t n_tokens, int32_t n_heads, int32_t head_dim, int32_t rope_offset, int32_t rope_dim,
                   double log_theta, int inverse, int in_place)
 {
-    overlap_next_launch();
     wait_for_previous_launch();
     __shared__ float s_cos[kMaxRopePairs], s_sin[kMaxRopePairs];
     const int pairs_per_head = head_dim / 2, p0 = rope_offset / 2, p1 = (rope_offset + rope_dim) / 2;
@@ -87,6 +86,7 @@ hydra_rope_kernel(const uint32_t* __restrict__ x, const int32_t* __restrict__ po
             }
         }
     }
+    overlap_next_launch();
 }
 
 // k[t, a, :] = [kv_up[t, a, 0:nope] | rope(k_pe[t, :])], v[t, a, :] = kv_up[t, a, nope:nope+dv]
@@ -96,7 +96,6 @@ hydra_mla_kv_assemble_kernel(const uint32_t* __restrict__ kv_up, const uint32_t*
                              int64_t n_tokens, int32_t n_heads, int32_t nope, int32_t rope_dim, int32_t dv,
                              double log_theta)
 {
-    overlap_next_launch();
     wait_for_previous_launch();
     __shared__ float s_cos[kMaxRopePairs], s_sin[kMaxRopePairs];
     __shared__ uint32_t s_pe[kMaxRopePairs];
@@ -123,6 +122,7 @@ hydra_mla_kv_assemble_kernel(const uint32_t* __restrict__ kv_up, const uint32_t*
             k[k0 + static_cast<int64_t>(a) * k_pairs + np + i] = s_pe[i];
         }
     }
+    overlap_next_launch();
 }
 
 // The adjoint: dkv_up[t, a, :] = [dk[t, a, 0:nope] | dv[t, a, :]],
@@ -133,7 +133,6 @@ hydra_mla_kv_assemble_bwd_kernel(const uint32_t* __restrict__ dk, const uint32_t
                                  uint32_t* __restrict__ dk_pe, int64_t n_tokens, int32_t n_heads, int32_t nope,
                                  int32_t rope_dim, int32_t dvd, double log_theta)
 {
-    overlap_next_launch();
     wait_for_previous_launch();
     __shared__ float s_cos[kMaxRopePairs], s_sin[kMaxRopePairs];
     const int np = nope / 2, rp = rope_dim / 2, vp = dvd / 2;
@@ -158,6 +157,7 @@ hydra_mla_kv_assemble_bwd_kernel(const uint32_t* __restrict__ dk, const uint32_t
             dk_pe[t * rp + i] = f2_to_bf2(sx * s_cos[i] - sy * s_sin[i], sx * s_sin[i] + sy * s_cos[i]);
         }
     }
+    overlap_next_launch();
 }
 
 inline bool aligned16_all(std::initializer_list<const void*> ptrs)
@@ -304,7 +304,6 @@ __global__ void __launch_bounds__(kVecThreads)
 hydra_rope_vec_kernel(const uint32_t* x, const int32_t* __restrict__ positions, uint32_t* y, const VecItems it, int32_t v0,
                       const Div by_rot, const Div by_copy, int inverse)
 {
-    overlap_next_launch();
     __shared__ __align__(16) float s_cos[kVecThreads], s_sin[kVecThreads];
     const uint32_t nv = by_rot.d, vph = by_rot.d + by_copy.d;
     const int my_tok = threadIdx.x / it.pairs, my_pair = threadIdx.x - my_tok * it.pairs;
@@ -349,6 +348,7 @@ hydra_rope_vec_kernel(const uint32_t* x, const int32_t* __restrict__ positions, 
             }
         }
     }
+    overlap_next_launch();
 }
 
 template <int kWords>
@@ -357,7 +357,6 @@ hydra_mla_kv_assemble_vec_kernel(const uint32_t* __restrict__ kv_up, const uint3
                                  const int32_t* __restrict__ positions, uint32_t* __restrict__ k, uint32_t* __restrict__ v,
                                  const VecItems it, uint32_t nv, const Div by_up, const Div by_rot)
 {
-    overlap_next_launch();
     __shared__ __align__(32) uint32_t s_pe[kVecThreads];
     const uint32_t vv = by_up.d - nv, rv = by_rot.d, k_vecs = nv + rv;
     const int my_tok = threadIdx.x / it.pairs, my_pair = threadIdx.x - my_tok * it.pairs;
@@ -396,6 +395,7 @@ hydra_mla_kv_assemble_vec_kernel(const uint32_t* __restrict__ kv_up, const uint3
             st_words<kWords>(kb, r * k_vecs + nv + i, w);
         }
     }
+    overlap_next_launch();
 }
 
 // The shared rotary key's gradient is the sum over the heads: each thread adds up one vector over every n-th head of its
@@ -406,7 +406,6 @@ hydra_mla_kv_assemble_bwd_vec_kernel(const uint32_t* __restrict__ dk, const uint
                                      const int32_t* __restrict__ positions, uint32_t* __restrict__ dkv_up,
                                      uint32_t* __restrict__ dk_pe, const VecItems it, uint32_t nv, const Div by_up, uint32_t rv)
 {
-    overlap_next_launch();
     __shared__ __align__(16) float s_part[kVecThreads * 2 * kWords];
     const uint32_t vv = by_up.d - nv, k_vecs = nv + rv;
     const int my_tok = threadIdx.x / it.pairs, my_pair = threadIdx.x - my_tok * it.pairs;
@@ -463,6 +462,7 @@ hydra_mla_kv_assemble_bwd_vec_kernel(const uint32_t* __restrict__ dk, const uint
             dk_pe[t0 * it.pairs + threadIdx.x] = f2_to_bf2(sx * cs + sy * sn, sy * cs - sx * sn);
         }
     }
+    overlap_next_launch();
 }
 
 // (exp and reciprocal of the special-function unit: a relative error of 2^-21, far below the bf16 result's 2^-9)
@@ -473,7 +473,6 @@ template <int kWords>
 __global__ void __launch_bounds__(256)
 hydra_gate_kernel(const void* __restrict__ out, const void* __restrict__ gate, void* __restrict__ y, int64_t n)
 {
-    overlap_next_launch();
     wait_for_previous_launch();
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; i < n; i += static_cast<int64_t>(gridDim.x) * 256) {
         const Words<kWords> o = ld_words<kWords>(out, i), g = ld_words<kWords>(gate, i);
@@ -485,6 +484,7 @@ hydra_gate_kernel(const void* __restrict__ out, const void* __restrict__ gate, v
         }
         st_words<kWords>(y, i, r);
     }
+    overlap_next_launch();
 }
 
 // d_out = dy * sigmoid(gate);  d_gate = dy * out * sigmoid(gate) * (1 - sigmoid(gate))
@@ -493,7 +493,6 @@ __global__ void __launch_bounds__(256)
 hydra_gate_bwd_kernel(const void* __restrict__ dy, const void* __restrict__ out, const void* __restrict__ gate,
                       void* __restrict__ d_out, void* __restrict__ d_gate, int64_t n)
 {
-    overlap_next_launch();
     wait_for_previous_launch();
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; i < n; i += static_cast<int64_t>(gridDim.x) * 256) {
         const Words<kWords> d = ld_words<kWords>(dy, i), o = ld_words<kWords>(out, i), g = ld_words<kWords>(gate, i);
@@ -508,6 +507,7 @@ hydra_gate_bwd_kernel(const void* __restrict__ dy, const void* __restrict__ out,
         st_words<kWords>(d_out, i, ro);
         st_words<kWords>(d_gate, i, rg);
     }
+    overlap_next_launch();
 }
 
 inline bool all_aligned32(std::initializer_list<const void*> ptrs)
