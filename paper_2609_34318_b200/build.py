@@ -17,7 +17,7 @@ SOURCES = ["api.cu", "fwd_kernel.cu", "fwd_short_kernel.cu", "bwd_kernels.cu", "
 # the tensor-core kernel files are compiled a second time for q / k heads of 128 (own symbol names)
 VARIANTS = [("fwd_kernel.cu", "d128", ["-DHYDRA_KERNEL_DQK=128"]), ("fwd_short_kernel.cu", "d128", ["-DHYDRA_KERNEL_DQK=128"]),
             ("bwd_kernels.cu", "d128", ["-DHYDRA_KERNEL_DQK=128"])]
-HEADERS = ["hydra_internal.h", "sm100_ptx.cuh", os.path.join("..", "..", "include", "hydra_attn.h"),
+HEADERS = ["hydra_internal.h", "once_per_device.h", "sm100_ptx.cuh", os.path.join("..", "..", "include", "hydra_attn.h"),
            os.path.join("..", "..", "include", "hydra_sched.h")]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

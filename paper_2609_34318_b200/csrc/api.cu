@@ -1063,20 +1063,23 @@ void prefetch_plans(const Problem& pb, int causal, bool any_part)
 // ---------------------------------------------------------------------------------------------
 // device properties and tensor maps
 // ---------------------------------------------------------------------------------------------
-struct DeviceInfo { int major = 0, sms = 0; bool known = false; };
 int32_t device_info(int* sms)
 {
-    static DeviceInfo info[64];
+    static std::atomic<int> majors[kMaxDevices] = {}, counts[kMaxDevices] = {};
+    static OncePerDevice asked;
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return HYDRA_ERR_CUDA;
-    if (!info[dev].known) {
-        if (cudaDeviceGetAttribute(&info[dev].major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&info[dev].sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            return HYDRA_ERR_CUDA;
-        info[dev].known = true;
-    }
-    if (info[dev].major != 10) return HYDRA_ERR_NOT_SM100;
-    if (sms) *sms = info[dev].sms;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return HYDRA_ERR_CUDA;
+    const cudaError_t e = asked(dev, [&] {
+        int major = 0, count = 0;
+        cudaError_t status = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
+        if (status == cudaSuccess) status = cudaDeviceGetAttribute(&count, cudaDevAttrMultiProcessorCount, dev);
+        majors[dev] = major;
+        counts[dev] = count;
+        return status;
+    });
+    if (e != cudaSuccess) return HYDRA_ERR_CUDA;
+    if (majors[dev] != 10) return HYDRA_ERR_NOT_SM100;
+    if (sms) *sms = counts[dev];
     return HYDRA_OK;
 }
 
@@ -1086,12 +1089,13 @@ using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, voi
                               CUtensorMapFloatOOBfill);
 EncodeFn encode_fn()
 {
-    static EncodeFn fn = nullptr;
+    static std::atomic<EncodeFn> found{nullptr};
+    EncodeFn fn = found.load();
     if (!fn) {
         void* p = nullptr;
         cudaDriverEntryPointQueryResult q;
         if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess)
-            fn = reinterpret_cast<EncodeFn>(p);
+            found = fn = reinterpret_cast<EncodeFn>(p);
     }
     return fn;
 }

@@ -629,11 +629,11 @@ static __device__ __align__(256) unsigned char g_noalloc_merge_tables[kNoAllocBy
 // Device address of the array on the current device (looked up once per device).
 cudaError_t noalloc_tables(unsigned char** out)
 {
-    static unsigned char* cached[64] = {};
+    static std::atomic<unsigned char*> cached[kMaxDevices] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     if (!cached[dev]) {
         void* ptr = nullptr;
         e = cudaGetSymbolAddress(&ptr, g_noalloc_merge_tables);

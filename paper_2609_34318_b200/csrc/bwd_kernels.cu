@@ -1495,43 +1495,28 @@ HYDRA_K(hydra_bwd_dq_from_ds_kernel)(const __grid_constant__ CUtensorMap map_k,
 }
 
 
-// cudaFuncSetAttribute applies to the device that is current when it is called, so the opt-in to more than
-// 48 KB of dynamic shared memory is made once per device ordinal, not once per process.
-template <class Kernel>
-cudaError_t configure_once_per_device(Kernel kernel, size_t smem_bytes, bool (&done)[64])
-{
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (done[dev]) return cudaSuccess;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes));
-    if (e == cudaSuccess) done[dev] = true;
-    return e;
-}
-
 cudaError_t HYDRA_K(launch_bwd_dq_from_ds)(const CUtensorMap& mk, const BwdParams& p, int grid,
                                   cudaStream_t stream)
 {
-    static bool configured[64] = {};
-    if (cudaError_t e = configure_once_per_device(HYDRA_K(hydra_bwd_dq_from_ds_kernel), HYDRA_K(bwd_dq_ds_smem_bytes)(), configured)) return e;
+    static OncePerDevice configured;
+    if (cudaError_t e = allow_dynamic_smem(HYDRA_K(hydra_bwd_dq_from_ds_kernel), HYDRA_K(bwd_dq_ds_smem_bytes)(), configured)) return e;
     return launch_overlapped(HYDRA_K(hydra_bwd_dq_from_ds_kernel), grid, dqs::kThreadsS, HYDRA_K(bwd_dq_ds_smem_bytes)(), stream, mk, p);
 }
 
 cudaError_t HYDRA_K(launch_bwd_dq)(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
                           const CUtensorMap& mdo, const BwdParams& p, int grid, cudaStream_t stream)
 {
-    static bool configured[64] = {};
-    if (cudaError_t e = configure_once_per_device(HYDRA_K(hydra_bwd_dq_kernel), HYDRA_K(bwd_dq_smem_bytes)(), configured)) return e;
+    static OncePerDevice configured;
+    if (cudaError_t e = allow_dynamic_smem(HYDRA_K(hydra_bwd_dq_kernel), HYDRA_K(bwd_dq_smem_bytes)(), configured)) return e;
     return launch_overlapped(HYDRA_K(hydra_bwd_dq_kernel), grid, kThreads, HYDRA_K(bwd_dq_smem_bytes)(), stream, mq, mk, mv, mdo, p);
 }
 
 cudaError_t HYDRA_K(launch_bwd_dkv)(const CUtensorMap& mq_sub, const CUtensorMap& mk, const CUtensorMap& mv,
                            const CUtensorMap& mdo_sub, const BwdParams& p, bool halves, int grid, cudaStream_t stream)
 {
-    static bool configured[2][64] = {};
+    static OncePerDevice configured[2];
     const auto kernel = halves ? HYDRA_K(hydra_bwd_dkv_kernel)<true> : HYDRA_K(hydra_bwd_dkv_kernel)<false>;
-    if (cudaError_t e = configure_once_per_device(kernel, HYDRA_K(bwd_dkv_smem_bytes)(), configured[halves])) return e;
+    if (cudaError_t e = allow_dynamic_smem(kernel, HYDRA_K(bwd_dkv_smem_bytes)(), configured[halves])) return e;
     return launch_overlapped_clusters(kernel, halves ? 2 : 1, grid, kThreads, HYDRA_K(bwd_dkv_smem_bytes)(), stream, mq_sub, mk, mv,
                                       mdo_sub, p);
 }

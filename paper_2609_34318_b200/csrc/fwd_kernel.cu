@@ -520,11 +520,10 @@ HYDRA_K(hydra_fwd_kernel)(const __grid_constant__ CUtensorMap map_q, const __gri
 // Kept per device ordinal: the shared-memory opt-in applies to the device that is current when it is made.
 int HYDRA_K(fwd_max_clusters)()
 {
-    static int cached_by_device[64];
-    static bool known[64] = {};
+    static std::atomic<int> clusters[kMaxDevices] = {};   // 0: not asked for yet
     int sms = 0, dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    if (known[dev]) return cached_by_device[dev];
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
+    if (const int known = clusters[dev].load()) return known;
     if (cudaFuncSetAttribute(HYDRA_K(hydra_fwd_kernel), cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(HYDRA_K(fwd_smem_bytes)())) != cudaSuccess)
         return 0;
@@ -535,8 +534,7 @@ int HYDRA_K(fwd_max_clusters)()
     cfg.dynamicSmemBytes = HYDRA_K(fwd_smem_bytes)();
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, HYDRA_K(hydra_fwd_kernel), &cfg) != cudaSuccess) n = 0;
-    cached_by_device[dev] = n;
-    known[dev] = n > 0;
+    clusters[dev].store(n);
     return n;
 }
 

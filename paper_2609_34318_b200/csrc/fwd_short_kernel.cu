@@ -546,18 +546,9 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
 cudaError_t HYDRA_K(launch_fwd_short)(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
                                       const FwdParams& p, bool halves, int grid, cudaStream_t stream)
 {
-    // the opt-in to more than 48 KB of dynamic shared memory is made once per device ordinal
-    static bool configured[64][2] = {};
+    static OncePerDevice configured[2];
     const auto kernel = halves ? HYDRA_K(hydra_fwd_short_kernel)<true> : HYDRA_K(hydra_fwd_short_kernel)<false>;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!configured[dev][halves]) {
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(HYDRA_K(fwd_short_smem_bytes)()));
-        if (e != cudaSuccess) return e;
-        configured[dev][halves] = true;
-    }
+    if (cudaError_t e = allow_dynamic_smem(kernel, HYDRA_K(fwd_short_smem_bytes)(), configured[halves])) return e;
     return launch_overlapped(kernel, grid, kThreads, HYDRA_K(fwd_short_smem_bytes)(), stream, mq, mk, mv, p);
 }
 

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include "../../include/hydra_attn.h"
+#include "once_per_device.h"
 
 namespace hydra {
 
@@ -191,22 +192,34 @@ template <auto kKernel, class... Args>
 cudaError_t launch_overlapped_spread(int grid, int block, cudaStream_t stream, Args&&... args)
 {
     constexpr int kSms = 148, kSmemPerSm = 227 * 1024, kMostPerSm = 4;
-    static bool configured[64] = {};
+    static OncePerDevice opt_in;
     size_t smem = 0;
     const int per_sm = (grid + kSms - 1) / kSms;
     if (per_sm < kMostPerSm) {
         int dev = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e != cudaSuccess) return e;
-        if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+        if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
         smem = static_cast<size_t>(kSmemPerSm / (per_sm + 1) / 1024 + 1) * 1024;
-        if (!configured[dev]) {
-            e = cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerSm / 2 / 1024 * 1024 + 1024);
-            if (e != cudaSuccess) return e;
-            configured[dev] = true;
-        }
+        e = opt_in(dev, [] {
+            return cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerSm / 2 / 1024 * 1024 + 1024);
+        });
+        if (e != cudaSuccess) return e;
     }
     return launch_overlapped(kKernel, grid, block, smem, stream, static_cast<Args&&>(args)...);
+}
+
+// The opt-in of a kernel to more than 48 KB of dynamic shared memory, once per device ordinal.
+template <class Kernel>
+cudaError_t allow_dynamic_smem(Kernel kernel, size_t smem_bytes, OncePerDevice& done)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    return done(dev, [&] {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes));
+    });
 }
 #endif
 
