@@ -477,7 +477,7 @@ hydra_ulysses_kernel(const Vec* __restrict__ src, Vec* __restrict__ dst, uint32_
     constexpr int kUnroll = 4;
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t n_warps = gridDim.x * (kThreads / 32);
-    if (kLong) {
+    if constexpr (kLong) {
         for (uint32_t r = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); r < rows; r += n_warps) {
             const uint32_t j = r / n, t = r - j * n, blk = r * cu, tok = (t * P + j) * cu;
             for (uint32_t w0 = lane; w0 < cu; w0 += 32 * kUnroll) {
@@ -490,26 +490,25 @@ hydra_ulysses_kernel(const Vec* __restrict__ src, Vec* __restrict__ dst, uint32_
                     if (w0 + e * 32 < cu) st_unit(dst + (kPack ? blk : tok) + w0 + e * 32, v[e]);
             }
         }
-        overlap_next_launch();
-        return;
-    }
-    for (uint32_t r0 = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); r0 < rows; r0 += n_warps * kUnroll) {
-        uint32_t blk[kUnroll], tok[kUnroll];
+    } else {
+        for (uint32_t r0 = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); r0 < rows; r0 += n_warps * kUnroll) {
+            uint32_t blk[kUnroll], tok[kUnroll];
 #pragma unroll
-        for (int e = 0; e < kUnroll; ++e) {
-            const uint32_t r = r0 + e * n_warps;
-            const uint32_t j = r / n, t = r - j * n;
-            blk[e] = r * cu;                               // block-major: [P][n][cu]
-            tok[e] = (t * P + j) * cu;                     // token-major: [n][P][cu]
-        }
-        for (uint32_t w = lane; w < cu; w += 32) {
-            Vec v[kUnroll];
+            for (int e = 0; e < kUnroll; ++e) {
+                const uint32_t r = r0 + e * n_warps;
+                const uint32_t j = r / n, t = r - j * n;
+                blk[e] = r * cu;                               // block-major: [P][n][cu]
+                tok[e] = (t * P + j) * cu;                     // token-major: [n][P][cu]
+            }
+            for (uint32_t w = lane; w < cu; w += 32) {
+                Vec v[kUnroll];
 #pragma unroll
-            for (int e = 0; e < kUnroll; ++e)
-                if (r0 + e * n_warps < rows) v[e] = ld_unit(src + (kPack ? tok[e] : blk[e]) + w);
+                for (int e = 0; e < kUnroll; ++e)
+                    if (r0 + e * n_warps < rows) v[e] = ld_unit(src + (kPack ? tok[e] : blk[e]) + w);
 #pragma unroll
-            for (int e = 0; e < kUnroll; ++e)
-                if (r0 + e * n_warps < rows) st_unit(dst + (kPack ? blk[e] : tok[e]) + w, v[e]);
+                for (int e = 0; e < kUnroll; ++e)
+                    if (r0 + e * n_warps < rows) st_unit(dst + (kPack ? blk[e] : tok[e]) + w, v[e]);
+            }
         }
     }
     overlap_next_launch();
