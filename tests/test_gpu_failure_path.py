@@ -18,12 +18,16 @@ from gpu_util import check, pairs_for, run_gpu, run_oracle
 
 pytestmark = pytest.mark.gpu
 
-CASES = {                       # name -> (kernel to stall, dS hand-off limit in bytes, forward's short-pair limit)
-    "forward_cta_pairs": ("HYDRA_STALL_FWD", 4 << 30, 0),
-    "forward_short_sequences": ("HYDRA_STALL_FWD", 4 << 30, 1 << 20),
-    "backward_key_side": ("HYDRA_STALL_BWD_DKV", 4 << 30, None),
-    "backward_query_side_from_ds": ("HYDRA_STALL_BWD_DQ", 4 << 30, None),
-    "backward_query_side_recomputing": ("HYDRA_STALL_BWD_DQ", 0, None),
+# name -> (kernel to stall, dS hand-off limit in bytes, forward's short-pair limit, lengths, heads, ring degree of each)
+TINY = ([7, 33, 128, 300], 4, [0, 0, 0, 1])                       # the 300-token sequence is cut and merged
+CASES = {
+    "forward_cta_pairs": ("HYDRA_STALL_FWD", 4 << 30, 0, TINY),
+    "forward_short_sequences": ("HYDRA_STALL_FWD", 4 << 30, 1 << 20, ([128] * 50, 3, [0] * 50)),   # 150 q tiles
+    "forward_halved_tiles": ("HYDRA_STALL_FWD", 4 << 30, 1 << 20, TINY),
+    "backward_key_side": ("HYDRA_STALL_BWD_DKV", 4 << 30, None, TINY),
+    "backward_key_side_clusters": ("HYDRA_STALL_BWD_DKV", 4 << 30, None, ([700], 2, [0])),         # 11 q sub-tiles
+    "backward_query_side_from_ds": ("HYDRA_STALL_BWD_DQ", 4 << 30, None, TINY),
+    "backward_query_side_recomputing": ("HYDRA_STALL_BWD_DQ", 0, None, TINY),
 }
 
 
@@ -32,15 +36,17 @@ def test_a_wait_that_runs_out_is_reported_and_the_next_call_is_correct(case):
     import paper_2609_34318_b200 as P
     from paper_2609_34318_b200.runner import AttnStep, bits_to_tensor
     kernel = getattr(P, CASES[case][0])
-    w = hw.workload("tiny")
-    x = w.tensors()
-    cu = w.cu()
-    lib_pairs, rows, ora_pairs = pairs_for(cu, [0, 0, 0, 1])      # the 300-token sequence is cut and merged
+    lengths, h, cp_r = CASES[case][3]
+    cu = hw.cu_seqlens(lengths)
+    rng = np.random.default_rng(len(case))
+    x = {n: hw.f32_to_bf16_bits(rng.standard_normal((int(cu[-1]), h, d)).astype(np.float32))
+         for n, d in (("q", hw.D_QK), ("k", hw.D_QK), ("v", hw.D_V), ("do", hw.D_V))}
+    lib_pairs, rows, ora_pairs = pairs_for(cu, cp_r) if any(cp_r) else (None, 0, None)
     P.hydra_set_bwd_scratch_limit(CASES[case][1])
     if CASES[case][2] is not None:
         P.hydra_set_fwd_short_len(CASES[case][2])
     try:
-        step = AttnStep(cu, w.n_heads, lib_pairs, rows)
+        step = AttnStep(cu, h, lib_pairs, rows)
         q, k, v, do = (bits_to_tensor(x[n]) for n in ("q", "k", "v", "do"))
         if kernel != P.HYDRA_STALL_FWD:
             step.forward(q, k, v)                                  # a good forward for the backward to follow
@@ -49,8 +55,8 @@ def test_a_wait_that_runs_out_is_reported_and_the_next_call_is_correct(case):
         P.hydra_debug_stall(kernel, 3_000_000)
         try:
             if kernel == P.HYDRA_STALL_FWD:
-                P.hydra_attn_fwd(q, k, v, cu, w.n_heads, lib_pairs, True, step.scale, step.out, step.lse,
-                                 step.o_part, step.lse_part, rows, step.workspace)
+                P.hydra_attn_fwd(q, k, v, cu, h, lib_pairs, True, step.scale, step.out, step.lse,
+                                 step.o_part if rows else None, step.lse_part if rows else None, rows, step.workspace)
             else:
                 step.backward(q, k, v, do)
             status, detail = step.poll()                           # synchronises the stream: the kernel returned
@@ -61,7 +67,7 @@ def test_a_wait_that_runs_out_is_reported_and_the_next_call_is_correct(case):
         assert P.hydra_status_string(status) == "HYDRA_ERR_DEVICE_TIMEOUT"
         assert 0 <= detail < 2 * torch.cuda.get_device_properties(0).multi_processor_count, (case, detail)
         # the context is intact: same problem again, hook off
-        got = run_gpu(x, cu, w.n_heads, lib_pairs, rows)
+        got = run_gpu(x, cu, h, lib_pairs, rows)
         ref = run_oracle(x, cu, pairs=ora_pairs)
         check(got, ref, label=f"after a timed-out {case}: ")
     finally:

@@ -45,7 +45,7 @@ def default_routing():
     [1, 1, 1, 2],                 # work items of a single row and a single key
     [63, 65, 64],                 # one key more and one key less than a step
     [129, 257, 64, 500, 127],     # one row more than a tile, one more than two
-    [2048],                       # the longest sequence the default routing sends here: 16 tiles, up to 32 steps
+    [2048],                       # 16 tiles of up to 32 steps in halves
     [200] * 40,                   # more work items than the two slots of every SM hold at once
     [1024] * 7,                   # tiles of up to 16 steps, the longest call whose slots pop two items ahead throughout
     [1025] * 6,                   # one step more: popped near the end of an item (162 tiles: not a halved call either)
@@ -186,9 +186,9 @@ def test_a_limit_set_by_the_caller_is_kept_to_by_a_few_longer_pairs_too():
             check(run_gpu(x, cu, h, backward=False), run_oracle(x, cu, backward=False), names=("out", "lse"))
 
 
-def test_chunked_short_pairs_write_partials_and_merge():
+@pytest.mark.parametrize("h", [2, 10])                 # 20 q tiles a head: halved tiles, and more tiles than SMs
+def test_chunked_short_pairs_write_partials_and_merge(h):
     """Short sequences cut into zigzag chunks: diagonal and full pairs with offsets, partial outputs, the merge."""
-    h = 2
     lengths = [300, 77, 512, 130]
     cu = hw.cu_seqlens(lengths)
     x = rand_inputs(5, int(cu[-1]), h)
@@ -197,8 +197,8 @@ def test_chunked_short_pairs_write_partials_and_merge():
     check(got, run_oracle(x, cu, pairs=ora_pairs), label="chunked short ")
 
 
-def test_non_causal_short_pairs():
-    h = 2
+@pytest.mark.parametrize("h", [2, 30])                 # 5 q tiles a head
+def test_non_causal_short_pairs(h):
     lengths = [100, 65, 257]
     cu = hw.cu_seqlens(lengths)
     x = rand_inputs(6, int(cu[-1]), h)
@@ -206,14 +206,13 @@ def test_non_causal_short_pairs():
     check(got, run_oracle(x, cu, causal=False), label="non-causal short ")
 
 
-@pytest.mark.parametrize("short_len", [FWD_SHORT_LEN_DEFAULT, 0])
-def test_output_that_is_16_but_not_32_byte_aligned(short_len):
+@pytest.mark.parametrize("short_len,h", [(FWD_SHORT_LEN_DEFAULT, 2), (FWD_SHORT_LEN_DEFAULT, 38), (0, 2)])   # 4 q tiles a head
+def test_output_that_is_16_but_not_32_byte_aligned(short_len, h):
     """The interface asks for 16-byte alignment; both forward kernels store 32 bytes at a time only when the
     address allows it."""
     import paper_2609_34318_b200 as P
     P.hydra_set_fwd_short_len(short_len)
     from paper_2609_34318_b200.runner import AttnStep, bits_to_tensor
-    h = 2
     lengths = [70, 300]
     cu = hw.cu_seqlens(lengths)
     T = int(cu[-1])
@@ -232,7 +231,7 @@ def test_output_that_is_16_but_not_32_byte_aligned(short_len):
     assert bool((raw[:off] == 0).all()) and bool((raw[off + T * h * DV * 2:] == 0).all())
 
 
-@pytest.mark.parametrize("short_len", [1 << 20, 0])
+@pytest.mark.parametrize("short_len,few_tiles", [(1 << 20, True), (1 << 20, False), (0, True)])
 @pytest.mark.parametrize("q_start,q_len,k_start,k_len", [
     (0, 300, 200, 100),       # the first 200 q rows come before every key: a whole tile without keys, one with some
     (10, 140, 149, 60),       # only the last q row sees a key (its own position)
@@ -240,14 +239,17 @@ def test_output_that_is_16_but_not_32_byte_aligned(short_len):
     (50, 200, 0, 0),          # an empty kv range
     (255, 5, 0, 260),         # five rows at the end of a long kv range
 ])
-def test_partials_of_hand_made_pairs_with_rows_that_see_no_key(short_len, q_start, q_len, k_start, k_len):
+def test_partials_of_hand_made_pairs_with_rows_that_see_no_key(short_len, few_tiles, q_start, q_len, k_start, k_len):
     """Rows of a pair that see no key get O = 0 and LSE = -inf (their weight in a merge is then 0): on both
-    forward kernels, for whole tiles without keys, for single rows, and for pairs with no visible key at all."""
+    forward kernels, for whole tiles without keys, for single rows, and for pairs with no visible key at all. (With no
+    more q tiles than SMs the short-sequence kernel shares every tile between two slots.)"""
     import oracle
     import paper_2609_34318_b200 as P
     from paper_2609_34318_b200.runner import AttnStep, bits_to_tensor
     P.hydra_set_fwd_short_len(short_len)
     lengths, h = [31, 300, 64], 2
+    if not few_tiles:
+        h = torch.cuda.get_device_properties(0).multi_processor_count // ((q_len + 127) // 128) + 1
     cu = hw.cu_seqlens(lengths)
     T = int(cu[-1])
     x = rand_inputs(q_start + k_len, T, h)
