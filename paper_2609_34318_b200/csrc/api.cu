@@ -712,14 +712,8 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
                  (work_all - work_short) * pb.h <= double{1 << 29})
             std::fill(is_short.begin(), is_short.end(), 1);
     }
-    // How far ahead the short kernel's slots pop: items of up to 8 steps two ahead, longer ones late, so that no slot sits on
-    // an item while others run dry. In a call whose tiles are all of up to 16 steps (1024 keys) two ahead throughout is
-    // better: late / two ahead us, 16384 tokens, 8 heads of 192, sequences of 520 tokens 66.7 / 64.9, of 900 84.6 / 77.5, of
-    // 1000 80.3 / 78.0; heads of 128 53.5 / 48.1, 68.9 / 58.6, 58.7 / 58.4. Longer tiles: 6000 tokens, 16 heads, sequences
-    // of 1100 tokens 54.8 / 64.6; 4096 tokens of 1500 36.2 / 42.2; 8192 log-normal ones 105.9 / 124.5. (A fixed line
-    // inside a call, at 12, 16 or 24 steps, was worse than either way on 1500-token sequences.)
-    constexpr int32_t kShortTile = 16, kShortItem = 8;
     int32_t longest_tile = 0;
+    int64_t short_cost = 0;
     std::vector<std::vector<GroupEntry>> groups(pb.pairs.size()), groups_short(pb.pairs.size());
     for (size_t pi = 0; pi < pb.pairs.size(); ++pi) {
         const auto& p = pb.pairs[pi];
@@ -729,6 +723,7 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
                 const int32_t n_kv = kv_steps_short(p, q0, rows, causal);
                 groups_short[pi].push_back(GroupEntry{q0, n_kv, rows, n_kv});
                 longest_tile = std::max(longest_tile, n_kv);
+                short_cost += n_kv + kItemOverhead;
             }
             continue;
         }
@@ -751,7 +746,18 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
             groups[pi].push_back(GroupEntry{qa, n_a, n_b, 2 * std::max(n_a, std::max(n_b, 0))});
         }
     }
-    plan.early_pops = longest_tile > kShortTile ? kShortItem : kShortTile;
+    // How far ahead the short kernel's slots pop: items of up to 8 steps two ahead, longer ones late, so that no slot sits on
+    // an item while others run dry. Two ahead throughout is better where no item is long: all of up to 16 steps (1024
+    // keys), or up to 24 and none over 0.6 of a slot's even share of the call. Late / two ahead us, 16384 tokens, 8 heads of
+    // 192, sequences of 520 tokens 66.7 / 64.9, of 900 84.6 / 77.5, of 1000 80.3 / 78.0; of 128 53.5 / 48.1, 68.9 / 58.6,
+    // 58.7 / 58.4; of 1150 90.4 / 88.7 and 70.3 / 69.3. Beyond: 6000 tokens, 16 heads, sequences of 1100 tokens 54.8 / 64.6;
+    // 4096 tokens of 1500 36.2 / 42.2; 8192 log-normal ones 105.9 / 124.5. (A fixed line inside a call, at 12, 16 or 24
+    // steps, was worse than either way on 1500-token sequences.)
+    constexpr int32_t kShortItem = 8, kShortTile = 16, kMidTile = 24;
+    const int64_t slots = 2 * plan_workers(1);
+    const bool early = longest_tile <= kShortTile ||
+                       (longest_tile <= kMidTile && (longest_tile + kItemOverhead) * slots * 10 <= short_cost * pb.h * 6);
+    plan.early_pops = early ? kMidTile : kShortItem;
     const std::vector<FwdItem> items = order_by_groups<FwdItem>(
         groups, pb.h, plan_workers(2),
         [](int32_t g, int32_t a, const GroupEntry& e) { return FwdItem{g, a, e.a, e.b, e.c, {0, 0, 0}}; });

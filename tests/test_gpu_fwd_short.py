@@ -134,6 +134,28 @@ def test_a_limit_set_to_the_library_s_own_value_is_kept_to(order):
     assert not torch.equal(got[-1], got[0]), "the two kernels' sums differ in their last bits"
 
 
+@pytest.mark.parametrize("length,copies", [(1100, 90), (1536, 45), (1537, 45)])   # tiles of up to 18, 24 and 25 steps
+def test_many_copies_of_a_sequence_give_the_same_bits(length, copies):
+    """In a call of many tiles of up to 24 steps the slots pop two items ahead, beyond that late: every copy of a sequence
+    comes out as every other, and as the oracle has the first."""
+    import paper_2609_34318_b200 as P
+    from paper_2609_34318_b200.runner import AttnStep, bits_to_tensor
+    P.hydra_set_fwd_short_len(1 << 20)
+    x = rand_inputs(length, length, 2)
+    step = AttnStep(hw.cu_seqlens([length] * copies), 2)
+    step.out.fill_(float("nan"))
+    step.lse.fill_(float("nan"))
+    step.forward(*(bits_to_tensor(x[n]).repeat(copies, 1, 1) for n in ("q", "k", "v")))
+    assert step.poll()[0] == 0
+    out = step.out.view(torch.int16).view(copies, length, 2, DV)
+    lse = step.lse.view(torch.int32).view(2, copies, length)
+    assert bool((out == out[:1]).all()) and bool((lse == lse[:, :1]).all())
+    ref = run_oracle(x, hw.cu_seqlens([length]), backward=False)
+    got = dict(out=step.out[:length].float().cpu().numpy().astype(np.float64),
+               lse=step.lse[:, :length].cpu().numpy().astype(np.float64))
+    check(got, ref, names=("out", "lse"))
+
+
 def test_random_length_mixes_and_both_kernels_agree():
     import paper_2609_34318_b200 as P
     rng = np.random.default_rng(11)
