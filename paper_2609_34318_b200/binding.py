@@ -307,7 +307,7 @@ def hydra_set_plan_prefetch(on: bool) -> None:
 
 def hydra_set_fwd_short_len(length: int) -> None:
     """Pairs with q and kv ranges of at most `length` tokens use the short-sequence forward kernel (0: off;
-    negative, the default: 1280, or 2048 with shared K / V heads or heads of 128)."""
+    negative, the default: 1280 to 3328 by head layout and size of the call, see the header)."""
     _lib.hydra_set_fwd_short_len(int(length))
 
 

@@ -425,15 +425,26 @@ void arena_note_use(const Plan& plan, int device, cudaStream_t stream)
 // Pairs whose q range and kv range are both at most this long go to the short-sequence forward kernel
 // (0: none do; negative: chosen by the library from the head layout). See build_fwd.
 std::atomic<int32_t> g_fwd_short_len{-1};
-// Where the two forward kernels take equal time on sequences of one length (32K tokens, 16 heads; ms, short-sequence /
-// CTA pairs): with a K / V head per query head at d_qk = 192, 0.165 / 0.191 at 512 tokens, 0.242 / 0.250 at 1024,
-// 0.326 / 0.316 at 1489, 0.399 / 0.373 at 2048; with shared K / V heads 0.225 / 0.252 at 1024, 0.379 / 0.373 at 2048,
-// 0.677 / 0.620 at 4096; at d_qk = 128 (where a slot of the short-sequence kernel has room for a second V stage)
-// 0.208 / 0.229 at 1024, 0.340 / 0.341 at 2048, 0.608 / 0.561 at 4096.
+// Where the two forward kernels take equal time. In calls of fewer than 20 q tiles per SM (16384 tokens of 16 heads have 15),
+// where the tail counts, at 1280 tokens with a K / V head per query head at d_qk = 192 and 2048 with shared K / V heads or at
+// d_qk = 128 (where a slot of the short-sequence kernel has room for a second V stage): CTA pairs / short-sequence kernel, 16384
+// tokens, 8 heads, sequences of 1281 to 1920 tokens 0.97-1.03, of 2047 and more 0.93-1.00. In larger calls, which have
+// sequences of many lengths cut into 256-row tiles to fill the CTA pairs with, at 1920 and 3328: 65536 tokens, 32 heads of 192,
+// 1281 tokens 1.08, 1600 1.20, 1920 1.13, 2047 1.00; with shared K / V heads 1281 1.27, 2047 1.05, 2900 1.07, 3200
+// 1.03, 3584 0.98; heads of 128 1281 1.28, 2600 1.09, 3200 1.05, 3584 0.99.
+constexpr int32_t kManyTilesPerSm = 20;
+int plan_workers(int per_worker_sms);
+bool many_q_tiles(const Problem& pb)
+{
+    int64_t n = 0;
+    for (const auto& p : pb.pairs) n += (p.q_len + TILE - 1) / TILE;
+    return n * pb.h >= int64_t{kManyTilesPerSm} * plan_workers(1);
+}
 int32_t fwd_short_len_for(const Problem& pb)
 {
     if (pb.fwd_short_set >= 0) return pb.fwd_short_set;
-    return (pb.dqk == D_QK && pb.kv_group == 1) ? 1280 : 2048;
+    const bool per_head = pb.dqk == D_QK && pb.kv_group == 1;
+    return many_q_tiles(pb) ? (per_head ? 1920 : 3328) : (per_head ? 1280 : 2048);
 }
 static_assert(FWD_SHORT_KEYS == SUB, "the short forward kernel reads K through the 64-row map of the CTA-pair kernel");
 
@@ -703,13 +714,18 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
             work_all += w;
             if (short_len > 0 && p.q_len <= short_len && p.k_len <= short_len) { is_short[pi] = 1; work_short += w; }
         }
-        if (work_short * 4 < work_all) std::fill(is_short.begin(), is_short.end(), 0);
         // The second launch is not worth its price either if little is left for it that the short kernel would run almost
-        // as fast: pairs up to twice the limit cost it at most a tenth more, and 2^29 positions (with those above the
-        // mask) take 0.2 ms. 4096 packed tokens, 16 heads, the longest sequence 1381 tokens: 75 us on both kernels,
-        // 59 on the short one alone. (Not against a limit set by the caller.)
-        else if (pb.fwd_short_set < 0 && work_short < work_all && longest <= 2 * short_len &&
-                 (work_all - work_short) * pb.h <= double{1 << 29})
+        // as fast (not against a limit set by the caller). In a small call: pairs of up to twice the limit and 2^29 positions
+        // (with those above the mask), which take 0.2 ms. 4096 packed tokens, 16 heads, the longest sequence 1381 tokens:
+        // 75 us on both kernels, 59 on the short one alone. In a large one pairs of up to a quarter more than the limit,
+        // however much they are of it: 65536 tokens, 16 heads, 24 sequences of 2016 tokens beside some of 300 639 us
+        // alone, 696 on both, 720 on CTA pairs; 16 query heads over two K / V heads, seven of 4160 767, 886, 886.
+        const bool automatic = pb.fwd_short_set < 0, many = many_q_tiles(pb);
+        if (automatic && many && int64_t{4} * longest <= 5 * short_len && work_short * 64 >= work_all)
+            std::fill(is_short.begin(), is_short.end(), 1);
+        else if (work_short * 4 < work_all)
+            std::fill(is_short.begin(), is_short.end(), 0);
+        else if (automatic && !many && longest <= 2 * short_len && (work_all - work_short) * pb.h <= double{1 << 29})
             std::fill(is_short.begin(), is_short.end(), 1);
     }
     int32_t longest_tile = 0;
