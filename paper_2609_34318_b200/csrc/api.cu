@@ -764,15 +764,16 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     }
     // How far ahead the short kernel's slots pop: items of up to 8 steps two ahead, longer ones late, so that no slot sits on
     // an item while others run dry. Two ahead throughout is better where no item is long: all of up to 16 steps (1024
-    // keys), or up to 24 and none over 0.6 of a slot's even share of the call. Late / two ahead us, 16384 tokens, 8 heads of
-    // 192, sequences of 520 tokens 66.7 / 64.9, of 900 84.6 / 77.5, of 1000 80.3 / 78.0; of 128 53.5 / 48.1, 68.9 / 58.6,
-    // 58.7 / 58.4; of 1150 90.4 / 88.7 and 70.3 / 69.3. Beyond: 6000 tokens, 16 heads, sequences of 1100 tokens 54.8 / 64.6;
-    // 4096 tokens of 1500 36.2 / 42.2; 8192 log-normal ones 105.9 / 124.5. (A fixed line inside a call, at 12, 16 or 24
-    // steps, was worse than either way on 1500-token sequences.)
+    // keys) and none over a slot's even share of the call, or all of up to 24 and none over 0.6 of it. Late / two ahead us:
+    // 16384 tokens, 8 heads of 192, sequences of 520 tokens 66.7 / 64.9, of 900 84.6 / 77.5, of 1000 80.3 / 78.0, of 1150
+    // 90.4 / 88.7; of 128 53.5 / 48.1, 68.9 / 58.6, 58.7 / 58.4, 70.3 / 69.3. Beyond the lines: 4 heads, 10 sequences of 1006
+    // tokens 25.0 / 26.7, 12 of 900 25.5 / 30.6; 16 heads, 6000 tokens of 1100 54.8 / 64.6, 4096 of 1500 36.2 / 42.2, 8192
+    // log-normal ones 105.9 / 124.5. (A fixed line inside a call, at 12, 16 or 24 steps, was worse than either way on
+    // 1500-token sequences.)
     constexpr int32_t kShortItem = 8, kShortTile = 16, kMidTile = 24;
     const int64_t slots = 2 * plan_workers(1);
-    const bool early = longest_tile <= kShortTile ||
-                       (longest_tile <= kMidTile && (longest_tile + kItemOverhead) * slots * 10 <= short_cost * pb.h * 6);
+    const int64_t share = longest_tile <= kShortTile ? 10 : longest_tile <= kMidTile ? 6 : 0;      // tenths of the even share
+    const bool early = (longest_tile + kItemOverhead) * slots * 10 <= short_cost * pb.h * share;
     plan.early_pops = early ? kMidTile : kShortItem;
     const std::vector<FwdItem> items = order_by_groups<FwdItem>(
         groups, pb.h, plan_workers(2),
