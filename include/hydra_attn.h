@@ -573,7 +573,8 @@ void hydra_set_plan_prefetch(int32_t on);
  * call's work, that call uses the CTA-pair kernel alone. Both compute the same function to the same tolerance
  * (not bit for bit: their summation orders differ). len = 0 switches the short-sequence kernel off; a negative
  * len (the default) lets the library choose: 1280 for heads of 192 with a K / V head per query head, 2048 with
- * shared K / V heads or heads of 128; 1920 and 3328 in calls of 20 or more 128-row q tiles (times heads) per SM;
+ * shared K / V heads or heads of 128; 1920 and 3328 in causal calls of whole sequences with 20 or more 128-row q
+ * tiles (times heads) per SM;
  * any length for a call with no more such tiles than the GPU has SMs, whose tiles the short-sequence kernel splits
  * between its two slots; and up to a quarter more than that limit (twice in smaller calls) where the pairs above it are
  * too little work for a second launch. A limit set by the caller is kept to exactly. Takes effect with the next call.

@@ -431,20 +431,26 @@ std::atomic<int32_t> g_fwd_short_len{-1};
 // tokens, 8 heads, sequences of 1281 to 1920 tokens 0.97-1.03, of 2047 and more 0.93-1.00. In larger calls, which have
 // sequences of many lengths cut into 256-row tiles to fill the CTA pairs with, at 1920 and 3328: 65536 tokens, 32 heads of 192,
 // 1281 tokens 1.08, 1600 1.20, 1920 1.13, 2047 1.00; with shared K / V heads 1281 1.27, 2047 1.05, 2900 1.07, 3200
-// 1.03, 3584 0.98; heads of 128 1281 1.28, 2600 1.09, 3200 1.05, 3584 0.99.
+// 1.03, 3584 0.98; heads of 128 1281 1.28, 2600 1.09, 3200 1.05, 3584 0.99. (Large calls of whole causal sequences, that
+// is. Chunk pairs off the diagonal keep CTA pairs busy without a mask: eleven sequences of 5685 tokens, 4 heads, cut in
+// chunks of 1421 445 us on CTA pairs, 495 on the other kernel, four of 12000, 16 heads, chunks of 1500 2810 and 3150.)
 constexpr int32_t kManyTilesPerSm = 20;
 int plan_workers(int per_worker_sms);
-bool many_q_tiles(const Problem& pb)
+bool many_q_tiles(const Problem& pb, int causal)
 {
     int64_t n = 0;
-    for (const auto& p : pb.pairs) n += (p.q_len + TILE - 1) / TILE;
-    return n * pb.h >= int64_t{kManyTilesPerSm} * plan_workers(1);
+    bool diagonal = causal != 0;
+    for (const auto& p : pb.pairs) {
+        n += (p.q_len + TILE - 1) / TILE;
+        diagonal = diagonal && p.q_start == p.k_start;
+    }
+    return diagonal && n * pb.h >= int64_t{kManyTilesPerSm} * plan_workers(1);
 }
-int32_t fwd_short_len_for(const Problem& pb)
+int32_t fwd_short_len_for(const Problem& pb, int causal)
 {
     if (pb.fwd_short_set >= 0) return pb.fwd_short_set;
     const bool per_head = pb.dqk == D_QK && pb.kv_group == 1;
-    return many_q_tiles(pb) ? (per_head ? 1920 : 3328) : (per_head ? 1280 : 2048);
+    return many_q_tiles(pb, causal) ? (per_head ? 1920 : 3328) : (per_head ? 1280 : 2048);
 }
 static_assert(FWD_SHORT_KEYS == SUB, "the short forward kernel reads K through the 64-row map of the CTA-pair kernel");
 
@@ -457,7 +463,7 @@ std::vector<uint8_t> make_key(int kind, int device, const Problem& pb, int causa
     };
     // the forward's tables depend on which pairs go to the short-sequence kernel: on the limit, and on who chose it
     const bool fwd = kind == HYDRA_WS_FWD;
-    const int32_t head[7] = {kind, device, pb.h, causal, pb.n_seqs, fwd ? fwd_short_len_for(pb) : 0,
+    const int32_t head[7] = {kind, device, pb.h, causal, pb.n_seqs, fwd ? fwd_short_len_for(pb, causal) : 0,
                              fwd && pb.fwd_short_set < 0};
     put(head, sizeof head);
     put(pb.cu.data(), pb.cu.size() * sizeof(int32_t));
@@ -684,7 +690,7 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     // bound by the length of a tile's chain of steps, and more, shorter chains per SM win; on long pairs its
     // operand sharing and its 256-row tiles do. A second launch has a price of its own (its start and its
     // tail), so the short kernel is used only if the short pairs carry at least a quarter of the call's work.
-    const int32_t short_len = fwd_short_len_for(pb);
+    const int32_t short_len = fwd_short_len_for(pb, causal);
     std::vector<uint8_t> is_short(pb.pairs.size(), 0);
     // A call with no more q tiles than SMs: what it takes is its longest tile's chain of steps. The short kernel then has
     // an idle slot beside every busy one and gives it the second half of the tile's keys, whatever their number (the
@@ -720,7 +726,7 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
         // 75 us on both kernels, 59 on the short one alone. In a large one pairs of up to a quarter more than the limit,
         // however much they are of it: 65536 tokens, 16 heads, 24 sequences of 2016 tokens beside some of 300 639 us
         // alone, 696 on both, 720 on CTA pairs; 16 query heads over two K / V heads, seven of 4160 767, 886, 886.
-        const bool automatic = pb.fwd_short_set < 0, many = many_q_tiles(pb);
+        const bool automatic = pb.fwd_short_set < 0, many = many_q_tiles(pb, causal);
         if (automatic && many && int64_t{4} * longest <= 5 * short_len && work_short * 64 >= work_all)
             std::fill(is_short.begin(), is_short.end(), 1);
         else if (work_short * 4 < work_all)
