@@ -280,15 +280,17 @@ int32_t hydra_grad_cast(const float* acc, void* grad, int64_t n_elements, void* 
  * (integer division); n_kv_heads must divide n_heads. k device bf16 [T, n_kv_heads, 192], v device bf16
  * [T, n_kv_heads, 128]; everything else as in hydra_attn_fwd / hydra_attn_bwd_accumulate, which are the
  * case n_kv_heads == n_heads.
- * In the backward dk, dv of a KV head are the SUM over the g query heads that read it: the work items of
- * the g query heads add into the same fp32 rows with reductions, so the order of the g terms, and with it
- * the last bits of dk / dv, may differ from run to run.
+ * In the backward dk, dv of a KV head are the SUM over the g query heads that read it. In calls with many
+ * key tiles one work item takes all g heads; otherwise the work items of a group add into the same fp32
+ * rows with reductions, so the order of the g terms, and with it the last bits of dk / dv, may differ from
+ * run to run.
  *   hydra_attn_bwd_accumulate_gqa  dq_acc device fp32 [T, n_heads, 192], dk_acc device fp32
  *                                  [T, n_kv_heads, 192], dv_acc device fp32 [T, n_kv_heads, 128]: the
  *                                  caller zeroes them and rounds them with hydra_grad_cast.
  *   hydra_attn_bwd_gqa             one shot: dq device bf16 [T, n_heads, 192], dk device bf16
  *                                  [T, n_kv_heads, 192], dv device bf16 [T, n_kv_heads, 128]. dk and dv are
- *                                  summed in fp32 in the workspace and rounded once; the workspace must
+ *                                  summed in fp32 (in the workspace if several work items share a row)
+ *                                  and rounded once; the workspace must
  *                                  have hydra_workspace_bytes_gqa(HYDRA_WS_BWD, ...) bytes (the per-head
  *                                  size plus 4 * (192 + 128) bytes per token and KV head), else
  *                                  HYDRA_ERR_WORKSPACE_TOO_SMALL. The banded form does not apply.

@@ -6,9 +6,11 @@
 #include <cmath>
 #include <cstddef>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <memory>
 #include <mutex>
+#include <queue>
 #include <vector>
 
 #include "hydra_internal.h"
@@ -253,6 +255,7 @@ struct Plan {
     int32_t halves = 0;              // forward: the short kernel's items are halves of tiles, two per thread block;
                                      // backward: two CTAs share every key-side item
     int32_t early_pops = 0;          // forward: FwdParams::early_pops
+    int32_t item_heads = 1;          // backward: query heads per key-side item (BwdParams::item_heads)
     int64_t ds_head_blocks = 0;      // backward: blocks of the dS hand-off buffer per head; -1: not usable
     // residency on the device (guarded by g_plan_mutex)
     int half = -1;                   // arena half the tables were last copied to
@@ -463,8 +466,8 @@ std::vector<uint8_t> make_key(int kind, int device, const Problem& pb, int causa
     };
     // the forward's tables depend on which pairs go to the short-sequence kernel: on the limit, and on who chose it
     const bool fwd = kind == HYDRA_WS_FWD;
-    const int32_t head[7] = {kind, device, pb.h, causal, pb.n_seqs, fwd ? fwd_short_len_for(pb, causal) : 0,
-                             fwd && pb.fwd_short_set < 0};
+    const int32_t head[8] = {kind, device, pb.h, causal, pb.n_seqs, fwd ? fwd_short_len_for(pb, causal) : 0,
+                             fwd && pb.fwd_short_set < 0, kind == HYDRA_WS_BWD ? pb.kv_group : 0};
     put(head, sizeof head);
     put(pb.cu.data(), pb.cu.size() * sizeof(int32_t));
     put(pb.pairs.data(), pb.pairs.size() * sizeof(hydra_pair_t));
@@ -946,6 +949,50 @@ bool key_tiles_halved(const Problem& pb, int causal)
     return longest > 8;
 }
 
+// Query heads that a key-side item visits where several share a K / V head. With all of a group in one item dk and dv are
+// complete in tensor memory: no fp32 sums in memory, no cast, K and V loaded and the accumulators written once. But such
+// items are few and long; the fewer heads an item takes, the better a small call fills the SMs. The queue is simulated for
+// every number of heads that divides the group (longest items first, as the kernel's list has them; a unit is a 64-row
+// sub-tile, about 1 us). Step in passes one after another, one head per item / as chosen here: 32768 tokens of 64 to 512,
+// 32 heads of 128 over 8, 1245 / 965 us; log-normal lengths, 8192 tokens, 32 heads over 8, 854 / 776, 16384 tokens, 16 over
+// 4, 1100 / 1038, 32768 tokens, 16 heads of 128 over 2, 1861 / 1832 (1, 2, 4, 8 heads per item: key side 959, 923, 908, 932
+// us, and the cast 23 us less with all 8).
+int32_t heads_per_key_item(const std::vector<std::vector<GroupEntry>>& groups, const Problem& pb, int workers)
+{
+    if (pb.kv_group <= 1) return 1;
+    constexpr int64_t kItem = 4, kItemSummed = 6, kCast = 8;    // beyond its sub-tiles: an item, one that adds in fp32; zeroing and cast
+    std::vector<int32_t> costs;
+    int64_t total = 0;
+    int32_t longest = 0;
+    for (const auto& g : groups)
+        for (const GroupEntry& e : g) { costs.push_back(e.cost); total += e.cost; longest = std::max(longest, e.cost); }
+    std::sort(costs.begin(), costs.end(), std::greater<int32_t>());
+    int64_t best = 0;
+    int32_t heads = 1;
+    for (int32_t d = pb.kv_group; d >= 1; --d) {
+        if (pb.kv_group % d) continue;
+        const int64_t item = d == pb.kv_group ? kItem : kItemSummed, copies = pb.h / d;
+        const int64_t even = (total * pb.h + static_cast<int64_t>(costs.size()) * copies * item + workers - 1) / workers;
+        int64_t end = std::max(even, longest * int64_t{d} + item);
+        // (with more items than that the list ends with short ones)
+        if (static_cast<int64_t>(costs.size()) * copies <= 16 * workers) {
+            std::priority_queue<int64_t, std::vector<int64_t>, std::greater<int64_t>> free;
+            for (int i = 0; i < workers; ++i) free.push(0);
+            end = 0;
+            for (int32_t c : costs)
+                for (int64_t k = 0; k < copies; ++k) {
+                    const int64_t t = free.top() + int64_t{c} * d + item;
+                    free.pop();
+                    free.push(t);
+                    end = std::max(end, t);
+                }
+        }
+        end += d == pb.kv_group ? 0 : kCast;
+        if (d == pb.kv_group || end < best) { best = end; heads = d; }
+    }
+    return heads;
+}
+
 void build_bwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& blob)
 {
     const int32_t n = static_cast<int32_t>(pb.pairs.size());
@@ -990,15 +1037,19 @@ void build_bwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
             }
             i = j;
         }
-        items = order_by_groups<GroupItem>(groups, pb.h, plan_workers(1), [&](int32_t g, int32_t a, const GroupEntry& e) {
-            return GroupItem{list_of[g].first, list_of[g].second, a, e.a};
+        const int32_t heads = by_q || plan.halves ? 1 : heads_per_key_item(groups, pb, plan_workers(1));
+        if (!by_q) plan.item_heads = heads;
+        for (auto& g : groups)
+            for (GroupEntry& e : g) e.cost *= heads;
+        items = order_by_groups<GroupItem>(groups, pb.h / heads, plan_workers(1), [&](int32_t g, int32_t a, const GroupEntry& e) {
+            return GroupItem{list_of[g].first, list_of[g].second, a * heads, e.a};
         });
     };
     std::vector<int32_t> lists_q, lists_k;
     std::vector<GroupItem> items_q, items_k;
+    plan.halves = key_tiles_halved(pb, causal);
     group_by(true, lists_q, items_q);
     group_by(false, lists_k, items_k);
-    plan.halves = key_tiles_halved(pb, causal);
     std::vector<PairDev> dev = device_pairs(pb);
     plan.ds_head_blocks = ds_layout(pb, causal, &dev);
     plan.off_pairs = append(blob, dev);
@@ -1696,12 +1747,20 @@ struct BwdTensors {
     void *dq, *dk, *dv;                 // bf16 outputs or fp32 accumulators
 };
 
+// Where dk and dv may be summed in fp32 when several key-side items share their rows (grouped query heads).
+struct KvSums {
+    float *dk, *dv;
+    size_t bytes;                       // dk's and dv's together
+    bool used;                          // set by bwd_run: the sums are there, the outputs are not written yet
+};
+
 // One backward over the pairs of `pb`: D = rowsum(dO*O) (if `first`), the key-side kernel, the query-side
 // kernel. dq and dk/dv are bf16 outputs or fp32 accumulators, each by its own flag. `ds` / `ds_room` is
-// where a dS hand-off buffer may go. With `first` false the status block keeps its flags and only the
+// where a dS hand-off buffer may go. `sums`: where dk and dv are summed if no item of the plan holds all query heads of a
+// K / V head (null: the outputs need no such sums). With `first` false the status block keeps its flags and only the
 // work-queue counters are cleared. `halves_of_call` is key_tiles_halved of the whole call, -1 if `pb` is all of it.
 int32_t bwd_run(const Problem& pb, int32_t n_kv_heads, int32_t causal, float softmax_scale, const BwdTensors& t,
-                bool accumulate_dq, bool accumulate_dkv, void* workspace, uint8_t* ds, size_t ds_room, uint64_t ds_limit, bool first,
+                KvSums* sums, bool accumulate_dq, bool accumulate_dkv, void* workspace, uint8_t* ds, size_t ds_room, uint64_t ds_limit, bool first,
                 int halves_of_call, int sms, cudaStream_t stream)
 {
     const int32_t n_heads = pb.h;
@@ -1716,9 +1775,12 @@ int32_t bwd_run(const Problem& pb, int32_t n_kv_heads, int32_t causal, float sof
     if (make_map(&mk, t.k, pb.Tk, n_kv_heads, pb.dqk, TILE) || make_map(&mv, t.v, pb.Tk, n_kv_heads, D_V, TILE) ||
         make_map(&mq_sub, t.q, pb.Tq, n_heads, pb.dqk, SUB) || make_map(&mdo_sub, t.dout, pb.Tq, n_heads, D_V, SUB))
         return HYDRA_ERR_CUDA;
+    if (sums) sums->used = plan->item_heads != n_heads / n_kv_heads;
+    const bool summed = sums && sums->used;
     if (first) {
         ScopedKernelTimer timer(K_PREP, stream);
-        if (launch_bwd_prep(t.dout, t.out, dsum, pb.Tq, n_heads, static_cast<StatusBlock*>(workspace), stream) != cudaSuccess)
+        if (launch_bwd_prep(t.dout, t.out, dsum, pb.Tq, n_heads, static_cast<StatusBlock*>(workspace), summed ? sums->dk : nullptr,
+                            summed ? sums->bytes : 0, stream) != cudaSuccess)
             return HYDRA_ERR_CUDA;
         g_launches += 1;
     } else if (launch_reset(static_cast<StatusBlock*>(workspace), true, stream) != cudaSuccess) {
@@ -1745,7 +1807,9 @@ int32_t bwd_run(const Problem& pb, int32_t n_kv_heads, int32_t causal, float sof
         bp.lists = lease.at<int32_t>(plan->off_lists2);
         bp.items = lease.at<GroupItem>(plan->off_items2);
         bp.n_items = plan->n_items2;
-        bp.accumulate = accumulate_dkv ? 1 : 0;
+        bp.item_heads = plan->item_heads;
+        bp.accumulate = accumulate_dkv || summed ? 1 : 0;
+        if (summed) { bp.dk = sums->dk; bp.dv = sums->dv; }
         bp.debug_stall_ns = g_debug_stall_ns[HYDRA_STALL_BWD_DKV].load();
         ScopedKernelTimer timer(K_DKV, stream);
         const bool halves = halves_of_call >= 0 ? halves_of_call != 0 : plan->halves != 0;
@@ -1897,6 +1961,7 @@ int32_t bwd_core(Problem& pb, const void* q, const void* k, const void* v, const
 {
     const int32_t n_heads = pb.h;
     if (n_kv_heads < 1 || n_heads % n_kv_heads) return HYDRA_ERR_INVALID_ARG;
+    pb.kv_group = n_heads / n_kv_heads;
     if (!(softmax_scale > 0.f) || !std::isfinite(softmax_scale)) return HYDRA_ERR_INVALID_ARG;
     if (!workspace || !aligned16(workspace)) return HYDRA_ERR_INVALID_ARG;
     const size_t need = kStatusBytes + align_up(static_cast<size_t>(pb.Tq) * n_heads * sizeof(float), 256);
@@ -1921,29 +1986,30 @@ int32_t bwd_core(Problem& pb, const void* q, const void* k, const void* v, const
     const BwdTensors t{q, k, v, out, dout, lse, dq, dk, dv};
     const size_t room = workspace_bytes > ds_off ? workspace_bytes - ds_off : 0;
 
-    // One-shot grouped-query form: the query heads of a group add into one dk / dv row, which only the
-    // accumulating epilogue can do. dk, dv are summed in fp32 in the workspace and rounded at the end; dq
-    // (one query head per row) is written as bf16 as usual.
+    // One-shot grouped-query form: where no key-side item holds all query heads of a group, they add into one dk / dv row,
+    // which only the accumulating epilogue can do: dk, dv are then summed in fp32 in the workspace (cleared by the D =
+    // rowsum(dO O) kernel) and rounded at the end. dq (one query head per row) is written as bf16 as usual.
     if (!accumulate && n_kv_heads != n_heads) {
         const size_t kv_bytes = bwd_kv_acc_bytes(pb, n_kv_heads);
         if (room < kv_bytes) return HYDRA_ERR_WORKSPACE_TOO_SMALL;
-        float* dk_acc = reinterpret_cast<float*>(ws + ds_off);
-        float* dv_acc = dk_acc + static_cast<size_t>(pb.Tk) * n_kv_heads * pb.dqk;
-        if (cudaMemsetAsync(dk_acc, 0, kv_bytes, stream) != cudaSuccess) return HYDRA_ERR_CUDA;
-        const BwdTensors tg{q, k, v, out, dout, lse, dq, dk_acc, dv_acc};
-        if (int32_t s = bwd_run(pb, n_kv_heads, causal, softmax_scale, tg, false, true, workspace,
+        KvSums sums{};
+        sums.dk = reinterpret_cast<float*>(ws + ds_off);
+        sums.dv = sums.dk + static_cast<size_t>(pb.Tk) * n_kv_heads * pb.dqk;
+        sums.bytes = kv_bytes;
+        if (int32_t s = bwd_run(pb, n_kv_heads, causal, softmax_scale, t, &sums, false, false, workspace,
                                 ws + ds_off + kv_bytes, room - kv_bytes, g_ds_limit_bytes.load(), true, -1, sms, stream))
             return s;
+        if (!sums.used) return HYDRA_OK;
         const size_t rk = static_cast<size_t>(n_kv_heads) * pb.dqk, rv = static_cast<size_t>(n_kv_heads) * D_V;
         for (const auto& run : covered_rows(pb, true)) {
             const size_t row = run.first, n = run.second - run.first;
             ScopedKernelTimer timer(K_CAST, stream);
-            if (launch_grad_cast(dk_acc + row * rk, static_cast<uint16_t*>(dk) + row * rk,
-                                 static_cast<int64_t>(n * rk), stream) != cudaSuccess ||
-                launch_grad_cast(dv_acc + row * rv, static_cast<uint16_t*>(dv) + row * rv,
-                                 static_cast<int64_t>(n * rv), stream) != cudaSuccess)
+            int launches = 0;
+            if (launch_grad_cast2(sums.dk + row * rk, static_cast<uint16_t*>(dk) + row * rk, static_cast<int64_t>(n * rk),
+                                  sums.dv + row * rv, static_cast<uint16_t*>(dv) + row * rv, static_cast<int64_t>(n * rv),
+                                  &launches, stream) != cudaSuccess)
                 return HYDRA_ERR_CUDA;
-            g_launches += 2;
+            g_launches += launches;
         }
         return HYDRA_OK;
     }
@@ -1970,7 +2036,7 @@ int32_t bwd_core(Problem& pb, const void* q, const void* k, const void* v, const
                 bool first = true;
                 for (const auto& band : bands) {
                     band_pb.pairs = band;
-                    if (int32_t s = bwd_run(band_pb, n_heads, causal, softmax_scale, tb, true, false, workspace,
+                    if (int32_t s = bwd_run(band_pb, n_heads, causal, softmax_scale, tb, nullptr, true, false, workspace,
                                             ws + ds_off + acc_bytes, scratch, scratch, first, halves, sms, stream))
                         return s;
                     first = false;
@@ -1990,7 +2056,7 @@ int32_t bwd_core(Problem& pb, const void* q, const void* k, const void* v, const
             }
         }
     }
-    return bwd_run(pb, n_kv_heads, causal, softmax_scale, t, accumulate, accumulate, workspace, ws + ds_off, room,
+    return bwd_run(pb, n_kv_heads, causal, softmax_scale, t, nullptr, accumulate, accumulate, workspace, ws + ds_off, room,
                    g_ds_limit_bytes.load(), true, -1, sms, stream);
 }
 }  // namespace

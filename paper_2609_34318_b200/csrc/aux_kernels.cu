@@ -326,13 +326,22 @@ __global__ void __launch_bounds__(32) hydra_reset_kernel(int32_t* block, int n)
     for (int i = threadIdx.x; i < n; i += 32) block[i] = 0;
 }
 
+// The whole grid clears n16 16-byte units (fp32 accumulators that the next kernel of the call adds into: a memset before the
+// call's kernels would be a launch of its own, and one that breaks the chain of overlapped launches).
+__device__ __forceinline__ void clear16(uint4* p, int64_t n16)
+{
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; i < n16; i += static_cast<int64_t>(gridDim.x) * kThreads)
+        p[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 // D[a, t] = sum_e dO[t, a, e] * O[t, a, e]; block 0 also clears the status block for the kernels that follow
 __global__ void __launch_bounds__(kThreads)
 hydra_bwd_prep_kernel(const uint4* __restrict__ dout, const uint4* __restrict__ out,
-                      float* __restrict__ dsum, int64_t T, int32_t h, StatusBlock* status)
+                      float* __restrict__ dsum, int64_t T, int32_t h, StatusBlock* status, uint4* zero, int64_t zero16)
 {
     overlap_next_launch();
     wait_for_previous_launch();
+    clear16(zero, zero16);
     if (blockIdx.x == 0 && threadIdx.x < sizeof(StatusBlock) / 4) reinterpret_cast<int32_t*>(status)[threadIdx.x] = 0;
     const int lane = threadIdx.x & (kLanesPerUnit - 1);
     const int64_t units = T * h;
@@ -358,10 +367,11 @@ hydra_bwd_prep_kernel(const uint4* __restrict__ dout, const uint4* __restrict__ 
 // The same with 32 bytes per lane (8 lanes per (row, head), 256-bit loads), for 32-byte aligned buffers.
 __global__ void __launch_bounds__(kThreads)
 hydra_bwd_prep_wide_kernel(const V8* __restrict__ dout, const V8* __restrict__ out, float* __restrict__ dsum,
-                           int64_t T, int32_t h, StatusBlock* status)
+                           int64_t T, int32_t h, StatusBlock* status, uint4* zero, int64_t zero16)
 {
     overlap_next_launch();
     wait_for_previous_launch();
+    clear16(zero, zero16);
     if (blockIdx.x == 0 && threadIdx.x < sizeof(StatusBlock) / 4) reinterpret_cast<int32_t*>(status)[threadIdx.x] = 0;
     constexpr int kLanes = 8, kUnits = kThreads / kLanes, kVecPerRow = D_V / 16;
     const int lane = threadIdx.x & (kLanes - 1);
@@ -410,6 +420,17 @@ hydra_grad_cast_kernel(const float4* acc, uint4* grad, int64_t n8, int64_t n, co
 
 // Sixteen elements per thread (two 32-byte loads, one 32-byte store), for 32-byte aligned buffers; the
 // elements past the last multiple of sixteen go one per thread.
+__device__ __forceinline__ void cast16(const V8* acc, V8* grad)
+{
+    const V8 a = ld_stream32(acc), b = ld_stream32(acc + 1);
+    uint32_t w[8];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        w[e] = pack_bf16x2(__uint_as_float(a.w[2 * e]), __uint_as_float(a.w[2 * e + 1]));
+        w[4 + e] = pack_bf16x2(__uint_as_float(b.w[2 * e]), __uint_as_float(b.w[2 * e + 1]));
+    }
+    st_global_v8(grad, w);
+}
 __global__ void __launch_bounds__(kThreads)
 hydra_grad_cast_wide_kernel(const V8* acc, V8* grad, int64_t n16, int64_t n, const float* acc_tail,
                             __nv_bfloat16* grad_tail)
@@ -418,19 +439,45 @@ hydra_grad_cast_wide_kernel(const V8* acc, V8* grad, int64_t n16, int64_t n, con
     wait_for_previous_launch();
     const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; i < n16; i += stride) {
-        const V8 a = ld_stream32(acc + 2 * i), b = ld_stream32(acc + 2 * i + 1);
-        uint32_t w[8];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            w[e] = pack_bf16x2(__uint_as_float(a.w[2 * e]), __uint_as_float(a.w[2 * e + 1]));
-            w[4 + e] = pack_bf16x2(__uint_as_float(b.w[2 * e]), __uint_as_float(b.w[2 * e + 1]));
-        }
-        st_global_v8(grad + i, w);
+        cast16(acc + 2 * i, grad + i);
     }
     if (blockIdx.x == 0) {
         const int64_t t = n16 * 16 + threadIdx.x;
         if (t < n) grad_tail[t] = __float2bfloat16_rn(acc_tail[t]);
     }
+}
+
+// The same for two gradients (dk and dv) whose sizes are multiples of sixteen elements: one launch less at the end of a call.
+__global__ void __launch_bounds__(kThreads)
+hydra_grad_cast2_wide_kernel(const V8* acc_a, V8* grad_a, int64_t n16_a, const V8* acc_b, V8* grad_b, int64_t n16_b)
+{
+    overlap_next_launch();
+    wait_for_previous_launch();
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; i < n16_a + n16_b; i += stride) {
+        if (i < n16_a) cast16(acc_a + 2 * i, grad_a + i);
+        else cast16(acc_b + 2 * (i - n16_a), grad_b + (i - n16_a));
+    }
+}
+
+cudaError_t launch_grad_cast2(const float* acc_a, void* grad_a, int64_t n_a, const float* acc_b, void* grad_b, int64_t n_b,
+                              int* launches, cudaStream_t stream)
+{
+    const uintptr_t all = reinterpret_cast<uintptr_t>(acc_a) | reinterpret_cast<uintptr_t>(grad_a) |
+                          reinterpret_cast<uintptr_t>(acc_b) | reinterpret_cast<uintptr_t>(grad_b);
+    if ((all & 31u) != 0 || ((n_a | n_b) & 15) != 0) {
+        *launches = 2;
+        if (cudaError_t e = launch_grad_cast(acc_a, grad_a, n_a, stream)) return e;
+        return launch_grad_cast(acc_b, grad_b, n_b, stream);
+    }
+    const int64_t n16 = (n_a + n_b) / 16;
+    if (n16 <= 0) return cudaSuccess;
+    *launches = 1;
+    const int64_t blocks = (n16 + kThreads - 1) / kThreads;
+    const int grid = static_cast<int>(blocks < 148 * 16 ? blocks : 148 * 16);
+    return launch_overlapped_spread<hydra_grad_cast2_wide_kernel>(grid, kThreads, stream, reinterpret_cast<const V8*>(acc_a),
+                                                                  static_cast<V8*>(grad_a), n_a / 16, reinterpret_cast<const V8*>(acc_b),
+                                                                  static_cast<V8*>(grad_b), n_b / 16);
 }
 
 cudaError_t launch_grad_cast(const float* acc, void* grad, int64_t n, cudaStream_t stream)
@@ -580,8 +627,10 @@ cudaError_t launch_reset(StatusBlock* status, bool keep_status, cudaStream_t str
 }
 
 cudaError_t launch_bwd_prep(const void* dout, const void* out, float* dsum, int64_t T, int32_t h, StatusBlock* status,
-                            cudaStream_t stream)
+                            void* zero, size_t zero_bytes, cudaStream_t stream)
 {
+    uint4* const z = static_cast<uint4*>(zero);
+    const int64_t z16 = static_cast<int64_t>(zero_bytes / 16);
     if (T * h == 0) return cudaSuccess;
     const int64_t passes = (T * h + kUnitsPerPass - 1) / kUnitsPerPass;
     const int grid = static_cast<int>(passes < 148 * 16 ? passes : 148 * 16);
@@ -589,10 +638,10 @@ cudaError_t launch_bwd_prep(const void* dout, const void* out, float* dsum, int6
         const int64_t wide_passes = (T * h + 2 * kUnitsPerPass - 1) / (2 * kUnitsPerPass);
         const int wide_grid = static_cast<int>(wide_passes < 148 * 16 ? wide_passes : 148 * 16);
         return launch_overlapped_spread<hydra_bwd_prep_wide_kernel>(wide_grid, kThreads, stream, static_cast<const V8*>(dout),
-                                 static_cast<const V8*>(out), dsum, T, h, status);
+                                 static_cast<const V8*>(out), dsum, T, h, status, z, z16);
     }
     return launch_overlapped_spread<hydra_bwd_prep_kernel>(grid, kThreads, stream, static_cast<const uint4*>(dout),
-                             static_cast<const uint4*>(out), dsum, T, h, status);
+                             static_cast<const uint4*>(out), dsum, T, h, status, z, z16);
 }
 
 }  // namespace hydra

@@ -206,29 +206,39 @@ enum : int { B_KVFULL = 0, B_KVEMPTY = 1, B_QFULL = 2, B_STAT = 5, B_QEMPTY = 8,
              B_VFULL = 18, B_ITEMFULL = 19, B_ITEMEMPTY = 19 + kSched, B_COUNT = 19 + 2 * kSched };
 static_assert(kDqk * TILE * 4u <= kDsStage, "the other CTA's part of dK fits the operand space");
 
-// Iterator over (pair of the kv chunk, 64-row q sub-tile).
+// Iterator over (query head of the item, pair of the kv chunk, 64-row q sub-tile). kHeads: items take BwdParams::item_heads
+// query heads, otherwise one (a build of its own: the loop over the heads in the one kernel cost batches of short sequences
+// with a K / V head per query head 4 %).
+template <bool kHeads>
 struct SubIter {
     const PairDev* pairs; const int32_t* list; int list_len; int r0; int causal; int even;
-    int li, u, nu; PairDev cur;
+    int li, u, nu; int head, heads; PairDev cur;             // heads: how many are left, the current one included
     __device__ void seek() {
-        while (li < list_len) {
-            if (li > 0) cur = pairs[list[li]];
-            nu = (cur.q_len + SUB - 1) / SUB;
-            u = 0;
-            if (causal) { const int i_min = r0 - cur.off; u = i_min > 0 ? i_min / SUB : 0; }
-            // with the dS hand-off a q tile is read as two sub-tiles: start at the even one (the extra
-            // sub-tile, if any, is fully masked and contributes zeros)
-            if (even) u &= ~1;
-            if (u < nu) return;
-            ++li;
+        for (;;) {
+            while (li < list_len) {
+                if (li > 0) cur = pairs[list[li]];
+                nu = (cur.q_len + SUB - 1) / SUB;
+                u = 0;
+                if (causal) { const int i_min = r0 - cur.off; u = i_min > 0 ? i_min / SUB : 0; }
+                // with the dS hand-off a q tile is read as two sub-tiles: start at the even one (the extra
+                // sub-tile, if any, is fully masked and contributes zeros)
+                if (even) u &= ~1;
+                if (u < nu) return;
+                ++li;
+            }
+            if (!kHeads || --heads <= 0) return;
+            ++head;
+            li = 0;
+            if (list_len > 1) cur = pairs[list[0]];
         }
     }
-    __device__ void init(const PairDev* p, const int32_t* l, int n, int r, int c, int ev, const PairDev& first) {
-        pairs = p; list = l; list_len = n; r0 = r; causal = c; even = ev; li = 0; u = 0; nu = 0; cur = first;
+    __device__ void init(const BwdParams& p, const GroupItem& item, const PairDev& first) {
+        pairs = p.pairs; list = p.lists + item.list_off; list_len = item.list_len; r0 = item.r0; causal = p.causal;
+        even = p.ds != nullptr; li = 0; u = 0; nu = 0; head = item.head; heads = kHeads ? p.item_heads : 1; cur = first;
         seek();
     }
     __device__ bool valid() const { return li < list_len; }
-    __device__ bool ends_within(int n) const { return li == list_len - 1 && u + n >= nu; }
+    __device__ bool ends_within(int n) const { return (!kHeads || heads == 1) && li == list_len - 1 && u + n >= nu; }
     __device__ void next() { if (++u >= nu) { ++li; seek(); } }
 };
 }  // namespace dkv
@@ -643,13 +653,14 @@ HYDRA_K(hydra_bwd_dq_kernel)(const __grid_constant__ CUtensorMap map_q, const __
 // kHalves: the two CTAs of a cluster share one kv tile, each visiting every other of its q sub-tiles; at the end CTA 0 gets
 // the other's dK through distributed shared memory and writes the tile's dK, CTA 1 its dV. For calls with no more than
 // half as many kv tiles as SMs, which take as long as their longest tile.
-template <bool kHalves>
+template <bool kHalves, bool kHeads>
 __global__ void __launch_bounds__(kThreads, 1)
 HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                      const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do,
                      const BwdParams p)
 {
     using namespace dkv;
+    using SubIter = dkv::SubIter<kHeads>;
     overlap_next_launch();
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -763,7 +774,7 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                 // lane 0 wrote this item's descriptors into the ring when it popped it (before the barrier above)
                 item = s_item[(kq - 1) % kSched];
                 first = s_first[(kq - 1) % kSched];
-                si.init(p.pairs, p.lists + item.list_off, item.list_len, item.r0, p.causal, p.ds != nullptr, first);
+                si.init(p, item, first);
                 sub_begin(si);
             }
             int raw_next = 0;
@@ -783,10 +794,10 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                         mbar_arrive_expect_tx(bar(B_QFULL + st), (kQkBoxes + 2) * kBox64);
                         for (int c = 0; c < kQkBoxes; ++c)
                             tma_load_3d(smem + kQ + st * kQkBoxes * kBox64 + c * kBox64, &map_q, bar(B_QFULL + st), c * 64,
-                                        item.head, tok);
+                                        si.head, tok);
                         for (int c = 0; c < 2; ++c)
                             tma_load_3d(smem + kDO + st * 2 * kBox64 + c * kBox64, &map_do, bar(B_QFULL + st), c * 64,
-                                        item.head, tok);
+                                        si.head, tok);
                     }
                     // The item's K and V come after its first Q and dO, which find a free stage while the item before still
                     // reads its K and V (80 KB that take some 3000 cycles to arrive then: between items this is what the
@@ -814,7 +825,7 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                         const int c = lane + 32 * e;
                         const int i = si.u * SUB + c;
                         const bool v = i < si.cur.q_len;
-                        const int64_t idx = static_cast<int64_t>(item.head) * p.T + si.cur.q_tok0 + i;
+                        const int64_t idx = static_cast<int64_t>(si.head) * p.T + si.cur.q_tok0 + i;
                         const float l = v ? __ldg(p.lse + idx) : neg_inf();
                         s_lse2[st][c] = (l == neg_inf()) ? neg_inf() : -(l * kLog2e);
                         s_dsum[st][c] = v ? -__ldg(p.dsum + idx) : 0.f;
@@ -856,9 +867,8 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                 PairDev first;
                 const int it = next_item(kq, item, first);
                 if (it < 0) break;
-                const int32_t* list = p.lists + item.list_off;
                 SubIter si;
-                si.init(p.pairs, list, item.list_len, item.r0, p.causal, p.ds != nullptr, first);
+                si.init(p, item, first);
                 sub_begin(si);
                 if (!si.valid()) continue;
                 if (issue_scores) {
@@ -964,7 +974,7 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
         const uint32_t tm_p = tm + kTmP + lane_base + g * 16;
         const uint32_t tm_ds = tm + kTmDS + lane_base + g * 16;
         uint32_t c_s = 0, c_pds = 0, gq = 0;
-        int ds_li = -1;                                // pair whose first hand-off block is in ds_blk0
+        int ds_li = -1, ds_head = 0;                   // pair and head whose first hand-off block is in ds_blk0
         int64_t ds_blk0 = 0;
         bool ok = true;
         for (uint32_t kq = 0; ok; ++kq) {
@@ -972,12 +982,11 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
             PairDev first;
             const int it = next_item(kq, item, first);
             if (it < 0) break;
-            const int32_t* list = p.lists + item.list_off;
             ds_li = -1;
             const int krow = item.r0 + r;              // kv row inside the chunk
             const bool row_valid = krow < first.k_len;
             const int64_t tok = static_cast<int64_t>(first.k_tok0) + krow;
-            // with shared KV heads (accumulating form only) the query heads of a group add into one dk / dv row
+            // with shared KV heads an item takes all query heads of a group, or several items add into one dk / dv row
             const int64_t kv_heads = p.h / p.kv_group;
             const int64_t kv_row = tok * kv_heads + item.head / p.kv_group;
             const int64_t dk_off = kv_row * kDqk + g * (kDqk / 2);
@@ -987,7 +996,7 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
             float* dkp_acc = static_cast<float*>(p.dk) + dk_off;         // accumulate mode: dk, dv are fp32
             float* dvp_acc = static_cast<float*>(p.dv) + dv_off;
             SubIter si;
-            si.init(p.pairs, list, item.list_len, item.r0, p.causal, p.ds != nullptr, first);
+            si.init(p, item, first);
             bool joint = false;                        // the other CTA of the cluster has sub-tiles of this tile too
             if (kHalves) {
                 SubIter second = si;
@@ -1067,11 +1076,12 @@ HYDRA_K(hydra_bwd_dkv_kernel)(const __grid_constant__ CUtensorMap map_q, const _
                 if (p.ds) {
                     // Hand dS^T to the query-side kernel (after P and dS have gone to the tensor core: off the
                     // chain S -> P, dS -> dV, dK).
-                    if (si.li != ds_li) {
+                    if (si.li != ds_li || (kHeads && si.head != ds_head)) {
                         ds_li = si.li;
+                        ds_head = si.head;
                         const DsGeom geo = ds_geom(si.cur.q_len, si.cur.off, p.causal);
                         const int jk = item.r0 / TILE;
-                        ds_blk0 = static_cast<int64_t>(item.head) * p.ds_head_blocks + si.cur.ds_base +
+                        ds_blk0 = static_cast<int64_t>(si.head) * p.ds_head_blocks + si.cur.ds_base +
                                   ds_rowstart(geo, jk) - ds_first(geo, jk);
                     }
                     // The block in memory is 8 chunks (8 q rows each) of 128 kv rows x 16 bytes: lane = kv row,
@@ -1514,9 +1524,12 @@ cudaError_t HYDRA_K(launch_bwd_dq)(const CUtensorMap& mq, const CUtensorMap& mk,
 cudaError_t HYDRA_K(launch_bwd_dkv)(const CUtensorMap& mq_sub, const CUtensorMap& mk, const CUtensorMap& mv,
                            const CUtensorMap& mdo_sub, const BwdParams& p, bool halves, int grid, cudaStream_t stream)
 {
-    static OncePerDevice configured[2];
-    const auto kernel = halves ? HYDRA_K(hydra_bwd_dkv_kernel)<true> : HYDRA_K(hydra_bwd_dkv_kernel)<false>;
-    if (cudaError_t e = allow_dynamic_smem(kernel, HYDRA_K(bwd_dkv_smem_bytes)(), configured[halves])) return e;
+    static OncePerDevice configured[3];
+    const bool heads = p.item_heads > 1;
+    if (halves && heads) return cudaErrorInvalidValue;     // (not planned: such calls have SMs to spare)
+    const auto kernel = halves ? HYDRA_K(hydra_bwd_dkv_kernel)<true, false>
+                               : (heads ? HYDRA_K(hydra_bwd_dkv_kernel)<false, true> : HYDRA_K(hydra_bwd_dkv_kernel)<false, false>);
+    if (cudaError_t e = allow_dynamic_smem(kernel, HYDRA_K(bwd_dkv_smem_bytes)(), configured[halves ? 1 : (heads ? 2 : 0)])) return e;
     return launch_overlapped_clusters(kernel, halves ? 2 : 1, grid, kThreads, HYDRA_K(bwd_dkv_smem_bytes)(), stream, mq_sub, mk, mv,
                                       mdo_sub, p);
 }

@@ -86,7 +86,8 @@ struct alignas(16) FwdShortItem {
 };
 static_assert(sizeof(FwdShortItem) == 32, "two 16-byte loads per work item");
 
-// Backward work item: one tile of one chunk and head, visiting every pair that shares the chunk.
+// Backward work item: one tile of one chunk and head, visiting every pair that shares the chunk (key side: for
+// BwdParams::item_heads query heads, of which `head` is the first).
 struct GroupItem {
     int32_t list_off;  // first entry of the chunk's pair list
     int32_t list_len;
@@ -250,6 +251,7 @@ struct BwdParams {
     int64_t T;
     int32_t h; int32_t causal;
     int32_t kv_group;           // query heads per KV head; k, v, dk, dv have h / kv_group heads
+    int32_t item_heads;         // key-side kernel: consecutive query heads (of one KV head) that an item visits
     float scale; float scale_log2;
     int32_t accumulate;
     void* ds;                   // dS hand-off buffer, or null: the query-side kernel recomputes S and dP
@@ -299,6 +301,9 @@ cudaError_t launch_merge(const MergeParams& p, cudaStream_t stream);
 // launch_merge plus the library's launch counter and per-kernel timer (defined beside them, in api.cu)
 cudaError_t launch_merge_counted(const MergeParams& p, cudaStream_t stream);
 cudaError_t launch_grad_cast(const float* acc, void* grad, int64_t n, cudaStream_t stream);
+// two gradients, in one launch where sizes and alignment allow it
+cudaError_t launch_grad_cast2(const float* acc_a, void* grad_a, int64_t n_a, const float* acc_b, void* grad_b, int64_t n_b,
+                              int* launches, cudaStream_t stream);
 cudaError_t launch_ulysses(bool pack, const void* src, void* dst, int64_t n_tokens, int32_t cp_u, int64_t chunk_units,
                            cudaStream_t stream);
 // the elementwise steps of a gated MLA block around the attention kernel (mla_ops.cu)
@@ -316,8 +321,8 @@ cudaError_t launch_gate_bwd(const void* dy, const void* out, const void* gate, v
                             cudaStream_t stream);
 // clears the status block (of which keep_status leaves all but the work-queue heads)
 cudaError_t launch_reset(StatusBlock* status, bool keep_status, cudaStream_t stream);
-// D = rowsum(dO * O); also clears the status block
+// D = rowsum(dO * O); also clears the status block and `zero_bytes` (a multiple of 16) at `zero`
 cudaError_t launch_bwd_prep(const void* dout, const void* out, float* dsum, int64_t T, int32_t h, StatusBlock* status,
-                            cudaStream_t stream);
+                            void* zero, size_t zero_bytes, cudaStream_t stream);
 
 }  // namespace hydra
