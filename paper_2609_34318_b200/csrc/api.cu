@@ -622,14 +622,19 @@ void order_items(std::vector<Item>& items, const std::vector<int32_t>& block_of,
     items.swap(sorted);
 }
 
-// The items of a plan come in groups (a pair, or a chunk) that repeat for every head with the same costs, so
-// the block order above (blocks = (group, head), longest block first, the items of a block longest first)
+// The items of a plan come in groups (a sequence: all of its pairs or chunks) that repeat for every head with the same costs,
+// so the block order above (blocks = (group, head), longest block first, the items of a block longest first)
 // needs only the GROUPS sorted, and the list is then written out in one pass. That matters because a
 // training loop meets new cu_seqlens with every micro-batch: sorting the 22 000 items of the many-short
 // workload took milliseconds on the host, as long as the kernels they feed. List scheduling ends within one
 // longest item of the even share, so when the longest item is under 5 % of that share the block order needs
 // no check; only otherwise (few, long, equal sequences: few items) is the queue simulated as above.
-struct GroupEntry { int32_t a, b, c, cost; };
+// A group is a whole sequence because its pairs share Q, K, V and dO, which items that run at the same time find in L2. With
+// a group per pair or chunk, which run far apart, sequences of 64 to 512 tokens cut in two (32768 tokens, 32 heads) read 1.67
+// GB in the forward, 2.08 on the key side and 1.58 on the query side, as whole sequences 1.19, 1.52 and 1.29 (step of 65536
+// tokens 3391 -> 3213 us). 32768 log-normal tokens, 16 heads, ring of 4, 3140 -> 2975 us; five sequences of 13107, 8 heads,
+// ring of 4, 8912 -> 8640; one of 65536 39444 -> 38900; heads of 128, 31598 tokens, 32 heads, ring of 2, 4207 -> 4030.
+struct GroupEntry { int32_t a, b, c, cost, of; };        // of: the pair or chunk
 // The groups longest first (their entries longest first inside), the number of items, and whether the block
 // order needs no check against the queue simulation.
 struct GroupOrder { std::vector<int32_t> order; int64_t n_items = 0; bool settled = true; };
@@ -668,7 +673,7 @@ std::vector<Item> order_by_groups(std::vector<std::vector<GroupEntry>>& groups, 
     for (int32_t g : go.order)
         for (int32_t a = 0; a < h; ++a)
             for (const GroupEntry& e : groups[g]) {
-                items.push_back(make(g, a, e));
+                items.push_back(make(a, e));
                 if (!go.settled) {
                     block_of.push_back(g * h + a);
                     cost.push_back(e.cost);
@@ -739,14 +744,15 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     }
     int32_t longest_tile = 0;
     int64_t short_cost = 0;
-    std::vector<std::vector<GroupEntry>> groups(pb.pairs.size()), groups_short(pb.pairs.size());
+    std::vector<std::vector<GroupEntry>> groups(pb.n_seqs), groups_short(pb.n_seqs);
     for (size_t pi = 0; pi < pb.pairs.size(); ++pi) {
         const auto& p = pb.pairs[pi];
+        const int32_t of = static_cast<int32_t>(pi);
         if (is_short[pi]) {
             for (int32_t q0 = 0; q0 < p.q_len; q0 += TILE) {
                 const int32_t rows = std::min(TILE, p.q_len - q0);
                 const int32_t n_kv = kv_steps_short(p, q0, rows, causal);
-                groups_short[pi].push_back(GroupEntry{q0, n_kv, rows, n_kv});
+                groups_short[p.seq].push_back(GroupEntry{q0, n_kv, rows, n_kv, of});
                 longest_tile = std::max(longest_tile, n_kv);
                 short_cost += n_kv + kItemOverhead;
             }
@@ -768,7 +774,7 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
             // of an item goes with the longer tile, not with the sum: a slab whose second tile is empty costs
             // as much per kv tile as a full one (measured: with the sum the slowest cluster of the 32K packed
             // workload ended 17 % after the mean, now 4 %)
-            groups[pi].push_back(GroupEntry{qa, n_a, n_b, 2 * std::max(n_a, std::max(n_b, 0))});
+            groups[p.seq].push_back(GroupEntry{qa, n_a, n_b, 2 * std::max(n_a, std::max(n_b, 0)), of});
         }
     }
     // How far ahead the short kernel's slots pop: items of up to 8 steps two ahead, longer ones late, so that no slot sits on
@@ -786,7 +792,7 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     plan.early_pops = early ? kMidTile : kShortItem;
     const std::vector<FwdItem> items = order_by_groups<FwdItem>(
         groups, pb.h, plan_workers(2),
-        [](int32_t g, int32_t a, const GroupEntry& e) { return FwdItem{g, a, e.a, e.b, e.c, {0, 0, 0}}; });
+        [](int32_t a, const GroupEntry& e) { return FwdItem{e.of, a, e.a, e.b, e.c, {0, 0, 0}}; });
     const std::vector<PairDev> dev_pairs = device_pairs(pb);
     plan.off_pairs = append(blob, dev_pairs);
     plan.off_items = append(blob, items);
@@ -795,8 +801,8 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     // micro-batch of short sequences has tens of thousands of them and a new one arrives with every step, so in
     // the common case (many items, none long: the block order is final) they are written straight into the
     // table, a group's entries once and then one copy per head with the head number set.
-    auto make_short = [&](int32_t g, int32_t a, const GroupEntry& e) {
-        const PairDev& d = dev_pairs[g];
+    auto make_short = [&](int32_t a, const GroupEntry& e) {
+        const PairDev& d = dev_pairs[e.of];
         FwdShortItem it{};
         it.q_tok0 = d.q_tok0 + e.a;
         it.k_tok0 = d.k_tok0;
@@ -816,7 +822,7 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
         for (size_t g = 0; g < groups_short.size(); ++g)
             for (int32_t a = 0; a < pb.h; ++a)
                 for (const GroupEntry& e : groups_short[g]) {
-                    FwdShortItem it = make_short(static_cast<int32_t>(g), a, e), rest = it;
+                    FwdShortItem it = make_short(a, e), rest = it;
                     const int32_t n0 = (e.b + 1) / 2;
                     rest.n_kv = static_cast<uint16_t>(e.b - n0);
                     if (rest.n_kv > 0) {
@@ -847,7 +853,7 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
         std::vector<FwdShortItem> block;
         for (int32_t g : go.order) {
             block.clear();
-            for (const GroupEntry& e : groups_short[g]) block.push_back(make_short(g, 0, e));
+            for (const GroupEntry& e : groups_short[g]) block.push_back(make_short(0, e));
             for (int32_t a = 0; a < pb.h; ++a) {
                 std::memcpy(dst, block.data(), block.size() * sizeof(FwdShortItem));
                 for (size_t i = 0; i < block.size(); ++i) dst[i].head = static_cast<uint16_t>(a);
@@ -1005,8 +1011,8 @@ void build_bwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
         };
         std::stable_sort(order.begin(), order.end(),
                          [&](int32_t a, int32_t b) { return range_less(key(a), key(b)); });
-        std::vector<std::vector<GroupEntry>> groups;       // one per chunk that has work
-        std::vector<std::pair<int32_t, int32_t>> list_of;  // its (list_off, list_len)
+        std::vector<std::vector<GroupEntry>> groups(pb.n_seqs);
+        std::vector<std::pair<int32_t, int32_t>> list_of;  // (list_off, list_len) of every chunk that has work
         int32_t i = 0;
         while (i < n) {
             int32_t j = i;
@@ -1024,7 +1030,7 @@ void build_bwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
             }
             const int32_t list_len = static_cast<int32_t>(lists.size()) - list_off;
             if (r.len > 0 && list_len > 0) {
-                groups.emplace_back();
+                const int32_t of = static_cast<int32_t>(list_of.size());
                 list_of.emplace_back(list_off, list_len);
                 for (int32_t r0 = 0; r0 < r.len; r0 += TILE) {
                     int32_t c = 0;
@@ -1032,7 +1038,7 @@ void build_bwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
                         const auto& p = pb.pairs[lists[list_off + t]];
                         c += by_q ? kv_tiles(p, r0, causal) : q_subs(p, r0, causal);
                     }
-                    groups.back().push_back(GroupEntry{r0, 0, 0, c});
+                    groups[r.seq].push_back(GroupEntry{r0, 0, 0, c, of});
                 }
             }
             i = j;
@@ -1041,8 +1047,8 @@ void build_bwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
         if (!by_q) plan.item_heads = heads;
         for (auto& g : groups)
             for (GroupEntry& e : g) e.cost *= heads;
-        items = order_by_groups<GroupItem>(groups, pb.h / heads, plan_workers(1), [&](int32_t g, int32_t a, const GroupEntry& e) {
-            return GroupItem{list_of[g].first, list_of[g].second, a * heads, e.a};
+        items = order_by_groups<GroupItem>(groups, pb.h / heads, plan_workers(1), [&](int32_t a, const GroupEntry& e) {
+            return GroupItem{list_of[e.of].first, list_of[e.of].second, a * heads, e.a};
         });
     };
     std::vector<int32_t> lists_q, lists_k;
