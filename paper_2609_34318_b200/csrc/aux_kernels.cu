@@ -79,7 +79,8 @@ hydra_lse_merge_kernel(const MergeParams p)
 {
     overlap_next_launch();
     wait_for_previous_launch();
-    const MergeItem item = p.items[blockIdx.x];
+    const int share = static_cast<int>(blockIdx.x) % p.split;      // of the item's units
+    const MergeItem item = p.items[static_cast<int>(blockIdx.x) / p.split];
     const MergeGroup g = p.groups[item.group];
     const int32_t* part_row = p.lists + g.list_off;
     const int rows = min(MERGE_ROWS, g.rows - item.row0);
@@ -94,9 +95,10 @@ hydra_lse_merge_kernel(const MergeParams p)
     // out alike, so their addresses advance by a constant; only the LSE addresses ([h, rows] layouts) need r and
     // a, which advance without a division. The offsets of the first batch of partials do not depend on the
     // unit at all and are formed once per block.
-    int u = threadIdx.x / kLanesPerUnit;
+    const int step = kUnitsPerPass * p.split;
+    int u = share * kUnitsPerPass + threadIdx.x / kLanesPerUnit;
     int r = u / p.h, a = u - r * p.h;
-    const int step_r = kUnitsPerPass / p.h, step_a = kUnitsPerPass - step_r * p.h;
+    const int step_r = step / p.h, step_a = step - step_r * p.h;
     const int64_t part_stride = static_cast<int64_t>(p.h) * kVecPerRow;         // uint4 per partial row
     const uint4* o_row = o_part + (static_cast<int64_t>(item.row0) * p.h + u) * kVecPerRow + lane;
     uint4* out_v = out + ((static_cast<int64_t>(g.out_tok0) + item.row0) * p.h + u) * kVecPerRow + lane;
@@ -108,7 +110,7 @@ hydra_lse_merge_kernel(const MergeParams p)
         off0[i] = pr0[i] * part_stride;
     }
 
-    for (; u < n_units; u += kUnitsPerPass, o_row += kUnitsPerPass * kVecPerRow, out_v += kUnitsPerPass * kVecPerRow) {
+    for (; u < n_units; u += step, o_row += step * kVecPerRow, out_v += step * kVecPerRow) {
         const int row = item.row0 + r;
         const float* lse_row = p.lse_part + static_cast<int64_t>(a) * p.part_rows + row;
         float* lse_out = p.lse + static_cast<int64_t>(a) * p.T + g.out_tok0 + row;
@@ -211,7 +213,8 @@ hydra_lse_merge_wide_kernel(const MergeParams p)
     overlap_next_launch();
     wait_for_previous_launch();
     constexpr int kLanes = 8, kUnits = kThreads / kLanes;
-    const MergeItem item = p.items[blockIdx.x];
+    const int share = static_cast<int>(blockIdx.x) % p.split;      // of the item's units
+    const MergeItem item = p.items[static_cast<int>(blockIdx.x) / p.split];
     const MergeGroup g = p.groups[item.group];
     const int32_t* part_row = p.lists + g.list_off;
     const int rows = min(MERGE_ROWS, g.rows - item.row0);
@@ -221,9 +224,10 @@ hydra_lse_merge_wide_kernel(const MergeParams p)
     constexpr int kVecPerRow = D_V / 16;          // 32-byte vectors per (row, head)
     constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
     const int n_units = rows * p.h;
-    int u = threadIdx.x / kLanes;
+    const int step = kUnits * p.split;
+    int u = share * kUnits + threadIdx.x / kLanes;
     int r = u / p.h, a = u - r * p.h;
-    const int step_r = kUnits / p.h, step_a = kUnits - step_r * p.h;
+    const int step_r = step / p.h, step_a = step - step_r * p.h;
     const int64_t part_stride = static_cast<int64_t>(p.h) * kVecPerRow;
     const V8* o_row = o_part + (static_cast<int64_t>(item.row0) * p.h + u) * kVecPerRow + lane;
     V8* out_v = out + ((static_cast<int64_t>(g.out_tok0) + item.row0) * p.h + u) * kVecPerRow + lane;
@@ -234,7 +238,7 @@ hydra_lse_merge_wide_kernel(const MergeParams p)
         pr0[i] = part_row[i < g.n_parts ? i : 0];
         off0[i] = pr0[i] * part_stride;
     }
-    for (; u < n_units; u += kUnits, o_row += kUnits * kVecPerRow, out_v += kUnits * kVecPerRow) {
+    for (; u < n_units; u += step, o_row += step * kVecPerRow, out_v += step * kVecPerRow) {
         const int row = item.row0 + r;
         const float* lse_row = p.lse_part + static_cast<int64_t>(a) * p.part_rows + row;
         float* lse_out = p.lse + static_cast<int64_t>(a) * p.T + g.out_tok0 + row;
@@ -597,11 +601,18 @@ cudaError_t launch_merge(const MergeParams& p, cudaStream_t stream)
     // Not launched ahead of the forward's end, unlike the other kernels of a call (the kernel behind it does start early): 432
     // chunk pairs of about 200 tokens, 4 heads 131 -> 127.5 us with their forward, 72 pairs, 16 heads 49.4 -> 47.3, one
     // rank's ring step of 64K tokens 5.54 -> 5.44 ms, 65536 tokens of short sequences cut in two 3.05 -> 3.015.
+    const bool wide = ((reinterpret_cast<uintptr_t>(p.o_part) | reinterpret_cast<uintptr_t>(p.out)) & 31u) == 0;
+    // An item (eight rows, all heads) is several passes of its block, each a round trip to memory behind the other: with
+    // fewer items than resident blocks as many blocks share one as fit at once. With its launch, one block per item / shared:
+    // 363 tokens, 16 heads, ring of 4 14.6 / 8.6 us, 1728 tokens, 32 heads, ring of 2 19.3 / 14.9, 1313 16.0 / 12.8.
+    constexpr int kResident = 148 * 4;
+    const int passes = (MERGE_ROWS * p.h + (wide ? 2 : 1) * kUnitsPerPass - 1) / ((wide ? 2 : 1) * kUnitsPerPass);
+    MergeParams shared = p;
+    shared.split = std::max(1, std::min(passes, kResident / p.n_items));
     auto launch = [&](auto kernel) {
-        kernel<<<p.n_items, kThreads, 0, stream>>>(p);
+        kernel<<<p.n_items * shared.split, kThreads, 0, stream>>>(shared);
         return cudaGetLastError();
     };
-    const bool wide = ((reinterpret_cast<uintptr_t>(p.o_part) | reinterpret_cast<uintptr_t>(p.out)) & 31u) == 0;
     if (wide) {
         if (p.accumulate) {
             if (four) return launch(hydra_lse_merge_wide_kernel<true, 4>);

@@ -272,6 +272,7 @@ struct MergeParams {
     int32_t h;
     int32_t accumulate;         // 1: the current (out, lse) rows are one more input of their merge
     int32_t max_parts;          // most partials any chunk has (chooses how many are requested together)
+    int32_t split;              // thread blocks that share an item (set by launch_merge)
 };
 
 // The tensor-core kernels exist once per supported q / k head dimension (the kernel files are compiled
