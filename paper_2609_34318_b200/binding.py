@@ -226,9 +226,16 @@ def _cu(cu_seqlens) -> np.ndarray:
     return np.ascontiguousarray(np.asarray(cu_seqlens, dtype=np.int32))
 
 
+_char_at = ctypes.c_char.from_buffer
+
+
 def _addr(array: np.ndarray) -> int:
-    """Address of an array's data (array.ctypes.data makes a ctypes object on the way: three times as long)."""
-    return array.__array_interface__["data"][0]
+    """Address of an array's data. __array_interface__ describes the whole type on the way: 1 us for a plain array, 6.5 us
+    for one of pairs; the buffer protocol takes 0.3 and 0.9 but wants a writable, non-empty array."""
+    try:
+        return ctypes.addressof(_char_at(array))
+    except (TypeError, ValueError):
+        return array.ctypes.data
 
 
 def as_pairs(pairs) -> Optional[np.ndarray]:
