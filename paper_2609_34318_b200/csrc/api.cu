@@ -1693,8 +1693,21 @@ int32_t fwd_core(Problem& pb, const void* q, const void* k, const void* v, int32
     if (int32_t s = lease.acquire(HYDRA_WS_FWD, pb, causal != 0, stream)) return s;
     const Plan* plan = &lease.plan();
     if (plan->n_items == 0 && plan->n_items2 == 0) return HYDRA_OK;
-    if (launch_reset(static_cast<StatusBlock*>(workspace), false, stream) != cudaSuccess) return HYDRA_ERR_CUDA;
+    // One item per SM before any SM gets two, or both halves of a tile on one SM.
+    const int short_grid = plan->halves ? plan->n_items2 / 2 : std::min(sms, plan->n_items2);
     FwdParams fp{};
+    // With no more items than slots nothing is popped from the queue, and the block at the workspace's start need not be
+    // cleared (one launch less: four sequences of 7 to 300 tokens, forward 11.5 -> 9.4 us). Not where the launches are
+    // recorded: every replay would have the number of the first.
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) return HYDRA_ERR_CUDA;
+    if (capturing == cudaStreamCaptureStatusNone && plan->n_items == 0 && plan->n_items2 <= 2 * short_grid) {
+        static std::atomic<uint32_t> calls{0};
+        do fp.call_tag = static_cast<int32_t>(calls.fetch_add(1) + 1u);
+        while (fp.call_tag == 0);
+    } else if (launch_reset(static_cast<StatusBlock*>(workspace), false, stream) != cudaSuccess) {
+        return HYDRA_ERR_CUDA;
+    }
     fp.pairs = lease.at<PairDev>(plan->off_pairs);
     fp.items = lease.at<FwdItem>(plan->off_items);
     fp.n_items = plan->n_items;
@@ -1726,10 +1739,8 @@ int32_t fwd_core(Problem& pb, const void* q, const void* k, const void* v, int32
         // short pairs: one CTA per SM with two work items in flight, K and V in boxes of 64 keys
         CUtensorMap mv_sub;
         if (make_map(&mv_sub, v, pb.Tk, n_kv_heads, D_V, FWD_SHORT_KEYS)) return HYDRA_ERR_CUDA;
-        // one item per SM before any SM gets two, or both halves of a tile on one SM
-        const int grid = plan->halves ? plan->n_items2 / 2 : std::min(sms, plan->n_items2);
         ScopedKernelTimer timer(K_FWD, stream);
-        if (ks->launch_fwd_short(mq, mk, mv_sub, fp, plan->halves != 0, grid, stream) != cudaSuccess) return HYDRA_ERR_CUDA;
+        if (ks->launch_fwd_short(mq, mk, mv_sub, fp, plan->halves != 0, short_grid, stream) != cudaSuccess) return HYDRA_ERR_CUDA;
         g_launches += 1;
     }
     lease.release();                                   // the tables have their reader on record
@@ -2618,8 +2629,8 @@ int32_t hydra_poll_status(void* workspace, void* cuda_stream, int32_t* device_st
     if (cudaStreamSynchronize(static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess) return HYDRA_ERR_CUDA;
     StatusBlock sb;
     if (cudaMemcpy(&sb, workspace, sizeof sb, cudaMemcpyDeviceToHost) != cudaSuccess) return HYDRA_ERR_CUDA;
-    *device_status = sb.status;
-    if (detail) *detail = sb.status ? sb.detail : -1;
+    *device_status = sb.call_tag == sb.error_tag ? sb.status : HYDRA_OK;
+    if (detail) *detail = *device_status ? sb.detail : -1;
     return HYDRA_OK;
 }
 

@@ -203,6 +203,8 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
             int raw1 = slot * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x), raw2 = 0;   // pops of the next item and of
             bool have1 = true, have2 = false;          // the one after it, if they have been asked for
             const int first_pop = kSlots * static_cast<int>(gridDim.x);
+            // (with no more items than slots every pop comes back empty, and the counter has not been cleared)
+            auto pop = [&]() -> int { return p.call_tag ? p.n_short : first_pop + atomicAdd(counter, 1); };
             bool pre = false;                          // Q and the first K tile of `cur` have been requested
             // round kq loads item kq - 1 (round 0: none) and hands over item kq on the way
             for (uint32_t kq = 0; ok; ++kq) {
@@ -216,11 +218,11 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
                     // (the pops are used in the order in which they were made: an early one must not be left over
                     // when a later one finds the queue empty)
                     if (!have1 && (n <= early || j >= n - kPopAhead)) {
-                        raw1 = first_pop + atomicAdd(counter, 1);
+                        raw1 = pop();
                         have1 = true;
                     }
                     if (!fetched && have1 && (n <= early || j >= n - 2)) { nxt_idx = fetch(raw1, nxt); fetched = true; }
-                    if (kq > 0 && j == 0 && n <= early) { raw2 = first_pop + atomicAdd(counter, 1); have2 = true; }
+                    if (kq > 0 && j == 0 && n <= early) { raw2 = pop(); have2 = true; }
                     // The next item's Q and first K tile are released by score products that are long issued
                     // when the last V stage comes free: ask for them first, and show the item to the issuer.
                     if (j == (n >= 2 ? n - 1 : n)) {
@@ -238,7 +240,14 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
                 have1 = have2;
                 have2 = false;
             }
-            if (blockIdx.x == 0 && slot == 0) probe.stop(p.status, QUEUE_FWD_SHORT);
+            if (blockIdx.x == 0 && slot == 0) {
+                if (p.call_tag) {                      // nothing has cleared the status block
+                    wait_for_previous_launch();        // (the test hook skips the one above)
+                    p.status->call_tag = p.call_tag;
+                    for (int i = 0; i < 4; ++i) p.status->probe_cycles[i] = p.status->probe_ns[i] = 0;
+                }
+                probe.stop(p.status, QUEUE_FWD_SHORT);
+            }
         }
     } else if (warp == kWarpMma + slot) {
         // ------------------------------------------------------------------ UMMA issuer
@@ -536,6 +545,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
         while (global_timer_ns() - t0 < 50000ull) { }
         if (tid == 0) {
             p.status->detail = blockIdx.x;
+            p.status->error_tag = p.call_tag;
             p.status->status = HYDRA_ERR_DEVICE_TIMEOUT;
         }
         __syncthreads();

@@ -113,6 +113,10 @@ struct StatusBlock {            // lives at the start of the workspace; zeroed b
     int32_t pad;
     int64_t detail;
     int32_t next_item[4];       // work-queue heads of the persistent kernels (forward, dK/dV, dQ, short forward)
+    // A call none of whose kernels pops from a queue is not worth a launch that clears this block. Its kernel writes call_tag,
+    // a number of the call's own, and with an error the same number as error_tag; `status` counts only while the two are
+    // equal, as they are (zero) wherever the block is cleared.
+    int32_t call_tag, error_tag;
     // SM clock seen from inside the tensor-core kernels: cycles and nanoseconds that passed in the
     // producer thread of CTA 0 between its first and its last instruction (same index as next_item)
     uint64_t probe_cycles[4];
@@ -231,6 +235,7 @@ struct FwdParams {
     const FwdShortItem* short_items;   // the pairs that go to the short-sequence kernel
     int32_t n_short;
     int32_t early_pops;         // short-sequence kernel: items of up to so many steps are popped two items ahead
+    int32_t call_tag;           // StatusBlock::call_tag of a call without a queue (short-sequence kernel), else 0
     void* out; float* lse; void* o_part; float* lse_part;
     int64_t T; int64_t part_rows;
     int32_t h; int32_t causal;
