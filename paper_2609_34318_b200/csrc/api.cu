@@ -717,6 +717,19 @@ GroupOrder order_groups(std::vector<std::vector<GroupEntry>>& groups, int32_t h,
     });
     const int64_t even = (total + workers - 1) / workers;
     go.settled = static_cast<int64_t>(longest + kItemOverhead) * 20 <= even;
+    if (go.settled) {
+        // No item is long: only the end of the list needs the longest-first order (a longest item's worth per worker). Before it
+        // the groups run as they lie in memory: a ragged tile's loads take rows of the next sequence along, which are then
+        // used while they are in L2. 32768 tokens of 64 to 512, 32 heads, read from memory, longest first / as they lie:
+        // forward 1.22 / 1.11 GB, key side 1.55 / 1.38, query side 1.12 / 1.06 (1.03 at least); step of 65536 2707 / 2660 us.
+        int64_t left = static_cast<int64_t>(workers) * (longest + kItemOverhead);
+        size_t tail = groups.size();
+        while (tail > 0 && left > 0) {
+            const int32_t g = go.order[--tail];
+            left -= (group_cost[g] + static_cast<int64_t>(groups[g].size()) * kItemOverhead) * h;
+        }
+        std::sort(go.order.begin(), go.order.begin() + static_cast<int64_t>(tail));
+    }
     return go;
 }
 template <class Item, class Make>
