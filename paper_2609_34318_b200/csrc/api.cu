@@ -311,6 +311,7 @@ struct Plan {
     int32_t halves = 0;              // forward: the short kernel's items are halves of tiles, two per thread block;
                                      // backward: two CTAs share every key-side item
     int32_t early_pops = 0;          // forward: FwdParams::early_pops
+    int32_t short_grid = 0;          // forward, halves: thread blocks the items have been dealt out to
     int32_t item_heads = 1;          // backward: query heads per key-side item (BwdParams::item_heads)
     int64_t ds_head_blocks = 0;      // backward: blocks of the dS hand-off buffer per head; -1: not usable
     // residency on the device (guarded by g_plan_mutex)
@@ -760,6 +761,51 @@ inline int32_t kv_steps_short(const hydra_pair_t& p, int32_t q0, int32_t rows, i
     return n_keys > 0 ? static_cast<int32_t>((n_keys + FWD_SHORT_KEYS - 1) / FWD_SHORT_KEYS) : 0;
 }
 
+// Tiles whose keys the two slots of a thread block share (short-sequence forward, calls of few tiles), dealt out longest first,
+// each to the thread block that has least to do: a longer tile as two parts, one per slot, short ones two at a time, a whole
+// one per slot (not in calls with a thread block for each).
+struct SharedTile { int32_t pair, q0, steps, head; };
+struct DealtTile { int32_t first, second, block, round; };      // second: the tile beside it; the same one: shared; -1: none
+struct Deal {
+    int32_t grid = 0, rounds = 0;
+    int64_t end = 0;                                    // of the longest thread block, in steps
+    std::vector<DealtTile> tiles;
+};
+Deal deal_shared_tiles(const std::vector<SharedTile>& tiles)
+{
+    constexpr int32_t kSharedSteps = 6;                 // a part of two steps is not worth the join
+    constexpr int32_t kOverhead = 3;                    // of a tile: load, join and store, in steps
+    Deal deal;
+    const int32_t n = static_cast<int32_t>(tiles.size());
+    deal.grid = std::min(plan_workers(1), n);
+    std::vector<int32_t> order(n), used(deal.grid, 0);
+    for (int32_t i = 0; i < n; ++i) order[i] = i;
+    if (n > deal.grid)                                  // (else as they lie: neighbours share K and V)
+        std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return tiles[x].steps > tiles[y].steps; });
+    using Load = std::pair<int64_t, int32_t>;           // (steps so far, thread block)
+    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> least;
+    for (int32_t c = 0; c < deal.grid; ++c) least.push({0, c});
+    for (int32_t i = 0; i < n; ++i) {
+        const int32_t t = order[i], steps = tiles[t].steps;
+        const int32_t block = least.top().second;
+        int64_t load = least.top().first + kOverhead;
+        least.pop();
+        DealtTile d{t, -1, block, used[block]++};
+        if (steps >= (n > deal.grid ? kSharedSteps : 2)) {
+            d.second = t;
+            load += (steps + 1) / 2;
+        } else {
+            if (n > deal.grid && i + 1 < n) d.second = order[++i];
+            load += steps;
+        }
+        deal.tiles.push_back(d);
+        deal.rounds = std::max(deal.rounds, used[block]);
+        deal.end = std::max(deal.end, load);
+        least.push({load, block});
+    }
+    return deal;
+}
+
 void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& blob)
 {
     // Which pairs go to the short-sequence kernel (one CTA per SM, two independent 128-row tiles in flight,
@@ -769,12 +815,17 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     // tail), so the short kernel is used only if the short pairs carry at least a quarter of the call's work.
     const int32_t short_len = fwd_short_len_for(pb, causal);
     std::vector<uint8_t> is_short(pb.pairs.size(), 0);
-    // A call with no more q tiles than SMs: what it takes is its longest tile's chain of steps. The short kernel then has
-    // an idle slot beside every busy one and gives it the second half of the tile's keys, whatever their number (the
-    // CTA-pair kernel would leave more than half of the SMs idle).
+    // A call of few q tiles takes as long as its longest tile's chain of steps. The short kernel's two slots then share the
+    // keys of a tile, whatever their number (deal_shared_tiles; the CTA-pair kernel would leave SMs idle): always with no more
+    // tiles than SMs, in calls of more where the queue is expected to take longer than the tiles dealt out. A step takes 0.93
+    // us in a slot whose neighbour idles, 1.25 to 1.4 beside a busy one; on CTA pairs a step's share of an SM is 0.5 to 0.6.
+    // Forward in passes one after another, 16 heads of 192 unless said, queue / shared, us: 1300 tokens 29.1 / 19.9, 2048 40.3 /
+    // 29.6, 4096, 8 heads 71.0 / 48.5, 8192, 4 heads 133 / 96, 4820 log-normal ones, 8 heads 41.5 / 33.7, 8192, 4 heads 53.0 /
+    // 39.4; beyond the line 3000 60.1 / 63.8, 4096 86.9 / 100, 2048, 32 heads 61.0 / 66.2, ten sequences of 410 34.1 / 40.8.
     // (A limit set by the caller is kept to.)
     // (A work item counts its steps in 16 bits: more keys than two items hold stay with the CTA-pair kernel.)
     constexpr int64_t kMostKeys = int64_t{UINT16_MAX} * FWD_SHORT_KEYS;
+    constexpr int64_t kMostShared = 5;                 // half tiles per SM: above 2.5 tiles per SM sharing never won
     int64_t n_tiles = 0;
     int32_t longest = 0, most_keys = 0;
     bool within = true;
@@ -785,8 +836,27 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
         within = within && p.q_len <= short_len && p.k_len <= short_len;
     }
     n_tiles *= pb.h;
-    const bool halves = short_len > 0 && n_tiles <= plan_workers(1) && most_keys <= 2 * kMostKeys &&
-                        (within || pb.fwd_short_set < 0);
+    std::vector<SharedTile> tiles;
+    Deal deal;
+    bool halves = short_len > 0 && 2 * n_tiles <= kMostShared * plan_workers(1) && most_keys <= 2 * kMostKeys &&
+                  (within || pb.fwd_short_set < 0);
+    if (halves) {
+        int64_t work = 0;
+        int32_t chain = 0;
+        for (size_t pi = 0; pi < pb.pairs.size(); ++pi) {
+            const auto& p = pb.pairs[pi];
+            for (int32_t a = 0; a < pb.h; ++a)
+                for (int32_t q0 = 0; q0 < p.q_len; q0 += TILE) {
+                    const int32_t steps = kv_steps_short(p, q0, std::min(TILE, p.q_len - q0), causal);
+                    chain = std::max(chain, steps + kItemOverhead);
+                    work += steps + kItemOverhead;
+                    tiles.push_back(SharedTile{static_cast<int32_t>(pi), q0, steps, a});
+                }
+        }
+        const int64_t queue = std::max<int64_t>(chain * 93, work * 60 / plan_workers(1));
+        deal = deal_shared_tiles(tiles);
+        halves = n_tiles <= plan_workers(1) || deal.end * 130 < queue;
+    }
     if (halves) {
         std::fill(is_short.begin(), is_short.end(), 1);
     } else {
@@ -886,32 +956,33 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     };
     const int short_workers = 2 * plan_workers(1);
     if (halves) {
-        // the first parts, then the second parts in the same order: slots 0 take items [0, n), slots 1 [n, 2 n)
-        std::vector<FwdShortItem> first, second;
-        for (size_t g = 0; g < groups_short.size(); ++g)
-            for (int32_t a = 0; a < pb.h; ++a)
-                for (const GroupEntry& e : groups_short[g]) {
-                    FwdShortItem it = make_short(a, e), rest = it;
-                    const int32_t n0 = (e.b + 1) / 2;
-                    rest.n_kv = static_cast<uint16_t>(e.b - n0);
-                    if (rest.n_kv > 0) {
-                        const int32_t skip = n0 * FWD_SHORT_KEYS;
-                        it.n_kv = static_cast<uint16_t>(n0);
-                        it.half = 1;
-                        rest.half = 2;
-                        rest.k_tok0 += skip;
-                        rest.k_len -= skip;
-                        rest.off -= skip;
-                    } else {
-                        rest.rows = 0;                      // nothing left for the other slot: it writes nothing
-                    }
-                    first.push_back(it);
-                    second.push_back(rest);
-                }
-        first.insert(first.end(), second.begin(), second.end());
-        plan.off_items2 = append(blob, first);
-        plan.n_items2 = static_cast<int32_t>(first.size());
+        auto entry = [&](const SharedTile& t) {
+            return GroupEntry{t.q0, t.steps, std::min(TILE, pb.pairs[t.pair].q_len - t.q0), t.steps, t.pair};
+        };
+        std::vector<FwdShortItem> table(static_cast<size_t>(deal.rounds) * 2 * deal.grid);      // (an item of no rows and no steps does nothing)
+        for (const DealtTile& t : deal.tiles) {
+            const SharedTile& one = tiles[t.first];
+            FwdShortItem it = make_short(one.head, entry(one)), other{};
+            if (t.second == t.first) {
+                const int32_t n0 = (one.steps + 1) / 2, skip = n0 * FWD_SHORT_KEYS;
+                other = it;
+                it.n_kv = static_cast<uint16_t>(n0);
+                it.half = 1;
+                other.n_kv = static_cast<uint16_t>(one.steps - n0);
+                other.half = 2;
+                other.k_tok0 += skip;
+                other.k_len -= skip;
+                other.off -= skip;
+            } else if (t.second >= 0) {
+                other = make_short(tiles[t.second].head, entry(tiles[t.second]));
+            }
+            table[static_cast<size_t>(2 * t.round) * deal.grid + t.block] = it;
+            table[static_cast<size_t>(2 * t.round + 1) * deal.grid + t.block] = other;
+        }
+        plan.off_items2 = append(blob, table);
+        plan.n_items2 = static_cast<int32_t>(table.size());
         plan.halves = 1;
+        plan.short_grid = deal.grid;
         return;
     }
     const GroupOrder go = order_groups(groups_short, pb.h, short_workers);
@@ -1706,15 +1777,15 @@ int32_t fwd_core(Problem& pb, const void* q, const void* k, const void* v, int32
     if (int32_t s = lease.acquire(HYDRA_WS_FWD, pb, causal != 0, stream)) return s;
     const Plan* plan = &lease.plan();
     if (plan->n_items == 0 && plan->n_items2 == 0) return HYDRA_OK;
-    // One item per SM before any SM gets two, or both halves of a tile on one SM.
-    const int short_grid = plan->halves ? plan->n_items2 / 2 : std::min(sms, plan->n_items2);
+    // One item per SM before any SM gets two, or what the items have been dealt out to.
+    const int short_grid = plan->halves ? plan->short_grid : std::min(sms, plan->n_items2);
     FwdParams fp{};
     // With no more items than slots nothing is popped from the queue, and the block at the workspace's start need not be
     // cleared (one launch less: four sequences of 7 to 300 tokens, forward 11.5 -> 9.4 us). Not where the launches are
     // recorded: every replay would have the number of the first.
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) return HYDRA_ERR_CUDA;
-    if (capturing == cudaStreamCaptureStatusNone && plan->n_items == 0 && plan->n_items2 <= 2 * short_grid) {
+    if (capturing == cudaStreamCaptureStatusNone && plan->n_items == 0 && (plan->halves || plan->n_items2 <= 2 * short_grid)) {
         static std::atomic<uint32_t> calls{0};
         do fp.call_tag = static_cast<int32_t>(calls.fetch_add(1) + 1u);
         while (fp.call_tag == 0);

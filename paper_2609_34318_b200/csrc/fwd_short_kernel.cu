@@ -82,7 +82,7 @@ constexpr int kPopAhead = 4;                          // steps before the end of
 enum : int {
     B_QFULL = 0, B_QEMPTY = 1, B_KFULL = 2, B_KEMPTY = 5, B_VFULL = 8, B_VEMPTY = 10, B_SFULL = 12, B_PFULL = 14,
     B_PVDONE = 16, B_OFREE = 17, B_ITEMFULL = 18, B_ITEMEMPTY = 18 + kSched, B_HALF = 18 + 2 * kSched,
-    B_PER_SLOT = 19 + 2 * kSched
+    B_HALFFREE = 19 + 2 * kSched, B_PER_SLOT = 20 + 2 * kSched      // (the two: slot 0's are used)
 };
 
 __device__ __forceinline__ float neg_inf() { return __int_as_float(0xff800000); }
@@ -91,8 +91,10 @@ __device__ __forceinline__ float neg_inf() { return __int_as_float(0xff800000); 
 
 size_t HYDRA_K(fwd_short_smem_bytes)() { return kSmemTotal + 1024; }
 
-// kHalves: every thread block has one q tile, whose keys its two slots share. (A build of its own: the join of the two parts
-// in the epilogue of the other would cost it 7 % on sequences of 64 to 512 tokens in instruction-cache misses.)
+// kHalves: the two slots share the keys of a thread block's longer q tiles, and the host has dealt the items out (entry (k *
+// kSlots + slot) * gridDim.x + blockIdx.x is a slot's k-th): for calls of few tiles, which take as long as their longest ones.
+// (A build of its own: the join of the two parts in the epilogue of the other would cost it 7 % on sequences of 64 to 512
+// tokens in instruction-cache misses.)
 template <bool kHalves>
 __global__ void __launch_bounds__(kThreads, 1)
 HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -119,7 +121,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
         for (int s = 0; s < kSlots; ++s)
             for (int i = 0; i < B_PER_SLOT; ++i) {
                 uint32_t count = 1u;
-                if ((i >= B_PFULL && i < B_PFULL + 2) || i == B_OFREE || i == B_HALF) count = 4u;   // softmax warps
+                if ((i >= B_PFULL && i < B_PFULL + 2) || i == B_OFREE || i == B_HALF || i == B_HALFFREE) count = 4u;   // softmax warps
                 if (i >= B_ITEMEMPTY && i < B_ITEMEMPTY + kSched) count = 5u;             // + its issuer
                 mbar_init(base + 8u * static_cast<uint32_t>(s * B_PER_SLOT + i), count);
             }
@@ -204,11 +206,24 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
             bool have1 = true, have2 = false;          // the one after it, if they have been asked for
             const int first_pop = kSlots * static_cast<int>(gridDim.x);
             // (with no more items than slots every pop comes back empty, and the counter has not been cleared)
-            auto pop = [&]() -> int { return p.call_tag ? p.n_short : first_pop + atomicAdd(counter, 1); };
+            int dealt = slot * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x);
+            auto pop = [&]() -> int {
+                if (kHalves) return dealt += first_pop;
+                return p.call_tag ? p.n_short : first_pop + atomicAdd(counter, 1);
+            };
+            uint32_t shared_tiles = 0;                 // whose second part this slot has run (slot 1)
             bool pre = false;                          // Q and the first K tile of `cur` have been requested
+            int last_half = 0;                         // part of the item before `cur`
             // round kq loads item kq - 1 (round 0: none) and hands over item kq on the way
             for (uint32_t kq = 0; ok; ++kq) {
                 const int n = cur.n_kv;
+                if (kHalves && last_half == 2) {       // slot 0 has read what this slot left in its operand space
+                    ok = mbar_wait(smem_u32(&bars[B_HALFFREE]), shared_tiles & 1u, abort_p, limit);
+                    if (!ok) break;
+                    fence_proxy_async_smem();          // (they were ordinary stores, what follows are asynchronous copies)
+                    ++shared_tiles;
+                }
+                last_half = cur.half;
                 if (n > 0 && !pre) { load_q(cur); load_k(cur, 0); }
                 if (n > 1) load_k(cur, 1);
                 pre = false;
@@ -226,7 +241,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
                     // The next item's Q and first K tile are released by score products that are long issued
                     // when the last V stage comes free: ask for them first, and show the item to the issuer.
                     if (j == (n >= 2 ? n - 1 : n)) {
-                        if (n >= 2 && nxt_idx >= 0 && nxt.n_kv > 0) { load_q(nxt); load_k(nxt, 0); pre = true; }
+                        if (n >= 2 && nxt_idx >= 0 && nxt.n_kv > 0 && !(kHalves && cur.half == 2)) { load_q(nxt); load_k(nxt, 0); pre = true; }
                         if (ok) publish(kq, nxt_idx, nxt);
                     }
                     if (j >= n) break;
@@ -351,6 +366,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
         const uint32_t tm_o = tm + lane_base;
         const uint32_t tm_s0 = tm + kTmS + lane_base;
         uint32_t g = 0;                                // steps of this slot so far
+        uint32_t joined = 0;                           // tiles joined with their second part (slot 0)
         bool ok = true;
         wait_for_previous_launch();
         for (uint32_t kq = 0; ok; ++kq) {
@@ -462,9 +478,9 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
             ok = wait(B_PVDONE, g - 1u);
             if (!ok) break;
             tc_fence_after_sync();
-            // A tile whose keys the two slots share: slot 1 leaves its unscaled O, maximum and sum in its own (now unused)
-            // operand space, a column of 128 rows after the other, and slot 0 joins them to its own. In such a launch
-            // every thread block has this one tile.
+            // A tile whose keys the two slots share: slot 1 leaves its unscaled O, maximum and sum in its own operand space,
+            // which is loaded again once slot 0 has read them, a column of 128 rows after the other, and slot 0 joins them to
+            // its own.
             const uint32_t half_buf = smem0 + kSlotBytes + r * 4u;
             constexpr uint32_t kColumn = TILE * 4;
             float mul0 = 1.f, mul1 = 0.f;
@@ -485,8 +501,9 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
                 continue;
             }
             if (kHalves && item.half == 1) {
-                ok = wait(B_HALF, 0u);
+                ok = wait(B_HALF, joined);
                 if (!ok) break;
+                ++joined;
                 const float m1 = ld_shared_f32(half_buf + D_V * kColumn), l1 = ld_shared_f32(half_buf + (D_V + 1) * kColumn);
                 const float m = fmaxf(m_run, m1);
                 if (m != neg_inf()) {                  // (a part without visible keys has maximum -inf: weight 0)
@@ -530,6 +547,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
                     }
                 }
             }
+            if (kHalves && item.half == 1) mbar_arrive_warp(bar(B_HALFFREE));
             if (row_valid)
                 *lse_dst = (l_run > 0.f) ? (m_run + __log2f(l_run)) * 0.6931471805599453f : neg_inf();
         }
