@@ -1350,7 +1350,7 @@ struct KernelSet {
     int (*fwd_max_clusters)();
     cudaError_t (*launch_fwd)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const FwdParams&, int,
                               cudaStream_t);
-    cudaError_t (*launch_fwd_short)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const FwdParams&, bool, int,
+    cudaError_t (*launch_fwd_short)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const FwdParams&, int32_t, bool, int,
                                     cudaStream_t);
     cudaError_t (*launch_bwd_dq)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const CUtensorMap&,
                                  const BwdParams&, int, cudaStream_t);
@@ -1780,6 +1780,7 @@ int32_t fwd_core(Problem& pb, const void* q, const void* k, const void* v, int32
     // One item per SM before any SM gets two, or what the items have been dealt out to.
     const int short_grid = plan->halves ? plan->short_grid : std::min(sms, plan->n_items2);
     FwdParams fp{};
+    int32_t call_tag = 0;
     // With no more items than slots nothing is popped from the queue, and the block at the workspace's start need not be
     // cleared (one launch less: four sequences of 7 to 300 tokens, forward 11.5 -> 9.4 us). Not where the launches are
     // recorded: every replay would have the number of the first.
@@ -1787,8 +1788,8 @@ int32_t fwd_core(Problem& pb, const void* q, const void* k, const void* v, int32
     if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) return HYDRA_ERR_CUDA;
     if (capturing == cudaStreamCaptureStatusNone && plan->n_items == 0 && (plan->halves || plan->n_items2 <= 2 * short_grid)) {
         static std::atomic<uint32_t> calls{0};
-        do fp.call_tag = static_cast<int32_t>(calls.fetch_add(1) + 1u);
-        while (fp.call_tag == 0);
+        do call_tag = static_cast<int32_t>(calls.fetch_add(1) + 1u);
+        while (call_tag == 0);
     } else if (launch_reset(static_cast<StatusBlock*>(workspace), false, stream) != cudaSuccess) {
         return HYDRA_ERR_CUDA;
     }
@@ -1824,7 +1825,7 @@ int32_t fwd_core(Problem& pb, const void* q, const void* k, const void* v, int32
         CUtensorMap mv_sub;
         if (make_map(&mv_sub, v, pb.Tk, n_kv_heads, D_V, FWD_SHORT_KEYS)) return HYDRA_ERR_CUDA;
         ScopedKernelTimer timer(K_FWD, stream);
-        if (ks->launch_fwd_short(mq, mk, mv_sub, fp, plan->halves != 0, short_grid, stream) != cudaSuccess) return HYDRA_ERR_CUDA;
+        if (ks->launch_fwd_short(mq, mk, mv_sub, fp, call_tag, plan->halves != 0, short_grid, stream) != cudaSuccess) return HYDRA_ERR_CUDA;
         g_launches += 1;
     }
     lease.release();                                   // the tables have their reader on record

@@ -91,6 +91,8 @@ __device__ __forceinline__ float neg_inf() { return __int_as_float(0xff800000); 
 
 size_t HYDRA_K(fwd_short_smem_bytes)() { return kSmemTotal + 1024; }
 
+// call_tag: StatusBlock::call_tag of a call without a queue, else 0. (Not a field of FwdParams: one more there made the CTA-pair
+// kernel, which does not use it, 2.7 % slower, one document of 16384 tokens, 8 heads 568 -> 584 us.)
 // kHalves: the two slots share the keys of a thread block's longer q tiles, and the host has dealt the items out (entry (k *
 // kSlots + slot) * gridDim.x + blockIdx.x is a slot's k-th): for calls of few tiles, which take as long as their longest ones.
 // (A build of its own: the join of the two parts in the epilogue of the other would cost it 7 % on sequences of 64 to 512
@@ -98,7 +100,7 @@ size_t HYDRA_K(fwd_short_smem_bytes)() { return kSmemTotal + 1024; }
 template <bool kHalves>
 __global__ void __launch_bounds__(kThreads, 1)
 HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                                const __grid_constant__ CUtensorMap map_v, const FwdParams p)
+                                const __grid_constant__ CUtensorMap map_v, const FwdParams p, const int32_t call_tag)
 {
     overlap_next_launch();
     extern __shared__ uint8_t smem_raw[];
@@ -209,7 +211,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
             int dealt = slot * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x);
             auto pop = [&]() -> int {
                 if (kHalves) return dealt += first_pop;
-                return p.call_tag ? p.n_short : first_pop + atomicAdd(counter, 1);
+                return call_tag ? p.n_short : first_pop + atomicAdd(counter, 1);
             };
             uint32_t shared_tiles = 0;                 // whose second part this slot has run (slot 1)
             bool pre = false;                          // Q and the first K tile of `cur` have been requested
@@ -256,9 +258,9 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
                 have2 = false;
             }
             if (blockIdx.x == 0 && slot == 0) {
-                if (p.call_tag) {                      // nothing has cleared the status block
+                if (call_tag) {                      // nothing has cleared the status block
                     wait_for_previous_launch();        // (the test hook skips the one above)
-                    p.status->call_tag = p.call_tag;
+                    p.status->call_tag = call_tag;
                     for (int i = 0; i < 4; ++i) p.status->probe_cycles[i] = p.status->probe_ns[i] = 0;
                 }
                 probe.stop(p.status, QUEUE_FWD_SHORT);
@@ -563,7 +565,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
         while (global_timer_ns() - t0 < 50000ull) { }
         if (tid == 0) {
             p.status->detail = blockIdx.x;
-            p.status->error_tag = p.call_tag;
+            p.status->error_tag = call_tag;
             p.status->status = HYDRA_ERR_DEVICE_TIMEOUT;
         }
         __syncthreads();
@@ -572,12 +574,12 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
 }
 
 cudaError_t HYDRA_K(launch_fwd_short)(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
-                                      const FwdParams& p, bool halves, int grid, cudaStream_t stream)
+                                      const FwdParams& p, int32_t call_tag, bool halves, int grid, cudaStream_t stream)
 {
     static OncePerDevice configured[2];
     const auto kernel = halves ? HYDRA_K(hydra_fwd_short_kernel)<true> : HYDRA_K(hydra_fwd_short_kernel)<false>;
     if (cudaError_t e = allow_dynamic_smem(kernel, HYDRA_K(fwd_short_smem_bytes)(), configured[halves])) return e;
-    return launch_overlapped(kernel, grid, kThreads, HYDRA_K(fwd_short_smem_bytes)(), stream, mq, mk, mv, p);
+    return launch_overlapped(kernel, grid, kThreads, HYDRA_K(fwd_short_smem_bytes)(), stream, mq, mk, mv, p, call_tag);
 }
 
 }  // namespace hydra

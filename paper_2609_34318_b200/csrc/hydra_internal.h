@@ -235,7 +235,6 @@ struct FwdParams {
     const FwdShortItem* short_items;   // the pairs that go to the short-sequence kernel
     int32_t n_short;
     int32_t early_pops;         // short-sequence kernel: items of up to so many steps are popped two items ahead
-    int32_t call_tag;           // StatusBlock::call_tag of a call without a queue (short-sequence kernel), else 0
     void* out; float* lse; void* o_part; float* lse_part;
     int64_t T; int64_t part_rows;
     int32_t h; int32_t causal;
@@ -292,7 +291,7 @@ struct MergeParams {
                                    const FwdParams& p, int grid, cudaStream_t stream);                                \
     size_t fwd_short_smem_bytes##SUFFIX();                                                                            \
     cudaError_t launch_fwd_short##SUFFIX(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv_sub,     \
-                                         const FwdParams& p, bool halves, int grid, cudaStream_t stream);             \
+                                         const FwdParams& p, int32_t call_tag, bool halves, int grid, cudaStream_t stream); \
     cudaError_t launch_bwd_dq##SUFFIX(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,            \
                                       const CUtensorMap& mdo, const BwdParams& p, int grid, cudaStream_t stream);     \
     cudaError_t launch_bwd_dq_from_ds##SUFFIX(const CUtensorMap& mk, const BwdParams& p, int grid,                    \
