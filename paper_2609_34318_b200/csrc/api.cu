@@ -11,6 +11,7 @@
 #include <memory>
 #include <mutex>
 #include <queue>
+#include <tuple>
 #include <vector>
 
 #include "hydra_internal.h"
@@ -312,6 +313,8 @@ struct Plan {
                                      // backward: two CTAs share every key-side item
     int32_t early_pops = 0;          // forward: FwdParams::early_pops
     int32_t short_grid = 0;          // forward, halves: thread blocks the items have been dealt out to
+    size_t off_segs = 0;             // forward: FwdSeg table of the short-sequence kernel's items
+    int32_t n_segs = 0;
     int32_t item_heads = 1;          // backward: query heads per key-side item (BwdParams::item_heads)
     int64_t ds_head_blocks = 0;      // backward: blocks of the dS hand-off buffer per head; -1: not usable
     // residency on the device (guarded by g_plan_mutex)
@@ -761,10 +764,56 @@ inline int32_t kv_steps_short(const hydra_pair_t& p, int32_t q0, int32_t rows, i
     return n_keys > 0 ? static_cast<int32_t>((n_keys + FWD_SHORT_KEYS - 1) / FWD_SHORT_KEYS) : 0;
 }
 
+// What the short-sequence forward makes its q tiles of: a pair, or consecutive q chunks that meet the same kv chunk, where that
+// saves tiles (a chunk's last tile is ragged: sequences of 121 tokens in chunks of 30 have ten tiles pair by pair, four by kv
+// chunk). `all` has the sum of the pairs' rows; `pairs` are their indices in order.
+// Forward, pair by pair / shared, us: 30000 tokens of 64 to 512, 16 heads, ring of 4 628 / 347, 12 sequences of 121 tokens, 16
+// heads, ring of 2 28.8 / 22.6, 26283 log-normal tokens, 16 heads, ring of 4 710 / 619, 65536 of 64 to 512, 32 heads, cut in two
+// 831 / 804.
+struct FwdRun {
+    hydra_pair_t all;
+    std::vector<int32_t> pairs;
+};
+std::vector<FwdRun> make_runs(const Problem& pb, const std::vector<uint8_t>& wanted)
+{
+    std::vector<int32_t> order;
+    for (size_t i = 0; i < pb.pairs.size(); ++i)
+        if (wanted[i] && pb.pairs[i].q_len > 0) order.push_back(static_cast<int32_t>(i));
+    bool cut = false;
+    for (int32_t i : order) cut = cut || pb.pairs[i].part_row >= 0;
+    auto key = [&](int32_t i) {
+        const auto& p = pb.pairs[i];
+        return std::make_tuple(p.seq, p.k_start, p.k_len, p.q_start);
+    };
+    if (cut) std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return key(x) < key(y); });
+    auto tiles = [](int32_t rows) { return (rows + TILE - 1) / TILE; };
+    std::vector<FwdRun> runs;
+    for (size_t i = 0, j = 0; i < order.size(); i = j) {
+        FwdRun run{pb.pairs[order[i]], {order[i]}};
+        int32_t separate = tiles(run.all.q_len);
+        for (j = i + 1; cut && j < order.size(); ++j) {
+            const auto& p = pb.pairs[order[j]];
+            if (p.seq != run.all.seq || p.k_start != run.all.k_start || p.k_len != run.all.k_len ||
+                p.q_start != run.all.q_start + run.all.q_len ||
+                pb.q_row(p.seq, p.q_start) != pb.q_row(p.seq, run.all.q_start) + run.all.q_len)
+                break;
+            run.all.q_len += p.q_len;
+            separate += tiles(p.q_len);
+            run.pairs.push_back(order[j]);
+        }
+        if (run.pairs.size() > 1 && tiles(run.all.q_len) == separate) {     // nothing saved
+            for (int32_t one : run.pairs) runs.push_back(FwdRun{pb.pairs[one], {one}});
+            continue;
+        }
+        runs.push_back(std::move(run));
+    }
+    return runs;
+}
+
 // Tiles whose keys the two slots of a thread block share (short-sequence forward, calls of few tiles), dealt out longest first,
 // each to the thread block that has least to do: a longer tile as two parts, one per slot, short ones two at a time, a whole
 // one per slot (not in calls with a thread block for each).
-struct SharedTile { int32_t pair, q0, steps, head; };
+struct SharedTile { int32_t run, q0, steps, head; };
 struct DealtTile { int32_t first, second, block, round; };      // second: the tile beside it; the same one: shared; -1: none
 struct Deal {
     int32_t grid = 0, rounds = 0;
@@ -830,11 +879,12 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     int32_t longest = 0, most_keys = 0;
     bool within = true;
     for (const auto& p : pb.pairs) {
-        n_tiles += (p.q_len + TILE - 1) / TILE;
         longest = std::max(longest, std::max(p.q_len, p.k_len));
         most_keys = std::max(most_keys, p.k_len);
         within = within && p.q_len <= short_len && p.k_len <= short_len;
     }
+    std::vector<FwdRun> runs = make_runs(pb, std::vector<uint8_t>(pb.pairs.size(), 1));
+    for (const FwdRun& run : runs) n_tiles += (run.all.q_len + TILE - 1) / TILE;
     n_tiles *= pb.h;
     std::vector<SharedTile> tiles;
     Deal deal;
@@ -843,14 +893,14 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     if (halves) {
         int64_t work = 0;
         int32_t chain = 0;
-        for (size_t pi = 0; pi < pb.pairs.size(); ++pi) {
-            const auto& p = pb.pairs[pi];
+        for (size_t ri = 0; ri < runs.size(); ++ri) {
+            const auto& p = runs[ri].all;
             for (int32_t a = 0; a < pb.h; ++a)
                 for (int32_t q0 = 0; q0 < p.q_len; q0 += TILE) {
                     const int32_t steps = kv_steps_short(p, q0, std::min(TILE, p.q_len - q0), causal);
                     chain = std::max(chain, steps + kItemOverhead);
                     work += steps + kItemOverhead;
-                    tiles.push_back(SharedTile{static_cast<int32_t>(pi), q0, steps, a});
+                    tiles.push_back(SharedTile{static_cast<int32_t>(ri), q0, steps, a});
                 }
         }
         const int64_t queue = std::max<int64_t>(chain * 93, work * 60 / plan_workers(1));
@@ -884,19 +934,21 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     int32_t longest_tile = 0;
     int64_t short_cost = 0;
     std::vector<std::vector<GroupEntry>> groups(pb.n_seqs), groups_short(pb.n_seqs);
+    if (!halves) runs = make_runs(pb, is_short);
+    for (size_t ri = 0; ri < runs.size(); ++ri) {
+        const auto& p = runs[ri].all;
+        for (int32_t q0 = 0; q0 < p.q_len; q0 += TILE) {
+            const int32_t rows = std::min(TILE, p.q_len - q0);
+            const int32_t n_kv = kv_steps_short(p, q0, rows, causal);
+            groups_short[p.seq].push_back(GroupEntry{q0, n_kv, rows, n_kv, static_cast<int32_t>(ri)});
+            longest_tile = std::max(longest_tile, n_kv);
+            short_cost += n_kv + kItemOverhead;
+        }
+    }
     for (size_t pi = 0; pi < pb.pairs.size(); ++pi) {
         const auto& p = pb.pairs[pi];
         const int32_t of = static_cast<int32_t>(pi);
-        if (is_short[pi]) {
-            for (int32_t q0 = 0; q0 < p.q_len; q0 += TILE) {
-                const int32_t rows = std::min(TILE, p.q_len - q0);
-                const int32_t n_kv = kv_steps_short(p, q0, rows, causal);
-                groups_short[p.seq].push_back(GroupEntry{q0, n_kv, rows, n_kv, of});
-                longest_tile = std::max(longest_tile, n_kv);
-                short_cost += n_kv + kItemOverhead;
-            }
-            continue;
-        }
+        if (is_short[pi]) continue;
         // One item = two consecutive 256-row UMMA tiles (A, then B) of a CTA pair. The slabs are aligned to
         // the END of the q chunk: with an odd number of 256-row tiles the chunk's FIRST tile goes alone (it
         // visits the fewest kv tiles), so the ragged last tile rides with a full neighbour instead of running
@@ -940,8 +992,29 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     // micro-batch of short sequences has tens of thousands of them and a new one arrives with every step, so in
     // the common case (many items, none long: the block order is final) they are written straight into the
     // table, a group's entries once and then one copy per head with the head number set.
+    // Where the rows of tiles that several pairs share go, once per tile (every head has the same).
+    std::vector<FwdSeg> segs;
+    std::map<std::pair<int32_t, int32_t>, int32_t> segs_of;        // (run, first row) -> FwdShortItem::segs
+    for (size_t ri = 0; ri < runs.size(); ++ri) {
+        const FwdRun& run = runs[ri];
+        if (run.pairs.size() < 2) continue;
+        for (int32_t q0 = 0; q0 < run.all.q_len; q0 += TILE) {
+            const size_t at = segs.size();
+            int32_t first = 0;                          // the pair's first row in the run
+            for (int32_t pi : run.pairs) {
+                const int32_t len = pb.pairs[pi].q_len;
+                if (first < q0 + TILE && first + len > q0) {
+                    const int32_t begin = std::max(0, first - q0);
+                    segs.push_back(FwdSeg{static_cast<int16_t>(begin), static_cast<int16_t>(dev_pairs[pi].to_part),
+                                          dev_pairs[pi].out_row0 + q0 - first});
+                }
+                first += len;
+            }
+            segs_of[{static_cast<int32_t>(ri), q0}] = static_cast<int32_t>(at << 8 | (segs.size() - at));
+        }
+    }
     auto make_short = [&](int32_t a, const GroupEntry& e) {
-        const PairDev& d = dev_pairs[e.of];
+        const PairDev& d = dev_pairs[runs[e.of].pairs[0]];
         FwdShortItem it{};
         it.q_tok0 = d.q_tok0 + e.a;
         it.k_tok0 = d.k_tok0;
@@ -952,12 +1025,15 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
         it.n_kv = static_cast<uint16_t>(e.b);
         it.rows = static_cast<uint8_t>(e.c);
         it.to_part = static_cast<uint8_t>(d.to_part);
+        if (runs[e.of].pairs.size() > 1) it.segs = segs_of.at({e.of, e.a});
         return it;
     };
+    plan.off_segs = append(blob, segs);
+    plan.n_segs = static_cast<int32_t>(segs.size());
     const int short_workers = 2 * plan_workers(1);
     if (halves) {
         auto entry = [&](const SharedTile& t) {
-            return GroupEntry{t.q0, t.steps, std::min(TILE, pb.pairs[t.pair].q_len - t.q0), t.steps, t.pair};
+            return GroupEntry{t.q0, t.steps, std::min(TILE, runs[t.run].all.q_len - t.q0), t.steps, t.run};
         };
         std::vector<FwdShortItem> table(static_cast<size_t>(deal.rounds) * 2 * deal.grid);      // (an item of no rows and no steps does nothing)
         for (const DealtTile& t : deal.tiles) {
@@ -1350,7 +1426,7 @@ struct KernelSet {
     int (*fwd_max_clusters)();
     cudaError_t (*launch_fwd)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const FwdParams&, int,
                               cudaStream_t);
-    cudaError_t (*launch_fwd_short)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const FwdParams&, int32_t, bool, int,
+    cudaError_t (*launch_fwd_short)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const FwdParams&, const FwdSeg*, int32_t, bool, int,
                                     cudaStream_t);
     cudaError_t (*launch_bwd_dq)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const CUtensorMap&,
                                  const BwdParams&, int, cudaStream_t);
@@ -1825,7 +1901,7 @@ int32_t fwd_core(Problem& pb, const void* q, const void* k, const void* v, int32
         CUtensorMap mv_sub;
         if (make_map(&mv_sub, v, pb.Tk, n_kv_heads, D_V, FWD_SHORT_KEYS)) return HYDRA_ERR_CUDA;
         ScopedKernelTimer timer(K_FWD, stream);
-        if (ks->launch_fwd_short(mq, mk, mv_sub, fp, call_tag, plan->halves != 0, short_grid, stream) != cudaSuccess) return HYDRA_ERR_CUDA;
+        if (ks->launch_fwd_short(mq, mk, mv_sub, fp, plan->n_segs ? lease.at<FwdSeg>(plan->off_segs) : nullptr, call_tag, plan->halves != 0, short_grid, stream) != cudaSuccess) return HYDRA_ERR_CUDA;
         g_launches += 1;
     }
     lease.release();                                   // the tables have their reader on record

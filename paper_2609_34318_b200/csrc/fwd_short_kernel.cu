@@ -97,10 +97,12 @@ size_t HYDRA_K(fwd_short_smem_bytes)() { return kSmemTotal + 1024; }
 // kSlots + slot) * gridDim.x + blockIdx.x is a slot's k-th): for calls of few tiles, which take as long as their longest ones.
 // (A build of its own: the join of the two parts in the epilogue of the other would cost it 7 % on sequences of 64 to 512
 // tokens in instruction-cache misses.)
-template <bool kHalves>
+// kSegs: some tiles hold rows of several pairs (`segs`; a build of its own for the same reason).
+template <bool kHalves, bool kSegs>
 __global__ void __launch_bounds__(kThreads, 1)
 HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                                const __grid_constant__ CUtensorMap map_v, const FwdParams p, const int32_t call_tag)
+                                const __grid_constant__ CUtensorMap map_v, const FwdParams p,
+                                const FwdSeg* segs, const int32_t call_tag)
 {
     overlap_next_launch();
     extern __shared__ uint8_t smem_raw[];
@@ -381,10 +383,18 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
             mbar_arrive_warp(bar(B_ITEMEMPTY + rs));
             if (idx < 0) break;
             const bool row_valid = r < item.rows;
-            const int64_t rows_total = item.to_part ? p.part_rows : p.T;
-            __nv_bfloat16* obase = static_cast<__nv_bfloat16*>(item.to_part ? p.o_part : p.out);
-            float* lbase = item.to_part ? p.lse_part : p.lse;
-            const int64_t orow = static_cast<int64_t>(item.out_row0) + r;
+            bool to_part = item.to_part != 0;
+            int64_t orow = static_cast<int64_t>(item.out_row0) + r;
+            if (kSegs && item.segs) {
+                const FwdSeg* seg = segs + (item.segs >> 8);
+                for (int i = 0; i < (item.segs & 255); ++i) {
+                    const FwdSeg one = seg[i];
+                    if (r >= one.begin) { to_part = one.to_part != 0; orow = static_cast<int64_t>(one.delta) + r; }
+                }
+            }
+            const int64_t rows_total = to_part ? p.part_rows : p.T;
+            __nv_bfloat16* obase = static_cast<__nv_bfloat16*>(to_part ? p.o_part : p.out);
+            float* lbase = to_part ? p.lse_part : p.lse;
             uint4* dst = reinterpret_cast<uint4*>(obase + (orow * p.h + item.head) * D_V);
             float* lse_dst = lbase + static_cast<int64_t>(item.head) * rows_total + orow;
             const int n_kv = item.n_kv;
@@ -574,12 +584,14 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
 }
 
 cudaError_t HYDRA_K(launch_fwd_short)(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
-                                      const FwdParams& p, int32_t call_tag, bool halves, int grid, cudaStream_t stream)
+                                      const FwdParams& p, const FwdSeg* segs, int32_t call_tag, bool halves, int grid,
+                                      cudaStream_t stream)
 {
-    static OncePerDevice configured[2];
-    const auto kernel = halves ? HYDRA_K(hydra_fwd_short_kernel)<true> : HYDRA_K(hydra_fwd_short_kernel)<false>;
-    if (cudaError_t e = allow_dynamic_smem(kernel, HYDRA_K(fwd_short_smem_bytes)(), configured[halves])) return e;
-    return launch_overlapped(kernel, grid, kThreads, HYDRA_K(fwd_short_smem_bytes)(), stream, mq, mk, mv, p, call_tag);
+    static OncePerDevice configured[4];
+    const auto kernel = segs ? (halves ? HYDRA_K(hydra_fwd_short_kernel)<true, true> : HYDRA_K(hydra_fwd_short_kernel)<false, true>)
+                             : (halves ? HYDRA_K(hydra_fwd_short_kernel)<true, false> : HYDRA_K(hydra_fwd_short_kernel)<false, false>);
+    if (cudaError_t e = allow_dynamic_smem(kernel, HYDRA_K(fwd_short_smem_bytes)(), configured[2 * (segs != nullptr) + halves])) return e;
+    return launch_overlapped(kernel, grid, kThreads, HYDRA_K(fwd_short_smem_bytes)(), stream, mq, mk, mv, p, segs, call_tag);
 }
 
 }  // namespace hydra

@@ -82,9 +82,16 @@ struct alignas(16) FwdShortItem {
     uint8_t to_part;   // 1: partial buffers, 0: out / lse
     uint16_t half;     // 0: all keys of the tile; 1, 2: its first and second part, run by the two slots of one thread
                        // block (the second hands its result to the first)
-    int32_t pad;
+    int32_t segs;      // 0: all rows as above; else index << 8 | number of the FwdSeg that say where the rows go
 };
 static_assert(sizeof(FwdShortItem) == 32, "two 16-byte loads per work item");
+
+// Rows of a tile that belong to one of several pairs: consecutive q chunks that meet the same kv chunk share their tiles.
+struct FwdSeg {
+    int16_t begin;     // first row of the tile; the segment ends where the next one begins
+    int16_t to_part;
+    int32_t delta;     // output row of tile row r is r + delta
+};
 
 // Backward work item: one tile of one chunk and head, visiting every pair that shares the chunk (key side: for
 // BwdParams::item_heads query heads, of which `head` is the first).
@@ -291,7 +298,8 @@ struct MergeParams {
                                    const FwdParams& p, int grid, cudaStream_t stream);                                \
     size_t fwd_short_smem_bytes##SUFFIX();                                                                            \
     cudaError_t launch_fwd_short##SUFFIX(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv_sub,     \
-                                         const FwdParams& p, int32_t call_tag, bool halves, int grid, cudaStream_t stream); \
+                                         const FwdParams& p, const FwdSeg* segs, int32_t call_tag, bool halves, int grid, \
+                                         cudaStream_t stream);                                                        \
     cudaError_t launch_bwd_dq##SUFFIX(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,            \
                                       const CUtensorMap& mdo, const BwdParams& p, int grid, cudaStream_t stream);     \
     cudaError_t launch_bwd_dq_from_ds##SUFFIX(const CUtensorMap& mk, const BwdParams& p, int grid,                    \
