@@ -589,6 +589,28 @@ void hydra_set_fwd_short_len(int32_t len);
  */
 double hydra_plan_build_seconds(int32_t which, const int32_t* cu_seqlens_host, int32_t n_seqs, int32_t n_heads,
                                 const hydra_pair_t* pairs, int32_t n_pairs, int32_t causal);
+/*
+ * Host only (no GPU needed): the work tables that a call of kind `which` (HYDRA_WS_FWD / MERGE / BWD) of hydra_attn_*_dims
+ * would run, for tests and tools that have to know which form a call takes. fields_out [HYDRA_PLAN_FIELDS] is described by
+ * the HYDRA_PLAN_* indices; the tables themselves, in the library's internal layout, are copied to tables_out if capacity > 0
+ * (HYDRA_ERR_WORKSPACE_TOO_SMALL, with fields_out written, if they are larger than that).
+ */
+enum {
+    HYDRA_PLAN_PAIRS = 0,       /* pairs the call works on (backward: after cut sequences have been joined)      */
+    HYDRA_PLAN_ITEMS,           /* work items: CTA-pair forward, merge, query-side backward                      */
+    HYDRA_PLAN_ITEMS2,          /* work items: short-sequence forward, key-side backward                         */
+    HYDRA_PLAN_SHARED,          /* 1: two slots share a q tile (forward), two CTAs a key tile (backward)         */
+    HYDRA_PLAN_GRID,            /* forward, SHARED: thread blocks; each has ITEMS2 / (2 * GRID) rounds           */
+    HYDRA_PLAN_SEGS,            /* forward: entries of the table of tiles that several pairs share               */
+    HYDRA_PLAN_ITEM_HEADS,      /* backward: query heads per key-side item                                       */
+    HYDRA_PLAN_OFF_ITEMS2,      /* byte offsets in the tables, and their size                                    */
+    HYDRA_PLAN_OFF_SEGS,
+    HYDRA_PLAN_BYTES,
+    HYDRA_PLAN_FIELDS
+};
+int32_t hydra_plan_describe(int32_t which, const int32_t* cu_seqlens_host, int32_t n_seqs, int32_t n_heads,
+                            int32_t n_kv_heads, int32_t d_qk, const hydra_pair_t* pairs, int32_t n_pairs, int32_t causal,
+                            int64_t* fields_out, void* tables_out, size_t capacity);
 void hydra_shutdown(void);
 
 #if defined(__GNUC__)

@@ -74,6 +74,8 @@ def _load() -> ctypes.CDLL:
     lib.hydra_set_plan_arena_bytes.restype = None
     lib.hydra_plan_build_seconds.restype = ctypes.c_double
     lib.hydra_plan_build_seconds.argtypes = [i32, vp, i32, i32, vp, i32, i32]
+    lib.hydra_plan_describe.restype = i32
+    lib.hydra_plan_describe.argtypes = [i32, vp, i32, i32, i32, i32, vp, i32, i32, vp, vp, sz]
     lib.hydra_set_plan_prefetch.argtypes = [i32]
     lib.hydra_set_plan_prefetch.restype = None
     lib.hydra_set_fwd_short_len.argtypes = [i32]
@@ -177,6 +179,7 @@ def _load() -> ctypes.CDLL:
 _lib = _load()
 LIBRARY_PATH = _build.OUT
 EXPORTS = ("hydra_version", "hydra_status_string", "hydra_launch_count", "hydra_set_wait_limit_ns", "hydra_debug_stall", "hydra_set_plan_arena_bytes", "hydra_set_plan_prefetch", "hydra_set_fwd_short_len", "hydra_plan_build_seconds",
+           "hydra_plan_describe",
            "hydra_shutdown", "hydra_usp_factor", "hydra_zigzag_pairs", "hydra_workspace_bytes",
            "hydra_attn_fwd", "hydra_lse_merge", "hydra_attn_bwd", "hydra_poll_status",
            "hydra_profile_enable", "hydra_profile_collect", "hydra_host_step_arena_bytes",
@@ -305,6 +308,31 @@ def hydra_plan_build_seconds(which: int, cu_seqlens, n_heads: int, pairs=None, c
     cu = _cu(cu_seqlens)
     pp, npairs, _keep = _pairs_arg(pairs)
     return float(_lib.hydra_plan_build_seconds(which, _addr(cu), len(cu) - 1, n_heads, pp, npairs, int(bool(causal))))
+
+
+PLAN_FIELDS = ("pairs", "items", "items2", "shared", "grid", "segs", "item_heads", "off_items2", "off_segs", "bytes")
+
+
+def hydra_plan_describe(which: int, cu_seqlens, n_heads: int, n_kv_heads: Optional[int] = None, d_qk: int = D_QK, pairs=None,
+                        causal: bool = True, tables: bool = False):
+    """Host-only: the form that a call of kind `which` takes, as a dict of PLAN_FIELDS (HYDRA_PLAN_* in the header), with
+    `tables` also the work tables themselves as an array of bytes."""
+    cu = _cu(cu_seqlens)
+    pp, npairs, _keep = _pairs_arg(pairs)
+    fields = np.zeros(len(PLAN_FIELDS), dtype=np.int64)
+
+    def call(out):
+        _check(_lib.hydra_plan_describe(which, _addr(cu), len(cu) - 1, n_heads, n_heads if n_kv_heads is None else n_kv_heads,
+                                        d_qk, pp, npairs, int(bool(causal)), _addr(fields),
+                                        None if out is None else _addr(out), 0 if out is None else out.size),
+               "hydra_plan_describe")
+    call(None)
+    named = dict(zip(PLAN_FIELDS, fields.tolist()))
+    if not tables:
+        return named
+    out = np.zeros(max(named["bytes"], 1), dtype=np.uint8)
+    call(out)
+    return named, out
 
 
 def hydra_set_plan_prefetch(on: bool) -> None:

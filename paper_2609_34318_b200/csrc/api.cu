@@ -309,12 +309,12 @@ struct Plan {
     std::vector<uint8_t> blob;       // the tables, as they go to the device
     size_t off_pairs = 0, off_items = 0, off_lists = 0, off_groups = 0, off_items2 = 0, off_lists2 = 0;
     int32_t n_items = 0, n_items2 = 0;
-    int32_t halves = 0;              // forward: the short kernel's items are halves of tiles, two per thread block;
+    int32_t halves = 0;              // forward: the short kernel's items are dealt out, longer tiles as a part per slot;
                                      // backward: two CTAs share every key-side item
     int32_t early_pops = 0;          // forward: FwdParams::early_pops
     int32_t short_grid = 0;          // forward, halves: thread blocks the items have been dealt out to
     size_t off_segs = 0;             // forward: FwdSeg table of the short-sequence kernel's items
-    int32_t n_segs = 0;
+    size_t n_segs = 0;
     int32_t item_heads = 1;          // backward: query heads per key-side item (BwdParams::item_heads)
     int64_t ds_head_blocks = 0;      // backward: blocks of the dS hand-off buffer per head; -1: not usable
     // residency on the device (guarded by g_plan_mutex)
@@ -994,12 +994,14 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     // table, a group's entries once and then one copy per head with the head number set.
     // Where the rows of tiles that several pairs share go, once per tile (every head has the same).
     std::vector<FwdSeg> segs;
-    std::map<std::pair<int32_t, int32_t>, int32_t> segs_of;        // (run, first row) -> FwdShortItem::segs
+    std::vector<size_t> tile_segs;                      // first entry of each tile of the shared runs, and the end
+    std::vector<size_t> run_tiles(runs.size(), 0);      // where a run's tiles begin in it
     for (size_t ri = 0; ri < runs.size(); ++ri) {
         const FwdRun& run = runs[ri];
         if (run.pairs.size() < 2) continue;
+        run_tiles[ri] = tile_segs.size();
         for (int32_t q0 = 0; q0 < run.all.q_len; q0 += TILE) {
-            const size_t at = segs.size();
+            tile_segs.push_back(segs.size());
             int32_t first = 0;                          // the pair's first row in the run
             for (int32_t pi : run.pairs) {
                 const int32_t len = pb.pairs[pi].q_len;
@@ -1010,9 +1012,9 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
                 }
                 first += len;
             }
-            segs_of[{static_cast<int32_t>(ri), q0}] = static_cast<int32_t>(at << 8 | (segs.size() - at));
         }
     }
+    tile_segs.push_back(segs.size());
     auto make_short = [&](int32_t a, const GroupEntry& e) {
         const PairDev& d = dev_pairs[runs[e.of].pairs[0]];
         FwdShortItem it{};
@@ -1025,11 +1027,15 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
         it.n_kv = static_cast<uint16_t>(e.b);
         it.rows = static_cast<uint8_t>(e.c);
         it.to_part = static_cast<uint8_t>(d.to_part);
-        if (runs[e.of].pairs.size() > 1) it.segs = segs_of.at({e.of, e.a});
+        if (runs[e.of].pairs.size() > 1) {
+            const size_t* at = &tile_segs[run_tiles[e.of] + e.a / TILE];
+            it.first_seg = static_cast<uint32_t>(at[0]);
+            it.half_segs = static_cast<uint16_t>((at[1] - at[0]) << 8);
+        }
         return it;
     };
     plan.off_segs = append(blob, segs);
-    plan.n_segs = static_cast<int32_t>(segs.size());
+    plan.n_segs = segs.size();
     const int short_workers = 2 * plan_workers(1);
     if (halves) {
         auto entry = [&](const SharedTile& t) {
@@ -1043,9 +1049,9 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
                 const int32_t n0 = (one.steps + 1) / 2, skip = n0 * FWD_SHORT_KEYS;
                 other = it;
                 it.n_kv = static_cast<uint16_t>(n0);
-                it.half = 1;
+                it.half_segs |= 1;
                 other.n_kv = static_cast<uint16_t>(one.steps - n0);
-                other.half = 2;
+                other.half_segs |= 2;
                 other.k_tok0 += skip;
                 other.k_len -= skip;
                 other.off -= skip;
@@ -1584,6 +1590,18 @@ void hydra_set_plan_prefetch(int32_t on) { g_plan_prefetch.store(on != 0); }
 // (a work item counts its 64-key steps in 16 bits)
 void hydra_set_fwd_short_len(int32_t len) { g_fwd_short_len.store(std::min(len, 1 << 21)); }
 
+namespace {
+// The tables of one call of kind `which`, as the call itself builds them.
+bool build_plan(int32_t which, const Problem& pb, int32_t causal, Plan& plan)
+{
+    if (which == HYDRA_WS_FWD) build_fwd(pb, causal != 0, plan, plan.blob);
+    else if (which == HYDRA_WS_MERGE) build_merge(pb, plan, plan.blob);
+    else if (which == HYDRA_WS_BWD) build_bwd(pb, causal != 0, plan, plan.blob);
+    else return false;
+    return true;
+}
+}  // namespace
+
 double hydra_plan_build_seconds(int32_t which, const int32_t* cu, int32_t n_seqs, int32_t n_heads,
                                 const hydra_pair_t* pairs, int32_t n_pairs, int32_t causal)
 {
@@ -1592,11 +1610,35 @@ double hydra_plan_build_seconds(int32_t which, const int32_t* cu, int32_t n_seqs
     pb.fwd_short_set = g_fwd_short_len.load();
     Plan plan;
     const auto t0 = std::chrono::steady_clock::now();
-    if (which == HYDRA_WS_FWD) build_fwd(pb, causal != 0, plan, plan.blob);
-    else if (which == HYDRA_WS_MERGE) build_merge(pb, plan, plan.blob);
-    else if (which == HYDRA_WS_BWD) build_bwd(pb, causal != 0, plan, plan.blob);
-    else return -1.0;
+    if (!build_plan(which, pb, causal, plan)) return -1.0;
     return std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
+}
+
+int32_t hydra_plan_describe(int32_t which, const int32_t* cu, int32_t n_seqs, int32_t n_heads, int32_t n_kv_heads,
+                            int32_t d_qk, const hydra_pair_t* pairs, int32_t n_pairs, int32_t causal,
+                            int64_t* fields_out, void* tables_out, size_t capacity)
+{
+    if (!fields_out || (capacity > 0 && !tables_out)) return HYDRA_ERR_INVALID_ARG;
+    if (!kernel_set(d_qk, D_V)) return HYDRA_ERR_UNSUPPORTED;
+    if (n_kv_heads < 1 || n_heads % n_kv_heads) return HYDRA_ERR_INVALID_ARG;
+    Problem pb;
+    if (int32_t s = make_problem(cu, n_seqs, n_heads, pairs, n_pairs, pb)) return s;
+    pb.dqk = d_qk;
+    pb.kv_group = n_heads / n_kv_heads;
+    pb.fwd_short_set = g_fwd_short_len.load();
+    if (which == HYDRA_WS_BWD) join_chunks(pb, causal);
+    Plan plan;
+    if (!build_plan(which, pb, causal, plan)) return HYDRA_ERR_INVALID_ARG;
+    const int64_t fields[HYDRA_PLAN_FIELDS] = {
+        static_cast<int64_t>(pb.pairs.size()), plan.n_items, plan.n_items2, plan.halves, plan.short_grid,
+        static_cast<int64_t>(plan.n_segs), plan.item_heads, static_cast<int64_t>(plan.off_items2),
+        static_cast<int64_t>(plan.off_segs), static_cast<int64_t>(plan.blob.size())};
+    std::copy(fields, fields + HYDRA_PLAN_FIELDS, fields_out);
+    if (capacity > 0) {
+        if (capacity < plan.blob.size()) return HYDRA_ERR_WORKSPACE_TOO_SMALL;
+        std::memcpy(tables_out, plan.blob.data(), plan.blob.size());
+    }
+    return HYDRA_OK;
 }
 
 int32_t hydra_usp_factor(int32_t degree, int32_t heads, int32_t* cp_u, int32_t* cp_r)

@@ -227,7 +227,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
                     fence_proxy_async_smem();          // (they were ordinary stores, what follows are asynchronous copies)
                     ++shared_tiles;
                 }
-                last_half = cur.half;
+                last_half = cur.half();
                 if (n > 0 && !pre) { load_q(cur); load_k(cur, 0); }
                 if (n > 1) load_k(cur, 1);
                 pre = false;
@@ -245,7 +245,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
                     // The next item's Q and first K tile are released by score products that are long issued
                     // when the last V stage comes free: ask for them first, and show the item to the issuer.
                     if (j == (n >= 2 ? n - 1 : n)) {
-                        if (n >= 2 && nxt_idx >= 0 && nxt.n_kv > 0 && !(kHalves && cur.half == 2)) { load_q(nxt); load_k(nxt, 0); pre = true; }
+                        if (n >= 2 && nxt_idx >= 0 && nxt.n_kv > 0 && !(kHalves && cur.half() == 2)) { load_q(nxt); load_k(nxt, 0); pre = true; }
                         if (ok) publish(kq, nxt_idx, nxt);
                     }
                     if (j >= n) break;
@@ -385,9 +385,9 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
             const bool row_valid = r < item.rows;
             bool to_part = item.to_part != 0;
             int64_t orow = static_cast<int64_t>(item.out_row0) + r;
-            if (kSegs && item.segs) {
-                const FwdSeg* seg = segs + (item.segs >> 8);
-                for (int i = 0; i < (item.segs & 255); ++i) {
+            if (kSegs && item.n_segs()) {
+                const FwdSeg* seg = segs + item.first_seg;
+                for (int i = 0; i < item.n_segs(); ++i) {
                     const FwdSeg one = seg[i];
                     if (r >= one.begin) { to_part = one.to_part != 0; orow = static_cast<int64_t>(one.delta) + r; }
                 }
@@ -496,7 +496,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
             const uint32_t half_buf = smem0 + kSlotBytes + r * 4u;
             constexpr uint32_t kColumn = TILE * 4;
             float mul0 = 1.f, mul1 = 0.f;
-            if (kHalves && item.half == 2) {
+            if (kHalves && item.half() == 2) {
                 st_shared_f32(half_buf + D_V * kColumn, m_run);
                 st_shared_f32(half_buf + (D_V + 1) * kColumn, l_run);
 #pragma unroll 1
@@ -512,7 +512,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
                 mbar_arrive_warp(smem_u32(&bars[B_HALF]));
                 continue;
             }
-            if (kHalves && item.half == 1) {
+            if (kHalves && item.half() == 1) {
                 ok = wait(B_HALF, joined);
                 if (!ok) break;
                 ++joined;
@@ -536,7 +536,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
                     tc_fence_before_sync();
                     mbar_arrive_warp(bar(B_OFREE));
                 }
-                if (kHalves && item.half == 1) {
+                if (kHalves && item.half() == 1) {
 #pragma unroll
                     for (int e = 0; e < 32; ++e)
                         o[e] = __float_as_uint(__uint_as_float(o[e]) * mul0 + ld_shared_f32(half_buf + (c0 + e) * kColumn) * mul1);
@@ -559,7 +559,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
                     }
                 }
             }
-            if (kHalves && item.half == 1) mbar_arrive_warp(bar(B_HALFFREE));
+            if (kHalves && item.half() == 1) mbar_arrive_warp(bar(B_HALFFREE));
             if (row_valid)
                 *lse_dst = (l_run > 0.f) ? (m_run + __log2f(l_run)) * 0.6931471805599453f : neg_inf();
         }

@@ -80,9 +80,13 @@ struct alignas(16) FwdShortItem {
     uint16_t n_kv;     // steps of FWD_SHORT_KEYS keys the tile visits; 0: its rows see no key
     uint8_t rows;      // q rows of the tile that exist (1..128)
     uint8_t to_part;   // 1: partial buffers, 0: out / lse
-    uint16_t half;     // 0: all keys of the tile; 1, 2: its first and second part, run by the two slots of one thread
-                       // block (the second hands its result to the first)
-    int32_t segs;      // 0: all rows as above; else index << 8 | number of the FwdSeg that say where the rows go
+    uint16_t half_segs;    // half() | n_segs() << 8 (one field: with two of a byte the kernel takes 16 registers more)
+    uint32_t first_seg;    // (a call has at most pairs + tiles of them, and of each fewer than 2^31)
+    // 0: all keys of the tile; 1, 2: its first and second part, run by the two slots of one thread block (the second hands its
+    // result to the first)
+    __host__ __device__ int half() const { return half_segs & 255; }
+    // 0: all rows as above; else how many FwdSeg (at most 128), from first_seg on, say where the rows go
+    __host__ __device__ int n_segs() const { return half_segs >> 8; }
 };
 static_assert(sizeof(FwdShortItem) == 32, "two 16-byte loads per work item");
 
