@@ -1432,7 +1432,7 @@ struct KernelSet {
     int (*fwd_max_clusters)();
     cudaError_t (*launch_fwd)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const FwdParams&, int,
                               cudaStream_t);
-    cudaError_t (*launch_fwd_short)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const FwdParams&, const FwdSeg*, int32_t, bool, int,
+    cudaError_t (*launch_fwd_short)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const FwdParams&, const FwdSeg*, uint64_t, bool, int,
                                     cudaStream_t);
     cudaError_t (*launch_bwd_dq)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const CUtensorMap&,
                                  const BwdParams&, int, cudaStream_t);
@@ -1867,6 +1867,22 @@ int32_t hydra_attn_fwd_local(const void* q, const void* k, const void* v, const 
 }
 
 namespace {
+// A number that no other call of this process has and that a workspace holds by chance once in 2^64: the calls counted from a
+// start of the process's own, in steps and mixed as in splitmix64 (Steele, Lea and Flood, 2014), a one-to-one function. Not 0.
+uint64_t next_call_tag()
+{
+    static std::atomic<uint64_t> calls{static_cast<uint64_t>(std::chrono::system_clock::now().time_since_epoch().count()) ^
+                                       static_cast<uint64_t>(std::chrono::steady_clock::now().time_since_epoch().count()) << 20};
+    uint64_t x;
+    do {
+        x = calls.fetch_add(0x9e3779b97f4a7c15ull);
+        x = (x ^ (x >> 30)) * 0xbf58476d1ce4e5b9ull;
+        x = (x ^ (x >> 27)) * 0x94d049bb133111ebull;
+        x ^= x >> 31;
+    } while (x == 0);
+    return x;
+}
+
 int32_t fwd_core(Problem& pb, const void* q, const void* k, const void* v, int32_t n_kv_heads, int32_t causal,
                  float softmax_scale, void* out, float* lse, void* o_part, float* lse_part, int64_t part_rows,
                  void* workspace, size_t workspace_bytes, void* cuda_stream)
@@ -1898,16 +1914,14 @@ int32_t fwd_core(Problem& pb, const void* q, const void* k, const void* v, int32
     // One item per SM before any SM gets two, or what the items have been dealt out to.
     const int short_grid = plan->halves ? plan->short_grid : std::min(sms, plan->n_items2);
     FwdParams fp{};
-    int32_t call_tag = 0;
+    uint64_t call_tag = 0;
     // With no more items than slots nothing is popped from the queue, and the block at the workspace's start need not be
     // cleared (one launch less: four sequences of 7 to 300 tokens, forward 11.5 -> 9.4 us). Not where the launches are
     // recorded: every replay would have the number of the first.
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) return HYDRA_ERR_CUDA;
     if (capturing == cudaStreamCaptureStatusNone && plan->n_items == 0 && (plan->halves || plan->n_items2 <= 2 * short_grid)) {
-        static std::atomic<uint32_t> calls{0};
-        do call_tag = static_cast<int32_t>(calls.fetch_add(1) + 1u);
-        while (call_tag == 0);
+        call_tag = next_call_tag();
     } else if (launch_reset(static_cast<StatusBlock*>(workspace), false, stream) != cudaSuccess) {
         return HYDRA_ERR_CUDA;
     }

@@ -102,7 +102,7 @@ template <bool kHalves, bool kSegs>
 __global__ void __launch_bounds__(kThreads, 1)
 HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                                 const __grid_constant__ CUtensorMap map_v, const FwdParams p,
-                                const FwdSeg* segs, const int32_t call_tag)
+                                const FwdSeg* segs, const uint64_t call_tag)
 {
     overlap_next_launch();
     extern __shared__ uint8_t smem_raw[];
@@ -584,7 +584,7 @@ HYDRA_K(hydra_fwd_short_kernel)(const __grid_constant__ CUtensorMap map_q, const
 }
 
 cudaError_t HYDRA_K(launch_fwd_short)(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
-                                      const FwdParams& p, const FwdSeg* segs, int32_t call_tag, bool halves, int grid,
+                                      const FwdParams& p, const FwdSeg* segs, uint64_t call_tag, bool halves, int grid,
                                       cudaStream_t stream)
 {
     static OncePerDevice configured[4];

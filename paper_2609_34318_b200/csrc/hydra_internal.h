@@ -119,15 +119,18 @@ struct MergeItem {
 };
 constexpr int MERGE_ROWS = 8;   // rows of a merge block
 
-struct StatusBlock {            // lives at the start of the workspace; zeroed before every call
+// Lives at the start of the workspace. Zeroed before the kernels of a call, except in forward calls with a call_tag, whose
+// workspace keeps what it held: there next_item is undefined and `status` counts as said below.
+struct StatusBlock {
     int32_t status;
     int32_t pad;
     int64_t detail;
     int32_t next_item[4];       // work-queue heads of the persistent kernels (forward, dK/dV, dQ, short forward)
     // A call none of whose kernels pops from a queue is not worth a launch that clears this block. Its kernel writes call_tag,
     // a number of the call's own, and with an error the same number as error_tag; `status` counts only while the two are
-    // equal, as they are (zero) wherever the block is cleared.
-    int32_t call_tag, error_tag;
+    // equal, as they are (zero) wherever the block is cleared. (64 mixed bits: a workspace may hold anything, and small
+    // numbers, which positions or token ids leave there, were taken for the first calls' own.)
+    uint64_t call_tag, error_tag;
     // SM clock seen from inside the tensor-core kernels: cycles and nanoseconds that passed in the
     // producer thread of CTA 0 between its first and its last instruction (same index as next_item)
     uint64_t probe_cycles[4];
@@ -302,7 +305,7 @@ struct MergeParams {
                                    const FwdParams& p, int grid, cudaStream_t stream);                                \
     size_t fwd_short_smem_bytes##SUFFIX();                                                                            \
     cudaError_t launch_fwd_short##SUFFIX(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv_sub,     \
-                                         const FwdParams& p, const FwdSeg* segs, int32_t call_tag, bool halves, int grid, \
+                                         const FwdParams& p, const FwdSeg* segs, uint64_t call_tag, bool halves, int grid, \
                                          cudaStream_t stream);                                                        \
     cudaError_t launch_bwd_dq##SUFFIX(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,            \
                                       const CUtensorMap& mdo, const BwdParams& p, int grid, cudaStream_t stream);     \

@@ -59,3 +59,31 @@ def test_any_workspace_will_do(lengths, h, fill):
             assert P.hydra_poll_status(ws)[0] == P.HYDRA_OK
             assert torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1])
     P.hydra_shutdown()
+
+
+SMALL_NUMBERS = """
+import numpy as np, torch
+import hydra_workloads as hw
+import paper_2609_34318_b200 as P
+cu = hw.cu_seqlens([7, 33])
+q, k, v = (torch.ones((40, 2, d), dtype=torch.bfloat16, device="cuda") for d in (hw.D_QK, hw.D_QK, hw.D_V))
+out, lse = torch.empty((40, 2, hw.D_V), dtype=torch.bfloat16, device="cuda"), torch.empty((2, 40), device="cuda")
+got = []
+for n in range(1, 9):                                  # the workspace held int32 tensors (positions, token ids) before
+    ws = torch.full((1024,), n, dtype=torch.int32, device="cuda").view(torch.uint8)
+    P.hydra_attn_fwd(q, k, v, cu, 2, None, True, 0.07, out, lse, None, None, 0, ws)
+    got.append(P.hydra_poll_status(ws)[0])
+print(got)
+assert got == [P.HYDRA_OK] * 8
+"""
+
+
+def test_small_numbers_in_the_workspace_are_no_error():
+    """The first calls of a process, in workspaces that hold a small number all over: the number of the call must not be one
+    that ordinary data hold."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    run = subprocess.run([sys.executable, "-c", SMALL_NUMBERS], capture_output=True, text=True, timeout=300, cwd=root)
+    assert run.returncode == 0, run.stdout + run.stderr
