@@ -584,7 +584,8 @@ void hydra_set_plan_prefetch(int32_t on);
 void hydra_set_fwd_short_len(int32_t len);
 /*
  * Host only (no GPU needed): seconds the host takes to build the work tables of one call of kind `which`
- * (HYDRA_WS_FWD / MERGE / BWD) for this problem, uncached. What a new cu_seqlens costs before its first launch.
+ * (HYDRA_WS_FWD / MERGE / BWD) for this problem, uncached. What a new cu_seqlens costs before its first launch. As in the
+ * call itself, the backward's tables are those of the pairs after cut sequences have been joined.
  * Negative on invalid arguments.
  */
 double hydra_plan_build_seconds(int32_t which, const int32_t* cu_seqlens_host, int32_t n_seqs, int32_t n_heads,

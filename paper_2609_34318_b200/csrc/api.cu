@@ -1592,8 +1592,9 @@ void hydra_set_fwd_short_len(int32_t len) { g_fwd_short_len.store(std::min(len, 
 
 namespace {
 // The tables of one call of kind `which`, as the call itself builds them.
-bool build_plan(int32_t which, const Problem& pb, int32_t causal, Plan& plan)
+bool build_plan(int32_t which, Problem& pb, int32_t causal, Plan& plan)
 {
+    if (which == HYDRA_WS_BWD) join_chunks(pb, causal);
     if (which == HYDRA_WS_FWD) build_fwd(pb, causal != 0, plan, plan.blob);
     else if (which == HYDRA_WS_MERGE) build_merge(pb, plan, plan.blob);
     else if (which == HYDRA_WS_BWD) build_bwd(pb, causal != 0, plan, plan.blob);
@@ -1626,7 +1627,6 @@ int32_t hydra_plan_describe(int32_t which, const int32_t* cu, int32_t n_seqs, in
     pb.dqk = d_qk;
     pb.kv_group = n_heads / n_kv_heads;
     pb.fwd_short_set = g_fwd_short_len.load();
-    if (which == HYDRA_WS_BWD) join_chunks(pb, causal);
     Plan plan;
     if (!build_plan(which, pb, causal, plan)) return HYDRA_ERR_INVALID_ARG;
     const int64_t fields[HYDRA_PLAN_FIELDS] = {

@@ -81,3 +81,13 @@ def test_the_workspace_holds_either_form():
         for h, hk, d in ((4, 4, 192), (8, 2, 128)):
             cut = P.hydra_workspace_bytes_dims(P.HYDRA_WS_BWD, cu, h, hk, d, 128, pairs)
             assert cut >= P.hydra_workspace_bytes_dims(P.HYDRA_WS_BWD, cu, h, hk, d, 128, None)
+
+
+def test_the_plan_timer_times_the_tables_that_the_call_builds():
+    """Sequences cut in 64 chunks have 2080 pairs each, or one, joined: without a mask all are listed."""
+    cu = np.arange(0, 101 * 512, 512, dtype=np.int32)
+    pairs, _, _, _ = P.hydra_zigzag_pairs(cu, 32)
+    assert P.hydra_plan_describe(P.HYDRA_WS_BWD, cu, 2, pairs=pairs)["pairs"] == 100
+    assert P.hydra_plan_describe(P.HYDRA_WS_BWD, cu, 2, pairs=pairs, causal=False)["pairs"] == len(pairs)
+    best = lambda causal: min(P.hydra_plan_build_seconds(P.HYDRA_WS_BWD, cu, 2, pairs, causal) for _ in range(5))
+    assert 2 * best(True) < best(False)
