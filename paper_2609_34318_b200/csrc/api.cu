@@ -197,10 +197,11 @@ bool join_chunks(Problem& pb, int32_t causal)
     by_q.reserve(pb.pairs.size());
     for (const auto& p : pb.pairs)
         if (p.q_len > 0 && p.k_len > 0) by_q.push_back(p);
-    std::sort(by_q.begin(), by_q.end(), [](const hydra_pair_t& a, const hydra_pair_t& b) {
+    auto less = [](const hydra_pair_t& a, const hydra_pair_t& b) {
         if (a.seq != b.seq) return a.seq < b.seq;
         return a.q_start != b.q_start ? a.q_start < b.q_start : a.k_start < b.k_start;
-    });
+    };
+    if (!std::is_sorted(by_q.begin(), by_q.end(), less)) std::sort(by_q.begin(), by_q.end(), less);     // (every call comes here)
     std::vector<hydra_pair_t> joined;
     bool any = false;
     for (size_t i = 0, j = 0; i < by_q.size(); i = j) {
@@ -732,7 +733,10 @@ GroupOrder order_groups(std::vector<std::vector<GroupEntry>>& groups, int32_t h,
             const int32_t g = go.order[--tail];
             left -= (group_cost[g] + static_cast<int64_t>(groups[g].size()) * kItemOverhead) * h;
         }
-        std::sort(go.order.begin(), go.order.begin() + static_cast<int64_t>(tail));
+        std::vector<uint8_t> early(groups.size(), 0);
+        for (size_t i = 0; i < tail; ++i) early[go.order[i]] = 1;
+        for (size_t g = 0, i = 0; g < groups.size(); ++g)       // (they are in order already: no sort)
+            if (early[g]) go.order[i++] = static_cast<int32_t>(g);
     }
     return go;
 }
@@ -766,48 +770,61 @@ inline int32_t kv_steps_short(const hydra_pair_t& p, int32_t q0, int32_t rows, i
 
 // What the short-sequence forward makes its q tiles of: a pair, or consecutive q chunks that meet the same kv chunk, where that
 // saves tiles (a chunk's last tile is ragged: sequences of 121 tokens in chunks of 30 have ten tiles pair by pair, four by kv
-// chunk). `all` has the sum of the pairs' rows; `pairs` are their indices in order.
+// chunk). `all` has the sum of the pairs' rows.
 // Forward, pair by pair / shared, us: 30000 tokens of 64 to 512, 16 heads, ring of 4 628 / 347, 12 sequences of 121 tokens, 16
 // heads, ring of 2 28.8 / 22.6, 26283 log-normal tokens, 16 heads, ring of 4 710 / 619, 65536 of 64 to 512, 32 heads, cut in two
 // 831 / 804.
+// Where no pair has partial rows the pairs are the runs, in their order.
 struct FwdRun {
     hydra_pair_t all;
-    std::vector<int32_t> pairs;
+    int32_t first, n;       // its pairs: FwdRuns::order[first .. first + n)
 };
-std::vector<FwdRun> make_runs(const Problem& pb, const std::vector<uint8_t>& wanted)
-{
-    std::vector<int32_t> order;
-    for (size_t i = 0; i < pb.pairs.size(); ++i)
-        if (wanted[i] && pb.pairs[i].q_len > 0) order.push_back(static_cast<int32_t>(i));
-    bool cut = false;
-    for (int32_t i : order) cut = cut || pb.pairs[i].part_row >= 0;
-    auto key = [&](int32_t i) {
-        const auto& p = pb.pairs[i];
-        return std::make_tuple(p.seq, p.k_start, p.k_len, p.q_start);
-    };
-    if (cut) std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return key(x) < key(y); });
-    auto tiles = [](int32_t rows) { return (rows + TILE - 1) / TILE; };
+struct FwdRuns {
     std::vector<FwdRun> runs;
-    for (size_t i = 0, j = 0; i < order.size(); i = j) {
-        FwdRun run{pb.pairs[order[i]], {order[i]}};
-        int32_t separate = tiles(run.all.q_len);
-        for (j = i + 1; cut && j < order.size(); ++j) {
-            const auto& p = pb.pairs[order[j]];
-            if (p.seq != run.all.seq || p.k_start != run.all.k_start || p.k_len != run.all.k_len ||
-                p.q_start != run.all.q_start + run.all.q_len ||
-                pb.q_row(p.seq, p.q_start) != pb.q_row(p.seq, run.all.q_start) + run.all.q_len)
-                break;
-            run.all.q_len += p.q_len;
-            separate += tiles(p.q_len);
-            run.pairs.push_back(order[j]);
+    std::vector<int32_t> order;
+    bool cut = false;       // some pair has partial rows
+};
+FwdRuns make_runs(const Problem& pb, const std::vector<uint8_t>& wanted)
+{
+    FwdRuns r;
+    r.order.reserve(pb.pairs.size());
+    for (size_t i = 0; i < pb.pairs.size(); ++i)
+        if (wanted[i] && pb.pairs[i].q_len > 0) {
+            r.order.push_back(static_cast<int32_t>(i));
+            r.cut = r.cut || pb.pairs[i].part_row >= 0;
         }
-        if (run.pairs.size() > 1 && tiles(run.all.q_len) == separate) {     // nothing saved
-            for (int32_t one : run.pairs) runs.push_back(FwdRun{pb.pairs[one], {one}});
+    r.runs.reserve(r.order.size());
+    auto alone = [&](size_t i) { r.runs.push_back(FwdRun{pb.pairs[r.order[i]], static_cast<int32_t>(i), 1}); };
+    if (!r.cut) {
+        for (size_t i = 0; i < r.order.size(); ++i) alone(i);
+        return r;
+    }
+    auto less = [&](int32_t x, int32_t y) {
+        const auto &a = pb.pairs[x], &b = pb.pairs[y];
+        if (a.seq != b.seq) return a.seq < b.seq;
+        if (a.k_start != b.k_start) return a.k_start < b.k_start;
+        return a.k_len != b.k_len ? a.k_len < b.k_len : a.q_start < b.q_start;
+    };
+    std::stable_sort(r.order.begin(), r.order.end(), less);
+    auto tiles = [](int32_t rows) { return (rows + TILE - 1) / TILE; };
+    for (size_t i = 0, j = 0; i < r.order.size(); i = j) {
+        hydra_pair_t all = pb.pairs[r.order[i]];
+        int32_t separate = tiles(all.q_len);
+        for (j = i + 1; j < r.order.size(); ++j) {
+            const auto& p = pb.pairs[r.order[j]];
+            if (p.seq != all.seq || p.k_start != all.k_start || p.k_len != all.k_len || p.q_start != all.q_start + all.q_len ||
+                pb.q_row(p.seq, p.q_start) != pb.q_row(p.seq, all.q_start) + all.q_len)
+                break;
+            all.q_len += p.q_len;
+            separate += tiles(p.q_len);
+        }
+        if (tiles(all.q_len) < separate) {
+            r.runs.push_back(FwdRun{all, static_cast<int32_t>(i), static_cast<int32_t>(j - i)});
             continue;
         }
-        runs.push_back(std::move(run));
+        for (size_t t = i; t < j; ++t) alone(t);        // one pair, or nothing saved
     }
-    return runs;
+    return r;
 }
 
 // Tiles whose keys the two slots of a thread block share (short-sequence forward, calls of few tiles), dealt out longest first,
@@ -883,7 +900,8 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
         most_keys = std::max(most_keys, p.k_len);
         within = within && p.q_len <= short_len && p.k_len <= short_len;
     }
-    std::vector<FwdRun> runs = make_runs(pb, std::vector<uint8_t>(pb.pairs.size(), 1));
+    FwdRuns made = make_runs(pb, std::vector<uint8_t>(pb.pairs.size(), 1));
+    const std::vector<FwdRun>& runs = made.runs;
     for (const FwdRun& run : runs) n_tiles += (run.all.q_len + TILE - 1) / TILE;
     n_tiles *= pb.h;
     std::vector<SharedTile> tiles;
@@ -934,9 +952,10 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     int32_t longest_tile = 0;
     int64_t short_cost = 0;
     std::vector<std::vector<GroupEntry>> groups(pb.n_seqs), groups_short(pb.n_seqs);
-    if (!halves) runs = make_runs(pb, is_short);
+    if (made.cut && std::find(is_short.begin(), is_short.end(), 0) != is_short.end()) made = make_runs(pb, is_short);
     for (size_t ri = 0; ri < runs.size(); ++ri) {
         const auto& p = runs[ri].all;
+        if (!is_short[made.order[runs[ri].first]]) continue;
         for (int32_t q0 = 0; q0 < p.q_len; q0 += TILE) {
             const int32_t rows = std::min(TILE, p.q_len - q0);
             const int32_t n_kv = kv_steps_short(p, q0, rows, causal);
@@ -998,13 +1017,13 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     std::vector<size_t> run_tiles(runs.size(), 0);      // where a run's tiles begin in it
     for (size_t ri = 0; ri < runs.size(); ++ri) {
         const FwdRun& run = runs[ri];
-        if (run.pairs.size() < 2) continue;
+        if (run.n < 2) continue;
         run_tiles[ri] = tile_segs.size();
         for (int32_t q0 = 0; q0 < run.all.q_len; q0 += TILE) {
             tile_segs.push_back(segs.size());
             int32_t first = 0;                          // the pair's first row in the run
-            for (int32_t pi : run.pairs) {
-                const int32_t len = pb.pairs[pi].q_len;
+            for (int32_t t = run.first; t < run.first + run.n; ++t) {
+                const int32_t pi = made.order[t], len = pb.pairs[pi].q_len;
                 if (first < q0 + TILE && first + len > q0) {
                     const int32_t begin = std::max(0, first - q0);
                     segs.push_back(FwdSeg{static_cast<int16_t>(begin), static_cast<int16_t>(dev_pairs[pi].to_part),
@@ -1016,7 +1035,8 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     }
     tile_segs.push_back(segs.size());
     auto make_short = [&](int32_t a, const GroupEntry& e) {
-        const PairDev& d = dev_pairs[runs[e.of].pairs[0]];
+        const FwdRun& run = runs[e.of];
+        const PairDev& d = dev_pairs[made.order[run.first]];
         FwdShortItem it{};
         it.q_tok0 = d.q_tok0 + e.a;
         it.k_tok0 = d.k_tok0;
@@ -1027,7 +1047,7 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
         it.n_kv = static_cast<uint16_t>(e.b);
         it.rows = static_cast<uint8_t>(e.c);
         it.to_part = static_cast<uint8_t>(d.to_part);
-        if (runs[e.of].pairs.size() > 1) {
+        if (run.n > 1) {
             const size_t* at = &tile_segs[run_tiles[e.of] + e.a / TILE];
             it.first_seg = static_cast<uint32_t>(at[0]);
             it.half_segs = static_cast<uint16_t>((at[1] - at[0]) << 8);
@@ -1356,18 +1376,17 @@ int32_t PlanLease::acquire(int kind, const Problem& pb, int causal, cudaStream_t
 // A forward of a new problem is followed, in training, by the merge and the backward of the same problem:
 // their tables are built on the host right after the forward kernel has been launched, while the GPU runs
 // it, instead of when their own calls arrive and the GPU has nothing to do (host work only: nothing is
-// uploaded). hydra_set_plan_prefetch(0) switches this off for forward-only use.
+// uploaded). hydra_set_plan_prefetch(0) switches this off for forward-only use. (The last use of `pb`: its pairs are joined.)
 std::atomic<int> g_plan_prefetch{1};
-void prefetch_plans(const Problem& pb, int causal, bool any_part)
+void prefetch_plans(Problem& pb, int causal, bool any_part)
 {
     if (!g_plan_prefetch.load()) return;
     int device = 0;
     if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return;
     std::lock_guard<std::mutex> lock(g_plan_mutex);
     if (any_part) find_or_build_plan(HYDRA_WS_MERGE, device, pb, 0);
-    Problem whole = pb;
-    join_chunks(whole, causal);                            // as the backward will
-    find_or_build_plan(HYDRA_WS_BWD, device, whole, causal);
+    join_chunks(pb, causal);                               // as the backward will
+    find_or_build_plan(HYDRA_WS_BWD, device, pb, causal);
 }
 
 // ---------------------------------------------------------------------------------------------

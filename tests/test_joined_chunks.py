@@ -91,3 +91,12 @@ def test_the_plan_timer_times_the_tables_that_the_call_builds():
     assert P.hydra_plan_describe(P.HYDRA_WS_BWD, cu, 2, pairs=pairs, causal=False)["pairs"] == len(pairs)
     best = lambda causal: min(P.hydra_plan_build_seconds(P.HYDRA_WS_BWD, cu, 2, pairs, causal) for _ in range(5))
     assert 2 * best(True) < best(False)
+
+
+def test_pairs_in_any_order_are_joined():
+    cu = np.array([0, 400, 700, 701], dtype=np.int32)
+    pairs, _, _, _ = P.hydra_zigzag_pairs(cu, 2)
+    turned = pairs[::-1].copy()
+    turned["group"] = pairs["group"].max() - turned["group"]
+    for got in (P.hydra_bwd_bands(cu, 4, turned, True, ROOM)[0], P.hydra_bwd_bands(cu, 4, pairs, True, ROOM)[0]):
+        assert [(int(p["seq"]), int(p["q_len"]), int(p["k_len"])) for p in got] == [(0, 400, 400), (1, 300, 300), (2, 1, 1)]

@@ -36,12 +36,16 @@ def rows_of(item, segs):
     return to_part, row
 
 
+@pytest.mark.parametrize("turned", [False, True])
 @pytest.mark.parametrize("lengths,cp_r,h", [
     ([121] * 6, 2, 3), ([7, 300, 129, 16], 4, 2), ([290] * 40, 1, 6), ([1280], 1, 16), ([1280, 30], [2, 0], 20), ([700, 1, 64], 0, 4),
 ])
-def test_every_row_goes_to_its_own_pair_once(all_pairs_short, lengths, cp_r, h):
+def test_every_row_goes_to_its_own_pair_once(all_pairs_short, lengths, cp_r, h, turned):
     cu = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
     pairs, rows, _, _ = P.hydra_zigzag_pairs(cu, cp_r)
+    if turned:                                         # groups may be listed in any order
+        pairs = pairs[::-1].copy()
+        pairs["group"] = pairs["group"].max() - pairs["group"]
     plan, items, segs = tables(cu, h, pairs)
     assert plan["items"] == 0
     seen = {True: np.zeros((h, rows), np.int64), False: np.zeros((h, int(cu[-1])), np.int64)}
