@@ -7,19 +7,25 @@ import torch
 import hydra_workloads as hw
 import oracle
 from gpu_util import check, pairs_for
+from test_plan_tables import tables
 
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("lengths,h,h_kv,d_qk,cp_r,causal", [
-    ([1300], 16, 16, 192, 0, True),                # 176 tiles, the longest in 21 steps
-    ([1100, 383, 64, 7, 129], 12, 12, 192, 0, True),   # long and short tiles in one call
-    ([1537], 18, 2, 128, 0, True),
-    ([2050], 14, 14, 192, 0, True),                # the last tile has two rows
-    ([1280], 20, 4, 192, 1, True),                 # chunk pairs, merged
-    ([900, 500], 14, 14, 128, 0, False),
+# shared: the most shared tiles of a thread block on 148 SMs, 0: the call goes to the queue
+@pytest.mark.parametrize("lengths,h,h_kv,d_qk,cp_r,causal,shared", [
+    ([1300], 16, 16, 192, 0, True, 1),             # 176 tiles, the longest in 21 steps
+    ([1100, 383, 64, 7, 129], 12, 12, 192, 0, True, 1),    # long and short tiles in one call
+    ([1537], 18, 2, 128, 0, True, 2),
+    ([2050], 14, 14, 192, 0, True, 2),             # the last tile has two rows
+    ([1280], 20, 4, 192, 1, True, 0),              # chunk pairs, merged
+    ([900, 500], 14, 14, 128, 0, False, 2),
+    ([10240], 4, 2, 128, 0, True, 3),              # the waits on a part come round to their first phase again
+    ([7992], 1, 1, 128, 2, True, 2),               # cut: tiles that hold rows of several pairs, shared
+    ([8166, 2216], 1, 1, 192, 2, True, 3),
+    ([3391, 7186], 2, 2, 192, [2, 1], True, 4),
 ])
-def test_tiles_dealt_out_and_shared(lengths, h, h_kv, d_qk, cp_r, causal):
+def test_tiles_dealt_out_and_shared(lengths, h, h_kv, d_qk, cp_r, causal, shared):
     import paper_2609_34318_b200 as P
     from paper_2609_34318_b200.runner import bits_to_tensor
     cu = hw.cu_seqlens(lengths)
@@ -28,6 +34,11 @@ def test_tiles_dealt_out_and_shared(lengths, h, h_kv, d_qk, cp_r, causal):
     x = {n: hw.f32_to_bf16_bits(rng.standard_normal((T, heads, d)).astype(np.float32))
          for n, heads, d in (("q", h, d_qk), ("k", h_kv, d_qk), ("v", h_kv, hw.D_V))}
     pairs, rows, _ = pairs_for(cu, cp_r) if cp_r else (None, 0, None)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        plan, items, segs = tables(cu, h, pairs, causal, h_kv, d_qk)
+        halves = items.reshape(-1, 2, plan["grid"])[:, 0]["half"] if plan["shared"] else np.zeros((1, 1))
+        assert (halves == 1).sum(axis=0).max() == shared
+        assert (len(segs) > 0) == (cp_r != 0 and shared > 0)
     scale = float(np.float32(1.0 / np.sqrt(np.float32(d_qk))))
     q, k, v = (bits_to_tensor(x[n]) for n in ("q", "k", "v"))
     ws = torch.randint(0, 256, (4096,), dtype=torch.uint8, device="cuda")

@@ -1,5 +1,6 @@
 """Key-side items that take several query heads of a K / V head (calls with many key tiles) and the sums in fp32 that other
-calls need, against the oracle: whole groups, part of a group, ragged tiles, cut sequences, heads of 192 and of 128."""
+calls need, against the oracle: whole groups, part of a group, ragged tiles, cut sequences (whose pairs are joined; several pairs
+per item: test_gpu_listed_pairs_backward), heads of 192 and of 128."""
 import numpy as np
 import pytest
 
@@ -11,14 +12,15 @@ pytestmark = pytest.mark.gpu
 DV = hw.D_V
 
 
-@pytest.mark.parametrize("lengths,h,h_kv,d_qk,cp_r", [
-    ([130] * 50, 8, 2, 192, 0),                    # 100 tiles of 2 K / V heads: every item holds a whole group
-    ([257, 64, 300] * 14, 8, 1, 128, 0),
-    ([300] * 24, 4, 2, 192, 1),                    # cut sequences: an item visits several pairs per head
-    ([1500, 700], 8, 2, 192, 0),                   # few long tiles: parts of a group, summed in fp32
-    ([129, 1, 64], 4, 1, 128, 0),                  # fewer tiles than SMs
+@pytest.mark.parametrize("lengths,h,h_kv,d_qk,cp_r,item_heads", [
+    ([130] * 50, 8, 2, 192, 0, 4),                 # 100 tiles of 2 K / V heads: every item holds a whole group
+    ([257, 64, 300] * 14, 8, 1, 128, 0, 4),        # two items per group
+    ([300] * 24, 4, 2, 192, 1, 2),                 # cut sequences, whose pairs are joined
+    ([1500, 700], 8, 2, 192, 0, 1),                # few long tiles: an item per query head, summed in fp32
+    ([600] * 8, 16, 1, 128, 0, 4),                 # four items per group, summed in fp32
+    ([129, 1, 64], 4, 1, 128, 0, 4),               # fewer tiles than SMs
 ])
-def test_items_of_several_query_heads(lengths, h, h_kv, d_qk, cp_r):
+def test_items_of_several_query_heads(lengths, h, h_kv, d_qk, cp_r, item_heads):
     import torch
     import paper_2609_34318_b200 as P
     from paper_2609_34318_b200.runner import bits_to_tensor
@@ -28,6 +30,7 @@ def test_items_of_several_query_heads(lengths, h, h_kv, d_qk, cp_r):
     x = {n: hw.f32_to_bf16_bits(rng.standard_normal((T, heads, d)).astype(np.float32))
          for n, heads, d in (("q", h, d_qk), ("k", h_kv, d_qk), ("v", h_kv, DV), ("do", h, DV))}
     lib_pairs, rows, ora_pairs = pairs_for(cu, cp_r) if cp_r else (None, 0, None)
+    assert P.hydra_plan_describe(P.HYDRA_WS_BWD, cu, h, h_kv, d_qk, lib_pairs)["item_heads"] == item_heads
     scale = float(np.float32(1.0 / np.sqrt(np.float32(d_qk))))
     q, k, v, do = (bits_to_tensor(x[n]) for n in ("q", "k", "v", "do"))
     out = torch.empty((T, h, DV), dtype=torch.bfloat16, device="cuda")
@@ -59,6 +62,7 @@ def test_items_of_several_query_heads(lengths, h, h_kv, d_qk, cp_r):
     for g in got:
         check(dict(out=f64(out), lse=f64(lse), dq=f64(g[0]), dk=f64(g[1]), dv=f64(g[2])),
               dict(out=o_ref, lse=l_ref, dq=ref[0], dk=ref[1], dv=ref[2]), label=f"{len(lengths)} sequences, {h}/{h_kv} heads: ")
-    if len(lengths) >= 24:                         # whole groups: nothing is added in memory, the sums do not depend on timing
+    # one item per row: nothing is added in memory; two: both orders of two additions to zero give the same sum
+    if h // h_kv <= 2 * item_heads:
         for a, b in zip(*got):
             assert torch.equal(a, b)

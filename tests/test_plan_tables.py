@@ -17,8 +17,8 @@ def all_pairs_short():
     P.hydra_set_fwd_short_len(-1)
 
 
-def tables(cu, h, pairs, causal=True):
-    plan, raw = P.hydra_plan_describe(P.HYDRA_WS_FWD, cu, h, pairs=pairs, causal=causal, tables=True)
+def tables(cu, h, pairs, causal=True, h_kv=None, d_qk=192):
+    plan, raw = P.hydra_plan_describe(P.HYDRA_WS_FWD, cu, h, h_kv, d_qk, pairs, causal, tables=True)
     items = raw[plan["off_items2"]:][:plan["items2"] * ITEM.itemsize].view(ITEM)
     segs = raw[plan["off_segs"]:][:plan["segs"] * SEG.itemsize].view(SEG)
     return plan, items, segs
