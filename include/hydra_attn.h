@@ -20,9 +20,10 @@
  *     arena (see hydra_set_plan_arena_bytes): a new (cu_seqlens, pairs, h) combination costs host
  *     work and an asynchronous copy on `cuda_stream`, no allocation and no wait.
  *   - The caller owns all tensors and the workspace; the library keeps no caller pointer.
- *   - A workspace carries the status word and the work-queue counters of the kernels of one call:
- *     each call clears them (on its stream) before it launches, so calls that may run at the same
- *     time need workspaces of their own; calls on one stream may share one.
+ *   - A workspace carries the status word and the work-queue counters of the kernels of one call,
+ *     whatever it held before: each call clears them (on its stream) before its kernels, or, where
+ *     none of them pops from a queue, marks the status word as its own. So calls that may run at the
+ *     same time need workspaces of their own; calls on one stream may share one.
  *   - Inputs must be finite: a tile that straddles the end of a sequence reads (and masks) the
  *     rows of its neighbour, and 0 * NaN is NaN.
  *   - Only compute capability 10.0 is supported; there is no fallback path.
@@ -117,6 +118,11 @@ int32_t hydra_zigzag_pairs(const int32_t* cu_seqlens_host, int32_t n_seqs, const
  * which both apply. The size assumes a causal call; a non-causal call needs about twice the buffer
  * and falls back to recomputation in a workspace sized here.
  *
+ * Cut sequences: the backward sums over pairs, so in a causal call (packed layout) a sequence whose pairs cover its causal
+ * triangle, every visible position once, runs as ONE pair, the sequence uncut. HYDRA_WS_BWD is the larger of the sizes of the
+ * pairs as listed and of the joined ones; the scratch limit, the banded form and hydra_bwd_bands go by the joined ones. Pairs
+ * with something missing or twice, calls without a mask and local layouts run as listed.
+ *
  * Banded form, for problems whose dS buffer is over that limit (long sequences). The band scratch is set
  * with hydra_set_bwd_band_scratch(bytes): a byte count >= 1 MiB, 0 (bands off), or HYDRA_BAND_AUTO (the
  * default): as much as the dS limit, for problems whose whole dS buffer is at most 16 times the limit
@@ -140,7 +146,8 @@ void hydra_set_bwd_band_scratch(uint64_t bytes);
  * Host only: the bands the banded backward would run for this problem with `scratch_bytes` of dS scratch.
  * Writes the clipped pairs of all bands, band after band, to pairs_out (capacity max_pairs; may be NULL
  * with max_pairs = 0 to count) and the band of each to band_out. Every visible (query, key) position of
- * the input pairs lies in exactly one clipped pair. n_bands_out = 0 means the problem cannot be banded
+ * the input pairs lies in exactly one clipped pair; a causal sequence whose listed pairs cover it whole is
+ * clipped as one pair, whatever chunks it was listed in. n_bands_out = 0 means the problem cannot be banded
  * with that scratch. Returns HYDRA_ERR_WORKSPACE_TOO_SMALL if max_pairs is too small (counts are still
  * written), HYDRA_ERR_INVALID_ARG on bad input.
  */
@@ -235,7 +242,8 @@ int32_t hydra_lse_merge_noalloc(const void* o_part, const float* lse_part, int64
  * Backward of the listed pairs, given the MERGED out and lse and the upstream gradient dout:
  *   D_i = <dout_i, out_i>;  P_ij = exp(s_ij - LSE_i);  dS_ij = P_ij (<dout_i, v_j> - D_i);
  *   dq_i = scale sum_j dS_ij k_j;  dk_j = scale sum_i dS_ij q_i;  dv_j = sum_i P_ij dout_i,
- * summed over all listed pairs that contain (i, j). The sums are accumulated on chip in fp32 and
+ * summed over all listed pairs that contain (i, j) (pairs that cover a whole causal sequence run as one: see
+ * hydra_workspace_bytes). The sums are accumulated on chip in fp32 and
  * written once as bf16, so results are deterministic. Rows of dq covered by no q chunk and rows of
  * dk/dv covered by no kv chunk are left untouched.
  * Requirement: any two pairs of a sequence have q ranges that are identical or disjoint, and kv
@@ -577,8 +585,8 @@ void hydra_set_plan_prefetch(int32_t on);
  * len (the default) lets the library choose: 1280 for heads of 192 with a K / V head per query head, 2048 with
  * shared K / V heads or heads of 128; 1920 and 3328 in causal calls of whole sequences with 20 or more 128-row q
  * tiles (times heads) per SM;
- * any length for a call with no more such tiles than the GPU has SMs, whose tiles the short-sequence kernel splits
- * between its two slots; and up to a quarter more than that limit (twice in smaller calls) where the pairs above it are
+ * any length for a call with no more such tiles than the GPU has SMs, or up to 2.5 times as many where that is expected to
+ * be faster, whose tiles the short-sequence kernel splits between its two slots; and up to a quarter more than that limit (twice in smaller calls) where the pairs above it are
  * too little work for a second launch. A limit set by the caller is kept to exactly. Takes effect with the next call.
  */
 void hydra_set_fwd_short_len(int32_t len);

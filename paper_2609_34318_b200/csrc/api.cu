@@ -201,7 +201,7 @@ bool join_chunks(Problem& pb, int32_t causal)
         if (a.seq != b.seq) return a.seq < b.seq;
         return a.q_start != b.q_start ? a.q_start < b.q_start : a.k_start < b.k_start;
     };
-    if (!std::is_sorted(by_q.begin(), by_q.end(), less)) std::sort(by_q.begin(), by_q.end(), less);     // (every call comes here)
+    if (!std::is_sorted(by_q.begin(), by_q.end(), less)) std::sort(by_q.begin(), by_q.end(), less);     // (in every call)
     std::vector<hydra_pair_t> joined;
     bool any = false;
     for (size_t i = 0, j = 0; i < by_q.size(); i = j) {
@@ -885,9 +885,10 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
     // keys of a tile, whatever their number (deal_shared_tiles; the CTA-pair kernel would leave SMs idle): always with no more
     // tiles than SMs, in calls of more where the queue is expected to take longer than the tiles dealt out. A step takes 0.93
     // us in a slot whose neighbour idles, 1.25 to 1.4 beside a busy one; on CTA pairs a step's share of an SM is 0.5 to 0.6.
-    // Forward in passes one after another, 16 heads of 192 unless said, queue / shared, us: 1300 tokens 29.1 / 19.9, 2048 40.3 /
-    // 29.6, 4096, 8 heads 71.0 / 48.5, 8192, 4 heads 133 / 96, 4820 log-normal ones, 8 heads 41.5 / 33.7, 8192, 4 heads 53.0 /
-    // 39.4; beyond the line 3000 60.1 / 63.8, 4096 86.9 / 100, 2048, 32 heads 61.0 / 66.2, ten sequences of 410 34.1 / 40.8.
+    // Forward in passes one after another, 16 heads of 192 unless said, queue / shared, us: one sequence of 1300 tokens 28.2 /
+    // 19.8, of 2048 39.1 / 29.4, of 4096, 8 heads 68.1 / 51.4, of 8192, 4 heads 126 / 94; 4820 tokens in five sequences of 341 to
+    // 2078, 8 heads 39.9 / 33.4; 8192 in seven of 341 to 2908, 4 heads 50.6 / 38.9; beyond the line one of 3000 60.1 / 63.8, of
+    // 4096 86.9 / 100, of 2048, 32 heads 61.0 / 66.2, ten of 410 34.1 / 40.8.
     // (A limit set by the caller is kept to.)
     // (A work item counts its steps in 16 bits: more keys than two items hold stay with the CTA-pair kernel.)
     constexpr int64_t kMostKeys = int64_t{UINT16_MAX} * FWD_SHORT_KEYS;
@@ -1061,7 +1062,8 @@ void build_fwd(const Problem& pb, int causal, Plan& plan, std::vector<uint8_t>& 
         auto entry = [&](const SharedTile& t) {
             return GroupEntry{t.q0, t.steps, std::min(TILE, runs[t.run].all.q_len - t.q0), t.steps, t.run};
         };
-        std::vector<FwdShortItem> table(static_cast<size_t>(deal.rounds) * 2 * deal.grid);      // (an item of no rows and no steps does nothing)
+        // (an item of no rows and no steps does nothing)
+        std::vector<FwdShortItem> table(static_cast<size_t>(deal.rounds) * 2 * deal.grid);
         for (const DealtTile& t : deal.tiles) {
             const SharedTile& one = tiles[t.first];
             FwdShortItem it = make_short(one.head, entry(one)), other{};
@@ -1203,7 +1205,7 @@ bool key_tiles_halved(const Problem& pb, int causal)
 // every number of heads that divides the group (longest items first, as the kernel's list has them; a unit is a 64-row
 // sub-tile, about 1 us). Step in passes one after another, one head per item / as chosen here: 32768 tokens of 64 to 512,
 // 32 heads of 128 over 8, 1245 / 965 us; log-normal lengths, 8192 tokens, 32 heads over 8, 854 / 776, 16384 tokens, 16 over
-// 4, 1100 / 1038, 32768 tokens, 16 heads of 128 over 2, 1861 / 1832 (1, 2, 4, 8 heads per item: key side 959, 923, 908, 932
+// 4, 1100 / 1038, 32768 tokens, 16 heads of 128 over 2, 1886 / 1852 (1, 2, 4, 8 heads per item: key side 959, 923, 908, 932
 // us, and the cast 23 us less with all 8).
 int32_t heads_per_key_item(const std::vector<std::vector<GroupEntry>>& groups, const Problem& pb, int workers)
 {
@@ -1451,8 +1453,8 @@ struct KernelSet {
     int (*fwd_max_clusters)();
     cudaError_t (*launch_fwd)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const FwdParams&, int,
                               cudaStream_t);
-    cudaError_t (*launch_fwd_short)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const FwdParams&, const FwdSeg*, uint64_t, bool, int,
-                                    cudaStream_t);
+    cudaError_t (*launch_fwd_short)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const FwdParams&,
+                                    const FwdSeg*, uint64_t, bool, int, cudaStream_t);
     cudaError_t (*launch_bwd_dq)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const CUtensorMap&,
                                  const BwdParams&, int, cudaStream_t);
     cudaError_t (*launch_bwd_dq_from_ds)(const CUtensorMap&, const BwdParams&, int, cudaStream_t);
@@ -1976,7 +1978,9 @@ int32_t fwd_core(Problem& pb, const void* q, const void* k, const void* v, int32
         CUtensorMap mv_sub;
         if (make_map(&mv_sub, v, pb.Tk, n_kv_heads, D_V, FWD_SHORT_KEYS)) return HYDRA_ERR_CUDA;
         ScopedKernelTimer timer(K_FWD, stream);
-        if (ks->launch_fwd_short(mq, mk, mv_sub, fp, plan->n_segs ? lease.at<FwdSeg>(plan->off_segs) : nullptr, call_tag, plan->halves != 0, short_grid, stream) != cudaSuccess) return HYDRA_ERR_CUDA;
+        const FwdSeg* segs = plan->n_segs ? lease.at<FwdSeg>(plan->off_segs) : nullptr;
+        if (ks->launch_fwd_short(mq, mk, mv_sub, fp, segs, call_tag, plan->halves != 0, short_grid, stream) != cudaSuccess)
+            return HYDRA_ERR_CUDA;
         g_launches += 1;
     }
     lease.release();                                   // the tables have their reader on record
@@ -2073,8 +2077,8 @@ struct KvSums {
 // K / V head (null: the outputs need no such sums). With `first` false the status block keeps its flags and only the
 // work-queue counters are cleared. `halves_of_call` is key_tiles_halved of the whole call, -1 if `pb` is all of it.
 int32_t bwd_run(const Problem& pb, int32_t n_kv_heads, int32_t causal, float softmax_scale, const BwdTensors& t,
-                KvSums* sums, bool accumulate_dq, bool accumulate_dkv, void* workspace, uint8_t* ds, size_t ds_room, uint64_t ds_limit, bool first,
-                int halves_of_call, int sms, cudaStream_t stream)
+                KvSums* sums, bool accumulate_dq, bool accumulate_dkv, void* workspace, uint8_t* ds, size_t ds_room,
+                uint64_t ds_limit, bool first, int halves_of_call, int sms, cudaStream_t stream)
 {
     const int32_t n_heads = pb.h;
     const KernelSet* ks = kernel_set(pb.dqk, D_V);

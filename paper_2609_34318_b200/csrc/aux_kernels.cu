@@ -602,9 +602,10 @@ cudaError_t launch_merge(const MergeParams& p, cudaStream_t stream)
     // chunk pairs of about 200 tokens, 4 heads 131 -> 127.5 us with their forward, 72 pairs, 16 heads 49.4 -> 47.3, one
     // rank's ring step of 64K tokens 5.54 -> 5.44 ms, 65536 tokens of short sequences cut in two 3.05 -> 3.015.
     const bool wide = ((reinterpret_cast<uintptr_t>(p.o_part) | reinterpret_cast<uintptr_t>(p.out)) & 31u) == 0;
-    // An item (eight rows, all heads) is several passes of its block, each a round trip to memory behind the other: with
-    // fewer items than resident blocks as many blocks share one as fit at once. With its launch, one block per item / shared:
-    // 363 tokens, 16 heads, ring of 4 14.6 / 8.6 us, 1728 tokens, 32 heads, ring of 2 19.3 / 14.9, 1313 16.0 / 12.8.
+    // An item (eight rows, all heads) is several passes of its block, each a round trip to memory behind the other: with fewer
+    // items than four blocks per SM, what most instances hold at once (the streaming 32-byte ones three, the 16-byte ones of two
+    // partials six), up to that many blocks share them. With its launch, one block per item / shared: 363 tokens, 16 heads, ring
+    // of 4 14.6 / 8.6 us, 1728 tokens, 32 heads, ring of 2 19.3 / 14.9, 1313 16.0 / 12.8.
     constexpr int kResident = 148 * 4;
     const int passes = (MERGE_ROWS * p.h + (wide ? 2 : 1) * kUnitsPerPass - 1) / ((wide ? 2 : 1) * kUnitsPerPass);
     MergeParams shared = p;
